@@ -5,35 +5,69 @@
 
 namespace gabp {
 
-// IEEE division, kept out of line so that the common path of rcp64 does not
+// IEEE division, kept out of line so that the common paths of div64 and rcp64 do not
 // carry its instructions.
-static __device__ __noinline__ double rcp64_slow(double d) { return 1.0 / d; }
+static __device__ __noinline__ double div64_slow(double a, double d) { return a / d; }
 
-// Reciprocal of a double by one step of Chebyshev's third-order iteration for 1/d:
-// with e = 1 - d y, y <- y (1 + e + e^2) = y + y (e + e^2).  If y = (1 - eps)/d, then
-// e = eps and the step gives (1 - eps^3)/d: the relative error is cubed (Newton's
-// y + y e would only square it).  The seed is the single-precision hardware
-// approximation (PTX rcp.approx.ftz.f32) of d rounded toward zero to 20 mantissa
-// bits, relative error below 2^-19, so one step leaves ~2^-57 plus the final
-// rounding: three FMAs on the (narrow) FP64 pipe instead of the four of two Newton
-// steps.  The float operand and the double seed are assembled from the IEEE-754
-// fields with integer operations, which keeps the conversions off the FP64 pipe.
-// Exponents outside [-120, 120] (and 0, subnormals, inf, NaN) take the IEEE division.
-__device__ __forceinline__ double rcp64(double d) {
-  const unsigned long long u = (unsigned long long)__double_as_longlong(d);
-  const unsigned hi = (unsigned)(u >> 32);
-  const int e = (int)((hi >> 20) & 0x7ffu) - 1023;
-  const unsigned fb = (hi & 0x80000000u) | ((unsigned)(e + 127) << 23) | ((hi & 0xfffffu) << 3);
+// Division off the FP64 pipe.  GB300 retires two FP64 operations per SM and clock (a warp's
+// FP64 instruction holds its scheduler's unit for 64 cycles) and bounds the FP64 rounds with
+// them, while the integer units stand idle: a quotient formed with integer instructions
+// (about 45 a warp) replaces four FP64 ones (three of a reciprocal iteration, one product).
+//
+// Reciprocal of d's 53-bit significand m in [1, 2): seed y (24 bits, PTX rcp.approx.ftz.f32 of
+// m cut to 24 bits, so |m y - 1| < 2^-21.5 with a margin), then the geometric series
+//   1 / m = y / (1 + s) = y (1 - s + s^2 - ...),   s = m y - 1  (exact, s^3 < 2^-64),
+// in fixed point.  Units: y 2^-24, m 2^-52, so m y wraps modulo 2^64 at 2^76 = 1 and its low
+// 64 bits, read as signed, are s itself.  Returns 1 / m in units of 2^-63 (error a few units).
+__device__ __forceinline__ unsigned long long rcp_sig64(unsigned dh, unsigned dl) {
   float yf;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(yf) : "f"(__uint_as_float(fb)));
-  const unsigned yb = __float_as_uint(yf);
-  const int ey = (int)((yb >> 23) & 0xffu) - 127;
-  const unsigned yhi = (yb & 0x80000000u) | ((unsigned)(ey + 1023) << 20) | ((yb >> 3) & 0xfffffu);
-  double y = __hiloint2double((int)yhi, (int)((yb & 7u) << 29));
-  const double r = fma(-d, y, 1.0);  // e
-  y = fma(y, fma(r, r, r), y);       // y (1 + e + e^2)
-  if (e < -120 || e > 120) y = rcp64_slow(d);
-  return y;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(yf) : "f"(__uint_as_float(0x3f800000u | ((dh & 0xfffffu) << 3) | (dl >> 29))));
+  const unsigned y = __float_as_uint(yf) - 0x3e800000u;  // y in (2^23, 2^24]: [0.5, 1] in units of 2^-24
+  const unsigned mh = (dh & 0xfffffu) | 0x100000u;
+  const long long s = (long long)((unsigned long long)dl * y + ((unsigned long long)(mh * y) << 32));
+  const int s32 = (int)(s >> 24);                                    // s in units of 2^-52
+  const long long t = s + (long long)__mulhi(s32, s32) * -16;        // s - s^2, units of 2^-76
+  const long long w = (long long)(int)(t >> 32) * (int)y + (long long)__umulhi((unsigned)t, y);  // y t, units of 2^-68
+  return ((unsigned long long)(y << 7) << 32) - (unsigned long long)(w >> 5);
+}
+
+// Exponent field of a high word, and whether quotients of two such operands are certain to be normal
+// (zero, subnormal, inf, NaN and the outer exponents take the IEEE division).
+__device__ __forceinline__ int exp_field64(unsigned hi) { return (int)((hi >> 20) & 0x7ffu); }
+__device__ __forceinline__ bool plain_exp64(int e) { return (unsigned)(e - 523) <= 1000u; }
+
+// a / d within 0.51 units in the last place (IEEE division's 0.50): the significands' 64-bit
+// product a (1 / d), normalised, rounded to 53 bits and put together with the exponent.
+__device__ __forceinline__ double div64(double a, double d) {
+  unsigned ah, al, dh, dl;
+  asm("mov.b64 {%0, %1}, %2;" : "=r"(al), "=r"(ah) : "d"(a));
+  asm("mov.b64 {%0, %1}, %2;" : "=r"(dl), "=r"(dh) : "d"(d));
+  const unsigned long long z = rcp_sig64(dh, dl);
+  const unsigned mh = ((ah & 0xfffffu) | 0x100000u) << 11 | (al >> 21), ml = al << 11;  // units of 2^-63
+  const unsigned zh = (unsigned)(z >> 32), zl = (unsigned)z;
+  const unsigned long long q =
+      (unsigned long long)mh * zh + ((unsigned long long)__umulhi(mh, zl) + __umulhi(ml, zh));  // units of 2^-62
+  const int sh = (unsigned)(q >> 32) < 0x40000000u ? 1 : 0;  // quotient of the significands below 1
+  const unsigned long long r = (q + (unsigned)(512 >> sh)) >> (10 - sh);
+  const int ea = exp_field64(ah), ed = exp_field64(dh);
+  const unsigned rh = ((unsigned)(r >> 32) + ((unsigned)(ea - ed + 1022 - sh) << 20)) ^ ((ah ^ dh) & 0x80000000u);
+  double v;
+  asm("mov.b64 %0, {%1, %2};" : "=d"(v) : "r"((unsigned)r), "r"(rh));
+  if (!plain_exp64(ea) || !plain_exp64(ed)) v = div64_slow(a, d);
+  return v;
+}
+
+// 1 / d in the same way (no product).
+__device__ __forceinline__ double rcp64(double d) {
+  unsigned dh, dl;
+  asm("mov.b64 {%0, %1}, %2;" : "=r"(dl), "=r"(dh) : "d"(d));
+  const unsigned long long r = (rcp_sig64(dh, dl) + 512u) >> 10;  // 2^52 .. 2^53 (1 / 1 carries into the exponent)
+  const int ed = exp_field64(dh);
+  const unsigned rh = ((unsigned)(r >> 32) + ((unsigned)(2044 - ed) << 20)) ^ (dh & 0x80000000u);
+  double v;
+  asm("mov.b64 %0, {%1, %2};" : "=d"(v) : "r"((unsigned)r), "r"(rh));
+  if (!plain_exp64(ed)) v = div64_slow(1.0, d);
+  return v;
 }
 
 // d == +0 or -0, tested on the bit pattern.  The two 32-bit halves come out of an

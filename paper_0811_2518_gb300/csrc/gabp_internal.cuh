@@ -4,8 +4,8 @@
 //   off-diagonal CSR in receiver layout: row i, slot e in [rp[i], rp[i+1]) with
 //   k = ci[e] holds the message k -> i.  av[e] = A_ik, ad[i] = A_ii.
 //   rev[e] is the slot of the reverse edge (row k, column i).
-//   FP64 path: M64[2][E] double2 {P, h} (h = P * mu, the information form of the
-//   mean message), N64[2][n] 32-byte node records {P~, h~, x, -}.
+//   FP64 path: M64[2][E] double2 {c, v} (the message P = -A c, h = P * mu = -c v, the
+//   information form), N64[2][n] 32-byte node records {P~, h~, x, -}.
 //   FP32 path: precision chains MP[2][E] float, coefficient pairs CF[E] float2,
 //   mean chains H[2][E][R] float, node rings.
 #pragma once
@@ -43,6 +43,8 @@ struct DevCtl {
   int max_iter;
   int check_from;    // first round whose iterate may be accepted (1 for GaBP)
   int stable;        // consecutive rounds with a stationary precision set
+  int cold;          // FP64 rounds: zero starting messages that are not in the store
+  int pad_;
   double bb;         // ||b||^2
   double tol2bb;     // tol^2 ||b||^2
   double rr;         // squared residual (or squared update) of the latest checked iterate
@@ -102,10 +104,10 @@ __device__ __forceinline__ void freeze_step(DevCtl *ctl, int fs, int t, double m
   }
 }
 
-// More than 16 units in the last place apart (any NaN, a sign change or a zero
+// More than `bar` units in the last place apart (any NaN, a sign change or a zero
 // against a non-zero counts as apart; two equal bit patterns do not).
-__device__ __forceinline__ bool ulp_apart(double u, double v) {
-  return (unsigned long long)(__double_as_longlong(u) - __double_as_longlong(v) + 16) > 32ull;
+__device__ __forceinline__ bool ulp_apart(double u, double v, unsigned bar = 16) {
+  return (unsigned long long)(__double_as_longlong(u) - __double_as_longlong(v) + bar) > 2ull * bar;
 }
 
 struct Graph {
@@ -130,6 +132,7 @@ struct Sell64 {
   bool vals_ok = false;  // sav matches the graph's values (cleared by gabp_set_values)
   int ns = 0;            // slices
   int Es = 0;            // positions (slots + padding)
+  int64_t far = 0;       // slots whose reverse edge lies far away in the message store
   int *srow = nullptr;   // [ns * 32] row of each slice lane, -1 past n
   int *sp = nullptr;     // [ns + 1] first position of each slice
   int *sci = nullptr;    // [Es] sender, -1 for padding
@@ -139,13 +142,13 @@ struct Sell64 {
 };
 
 struct Work64 {
-  double2 *M[2] = {nullptr, nullptr};  // messages at the sliced positions
+  double2 *M[2] = {nullptr, nullptr};  // messages {c, v} at the sliced positions (P = -A c, h = -c v)
   NodeRec64 *N[2] = {nullptr, nullptr};
   bool valid = false;   // a solve has completed; messages/records are readable
   int result_round = 0;
   Sell64 sl;
   unsigned *bar = nullptr;  // grid barrier of the cooperative rounds: arrivals, generation, error flag
-  double *C = nullptr;      // [Es] frozen coefficients c = -A / (P~ - P) (options.freeze_precisions)
+  double *C = nullptr;      // [Es] frozen coefficients c = A / (P~ - P) (options.freeze_precisions)
 };
 
 struct Work32 {

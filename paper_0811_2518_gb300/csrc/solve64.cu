@@ -4,7 +4,13 @@
 //   P~_i = A_ii + sum_{k in N(i)} P_ki,    h~_i = b_i + sum_{k in N(i)} h_ki,
 //   P_ij = -A_ij^2 / (P~_i - P_ji),        h_ij = P_ij mu_ij = -A_ij (h~_i - h_ji) / (P~_i - P_ji),
 //   x_i  = h~_i / P~_i                     (marginal mean, Algorithm 1 step 4).
-// Messages are kept in information form (P, h = P mu); mu_ij of the paper is h_ij / P_ij.
+// Messages are in information form (P, h = P mu); mu_ij of the paper is h_ij / P_ij.  A slot
+// stores message k -> i as the pair {c, v} it is a product of: the cavity mean aggregate
+// v = h~_k - h_ik and c = A_ik / (P~_k - P_ik), so that
+//   P_ki = -A_ik c,    h_ki = -c v.
+// Every use of a message is then one fused multiply-add: the sums P~ -= A c, h~ -= c v and the
+// cavities P~_k + A c, h~_k + c v, five FP64 instructions per slot with the residual's (eleven
+// with stored products P, h and a reciprocal on the FP64 pipe), and no product is rounded.
 //
 // Round t of the parallel schedule reads round t-1 only (two message stores that
 // swap roles, paper Sec. "The Gaussian BP Algorithm", scheduling paragraph):
@@ -15,12 +21,17 @@
 // gathered anyway, so the residual of round t-1's iterate costs one FMA per slot;
 // the stop rule therefore decides about x^{(t-1)} during round t.
 //
+// Two forms of a round give the same bits, since both evaluate one formula on the same values:
+//   gather     the reverse message i -> k of round t-1 is read from row k's slot;
+//   recompute  it is formed again from what row i held at round t-2, its own record and the slot's
+//              own in-message (the store of round t, not yet overwritten): two more FP64 instructions
+//              and a division on the integer units, and no random access to the message store.
+//
 // Layout (Sell64): rows are ordered by degree inside windows of kSellWindow rows
 // and cut into slices of 32; one warp runs a slice, one lane a row, and slot j of
-// the slice's rows is one contiguous 32-wide line.  The round is bound by the FP64
-// pipe (a Newton reciprocal and ~12 FP64 operations per slot on GB300's narrow FP64
-// units), so what matters is that every lane of every FP64 instruction does work:
-// rows of equal degree share a warp, and the row epilogue runs on all 32 lanes.
+// the slice's rows is one contiguous 32-wide line.  A warp's FP64 instruction costs
+// the same however many of its lanes work, so every lane of it should: rows of equal
+// degree share a warp, and the row epilogue runs on all 32 lanes.
 #include "gabp_internal.cuh"
 #include "devutil.cuh"
 #include "cluster.cuh"
@@ -28,23 +39,20 @@
 #include <cooperative_groups.h>
 
 #include <algorithm>
+#include <type_traits>
 #include <vector>
 
 namespace gabp {
 
 constexpr int kSellWindow = 4096;  // rows sorted by degree within windows of this many (a multiple of 32)
 
-// Slots per lane whose loads the FP64 node round issues together, and the blocks per SM its
-// register budget is sized for (__launch_bounds__).  Measured on the 2^20 random graph: 2 slots and
-// 3 blocks (24 warps per SM) 0.558 ms per round; 4 blocks (64 registers) 0.589; 2 blocks 0.73;
-// 1 slot with 4 blocks 0.633; 4 slots with 2 blocks 0.678.
-#ifndef GABP_K64_UNROLL
-#define GABP_K64_UNROLL 2
-#endif
-#ifndef GABP_K64_MINB
-#define GABP_K64_MINB 3
-#endif
-constexpr int kU64 = GABP_K64_UNROLL;
+// Slots per lane whose loads a round issues together, and the blocks per SM its register budget
+// is sized for (__launch_bounds__).  Recompute form on the 2^20 random graph of degree 16: 2 slots and
+// 4 blocks (64 registers, 32 warps an SM) 276 us per round; 3 blocks 286; 1 slot with 4 blocks 284, with
+// 5 blocks 282.  Gather form on the 128^3 grid: 3 slots and 4 blocks 164 us per round, 2 slots 169,
+// 3 slots with 3 or 5 blocks 170 / 185.
+constexpr int kURec = 2, kUGather = 3, kUCoop = 2, kU64 = 2;
+constexpr int kMinBlocks64 = 4;
 
 struct Args64 {
   int n;
@@ -63,6 +71,7 @@ struct Args64 {
   double *C;   // [Es] frozen coefficients (freeze != 0)
   int freeze;  // options.freeze_precisions on a plain node solve
   int wide;    // plain node rounds of a matrix of long rows: k64_wide
+  int rec;     // plain node rounds with a launch each: the recompute form
 };
 
 // Warp / lane of the calling thread and the number of warps in the grid.
@@ -72,6 +81,17 @@ struct WarpPos {
 __device__ __forceinline__ WarpPos warp_pos() {
   return WarpPos{(int)(threadIdx.x & 31), (int)((blockIdx.x * kBlock + threadIdx.x) >> 5),
                  (int)((gridDim.x * kBlock) >> 5)};
+}
+
+// The slice a warp takes in its pass m over the grid (ns or more: none).  Inside a window of kSellWindow
+// rows the slices get narrower (rows sorted by degree), and a fixed stride would hand a warp slices of
+// like width in every pass (28 % of the round with idle warps on the 2^20 random graph); turning each
+// pass by the golden section of a window's 128 slices spreads every warp's slices over the window:
+// 347 -> 286 us per round there, unchanged on grids.
+__device__ __forceinline__ int pass_slice(const WarpPos &w, int m) {
+  constexpr int kSlices = kSellWindow / 32, kGolden = 79;  // 128 / 1.618
+  const int turn = (kGolden + kSlices - w.nwarps % kSlices) % kSlices;
+  return m * w.nwarps + (w.warp + m * turn) % w.nwarps;
 }
 
 // Round bookkeeping shared by the FP64 round kernels: this round checked
@@ -151,10 +171,6 @@ __device__ __forceinline__ void decide64(DevCtl *ctl, int t, double rr, double b
 template <bool COOP> __device__ __forceinline__ int ld_idx(const int *p) { return COOP ? __ldg(p) : __ldcs(p); }
 template <bool COOP> __device__ __forceinline__ double ld_val(const double *p) { return COOP ? __ldg(p) : __ldcs(p); }
 template <bool COOP> __device__ __forceinline__ double2 ld_msg(const double2 *p) { return COOP ? __ldcg(p) : __ldcs(p); }
-template <bool COOP> __device__ __forceinline__ double ld_msgh(const double2 *p) {
-  const double *q = reinterpret_cast<const double *>(p) + 1;
-  return COOP ? __ldcg(q) : __ldcs(q);
-}
 template <bool COOP> __device__ __forceinline__ NodeRec64 ld_rec(const NodeRec64 *p) {
   if (!COOP) return *p;
   const double2 *r = reinterpret_cast<const double2 *>(p);
@@ -162,70 +178,101 @@ template <bool COOP> __device__ __forceinline__ NodeRec64 ld_rec(const NodeRec64
   return NodeRec64{q.x, q.y, q1.x, q1.y};
 }
 
+// Message k -> i of round t as {c, v} from node k's record at t-1 and the reverse message rv
+// (i -> k at t-1).  bad: a cavity precision P_{k\i} of exactly 0.
+__device__ __forceinline__ double2 message64(double A, const NodeRec64 &nk, const double2 &rv, int &bad) {
+  const double den = fma(A, rv.x, nk.P);  // cavity precision P_{k\i}
+  bad |= is_zero64(den);
+  return make_double2(div64(A, den), fma(rv.x, rv.y, nk.h));
+}
+// The reverse message i -> k of round t-1 by the same formula, from row i's aggregates at t-2
+// (P2, h2) and the slot's own in-message at t-2 (recompute form; its cavity was checked by row k).
+__device__ __forceinline__ double2 reverse64(double A, double P2, double h2, const double2 &m2) {
+  return make_double2(div64(A, fma(A, m2.x, P2)), fma(m2.x, m2.y, h2));
+}
+
+// Where round t takes its reverse messages from.  A cold run starts with zero messages that are
+// never stored: round 1 has no reverse message (kZero), and in the recompute form round 2's own
+// in-messages at t-2 are zero (kRecZero).  Round 1 of a warm run gathers in either form.
+enum RevFrom { kGather, kRec, kZero, kRecZero };
+template <bool REC>
+__device__ __forceinline__ RevFrom round_source(int t, int cold) {
+  if (t == 1) return cold ? kZero : kGather;
+  return !REC ? kGather : t == 2 && cold ? kRecZero : kRec;
+}
+
 // One slice of a plain round (node variant, no acceleration), a lane per row.
 // MODE 0: Algorithm 2's round.  MODE 1 (freeze screen): the same, flagging rows whose
 // P~_i moved since the previous round.  MODE 2 (freeze verify): the same, flagging
 // precision messages that moved since the previous round (the slot's own previous
-// message) and storing each slot's coefficient c = -A / (P~_k - P_ik) and each row's
-// 1/P~ (the record's spare slot).  MODE 3 (frozen precisions): only the mean
-// messages, h_ki = c (h~_k - h_ik), with the stored coefficients; P~ and 1/P~
-// carried over.  All modes form x and the residual of the previous iterate as the
-// round kernels do.
-template <bool COOP, int MODE>
+// message; P_ki = -A c moves as c does) and storing each slot's coefficient
+// c = A / (P~_k - P_ik) and each row's 1/P~ (the record's spare slot).  The first
+// verification of a solve takes a bar of 8 units in the last place, which tells a message
+// that still converges from one that rounds; where the stagnant messages jitter by more
+// (3D grids: up to 16), the later ones, after longer screens, take the screen's 16.  MODE 3 (frozen precisions): only the mean
+// messages, h_ki = -c v, with the stored coefficients; P~ and 1/P~ carried over.
+// All modes form x and the residual of the previous iterate as the round kernels do.
+// FROM: where the reverse messages come from (round_source), a template parameter because a
+// branch on it between a slot's loads would keep them from being issued together.  In the
+// recompute form Nout and Mout hold round t-2 until they are written.
+template <bool COOP, int MODE, RevFrom FROM>
 __device__ __forceinline__ void plain_slice(const Args64 &a, int sl, int lane, const double *__restrict__ b,
                                             const double2 *__restrict__ Min, double2 *__restrict__ Mout,
                                             const NodeRec64 *__restrict__ Nin, NodeRec64 *__restrict__ Nout,
                                             double &rr, int &bad, int &moving) {
+  constexpr bool REC = FROM == kRec || FROM == kRecZero;
+  constexpr int U = COOP ? kUCoop : REC ? kURec : kUGather;
   const int i = COOP ? __ldg(a.srow + sl * 32 + lane) : a.srow[sl * 32 + lane];
   const int q0 = COOP ? __ldg(a.sp + sl) : a.sp[sl];
   const int p0 = q0 + lane, wd = ((COOP ? __ldg(a.sp + sl + 1) : a.sp[sl + 1]) - q0) >> 5;
+  double P2 = 0.0, h2 = 0.0;
+  if (REC && i >= 0) {
+    const double2 q = *reinterpret_cast<const double2 *>(Nout + i);
+    P2 = q.x;
+    h2 = q.y;
+  }
+  const unsigned bar = MODE == 2 ? (__ldcg(&a.ctl->pfail) ? 16 : 8) : 0;
   double accP = 0.0, acch = 0.0, accr = 0.0;
-  for (int j = 0; j < wd; j += kU64) {
-    int k[kU64];
-    double A[kU64], c[kU64], rh[kU64];
-    double2 rv[kU64];
-    NodeRec64 nk[kU64];
+  for (int j = 0; j < wd; j += U) {
+    int k[U];
+    double A[U], c[U];
+    double2 rv[U];
+    NodeRec64 nk[U];
 #pragma unroll
-    for (int u = 0; u < kU64; ++u) {
+    for (int u = 0; u < U; ++u) {
       const int pos = p0 + 32 * (j + u);
       k[u] = j + u < wd ? ld_idx<COOP>(a.sci + pos) : -1;
       if (k[u] >= 0) {
         A[u] = ld_val<COOP>(a.sav + pos);
-        const int rp = ld_idx<COOP>(a.srev + pos);
-        if (MODE == 3) {
-          c[u] = COOP ? __ldcg(a.C + pos) : __ldcs(a.C + pos);  // written by this launch when COOP
-          rh[u] = ld_msgh<COOP>(Min + rp);  // mean message i -> k of round t-1
-        } else {
-          rv[u] = ld_msg<COOP>(Min + rp);   // message i -> k of round t-1
-          if (MODE == 2) rh[u] = ld_msg<COOP>(Min + pos).x;  // this slot's precision message at t-1
-        }
+        if (FROM == kGather) rv[u] = ld_msg<COOP>(Min + ld_idx<COOP>(a.srev + pos));  // i -> k of round t-1
+        else if (FROM == kRec) rv[u] = __ldcs(Mout + pos);  // the own in-message at t-2
+        else rv[u] = make_double2(0.0, 0.0);
+        if (MODE == 3) c[u] = COOP ? __ldcg(a.C + pos) : __ldcs(a.C + pos);  // written by this launch when COOP
+        if (MODE == 2) c[u] = ld_msg<COOP>(Min + pos).x;  // this slot's coefficient at t-1
       }
     }
 #pragma unroll
-    for (int u = 0; u < kU64; ++u)
+    for (int u = 0; u < U; ++u)
       if (k[u] >= 0) nk[u] = ld_rec<COOP>(Nin + k[u]);  // node k at round t-1
 #pragma unroll
-    for (int u = 0; u < kU64; ++u) {
+    for (int u = 0; u < U; ++u) {
       if (k[u] < 0) continue;
       const int pos = p0 + 32 * (j + u);
       if (MODE == 3) {
-        const double hn = __dmul_rn(c[u], nk[u].h - rh[u]);
+        const double v = fma(rv[u].x, rv[u].y, nk[u].h);
         double *dst = reinterpret_cast<double *>(Mout + pos) + 1;
-        if (COOP) *dst = hn; else __stcs(dst, hn);
-        acch = __dadd_rn(acch, hn);
+        if (COOP) *dst = v; else __stcs(dst, v);
+        acch = fma(-c[u], v, acch);
       } else {
-        const double den = nk[u].P - rv[u].x;  // cavity precision P_{k\i}
-        bad |= is_zero64(den);
-        const double cin = -A[u] * rcp64(den);
-        // the aggregates add the stored (rounded) messages, as Algorithm 2 sums them
-        const double2 m = make_double2(__dmul_rn(cin, A[u]), __dmul_rn(cin, nk[u].h - rv[u].y));
+        if (REC) rv[u] = reverse64(A[u], P2, h2, rv[u]);
+        const double2 m = message64(A[u], nk[u], rv[u], bad);
         if (COOP) Mout[pos] = m; else __stcs(Mout + pos, m);
         if (MODE == 2) {
-          moving |= ulp_apart(m.x, rh[u]);
-          a.C[pos] = cin;
+          moving |= ulp_apart(m.x, c[u], bar);
+          a.C[pos] = m.x;
         }
-        accP = __dadd_rn(accP, m.x);
-        acch = __dadd_rn(acch, m.y);
+        accP = fma(-A[u], m.x, accP);
+        acch = fma(-m.x, m.y, acch);
       }
       accr = fma(A[u], nk[u].x, accr);
     }
@@ -240,8 +287,8 @@ __device__ __forceinline__ void plain_slice(const Args64 &a, int sl, int lane, c
       const double P = d + accP, h = bi + acch;
       bad |= is_zero64(P);
       if (MODE == 1) moving |= ulp_apart(P, own.P);
-      const double ip = rcp64(P);
-      Nout[i] = NodeRec64{P, h, h * ip, MODE == 2 ? ip : h * ip};
+      const double x = div64(h, P);
+      Nout[i] = NodeRec64{P, h, x, MODE == 2 ? rcp64(P) : x};
     }
     const double r = bi - fma(d, own.x, accr);
     rr = fma(r, r, rr);
@@ -252,7 +299,8 @@ __device__ __forceinline__ void plain_slice(const Args64 &a, int sl, int lane, c
 // Warm start (warm = 1): round 0 takes the messages already in M0 (a previous
 // solve's, or imported ones) and forms the aggregates from them with this b:
 // any starting messages lead to the same fixed point when the iteration converges.
-__global__ void __launch_bounds__(kBlock) k64_init(Args64 a, double tol, int max_iter, int warm) {
+// cold = 1: M0 was not cleared, and the rounds take zero starting messages without reading it.
+__global__ void __launch_bounds__(kBlock) k64_init(Args64 a, double tol, int max_iter, int warm, int cold) {
   const double *b = a.ctl->b;
   const WarpPos w = warp_pos();
   double bb = 0.0;
@@ -266,8 +314,8 @@ __global__ void __launch_bounds__(kBlock) k64_init(Args64 a, double tol, int max
         const int pos = p0 + 32 * j + w.lane;
         if (a.sci[pos] < 0) break;
         const double2 m = a.M0[pos];
-        P += m.x;
-        h += m.y;
+        P = fma(-a.sav[pos], m.x, P);
+        h = fma(-m.x, m.y, h);
       }
     }
     const double x0 = h / P;
@@ -285,6 +333,7 @@ __global__ void __launch_bounds__(kBlock) k64_init(Args64 a, double tol, int max
     c->max_iter = max_iter;
     c->check_from = 1;
     c->stable = 0;
+    c->cold = cold;
     c->edge_bad = 0;
     c->rr = tot[0];
     c->arrive = 0;
@@ -320,15 +369,26 @@ enum { ACC_NONE = 0, ACC_AITKEN = 1, ACC_STEFFENSEN = 2 };
 
 // One plain round over this kernel's slices in mode MODE of plain_slice, then the
 // block sums and, in the last block, the freeze state's step and the decision.
-template <int MODE>
+template <int MODE, bool REC>
 __device__ __forceinline__ void plain_round(const Args64 &a, DevCtl *ctl, int t, const double *__restrict__ b,
                                             const double2 *__restrict__ Min, double2 *__restrict__ Mout,
                                             const NodeRec64 *__restrict__ Nin, NodeRec64 *__restrict__ Nout,
                                             const WarpPos &w) {
   double rr = 0.0;
   int bad = 0, moving = 0;
-  for (int sl = w.warp; sl < a.ns; sl += w.nwarps)
-    plain_slice<false, MODE>(a, sl, w.lane, b, Min, Mout, Nin, Nout, rr, bad, moving);
+  const RevFrom from = round_source<REC>(t, ctl->cold);
+  auto rows = [&](auto f) {
+    for (int m = 0; m * w.nwarps < a.ns; ++m) {
+      const int sl = pass_slice(w, m);
+      if (sl < a.ns)
+        plain_slice<false, MODE, decltype(f)::value>(a, sl, w.lane, b, Min, Mout, Nin, Nout, rr, bad, moving);
+    }
+  };
+  // the freeze verifies after two screened rounds at the earliest: no starting messages in modes 2 and 3
+  if (REC && from == kRec) rows(std::integral_constant<RevFrom, REC ? kRec : kGather>());
+  else if (MODE >= 2 || from == kGather) rows(std::integral_constant<RevFrom, kGather>());
+  else if (from == kZero) rows(std::integral_constant<RevFrom, MODE >= 2 ? kGather : kZero>());
+  else rows(std::integral_constant<RevFrom, REC && MODE < 2 ? kRecZero : kGather>());
   constexpr int NV = MODE > 0 ? 3 : 2;  // the moving count only when the freeze is on
   double v[NV], tot[NV];
   int modes[NV];
@@ -358,6 +418,7 @@ __global__ void __launch_bounds__(kBlock) k64_wide(Args64 a) {
   const NodeRec64 *__restrict__ Nin = (t & 1) ? a.N0 : a.N1;
   NodeRec64 *__restrict__ Nout = (t & 1) ? a.N1 : a.N0;
   const WarpPos w = warp_pos();
+  const RevFrom from = round_source<true>(t, ctl->cold);
   double rr = 0.0;
   int bad = 0;
   for (int q = w.warp; q < a.ns * 32; q += w.nwarps) {
@@ -365,21 +426,23 @@ __global__ void __launch_bounds__(kBlock) k64_wide(Args64 a) {
     if (i < 0) continue;  // warp-uniform
     const int sl = q >> 5, r = q & 31;
     const int p0 = a.sp[sl] + r, wd = (a.sp[sl + 1] - a.sp[sl]) >> 5;
+    const double2 n2 = *reinterpret_cast<const double2 *>(Nout + i);  // the row's {P~, h~} at t-2
+    __syncwarp();  // read by every lane before lane 0 writes round t there
     double accP = 0.0, acch = 0.0, accr = 0.0;
     for (int j = w.lane; j < wd; j += 32) {
       const int pos = p0 + 32 * j;
       const int k = __ldcs(a.sci + pos);
       if (k < 0) continue;
       const double A = __ldcs(a.sav + pos);
-      const double2 rv = __ldcs(Min + __ldcs(a.srev + pos));  // message i -> k of round t-1
-      const NodeRec64 nk = Nin[k];                              // node k at round t-1
-      const double den = nk.P - rv.x;
-      bad |= is_zero64(den);
-      const double cin = -A * rcp64(den);
-      const double2 m = make_double2(__dmul_rn(cin, A), __dmul_rn(cin, nk.h - rv.y));
+      double2 rv = make_double2(0.0, 0.0);  // message i -> k of round t-1, recomputed from round 2 on
+      if (from == kGather) rv = __ldcs(Min + __ldcs(a.srev + pos));
+      else if (from == kRec) rv = __ldcs(Mout + pos);
+      if (from == kRec || from == kRecZero) rv = reverse64(A, n2.x, n2.y, rv);
+      const NodeRec64 nk = Nin[k];  // node k at round t-1
+      const double2 m = message64(A, nk, rv, bad);
       __stcs(Mout + pos, m);
-      accP = __dadd_rn(accP, m.x);
-      acch = __dadd_rn(acch, m.y);
+      accP = fma(-A, m.x, accP);
+      acch = fma(-m.x, m.y, acch);
       accr = fma(A, nk.x, accr);
     }
 #pragma unroll
@@ -393,8 +456,8 @@ __global__ void __launch_bounds__(kBlock) k64_wide(Args64 a) {
       const NodeRec64 own = Nin[i];
       const double P = d + accP, h = bi + acch;
       bad |= is_zero64(P);
-      const double ip = rcp64(P);
-      Nout[i] = NodeRec64{P, h, h * ip, h * ip};
+      const double x = div64(h, P);
+      Nout[i] = NodeRec64{P, h, x, x};
       const double rres = bi - fma(d, own.x, accr);
       rr = fma(rres, rres, rr);
     }
@@ -411,8 +474,8 @@ __global__ void __launch_bounds__(kBlock) k64_wide(Args64 a) {
 // a time, except that a failed verification returns it to 0: so one of the three
 // runs, or k64_frz<2> and then k64_frz<1> (two rounds; the round count and the stop
 // rule live on the device, so a launch slot may hold two rounds).
-template <int MODE>
-__global__ void __launch_bounds__(kBlock, GABP_K64_MINB) k64_frz(Args64 a) {
+template <int MODE, bool REC = false>
+__global__ void __launch_bounds__(kBlock, MODE == 2 ? 3 : kMinBlocks64) k64_frz(Args64 a) {
   DevCtl *ctl = a.ctl;
   if (ctl->done || ctl->fstate != MODE - 1) return;
   const int t = ctl->round + 1;
@@ -420,7 +483,7 @@ __global__ void __launch_bounds__(kBlock, GABP_K64_MINB) k64_frz(Args64 a) {
   double2 *__restrict__ Mout = (t & 1) ? a.M1 : a.M0;
   const NodeRec64 *__restrict__ Nin = (t & 1) ? a.N0 : a.N1;
   NodeRec64 *__restrict__ Nout = (t & 1) ? a.N1 : a.N0;
-  plain_round<MODE>(a, ctl, t, ctl->b, Min, Mout, Nin, Nout, warp_pos());
+  plain_round<MODE, REC>(a, ctl, t, ctl->b, Min, Mout, Nin, Nout, warp_pos());
 }
 
 // Fused node-centric round (GABP_VARIANT_NODE): a warp per slice, a lane per row.
@@ -432,8 +495,8 @@ __global__ void __launch_bounds__(kBlock, GABP_K64_MINB) k64_frz(Args64 a) {
 // keeps the cycle's starting iterate x_n in the spare slot; the second also sums
 // <d, D> and <D, D> (d = x_{n+2} - x_{n+1}, D = x_{n+2} - 2 x_{n+1} + x_n), whose
 // quotient, the scalar step lam, its last block stores for k64_steff.
-template <int ACC>
-__global__ void __launch_bounds__(kBlock, GABP_K64_MINB) k64_node(Args64 a) {
+template <int ACC, bool REC = false>
+__global__ void __launch_bounds__(kBlock, ACC ? 3 : kMinBlocks64) k64_node(Args64 a) {
   constexpr bool AIT = ACC == ACC_AITKEN;
   constexpr bool STF = ACC == ACC_STEFFENSEN;
   DevCtl *ctl = a.ctl;
@@ -446,7 +509,7 @@ __global__ void __launch_bounds__(kBlock, GABP_K64_MINB) k64_node(Args64 a) {
   NodeRec64 *__restrict__ Nout = (t & 1) ? a.N1 : a.N0;
   const WarpPos w = warp_pos();
   if (ACC == ACC_NONE) {
-    plain_round<0>(a, ctl, t, b, Min, Mout, Nin, Nout, w);
+    plain_round<0, REC>(a, ctl, t, b, Min, Mout, Nin, Nout, w);
     return;
   }
   double rr = 0.0, sdD = 0.0, sDD = 0.0;
@@ -478,15 +541,10 @@ __global__ void __launch_bounds__(kBlock, GABP_K64_MINB) k64_node(Args64 a) {
 #pragma unroll
       for (int u = 0; u < kU64; ++u) {
         if (k[u] >= 0) {
-          const double den = nk[u].P - rv[u].x;  // cavity precision P_{k\i}
-          bad |= is_zero64(den);
-          const double cin = -A[u] * rcp64(den);
-          // the aggregates add the stored (rounded) messages, as Algorithm 2 sums them: no
-          // contraction of a product into the sum
-          const double2 m = make_double2(__dmul_rn(cin, A[u]), __dmul_rn(cin, nk[u].h - rv[u].y));
+          const double2 m = message64(A[u], nk[u], rv[u], bad);
           __stcs(Mout + p0 + 32 * (j + u), m);
-          accP = __dadd_rn(accP, m.x);
-          acch = __dadd_rn(acch, m.y);
+          accP = fma(-A[u], m.x, accP);
+          acch = fma(-m.x, m.y, acch);
           accr = fma(A[u], AIT ? nk[u].pad : nk[u].x, accr);
         }
       }
@@ -496,7 +554,7 @@ __global__ void __launch_bounds__(kBlock, GABP_K64_MINB) k64_node(Args64 a) {
       const double P = d + accP, h = bi + acch;
       bad |= is_zero64(P);
       const NodeRec64 own = Nin[i];
-      const double xt = h * rcp64(P);
+      const double xt = div64(h, P);
       double yt = xt;
       if (AIT && t >= 2) yt = aitken64(Nout[i].x, own.x, xt);
       if (STF) {
@@ -557,7 +615,7 @@ constexpr int kCoopMaxSlices = 4096;
 constexpr long long kCoopBarrierLimit = 4000000000LL;
 
 template <bool FRZ>
-__global__ void __launch_bounds__(kCoopThreads, FRZ ? 8 : 0) k64_coop(Args64 a, unsigned *bar, int *err, int max_rounds) {
+__global__ void __launch_bounds__(kCoopThreads, FRZ ? 8 : 12) k64_coop(Args64 a, unsigned *bar, int *err, int max_rounds) {
   DevCtl *ctl = a.ctl;
   __shared__ int s_last, s_go;
   __shared__ unsigned s_gen;
@@ -565,6 +623,7 @@ __global__ void __launch_bounds__(kCoopThreads, FRZ ? 8 : 0) k64_coop(Args64 a, 
   const int warp = (blockIdx.x * kCoopThreads + threadIdx.x) >> 5;
   const int nwarps = (gridDim.x * kCoopThreads) >> 5;
   const double *__restrict__ b = ctl->b;
+  const int cold = ctl->cold;
   for (int iter = 0; iter < max_rounds; ++iter) {
     const int t = __ldcg(&ctl->round) + 1;
     const int fs = FRZ ? __ldcg(&ctl->fstate) : -1;
@@ -575,10 +634,11 @@ __global__ void __launch_bounds__(kCoopThreads, FRZ ? 8 : 0) k64_coop(Args64 a, 
     double rr = 0.0;
     int bad = 0, moving = 0;
     for (int sl = warp; sl < a.ns; sl += nwarps) {
-      if (!FRZ) plain_slice<true, 0>(a, sl, lane, b, Min, Mout, Nin, Nout, rr, bad, moving);
-      else if (fs == 0) plain_slice<true, 1>(a, sl, lane, b, Min, Mout, Nin, Nout, rr, bad, moving);
-      else if (fs == 1) plain_slice<true, 2>(a, sl, lane, b, Min, Mout, Nin, Nout, rr, bad, moving);
-      else plain_slice<true, 3>(a, sl, lane, b, Min, Mout, Nin, Nout, rr, bad, moving);
+      if (!FRZ && t == 1 && cold) plain_slice<true, 0, kZero>(a, sl, lane, b, Min, Mout, Nin, Nout, rr, bad, moving);
+      else if (!FRZ) plain_slice<true, 0, kGather>(a, sl, lane, b, Min, Mout, Nin, Nout, rr, bad, moving);
+      else if (fs == 0) plain_slice<true, 1, kGather>(a, sl, lane, b, Min, Mout, Nin, Nout, rr, bad, moving);
+      else if (fs == 1) plain_slice<true, 2, kGather>(a, sl, lane, b, Min, Mout, Nin, Nout, rr, bad, moving);
+      else plain_slice<true, 3, kGather>(a, sl, lane, b, Min, Mout, Nin, Nout, rr, bad, moving);
     }
     // grid barrier; the last block to arrive reduces and decides
     constexpr int NV = FRZ ? 3 : 2;
@@ -672,6 +732,7 @@ __global__ void __launch_bounds__(32 * NW) k64_cluster(Args64 a, int max_rounds)
   DevCtl *ctl = a.ctl;
   const double *__restrict__ b = ctl->b;
   const int t0 = ctl->round;  // read by every CTA before the first barrier, written only after it
+  const int cold = ctl->cold;
   const StopRule rule = stop_rule(ctl);  // CTA 0 writes none of these fields
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
   const int warp = (int)(rank * NW) + wib;
@@ -686,10 +747,11 @@ __global__ void __launch_bounds__(32 * NW) k64_cluster(Args64 a, int max_rounds)
     double rr = 0.0;
     int bad = 0, moving = 0;
     for (int sl = warp; sl < a.ns; sl += nwarps) {
-      if (!FRZ) plain_slice<true, 0>(a, sl, lane, b, Min, Mout, Nin, Nout, rr, bad, moving);
-      else if (fs == 0) plain_slice<true, 1>(a, sl, lane, b, Min, Mout, Nin, Nout, rr, bad, moving);
-      else if (fs == 1) plain_slice<true, 2>(a, sl, lane, b, Min, Mout, Nin, Nout, rr, bad, moving);
-      else plain_slice<true, 3>(a, sl, lane, b, Min, Mout, Nin, Nout, rr, bad, moving);
+      if (!FRZ && t == 1 && cold) plain_slice<true, 0, kZero>(a, sl, lane, b, Min, Mout, Nin, Nout, rr, bad, moving);
+      else if (!FRZ) plain_slice<true, 0, kGather>(a, sl, lane, b, Min, Mout, Nin, Nout, rr, bad, moving);
+      else if (fs == 0) plain_slice<true, 1, kGather>(a, sl, lane, b, Min, Mout, Nin, Nout, rr, bad, moving);
+      else if (fs == 1) plain_slice<true, 2, kGather>(a, sl, lane, b, Min, Mout, Nin, Nout, rr, bad, moving);
+      else plain_slice<true, 3, kGather>(a, sl, lane, b, Min, Mout, Nin, Nout, rr, bad, moving);
     }
     // flags: bit 0 a zero cavity or node precision, bit 1 a precision moved (the freeze's screen)
     const ClusterSums tot =
@@ -789,7 +851,7 @@ __global__ void __launch_bounds__(32 * NW) k64_chip(Args64 a, ChipShape c, int m
         const int pos = p0 + e, li = lb + e;
         const int k = a.sci[pos];
         savl[li] = a.sav[pos];
-        Ml0[li] = a.M0[pos];
+        Ml0[li] = ctl->cold ? make_double2(0.0, 0.0) : a.M0[pos];
         Ml1[li] = a.M1[pos];
         int kr = -1, rr = 0;
         if (k >= 0) {
@@ -842,13 +904,10 @@ __global__ void __launch_bounds__(32 * NW) k64_chip(Args64 a, ChipShape c, int m
 #pragma unroll
         for (int u = 0; u < kUChip; ++u) {
           if (kr[u] < 0) continue;
-          const double den = nk[u].P - rv[u].x;
-          bad |= is_zero64(den);
-          const double cin = -A[u] * rcp64(den);
-          const double2 m = make_double2(__dmul_rn(cin, A[u]), __dmul_rn(cin, nk[u].h - rv[u].y));
+          const double2 m = message64(A[u], nk[u], rv[u], bad);
           Mout[lb + 32 * (j + u) + lane] = m;
-          accP = __dadd_rn(accP, m.x);
-          acch = __dadd_rn(acch, m.y);
+          accP = fma(-A[u], m.x, accP);
+          acch = fma(-m.x, m.y, acch);
           accr = fma(A[u], nk[u].x, accr);
         }
       }
@@ -857,8 +916,8 @@ __global__ void __launch_bounds__(32 * NW) k64_chip(Args64 a, ChipShape c, int m
         const NodeRec64 own = Rin[lr];
         const double P = d + accP, h = bi + acch;
         bad |= is_zero64(P);
-        const double ip = rcp64(P);
-        Rout[lr] = NodeRec64{P, h, h * ip, h * ip};
+        const double x = div64(h, P);
+        Rout[lr] = NodeRec64{P, h, x, x};
         const double res = bi - fma(d, own.x, accr);
         rr = fma(res, res, rr);
       }
@@ -894,7 +953,8 @@ __global__ void __launch_bounds__(32 * NW) k64_chip(Args64 a, ChipShape c, int m
 
 // Steffensen's iterations, the step after a cycle's second round t: "y replaces
 // x_n and GaBP runs again".  The mean messages of round t move by the cycle's
-// scalar step, h <- h^(t) - lam (h^(t) - h^(t-1)) (the precision messages stay),
+// scalar step, h <- h^(t) - lam (h^(t) - h^(t-1)) (the precision messages stay:
+// h = -c v moves with v <- v^(t) - lam (v^(t) - v^(t-1) c^(t-1) / c^(t))),
 // and every node record is rebuilt from them: h~ = b + sum h, x = h~ / P~.  With
 // stationary precisions these means are exactly y = x^(t) - lam (x^(t) - x^(t-1)).
 // Launched after every round; it acts once per even round that has not stopped
@@ -917,15 +977,16 @@ __global__ void __launch_bounds__(kBlock) k64_steff(Args64 a) {
     for (int j = 0; j < wd; ++j) {
       const int pos = p0 + 32 * j;
       if (a.sci[pos] < 0) break;
-      const double ht = Mt[pos].y;
-      const double hn = ht - lam * (ht - Mp[pos].y);
-      Mt[pos].y = hn;
-      acch = __dadd_rn(acch, hn);
+      const double2 mt = Mt[pos], mp = Mp[pos];
+      const double q = is_zero64(mt.x) ? 1.0 : div64(mp.x, mt.x);
+      const double vn = mt.y - lam * (mt.y - mp.y * q);
+      Mt[pos].y = vn;
+      acch = fma(-mt.x, vn, acch);
     }
     if (i >= 0) {
       const NodeRec64 own = Nt[i];
       const double h = b[i] + acch;
-      const double x = h * rcp64(own.P);
+      const double x = div64(h, own.P);
       Nt[i] = NodeRec64{own.P, h, x, x};
     }
   }
@@ -962,10 +1023,7 @@ __global__ void __launch_bounds__(kBlock) k64_edge_msg(Args64 a) {
     const double A = __ldcs(a.sav + pos);
     const double2 rv = __ldcs(Min + __ldcs(a.srev + pos));
     const NodeRec64 nk = Nin[k];
-    const double den = nk.P - rv.x;
-    bad |= is_zero64(den);
-    const double cin = -A * rcp64(den);
-    __stcs(Mout + pos, make_double2(__dmul_rn(cin, A), __dmul_rn(cin, nk.h - rv.y)));
+    __stcs(Mout + pos, message64(A, nk, rv, bad));
   }
   if (__syncthreads_or(bad) && threadIdx.x == 0) atomicOr(&ctl->edge_bad, 1);
 }
@@ -992,15 +1050,16 @@ __global__ void __launch_bounds__(kBlock) k64_edge_agg(Args64 a) {
       const int k = __ldcs(a.sci + pos);
       if (k < 0) break;
       const double2 m = __ldcs(Mnew + pos);
-      accP += m.x;
-      acch += m.y;
-      accr = fma(__ldcs(a.sav + pos), Nin[k].x, accr);
+      const double A = __ldcs(a.sav + pos);
+      accP = fma(-A, m.x, accP);
+      acch = fma(-m.x, m.y, acch);
+      accr = fma(A, Nin[k].x, accr);
     }
     if (i >= 0) {
       const double bi = b[i], d = a.ad[i];
       const double P = d + accP, h = bi + acch;
       bad |= is_zero64(P);
-      Nout[i] = NodeRec64{P, h, h * rcp64(P), 0.0};
+      Nout[i] = NodeRec64{P, h, div64(h, P), 0.0};
       const double r = bi - fma(d, Nin[i].x, accr);
       rr = fma(r, r, rr);
     }
@@ -1020,11 +1079,11 @@ __global__ void k64_finalize(int n, const NodeRec64 *__restrict__ N, double *__r
   if (i < n) x[i] = aitken ? N[i].pad : N[i].x;
 }
 
-// Messages of the returned round in the layout of the input CSR.  M is indexed by
-// position c2s[e] of compact slot e (the sliced layout), or by e itself when c2s
-// is null.
+// Messages of the returned round in the layout of the input CSR.  With the sliced
+// layout's c2s, M holds {c, v} at position c2s[e] of compact slot e and A_ik is av[e];
+// without (c2s null), M holds {P, h} at e itself.
 __global__ void k64_messages(int n, const int *__restrict__ rowptr, const int *__restrict__ dpos,
-                             const int *__restrict__ rp, const int *__restrict__ c2s,
+                             const int *__restrict__ rp, const int *__restrict__ c2s, const double *__restrict__ av,
                              const double2 *__restrict__ M, double *__restrict__ P, double *__restrict__ hm) {
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
@@ -1034,8 +1093,8 @@ __global__ void k64_messages(int n, const int *__restrict__ rowptr, const int *_
   for (int q = 0; q < deg; ++q) {
     int p = a + q + (q >= d ? 1 : 0);
     double2 m = M[c2s ? c2s[e0 + q] : e0 + q];
-    P[p] = m.x;
-    hm[p] = m.y;
+    P[p] = c2s ? -av[e0 + q] * m.x : m.x;
+    hm[p] = c2s ? -m.x * m.y : m.y;
   }
 }
 
@@ -1055,15 +1114,25 @@ __global__ void k_sell_fill(int nq, const int *__restrict__ srow, const int *__r
   }
 }
 
-// Reverse positions and values (values again after gabp_set_values).
+// Reverse positions, with the count of those far away, and values (far null: the values alone,
+// again after gabp_set_values).
+constexpr int kFarSlots = 1 << 21;
 __global__ void k_sell_rev_vals(int E, const int *__restrict__ c2s, const int *__restrict__ rev,
                                 const double *__restrict__ av, int *__restrict__ srev, double *__restrict__ sav,
-                                int with_rev) {
+                                unsigned *__restrict__ far) {
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= E) return;
-  const int pos = c2s[e];
-  if (with_rev) srev[pos] = c2s[rev[e]];
-  sav[pos] = av[e];
+  int f = 0;
+  if (e < E) {
+    const int pos = c2s[e];
+    if (far) {
+      const int rp = c2s[rev[e]];
+      srev[pos] = rp;
+      f = abs(rp - pos) > kFarSlots;
+    }
+    sav[pos] = av[e];
+  }
+  const int nf = __syncthreads_count(f);
+  if (nf && threadIdx.x == 0) atomicAdd(far, (unsigned)nf);
 }
 
 __global__ void k64_marginals(int n, const NodeRec64 *__restrict__ N, double *__restrict__ Pi) {
@@ -1198,10 +1267,16 @@ static gabp_status ensure_sell64(gabp_handle h) {
     GABP_CUDA(cudaMemsetAsync(S.sav, 0, sizeof(double) * Ea, h->stream));
     const int nq = ns * 32;
     k_sell_fill<<<(nq + kBlock - 1) / kBlock, kBlock, 0, h->stream>>>(nq, S.srow, S.sp, g.rp, g.ci, S.c2s, S.sci);
+    unsigned far = 0;
+    unsigned *dfar = &h->ctl->arrive;  // the control block is idle here; every run clears it
+    GABP_CUDA(cudaMemsetAsync(dfar, 0, sizeof(unsigned), h->stream));
     if (E > 0)
-      k_sell_rev_vals<<<(E + kBlock - 1) / kBlock, kBlock, 0, h->stream>>>(E, S.c2s, g.rev, g.av, S.srev, S.sav, 1);
+      k_sell_rev_vals<<<(E + kBlock - 1) / kBlock, kBlock, 0, h->stream>>>(E, S.c2s, g.rev, g.av, S.srev, S.sav, dfar);
     GABP_CUDA(cudaGetLastError());
+    GABP_CUDA(cudaMemcpyAsync(&far, dfar, sizeof(unsigned), cudaMemcpyDeviceToHost, h->stream));
+    GABP_CUDA(cudaMemsetAsync(dfar, 0, sizeof(unsigned), h->stream));
     GABP_CUDA(cudaStreamSynchronize(h->stream));  // the host vectors are released on return
+    S.far = far;
     S.ready = true;
     S.vals_ok = true;
     h->tuned_L64 = 1;  // one row per lane
@@ -1234,7 +1309,8 @@ static gabp_status ensure_sell64(gabp_handle h) {
     }
   } else if (!S.vals_ok) {
     if (E > 0)
-      k_sell_rev_vals<<<(E + kBlock - 1) / kBlock, kBlock, 0, h->stream>>>(E, S.c2s, g.rev, g.av, S.srev, S.sav, 0);
+      k_sell_rev_vals<<<(E + kBlock - 1) / kBlock, kBlock, 0, h->stream>>>(E, S.c2s, g.rev, g.av, S.srev, S.sav,
+                                                                           nullptr);
     GABP_CUDA(cudaGetLastError());
     S.vals_ok = true;
   }
@@ -1283,6 +1359,12 @@ static Args64 args64(gabp_handle h) {
   a.C = h->w64.C;
   a.freeze = h->opt.freeze_precisions && h->opt.variant == GABP_VARIANT_NODE && h->opt.accel == ACC_NONE &&
              h->w64.C != nullptr;
+  // Recompute the reverse messages when more than a quarter of them lie further than kFarSlots positions
+  // (32 MB of messages) from the slot that needs them: such reads come from DRAM, a 32-byte sector each.
+  // Both forms measured, gather / recompute: random graphs of degree 16 with 200,000 rows (12 % far) 76 / 79
+  // us per round, 400,000 (45 %) 145 / 128, 2^20 (77 %) 449 / 276; 10^6 rows of degree 6 (42 %) 193 / 122;
+  // 64^3 and 128^3 grids (none far) 34 / 39 and 164 / 203.
+  a.rec = S.far > (int64_t)h->g.E / 4;
   // long rows and too few slices to give every SM eight warps: a warp per row instead
   a.wide = !a.freeze && h->opt.variant == GABP_VARIANT_NODE && h->opt.accel == ACC_NONE && S.ns > 0 &&
            (double)S.Es >= 64.0 * 32.0 * S.ns && S.ns < 8 * h->num_sms;
@@ -1308,10 +1390,18 @@ static void launch_round(gabp_handle h, const Args64 &a) {
     k64_wide<<<resident_grid(h->num_sms, k64_wide), kBlock, 0, h->stream>>>(a);
   } else if (a.freeze) {
     k64_frz<3><<<slice_grid(h, k64_frz<3>), kBlock, 0, h->stream>>>(a);
-    k64_frz<2><<<slice_grid(h, k64_frz<2>), kBlock, 0, h->stream>>>(a);
-    k64_frz<1><<<slice_grid(h, k64_frz<1>), kBlock, 0, h->stream>>>(a);
+    if (a.rec) {
+      k64_frz<2, true><<<slice_grid(h, k64_frz<2, true>), kBlock, 0, h->stream>>>(a);
+      k64_frz<1, true><<<slice_grid(h, k64_frz<1, true>), kBlock, 0, h->stream>>>(a);
+    } else {
+      k64_frz<2><<<slice_grid(h, k64_frz<2>), kBlock, 0, h->stream>>>(a);
+      k64_frz<1><<<slice_grid(h, k64_frz<1>), kBlock, 0, h->stream>>>(a);
+    }
   } else {
-    k64_node<ACC_NONE><<<slice_grid(h, k64_node<ACC_NONE>), kBlock, 0, h->stream>>>(a);
+    if (a.rec)
+      k64_node<ACC_NONE, true><<<slice_grid(h, k64_node<ACC_NONE, true>), kBlock, 0, h->stream>>>(a);
+    else
+      k64_node<ACC_NONE, false><<<slice_grid(h, k64_node<ACC_NONE, false>), kBlock, 0, h->stream>>>(a);
   }
 }
 
@@ -1356,6 +1446,16 @@ gabp_status solve64(gabp_handle h, const double *b, double *x, double tol, int m
   if (h->opt.freeze_precisions && !h->w64.C)  // the frozen coefficients' store
     GABP_CUDA(cudaMalloc(&h->w64.C, sizeof(double) * Es));
   Args64 a = args64(h);
+  // small and medium graphs: every round in one cluster or cooperative launch
+  const int coop_grid = a.freeze ? h->coop64f : h->coop64;
+  const bool clus = !a.wide && h->w64.sl.ns <= kClusterMaxSlices && h->opt.variant == GABP_VARIANT_NODE &&
+                    h->opt.accel == ACC_NONE && h->clu64 > 0;
+  const bool coop = !clus && !a.wide && h->w64.sl.ns <= kCoopMaxSlices && h->opt.variant == GABP_VARIANT_NODE &&
+                    h->opt.accel == ACC_NONE && coop_grid > 0;
+  // zero starting messages that need no store (the accelerated, the edge and the one-launch freeze
+  // rounds read M0)
+  const bool cold = !warm && h->opt.variant == GABP_VARIANT_NODE && h->opt.accel == ACC_NONE &&
+                    !(a.freeze && (clus || coop));
   // round-0 state (Algorithm 1 step 1): control block pointed at b, zero messages
   auto init = [&]() -> gabp_status {
     GABP_CUDA(cudaMemsetAsync(h->ctl, 0, sizeof(DevCtl), h->stream));
@@ -1374,20 +1474,15 @@ gabp_status solve64(gabp_handle h, const double *b, double *x, double tol, int m
       GABP_CUDA(cudaMemcpyAsync(&h->ctl->hist, &hp, sizeof(hp), cudaMemcpyHostToDevice, h->stream));
       GABP_CUDA(cudaMemcpyAsync(&h->ctl->hist_cap, &cap, sizeof(cap), cudaMemcpyHostToDevice, h->stream));
     }
-    if (!warm) GABP_CUDA(cudaMemsetAsync(h->w64.M[0], 0, sizeof(double2) * Es, h->stream));
-    k64_init<<<blocks_for(a.ns, kBlock / 32, h->max_blocks), kBlock, 0, h->stream>>>(a, tol, max_iter, warm ? 1 : 0);
+    if (!warm && !cold) GABP_CUDA(cudaMemsetAsync(h->w64.M[0], 0, sizeof(double2) * Es, h->stream));
+    k64_init<<<blocks_for(a.ns, kBlock / 32, h->max_blocks), kBlock, 0, h->stream>>>(a, tol, max_iter, warm ? 1 : 0,
+                                                                                       cold ? 1 : 0);
     GABP_CUDA(cudaGetLastError());
     GABP_CUDA(cudaStreamSynchronize(h->stream));  // also retires the pageable copy of bptr
     return GABP_OK;
   };
   if ((s = init()) != GABP_OK) return s;
 
-  // small and medium graphs: every round in one cooperative launch
-  const int coop_grid = a.freeze ? h->coop64f : h->coop64;
-  const bool clus = !a.wide && h->w64.sl.ns <= kClusterMaxSlices && h->opt.variant == GABP_VARIANT_NODE &&
-                    h->opt.accel == ACC_NONE && h->clu64 > 0;
-  const bool coop = !clus && !a.wide && h->w64.sl.ns <= kCoopMaxSlices && h->opt.variant == GABP_VARIANT_NODE &&
-                    h->opt.accel == ACC_NONE && coop_grid > 0;
   const bool use_graph = !coop && !clus && h->stream != nullptr && h->opt.graphs;
   cudaGraphExec_t ge = nullptr;
   if (use_graph) {
@@ -1494,6 +1589,8 @@ gabp_status solve64(gabp_handle h, const double *b, double *x, double tol, int m
   h->stats.refine_steps = 0;
   h->stats.freeze_round = a.freeze ? c.fround : 0;
   h->stats.freeze_checks = a.freeze ? c.fchecks : 0;
+  if (cold && c.result_round == 0)  // the messages of round 0
+    GABP_CUDA(cudaMemsetAsync(h->w64.M[0], 0, sizeof(double2) * Es, h->stream));
   if (warm && c.bb == 0.0) {  // b = 0: x = 0 (the warm round-0 records hold the old messages' mean)
     GABP_CUDA(cudaMemsetAsync(x, 0, sizeof(double) * g.n, h->stream));
   } else {
@@ -1512,23 +1609,27 @@ gabp_status messages64(gabp_handle h, double *P, double *hm) {
   if (!h->w64.valid) return GABP_ERR_INVALID;
   Graph &g = h->g;
   k64_messages<<<(g.n + kBlock - 1) / kBlock, kBlock, 0, h->stream>>>(
-      g.n, g.rowptr, g.dpos, g.rp, h->w64.sl.c2s, h->w64.M[h->w64.result_round & 1], P, hm);
+      g.n, g.rowptr, g.dpos, g.rp, h->w64.sl.c2s, g.av, h->w64.M[h->w64.result_round & 1], P, hm);
   GABP_CUDA(cudaGetLastError());
   GABP_CUDA(cudaStreamSynchronize(h->stream));
   return GABP_OK;
 }
 
-// Inverse of k64_messages: input-layout messages into the sliced positions.
+// Inverse of k64_messages: input-layout messages into the sliced positions as {c, v}.  A
+// mean message without a precision message (P = 0, h != 0) takes a c of 2^-300, whose
+// precision vanishes against any aggregate.
 __global__ void k64_load_messages(int n, const int *__restrict__ rowptr, const int *__restrict__ dpos,
                                   const int *__restrict__ rp, const int *__restrict__ c2s,
-                                  const double *__restrict__ P, const double *__restrict__ hm,
-                                  double2 *__restrict__ M) {
+                                  const double *__restrict__ av, const double *__restrict__ P,
+                                  const double *__restrict__ hm, double2 *__restrict__ M) {
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   int a = rowptr[i], d = dpos[i], e0 = rp[i], deg = rp[i + 1] - rp[i];
   for (int q = 0; q < deg; ++q) {
     int p = a + q + (q >= d ? 1 : 0);
-    M[c2s[e0 + q]] = make_double2(P[p], hm[p]);
+    double c = -P[p] / av[e0 + q];
+    if (c == 0.0 && hm[p] != 0.0) c = 0x1p-300;
+    M[c2s[e0 + q]] = make_double2(c, hm[p] == 0.0 ? 0.0 : -hm[p] / c);
   }
 }
 
@@ -1537,7 +1638,7 @@ gabp_status load_messages64(gabp_handle h, const double *P, const double *hm) {
   if (s != GABP_OK) return s;
   Graph &g = h->g;
   k64_load_messages<<<(g.n + kBlock - 1) / kBlock, kBlock, 0, h->stream>>>(g.n, g.rowptr, g.dpos, g.rp,
-                                                                           h->w64.sl.c2s, P, hm, h->w64.M[0]);
+                                                                           h->w64.sl.c2s, g.av, P, hm, h->w64.M[0]);
   GABP_CUDA(cudaGetLastError());
   GABP_CUDA(cudaStreamSynchronize(h->stream));
   h->w64.result_round = 0;
@@ -1547,8 +1648,8 @@ gabp_status load_messages64(gabp_handle h, const double *P, const double *hm) {
 
 gabp_status messages64_from(gabp_handle h, const double2 *M, double *P, double *hm) {
   Graph &g = h->g;
-  k64_messages<<<(g.n + kBlock - 1) / kBlock, kBlock, 0, h->stream>>>(g.n, g.rowptr, g.dpos, g.rp, nullptr, M, P,
-                                                                       hm);
+  k64_messages<<<(g.n + kBlock - 1) / kBlock, kBlock, 0, h->stream>>>(g.n, g.rowptr, g.dpos, g.rp, nullptr, nullptr, M,
+                                                                       P, hm);
   GABP_CUDA(cudaGetLastError());
   GABP_CUDA(cudaStreamSynchronize(h->stream));
   return GABP_OK;
