@@ -97,7 +97,8 @@ typedef struct {
                            schedule "round" below reads "sweep").  Screen: after two consecutive
                            rounds in which no node's P~_i moved by more than 16 units in the last
                            place (~2^-48 relative), one round checks every precision message against its previous
-                           round's the same way while it stores each edge's coefficient
+                           round's the same way (parallel schedule: the first
+                           time with a bar of 8 units) while it stores each edge's coefficient
                            -A_ki / P_k\i and each node's 1/P~; if none moved, later rounds update
                            the mean messages only (the precisions do not depend on b), else the
                            screen resumes.  Every round up to the stored one is bitwise the plain

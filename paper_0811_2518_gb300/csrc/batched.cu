@@ -4,10 +4,17 @@
 //
 // The precision messages depend on A only (eq_prec and eq_prec_message have no
 // b in them), so the FP32 precision phase and the frozen coefficient pairs of
-// solve32.cu serve every right-hand side.  The mean iteration is the recompute
-// form of solve32.cu, run for RP columns at once:
-//   h_{i->k}^{(t-1)} = c_out (h~_i^{(t-2)} - h_{k->i}^{(t-2)}),
-//   h_{k->i}^{(t)}   = c_in  (h~_k^{(t-1)} - h_{i->k}^{(t-1)}).
+// solve32.cu serve every right-hand side.  The mean messages of round t are
+//   h_{k->i}^{(t)} = c_in (h~_k^{(t-1)} - h_{i->k}^{(t-1)}),
+// run for RP columns at once, and the message store, E x RP floats, is the traffic.  Only the
+// messages of EVEN rounds are stored, one array:
+//   even t   row i forms the reverse message of round t-1 again from what it held at t-2,
+//            h_{i->k}^{(t-1)} = c_out (h~_i^{(t-2)} - h_{k->i}^{(t-2)}), its own slot, which it
+//            overwrites with h_{k->i}^{(t)};
+//   odd t    the reverse message of round t-1 is the stored one of the reverse edge, read from row
+//            k's slot; nothing is written but the aggregates.
+// A pair of rounds moves three messages per slot where the recompute form in every round (two
+// stores) moves four.
 // Layout: slot-major, column-minor -- H[e][r], NH[i][r] -- so a warp that owns a
 // row reads one coefficient pair and one column index per slot (broadcast) and
 // moves RP contiguous floats for the slot's messages and for the sender's
@@ -73,9 +80,10 @@ struct ArgsB {
   int n, RP;
   const int *__restrict__ rp;
   const int *__restrict__ ci;
+  const int *__restrict__ rev;
   const float2 *__restrict__ CF;
   const float *__restrict__ invP;
-  float *H0, *H1;
+  float *H;  // [E][RP] messages of the latest even round
   float *NH0, *NH1, *NH2;
   const float *rhs;
   DevCtl *ctl;
@@ -127,67 +135,75 @@ __device__ bool col_reduce(const double (&acc)[NV][VEC], int RP, double *red, do
   return true;
 }
 
-// Round t of the batched frozen-precision mean iteration (one warp per row).
-// Stops when every column with a nonzero iterate has ||dx_r|| <= inner_tol ||x_r||.
+// Slots of a row whose loads are issued together, and the blocks per SM of the register budget.  A
+// round is bound by HBM (128^3 grid, 64 columns: 6.9 GB on average, 1.01 ms at the measured copy rate) and
+// by the bytes its warps keep in flight: 2 slots and 6 blocks 1.33 ms per round (1.68 with four messages a
+// pair of rounds); 7 or 8 blocks the same, 3 slots with 6 / 5 / 4 blocks 1.37 / 1.42 / 1.74, 1 with 8 1.47.
+#ifndef GABP_KB_U
+#define GABP_KB_U 2
+#endif
+#ifndef GABP_KB_MINB
+#define GABP_KB_MINB 6
+#endif
 template <int VEC>
-__global__ void __launch_bounds__(kBlock, 6) kb_mean(ArgsB a) {
-  DevCtl *ctl = a.ctl;
-  if (ctl->done) return;
-  const int t = ctl->round + 1;
+constexpr int kBU = VEC == 4 ? 2 : GABP_KB_U;
+
+// Rounds by what their reverse messages come from: none in round 1 (zero messages), the row's own
+// aggregate in round 2 (its stored messages are the zero ones, not read), then as above.
+enum BKind { kBFirst, kBSecond, kBEven, kBOdd };
+
+// NU slots e .. e + NU - 1 of one row: messages k -> i of this round added to acc, stored in even rounds.
+template <int VEC, BKind KIND, int NU>
+__device__ __forceinline__ void kb_slots(const ArgsB &a, int e, int c0, const float *__restrict__ Hm1,
+                                         const float (&hi2)[VEC], float (&acc)[VEC]) {
   const int RP = a.RP;
-  float *__restrict__ Hc = (t & 1) ? a.H1 : a.H0;  // holds t-2, becomes t
-  const float *__restrict__ Hm1 = ring3b(a.NH0, a.NH1, a.NH2, t + 2);
-  const float *__restrict__ Hm2 = ring3b(a.NH0, a.NH1, a.NH2, t + 1);
-  float *__restrict__ Ht = ring3b(a.NH0, a.NH1, a.NH2, t);
-  const int lane = threadIdx.x & 31;
+  int k[NU], rv[NU];
+  float2 cf[NU];
+  float hs[NU][VEC], hk[NU][VEC];
+#pragma unroll
+  for (int u = 0; u < NU; ++u) {
+    k[u] = a.ci[e + u];
+    cf[u] = a.CF[e + u];
+    if (KIND == kBOdd) rv[u] = a.rev[e + u];
+  }
+#pragma unroll
+  for (int u = 0; u < NU; ++u) {
+    if (KIND == kBEven) ldv_cs<VEC>(a.H + (size_t)(e + u) * RP + c0, hs[u]);
+    if (KIND == kBOdd) ldv_cs<VEC>(a.H + (size_t)rv[u] * RP + c0, hs[u]);
+    ldv<VEC>(Hm1 + (size_t)k[u] * RP + c0, hk[u]);
+  }
+#pragma unroll
+  for (int u = 0; u < NU; ++u) {
+    float hn[VEC];
+#pragma unroll
+    for (int v = 0; v < VEC; ++v) {
+      const float hout = KIND == kBFirst ? 0.f                               // message i -> k at t-1
+                         : KIND == kBOdd ? hs[u][v]
+                                         : cf[u].y * (hi2[v] - (KIND == kBEven ? hs[u][v] : 0.f));
+      hn[v] = cf[u].x * (hk[u][v] - hout);                                   // message k -> i at t
+      acc[v] += hn[v];
+    }
+    if (KIND == kBEven || KIND == kBSecond) stv_cs<VEC>(a.H + (size_t)(e + u) * RP + c0, hn);
+  }
+}
+
+template <int VEC, BKind KIND>
+__device__ __forceinline__ void kb_rows(const ArgsB &a, const float *__restrict__ Hm1, const float *__restrict__ Hm2,
+                                        float *__restrict__ Ht, float (&acc2)[2][VEC]) {
+  constexpr int NU = kBU<VEC>;
+  const int RP = a.RP;
+  const int c0 = (threadIdx.x & 31) * VEC;
   const int warp = (blockIdx.x * kBlock + threadIdx.x) >> 5;
   const int nwarps = (gridDim.x * kBlock) >> 5;
-  const int c0 = lane * VEC;
-  float acc2[2][VEC];
-#pragma unroll
-  for (int v = 0; v < VEC; ++v) acc2[0][v] = acc2[1][v] = 0.f;
   for (int i = warp; i < a.n; i += nwarps) {
     float hi2[VEC], acc[VEC];
-    if (t >= 2) ldv<VEC>(Hm2 + (size_t)i * RP + c0, hi2);
+    if (KIND == kBEven || KIND == kBSecond) ldv<VEC>(Hm2 + (size_t)i * RP + c0, hi2);
 #pragma unroll
     for (int v = 0; v < VEC; ++v) acc[v] = 0.f;
-    const int e0 = a.rp[i], e1 = a.rp[i + 1];
-    int e = e0;
-    for (; e + 1 < e1; e += 2) {  // two slots with their loads issued together
-      const int k0 = a.ci[e], k1 = a.ci[e + 1];
-      const float2 cf0 = a.CF[e], cf1 = a.CF[e + 1];
-      float hs0[VEC], hs1[VEC], hk0[VEC], hk1[VEC], hn0[VEC], hn1[VEC];
-      ldv_cs<VEC>(Hc + (size_t)e * RP + c0, hs0);
-      ldv_cs<VEC>(Hc + (size_t)(e + 1) * RP + c0, hs1);
-      ldv<VEC>(Hm1 + (size_t)k0 * RP + c0, hk0);
-      ldv<VEC>(Hm1 + (size_t)k1 * RP + c0, hk1);
-#pragma unroll
-      for (int v = 0; v < VEC; ++v) {
-        const float ho0 = t >= 2 ? cf0.y * (hi2[v] - hs0[v]) : 0.f;  // messages i -> k at t-1
-        const float ho1 = t >= 2 ? cf1.y * (hi2[v] - hs1[v]) : 0.f;
-        hn0[v] = cf0.x * (hk0[v] - ho0);                             // messages k -> i at t
-        hn1[v] = cf1.x * (hk1[v] - ho1);
-        acc[v] += hn0[v];
-        acc[v] += hn1[v];
-      }
-      stv_cs<VEC>(Hc + (size_t)e * RP + c0, hn0);
-      stv_cs<VEC>(Hc + (size_t)(e + 1) * RP + c0, hn1);
-    }
-    if (e < e1) {
-      const int k = a.ci[e];
-      const float2 cf = a.CF[e];
-      float hs[VEC], hk[VEC];
-      ldv_cs<VEC>(Hc + (size_t)e * RP + c0, hs);
-      ldv<VEC>(Hm1 + (size_t)k * RP + c0, hk);
-      float hn[VEC];
-#pragma unroll
-      for (int v = 0; v < VEC; ++v) {
-        const float hout = t >= 2 ? cf.y * (hi2[v] - hs[v]) : 0.f;  // message i -> k at t-1
-        hn[v] = cf.x * (hk[v] - hout);                              // message k -> i at t
-        acc[v] += hn[v];
-      }
-      stv_cs<VEC>(Hc + (size_t)e * RP + c0, hn);
-    }
+    int e = a.rp[i];
+    const int e1 = a.rp[i + 1];
+    for (; e + NU <= e1; e += NU) kb_slots<VEC, KIND, NU>(a, e, c0, Hm1, hi2, acc);
+    for (; e < e1; ++e) kb_slots<VEC, KIND, 1>(a, e, c0, Hm1, hi2, acc);
     float rh[VEC], hp[VEC], hnew[VEC];
     ldv<VEC>(a.rhs + (size_t)i * RP + c0, rh);
     ldv<VEC>(Hm1 + (size_t)i * RP + c0, hp);
@@ -200,6 +216,29 @@ __global__ void __launch_bounds__(kBlock, 6) kb_mean(ArgsB a) {
       acc2[1][v] = fmaf(x, x, acc2[1][v]);
     }
     stv<VEC>(Ht + (size_t)i * RP + c0, hnew);
+  }
+}
+
+// Round t of the batched frozen-precision mean iteration (one warp per row).
+// Stops when every column with a nonzero iterate has ||dx_r|| <= inner_tol ||x_r||.
+template <int VEC>
+__global__ void __launch_bounds__(kBlock, GABP_KB_MINB) kb_mean(ArgsB a) {
+  DevCtl *ctl = a.ctl;
+  if (ctl->done) return;
+  const int t = ctl->round + 1;
+  const int RP = a.RP;
+  const float *__restrict__ Hm1 = ring3b(a.NH0, a.NH1, a.NH2, t + 2);
+  const float *__restrict__ Hm2 = ring3b(a.NH0, a.NH1, a.NH2, t + 1);
+  float *__restrict__ Ht = ring3b(a.NH0, a.NH1, a.NH2, t);
+  float acc2[2][VEC];
+#pragma unroll
+  for (int v = 0; v < VEC; ++v) acc2[0][v] = acc2[1][v] = 0.f;
+  if (t & 1) {
+    if (t == 1) kb_rows<VEC, kBFirst>(a, Hm1, Hm2, Ht, acc2);
+    else kb_rows<VEC, kBOdd>(a, Hm1, Hm2, Ht, acc2);
+  } else {
+    if (t == 2) kb_rows<VEC, kBSecond>(a, Hm1, Hm2, Ht, acc2);
+    else kb_rows<VEC, kBEven>(a, Hm1, Hm2, Ht, acc2);
   }
   double accd[2][VEC];
 #pragma unroll
@@ -335,20 +374,75 @@ struct ArgsBS {
   const float2 *__restrict__ sCF;
   const float *__restrict__ sinvP;
   const float *__restrict__ srhs;  // [n][RP] new order
-  float *sH;                       // [E][RP] serial slot order
+  const int *__restrict__ srev;
+  int n1, e1;                      // two colours: the first row of colour 1 and its first slot
+  float *sH;                       // [E][RP] serial slot order (two colours: the slots from e1 on)
   float *hfire;                    // [n][RP] new order
   DevCtl *ctl;
   double *red;
   double *col;                     // [2][RP] pass sums, then [2][RP] sweep sums, [RP] previous step
 };
 
+// As above for the serial sweeps: 3 slots and 5 blocks (two colours, 128^3 grid, 64 columns: 1.49 ms per
+// sweep, 1.82 with four messages a pair of slots); 2 and 6 the same, 3 and 6 1.51, 3 and 4 1.58, 4 and 5 1.59.
 #ifndef GABP_KBS_U
 #define GABP_KBS_U 3
 #endif
 #ifndef GABP_KBS_MINB
-#define GABP_KBS_MINB 6
+#define GABP_KBS_MINB 5
 #endif
 constexpr int kBsU = GABP_KBS_U;  // slots of a row whose loads are issued together
+
+// The end of a pass: per-column sums over the grid; the last block adds them to the sweep's and, after
+// the sweep's last pass, takes the per-column decision.
+template <int VEC>
+__device__ __forceinline__ void kbs_finish(const ArgsBS &a, const float (&acc2)[2][VEC], bool last) {
+  DevCtl *ctl = a.ctl;
+  const int RP = a.RP;
+  double accd[2][VEC];
+#pragma unroll
+  for (int v = 0; v < VEC; ++v) {
+    accd[0][v] = (double)acc2[0][v];
+    accd[1][v] = (double)acc2[1][v];
+  }
+  if (col_reduce<VEC, 2>(accd, a.RP, a.red, a.col, &ctl->arrive)) {
+    // the last block: add the pass to the sweep's per-column sums
+    double *sw = a.col + 2 * RP, *prev = a.col + 4 * RP;
+    for (int r = threadIdx.x; r < 2 * RP; r += kBlock) sw[r] += a.col[r];
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      if (last) {  // the sweep is complete: per-column decision
+        const int t = ctl->round + 1;
+        ctl->round = t;
+        int notdone = 0;
+        bool finite = true;
+        for (int r = 0; r < RP; ++r) {
+          const double dd = sw[r], xx = sw[RP + r], pv = prev[r];
+          if (!isfinite(dd) || !isfinite(xx)) finite = false;
+          double f2 = 1.0;
+          if (t >= 3 && pv > 0.0) {
+            const double q = sqrt(dd / pv);
+            f2 = q < 0.8 ? fmax(1.0, (q / (1.0 - q)) * (q / (1.0 - q))) : 16.0;
+          }
+          if (xx > 0.0 && !(dd * f2 <= ctl->tol2bb * xx)) ++notdone;
+          prev[r] = dd;
+          sw[r] = 0.0;
+          sw[RP + r] = 0.0;
+        }
+        ctl->rr = (double)notdone;
+        if (!finite) {
+          ctl->status = GABP_DIVERGED; ctl->iters = t; ctl->result_round = t; ctl->done = 1;
+        } else if (t >= 2 && notdone == 0) {
+          ctl->status = GABP_OK; ctl->iters = t; ctl->result_round = t; ctl->done = 1;
+        } else if (t >= ctl->max_iter) {
+          ctl->status = GABP_NOT_CONVERGED; ctl->iters = t; ctl->result_round = t; ctl->done = 1;
+        }
+      }
+      ctl->arrive = 0;
+      __threadfence();
+    }
+  }
+}
 
 template <int VEC>
 __global__ void __launch_bounds__(kBlock, GABP_KBS_MINB) kbs_pass(ArgsBS a, int c, int skip0, int skipn) {
@@ -437,54 +531,93 @@ __global__ void __launch_bounds__(kBlock, GABP_KBS_MINB) kbs_pass(ArgsBS a, int 
       stv<VEC>(a.hfire + (size_t)j * RP + c0, hnew);
     }
   }
-  double accd[2][VEC];
+  kbs_finish<VEC>(a, acc2, c == a.C - 1);
+}
+
+// Pass C of a sweep of two colours (grids, trees, the augmented least-squares systems), where a pass
+// visits whole rows of the other colour and nothing else.  Only the messages into colour 1 are kept:
+//   pass 0 (colour 0 fires, rows of colour 1)  as kbs_pass: the slot's own message, overwritten;
+//   pass 1 (colour 1 fires, rows of colour 0)  the reverse message j -> k is the one pass 0 has just
+//          stored in row k, read from there; the messages into colour 0 are used and not stored.
+// A sweep moves three messages per pair of slots instead of four.  The first sweep starts from zero
+// messages: hfire of colour 1 is 0 and the store is not read.
+template <int VEC, int PASS, bool START, int NU>
+__device__ __forceinline__ void kbs2_slots(const ArgsBS &a, int e, int c0, const float (&hj)[VEC], float (&acc)[VEC]) {
+  const int RP = a.RP;
+  int k[NU], q[NU];
+  float2 cf[NU];
+  float hs[NU][VEC], hk[NU][VEC];
 #pragma unroll
-  for (int v = 0; v < VEC; ++v) {
-    accd[0][v] = (double)acc2[0][v];
-    accd[1][v] = (double)acc2[1][v];
+  for (int u = 0; u < NU; ++u) {
+    k[u] = a.sci[e + u];
+    cf[u] = a.sCF[e + u];
+    q[u] = (PASS == 0 ? e + u : a.srev[e + u]) - a.e1;
   }
-  if (col_reduce<VEC, 2>(accd, RP, a.red, a.col, &ctl->arrive)) {
-    // the last block: add the pass to the sweep's per-column sums
-    double *sw = a.col + 2 * RP, *prev = a.col + 4 * RP;
-    for (int r = threadIdx.x; r < 2 * RP; r += kBlock) sw[r] += a.col[r];
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      if (c == a.C - 1) {  // the sweep is complete: per-column decision
-        const int t = ctl->round + 1;
-        ctl->round = t;
-        int notdone = 0;
-        bool finite = true;
-        for (int r = 0; r < RP; ++r) {
-          const double dd = sw[r], xx = sw[RP + r], pv = prev[r];
-          if (!isfinite(dd) || !isfinite(xx)) finite = false;
-          double f2 = 1.0;
-          if (t >= 3 && pv > 0.0) {
-            const double q = sqrt(dd / pv);
-            f2 = q < 0.8 ? fmax(1.0, (q / (1.0 - q)) * (q / (1.0 - q))) : 16.0;
-          }
-          if (xx > 0.0 && !(dd * f2 <= ctl->tol2bb * xx)) ++notdone;
-          prev[r] = dd;
-          sw[r] = 0.0;
-          sw[RP + r] = 0.0;
-        }
-        ctl->rr = (double)notdone;
-        if (!finite) {
-          ctl->status = GABP_DIVERGED; ctl->iters = t; ctl->result_round = t; ctl->done = 1;
-        } else if (t >= 2 && notdone == 0) {
-          ctl->status = GABP_OK; ctl->iters = t; ctl->result_round = t; ctl->done = 1;
-        } else if (t >= ctl->max_iter) {
-          ctl->status = GABP_NOT_CONVERGED; ctl->iters = t; ctl->result_round = t; ctl->done = 1;
-        }
-      }
-      ctl->arrive = 0;
-      __threadfence();
+#pragma unroll
+  for (int u = 0; u < NU; ++u) {
+    if (!START || PASS == 1) ldv_cs<VEC>(a.sH + (size_t)q[u] * RP + c0, hs[u]);
+    ldv<VEC>(a.hfire + (size_t)k[u] * RP + c0, hk[u]);
+  }
+#pragma unroll
+  for (int u = 0; u < NU; ++u) {
+    float hn[VEC];
+#pragma unroll
+    for (int v = 0; v < VEC; ++v) {
+      const float hout = PASS == 1 ? hs[u][v] : START ? 0.f : cf[u].y * (hj[v] - hs[u][v]);
+      hn[v] = cf[u].x * (hk[u][v] - hout);
+      acc[v] += hn[v];
     }
+    if (PASS == 0) stv_cs<VEC>(a.sH + (size_t)q[u] * RP + c0, hn);
   }
+}
+
+template <int VEC, int PASS, bool START>
+__device__ __forceinline__ void kbs2_rows(const ArgsBS &a, int j0, int j1, float (&acc2)[2][VEC]) {
+  constexpr int NU = VEC == 4 ? 2 : kBsU;
+  const int RP = a.RP;
+  const int c0 = (threadIdx.x & 31) * VEC;
+  const int warp = (blockIdx.x * kBlock + threadIdx.x) >> 5;
+  const int nwarps = (gridDim.x * kBlock) >> 5;
+  for (int j = j0 + warp; j < j1; j += nwarps) {
+    float hj[VEC], acc[VEC];
+    ldv<VEC>(a.hfire + (size_t)j * RP + c0, hj);
+#pragma unroll
+    for (int v = 0; v < VEC; ++v) acc[v] = 0.f;
+    int e = a.srp[j];
+    const int e1 = a.srp[j + 1];
+    for (; e + NU <= e1; e += NU) kbs2_slots<VEC, PASS, START, NU>(a, e, c0, hj, acc);
+    for (; e < e1; ++e) kbs2_slots<VEC, PASS, START, 1>(a, e, c0, hj, acc);
+    float rh[VEC], hnew[VEC];
+    ldv<VEC>(a.srhs + (size_t)j * RP + c0, rh);
+    const float ip = a.sinvP[j];
+#pragma unroll
+    for (int v = 0; v < VEC; ++v) {
+      hnew[v] = rh[v] + acc[v];
+      const float x = hnew[v] * ip, dx = (hnew[v] - hj[v]) * ip;
+      acc2[0][v] = fmaf(dx, dx, acc2[0][v]);
+      acc2[1][v] = fmaf(x, x, acc2[1][v]);
+    }
+    stv<VEC>(a.hfire + (size_t)j * RP + c0, hnew);
+  }
+}
+
+template <int VEC, int PASS>
+__global__ void __launch_bounds__(kBlock, GABP_KBS_MINB) kbs2_pass(ArgsBS a) {
+  DevCtl *ctl = a.ctl;
+  if (ctl->done) return;
+  float acc2[2][VEC];
+#pragma unroll
+  for (int v = 0; v < VEC; ++v) acc2[0][v] = acc2[1][v] = 0.f;
+  const int j0 = PASS == 0 ? a.n1 : 0, j1 = PASS == 0 ? a.n : a.n1;
+  if (PASS == 0 && ctl->round == 0) kbs2_rows<VEC, PASS, true>(a, j0, j1, acc2);
+  else kbs2_rows<VEC, PASS, false>(a, j0, j1, acc2);
+  kbs_finish<VEC>(a, acc2, PASS == 1);
 }
 
 // new-order rows of an [n][RP] FP32 array from the input order; the inner
 // solve starts with h~ = r
-__global__ void kbs_init(int n, int RP, const int *__restrict__ oid, const float *__restrict__ rhs,
+// (rows from n1 on: with 0, they have not fired)
+__global__ void kbs_init(int n, int n1, int RP, const int *__restrict__ oid, const float *__restrict__ rhs,
                          float *__restrict__ srhs, float *__restrict__ hfire) {
   const int lane = threadIdx.x & 31;
   const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -494,7 +627,7 @@ __global__ void kbs_init(int n, int RP, const int *__restrict__ oid, const float
     for (int r = lane; r < RP; r += 32) {
       const float v = rhs[src + r];
       srhs[dst + r] = v;
-      hfire[dst + r] = v;
+      hfire[dst + r] = j < n1 ? v : 0.f;
     }
   }
 }
@@ -543,7 +676,7 @@ __global__ void kb_ctl_reset(DevCtl *c, int max_iter, double tol2) {
 
 struct WorkB {
   int RP = 0;
-  float *H[2] = {nullptr, nullptr};
+  float *H = nullptr;
   float *NH[3] = {nullptr, nullptr, nullptr};
   float *rhs = nullptr;
   double *X = nullptr, *Bt = nullptr;
@@ -559,7 +692,7 @@ struct WorkB {
 void free_wb(gabp_handle h) {
   WorkB *w = h->wb;
   if (!w) return;
-  cudaFree(w->H[0]); cudaFree(w->H[1]);
+  cudaFree(w->H);
   for (int j = 0; j < 3; ++j) cudaFree(w->NH[j]);
   cudaFree(w->rhs); cudaFree(w->X); cudaFree(w->Bt); cudaFree(w->red); cudaFree(w->col); cudaFree(w->arrive);
   cudaFree(w->sH); cudaFree(w->hfire); cudaFree(w->srhs);
@@ -574,9 +707,7 @@ static gabp_status ensure_wb(gabp_handle h, int RP) {
   free_wb(h);
   h->wb = new WorkB();
   WorkB *w = h->wb;
-  const size_t E = (size_t)(h->g.E > 0 ? h->g.E : 1), n = (size_t)h->g.n;
-  GABP_CUDA(cudaMalloc(&w->H[0], sizeof(float) * E * RP));
-  GABP_CUDA(cudaMalloc(&w->H[1], sizeof(float) * E * RP));
+  const size_t n = (size_t)h->g.n;
   for (int j = 0; j < 3; ++j) GABP_CUDA(cudaMalloc(&w->NH[j], sizeof(float) * n * RP));
   GABP_CUDA(cudaMalloc(&w->rhs, sizeof(float) * n * RP));
   GABP_CUDA(cudaMalloc(&w->X, sizeof(double) * n * RP));
@@ -628,25 +759,32 @@ static gabp_status batched_chunk(gabp_handle h, int R, const double *B, double *
   std::vector<double> bb(R), rr(R);
   for (int r = 0; r < R; ++r) bb[r] = rr[r] = colh[r];
   ArgsB a;
-  a.n = g.n; a.RP = RP; a.rp = g.rp; a.ci = g.ci; a.CF = w32.CF; a.invP = w32.invP;
-  a.H0 = w.H[0]; a.H1 = w.H[1]; a.NH0 = w.NH[0]; a.NH1 = w.NH[1]; a.NH2 = w.NH[2];
+  const bool serial = h->opt.schedule == 1;
+  if (!serial && !w.H) GABP_CUDA(cudaMalloc(&w.H, sizeof(float) * E * RP));
+  a.n = g.n; a.RP = RP; a.rp = g.rp; a.ci = g.ci; a.rev = g.rev; a.CF = w32.CF; a.invP = w32.invP;
+  a.H = w.H; a.NH0 = w.NH[0]; a.NH1 = w.NH[1]; a.NH2 = w.NH[2];
   a.rhs = w.rhs; a.ctl = h->ctl; a.red = w.red; a.col = w.col;
   const double itol = h->opt.inner_tol;
-  const bool serial = h->opt.schedule == 1;
   ArgsBS as;
-  int nb_ser = 1;
+  int nb_ser = 1, nb_two[2] = {1, 1};
+  bool two = false;  // two colours
   if (serial) {
     if ((s = serial_freeze32(h, w32.CF, w32.invP)) != GABP_OK) return s;
     WorkS &ws = h->ws;
+    two = ws.C == 2;
+    as.n1 = two ? ws.cstart[1] : g.n;
+    as.e1 = two ? ws.srp_h[as.n1] : 0;
     if (!w.sH) {
-      GABP_CUDA(cudaMalloc(&w.sH, sizeof(float) * E * RP));
+      GABP_CUDA(cudaMalloc(&w.sH, sizeof(float) * (E - as.e1) * RP));
       GABP_CUDA(cudaMalloc(&w.hfire, sizeof(float) * g.n * RP));
       GABP_CUDA(cudaMalloc(&w.srhs, sizeof(float) * g.n * RP));
     }
     as.n = g.n; as.C = ws.C; as.RP = RP; as.co = ws.co; as.sci = ws.sci; as.scol = ws.scol; as.srp = ws.srp;
-    as.sCF = ws.sCF; as.sinvP = ws.sinvP; as.srhs = w.srhs; as.sH = w.sH; as.hfire = w.hfire;
+    as.srev = ws.srev; as.sCF = ws.sCF; as.sinvP = ws.sinvP; as.srhs = w.srhs; as.sH = w.sH; as.hfire = w.hfire;
     as.ctl = h->ctl; as.red = w.red; as.col = w.col;
     nb_ser = grid_of(kbs_pass<VEC>);
+    nb_two[0] = grid_of(kbs2_pass<VEC, 0>);
+    nb_two[1] = grid_of(kbs2_pass<VEC, 1>);
   }
   int total_inner = 0;
   auto all_done = [&]() {
@@ -656,7 +794,7 @@ static gabp_status batched_chunk(gabp_handle h, int R, const double *B, double *
   };
   bool diverged = false;
   for (int step = 0; step < h->opt.max_refine && !all_done() && total_inner < max_iter; ++step) {
-    GABP_CUDA(cudaMemsetAsync(serial ? w.sH : w.H[0], 0, sizeof(float) * E * RP, h->stream));
+    if (serial && !two) GABP_CUDA(cudaMemsetAsync(w.sH, 0, sizeof(float) * E * RP, h->stream));
     const int cap = std::min(h->opt.inner_max_iter, std::max(1, max_iter - total_inner));
     double worst_ratio = 0.0;  // the column furthest from its target sets the inner tolerance
     for (int r = 0; r < R; ++r)
@@ -664,11 +802,17 @@ static gabp_status batched_chunk(gabp_handle h, int R, const double *B, double *
     const double it_tol = inner_target(itol, tol, 1.0, worst_ratio);
     if (serial) {
       WorkS &ws = h->ws;
-      kbs_init<<<std::max(1, (g.n + 7) / 8), kBlock, 0, h->stream>>>(g.n, RP, ws.oid, w.rhs, w.srhs, w.hfire);
+      kbs_init<<<std::max(1, (g.n + 7) / 8), kBlock, 0, h->stream>>>(g.n, as.n1, RP, ws.oid, w.rhs, w.srhs,
+                                                                             w.hfire);
       kbs_ctl_reset<<<1, 1, 0, h->stream>>>(h->ctl, cap, it_tol * it_tol, w.col, RP);
       h->prof.launches += 2;
       GABP_CUDA(cudaGetLastError());
       s = run_rounds(h, &w.sgraph, &w.sgraph_key, RP | (ws.C << 16), [&] {
+        if (two) {
+          kbs2_pass<VEC, 0><<<nb_two[0], kBlock, shmem, h->stream>>>(as);
+          kbs2_pass<VEC, 1><<<nb_two[1], kBlock, shmem, h->stream>>>(as);
+          return;
+        }
         for (int c = 0; c < ws.C; ++c)
           kbs_pass<VEC><<<nb_ser, kBlock, shmem, h->stream>>>(as, c, ws.cstart[c], ws.cstart[c + 1] - ws.cstart[c]);
       }, cap, PH_MEAN32);
