@@ -44,7 +44,7 @@ struct DevCtl {
   int check_from;    // first round whose iterate may be accepted (1 for GaBP)
   int stable;        // consecutive rounds with a stationary precision set
   int cold;          // FP64 rounds: zero starting messages that are not in the store
-  int pad_;
+  int start;         // FP32 mean rounds: the round the run started from (0: zero messages)
   double bb;         // ||b||^2
   double tol2bb;     // tol^2 ||b||^2
   double rr;         // squared residual (or squared update) of the latest checked iterate
@@ -169,6 +169,11 @@ struct Work32 {
   DevCtl *ctlR = nullptr;                         // per-RHS control (refinement)
   int *rhs_active = nullptr;
   float2 *NQ[3] = {nullptr, nullptr, nullptr};    // [n] {P~, h~} ring of the joint rounds
+  // mean rounds of a dense matrix: [n][ld] coefficients and messages, partial column sums
+  float *dCin = nullptr, *dCout = nullptr, *dH = nullptr, *dSp = nullptr;
+  int dense_ld = 0;                               // row length there (0: those rounds do not run)
+  int dense_grid = 0;
+  bool dense_packed = false;                      // dCin, dCout hold CF
   struct RefineCtl *rc = nullptr;                 // device-resident refinement loop state
   struct RefineCtl *rc_host = nullptr;            // pinned copy read after a device-loop solve
   double *Bd = nullptr;                           // [n] right-hand side staged for the device loop

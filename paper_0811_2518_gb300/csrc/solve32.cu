@@ -76,6 +76,9 @@ void with_shape(int code, F &&f) {
 struct Args32 {
   int n;
   int dense;  // complete pattern (a dense matrix): k32_mean derives the sender from the slot
+  int ld;     // row length of the dense mean rounds' arrays (0: k32_mean runs the mean rounds)
+  float *Cin, *Cout, *Hd;  // [n][ld] coefficients c_in, c_out and stored messages of those rounds
+  float *Sp;               // [gridDim][ld] partial column sums
   const int *__restrict__ rp;
   const int *__restrict__ ci;
   const float *__restrict__ av;
@@ -353,6 +356,25 @@ __global__ void __launch_bounds__(kBlock) k32_coef(Args32 a, int T) {
   }
 }
 
+// The decision after mean round t, from the squared norms tot of its update and iterate.
+__device__ __forceinline__ void mean_decide(const Args32 &a, DevCtl *ctl, int t, const double (&tot)[2]) {
+  ctl->round = t;
+  ctl->rr = tot[0];
+  ctl->xx = tot[1];
+  if (ctl->no_stop) {
+    // autotuning run: no decision
+  } else if (!isfinite(tot[0]) || !isfinite(tot[1])) {
+    ctl->status = GABP_DIVERGED; ctl->iters = t; ctl->result_round = t; ctl->done = 1;
+  } else if (t >= 2 && tot[0] <= ctl->tol2bb * tot[1]) {
+    ctl->status = GABP_OK; ctl->iters = t; ctl->result_round = t; ctl->done = 1;
+  } else if (t >= ctl->max_iter) {
+    ctl->status = GABP_NOT_CONVERGED; ctl->iters = t; ctl->result_round = t; ctl->done = 1;
+  }
+  if (a.use_cond && ctl->done) cudaGraphSetConditional(a.cond, 0);
+  ctl->arrive = 0;
+  __threadfence();
+}
+
 // ---------------------------------------------------------------------------- mean phase, one RHS
 // Round t of the frozen-precision mean iteration (recompute form).  The inner
 // solve stops when ||x^(t) - x^(t-1)|| <= inner_tol ||x^(t)|| (node-local
@@ -425,22 +447,183 @@ __global__ void __launch_bounds__(kBlock) k32_mean(Args32 a) {
   const int modes[2] = {0, 0};
   block_sum<2>(v);
   if (last_block_reduce<2>(v, modes, a.partials, &ctl->arrive, tot) && threadIdx.x == 0) {
-    ctl->round = t;
-    ctl->rr = tot[0];
-    ctl->xx = tot[1];
-    if (ctl->no_stop) {
-      // autotuning run: no decision
-    } else if (!isfinite(tot[0]) || !isfinite(tot[1])) {
-      ctl->status = GABP_DIVERGED; ctl->iters = t; ctl->result_round = t; ctl->done = 1;
-    } else if (t >= 2 && tot[0] <= ctl->tol2bb * tot[1]) {
-      ctl->status = GABP_OK; ctl->iters = t; ctl->result_round = t; ctl->done = 1;
-    } else if (t >= ctl->max_iter) {
-      ctl->status = GABP_NOT_CONVERGED; ctl->iters = t; ctl->result_round = t; ctl->done = 1;
-    }
-    if (a.use_cond && ctl->done) cudaGraphSetConditional(a.cond, 0);
-    ctl->arrive = 0;
-    __threadfence();
+    mean_decide(a, ctl, t, tot);
   }
+}
+
+// ---------------------------------------------------------------------------- mean phase, dense matrix
+// Mean rounds of a complete pattern on full n x ld arrays (column k of row i at i ld + k; the diagonal
+// and the padding columns hold zeros, which make zero messages).  With every slot (i, k) come c_in =
+// c_ki and c_out = c_ik, so that what a column of the matrix sends needs no transposed access:
+//   write rounds     as k32_mean (recompute form): message k -> i of round t into slot (i, k); on the
+//                    way column k collects S_k = sum_i c_ik h_{k->i}^{(t)}, the messages' part of what
+//                    node k will receive next;
+//   product rounds   node i receives sum_k c_ki (h~_k^{(t)} - h_{i->k}^{(t)}) = sum_k c_ki h~_k^{(t)} - S_i:
+//                    a matrix-vector product with c_in alone, no message read or written.
+// The two alternate, so a pair of rounds moves 20 bytes a slot where k32_mean moves 32 (both
+// coefficients, message read and write, in every round).  HBM bounds both: 8192 points, 162 us a write
+// round (158 at the measured copy rate) and 50 us a product round (39), against 237 us with k32_mean.
+// A CTA owns a range of rows, 4 at a time; thread x owns columns 4 x, 4 x + 4 kBlock, ..., whose sums S
+// it keeps in shared memory; the CTAs' sums go to Sp and are added in CTA order.
+constexpr int kDenseRows = 4;  // rows whose loads are issued together
+// Smallest dense matrix of these rounds; below, the launches bound either.  Whole solves, k32_mean / these:
+// 300 points 3.0 / 2.6 ms, 800 4.4 / 3.0, 2000 9.4 / 4.5, 4096 24.5 / 9.7, 8192 54.3 / 27.9.
+constexpr int kDenseMin = 256;
+
+__device__ __forceinline__ int dense_group0(int n, int b, int nb) {  // first row group of CTA b
+  return (int)((int64_t)((n + kDenseRows - 1) / kDenseRows) * b / nb);
+}
+
+// c_in, c_out and, for an inner solve that starts from the joint rounds' state, the messages of its start
+// round from the row-CSR arrays; zeros on the diagonal and in the padding.
+__global__ void __launch_bounds__(kBlock) k32_dense_pack(Args32 a, int with_h) {
+  constexpr int U = 4;  // columns a thread whose loads are issued together
+  const float *__restrict__ Hs = (a.ctl->start & 1) ? a.H1 : a.H0;
+  for (int i = blockIdx.x; i < a.n; i += gridDim.x) {
+    const int64_t e0 = (int64_t)i * (a.n - 1), o = (int64_t)i * a.ld;
+    for (int k0 = threadIdx.x; k0 < a.ld; k0 += U * kBlock) {
+      float2 cf[U];
+      float hs[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int k = k0 + u * kBlock;
+        const bool in = k < a.n && k != i;
+        const int64_t e = e0 + k - (k > i);
+        cf[u] = in ? __ldcs(a.CF + e) : make_float2(0.f, 0.f);
+        hs[u] = in && with_h ? __ldcs(Hs + e) : 0.f;
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int k = k0 + u * kBlock;
+        if (k >= a.ld) break;
+        __stcs(a.Cin + o + k, cf[u].x);
+        __stcs(a.Cout + o + k, cf[u].y);
+        if (with_h) __stcs(a.Hd + o + k, hs[u]);
+      }
+    }
+  }
+}
+
+// The 4 rows from i0 of a write round: row sums into acc, column sums into cs (shared).  ZERO: the stored
+// messages are the zero ones a run starts from (not read).
+template <bool ZERO>
+__device__ __forceinline__ void dense_write_rows(const Args32 &a, int i0, const float *__restrict__ Hm1,
+                                                 const float *__restrict__ Hm2, float *cs, float (&acc)[kDenseRows]) {
+  float h2[kDenseRows];
+#pragma unroll
+  for (int r = 0; r < kDenseRows; ++r) h2[r] = Hm2[min(i0 + r, a.n - 1)];
+  for (int c = 4 * threadIdx.x; c < a.ld; c += 4 * kBlock) {
+    float4 ci[kDenseRows], co[kDenseRows], hs[kDenseRows];
+#pragma unroll
+    for (int r = 0; r < kDenseRows; ++r) {
+      const int64_t o = (int64_t)min(i0 + r, a.n - 1) * a.ld + c;
+      ci[r] = __ldcs(reinterpret_cast<const float4 *>(a.Cin + o));
+      co[r] = __ldcs(reinterpret_cast<const float4 *>(a.Cout + o));
+      hs[r] = ZERO ? make_float4(0.f, 0.f, 0.f, 0.f) : __ldcs(reinterpret_cast<const float4 *>(a.Hd + o));
+    }
+    const float4 hk = *reinterpret_cast<const float4 *>(Hm1 + c);
+    float4 s = *reinterpret_cast<const float4 *>(cs + c);
+#pragma unroll
+    for (int r = 0; r < kDenseRows; ++r) {
+      if (i0 + r >= a.n) break;
+      float4 hn;
+      hn.x = ci[r].x * (hk.x - co[r].x * (h2[r] - hs[r].x));
+      hn.y = ci[r].y * (hk.y - co[r].y * (h2[r] - hs[r].y));
+      hn.z = ci[r].z * (hk.z - co[r].z * (h2[r] - hs[r].z));
+      hn.w = ci[r].w * (hk.w - co[r].w * (h2[r] - hs[r].w));
+      __stcs(reinterpret_cast<float4 *>(a.Hd + (int64_t)(i0 + r) * a.ld + c), hn);
+      acc[r] += (hn.x + hn.y) + (hn.z + hn.w);
+      s.x = fmaf(co[r].x, hn.x, s.x);
+      s.y = fmaf(co[r].y, hn.y, s.y);
+      s.z = fmaf(co[r].z, hn.z, s.z);
+      s.w = fmaf(co[r].w, hn.w, s.w);
+    }
+    *reinterpret_cast<float4 *>(cs + c) = s;
+  }
+}
+
+// The 4 rows from i0 of a product round.
+__device__ __forceinline__ void dense_product_rows(const Args32 &a, int i0, const float *__restrict__ Hm1,
+                                                   float (&acc)[kDenseRows]) {
+  for (int c = 4 * threadIdx.x; c < a.ld; c += 4 * kBlock) {
+    float4 ci[kDenseRows];
+#pragma unroll
+    for (int r = 0; r < kDenseRows; ++r)
+      ci[r] = __ldcs(reinterpret_cast<const float4 *>(a.Cin + (int64_t)min(i0 + r, a.n - 1) * a.ld + c));
+    const float4 hk = *reinterpret_cast<const float4 *>(Hm1 + c);
+#pragma unroll
+    for (int r = 0; r < kDenseRows; ++r)
+      acc[r] += fmaf(ci[r].x, hk.x, ci[r].y * hk.y) + fmaf(ci[r].z, hk.z, ci[r].w * hk.w);
+  }
+}
+
+__global__ void __launch_bounds__(kBlock, 2) k32_dense(Args32 a) {
+  DevCtl *ctl = a.ctl;
+  if (ctl->done) return;
+  extern __shared__ __align__(16) float cs[];  // [ld] column sums of this CTA's rows
+  __shared__ float red[kDenseRows][kBlock / 32];
+  __shared__ float sfrom[kBlock / 32][32];
+  const int t = ctl->round + 1, start = ctl->start;
+  const bool write = ((t ^ start) & 1) == 0;
+  const float *__restrict__ Hm1 = ring3(a.NH0, a.NH1, a.NH2, t + 2);
+  const float *__restrict__ Hm2 = ring3(a.NH0, a.NH1, a.NH2, t + 1);
+  float *__restrict__ Ht = ring3(a.NH0, a.NH1, a.NH2, t);
+  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+  const int g0 = dense_group0(a.n, blockIdx.x, gridDim.x), g1 = dense_group0(a.n, blockIdx.x + 1, gridDim.x);
+  if (write)
+    for (int c = threadIdx.x; c < a.ld; c += kBlock) cs[c] = 0.f;  // each thread clears others' columns too
+  __syncthreads();
+  float dxx = 0.f, xx = 0.f;
+  for (int g = g0; g < g1; ++g) {
+    const int i0 = g * kDenseRows;
+    float acc[kDenseRows] = {};
+    if (!write) {
+      dense_product_rows(a, i0, Hm1, acc);
+      // S of every eighth group of 32 rows: lane = row, the warps share the CTAs' sums
+      if (t > 1 && ((g - g0) & 7) == 0) {
+        float sv = 0.f;
+        if (i0 + lane < a.ld)
+          for (int b = wib; b < (int)gridDim.x; b += kBlock / 32) sv += __ldcg(a.Sp + (int64_t)b * a.ld + i0 + lane);
+        __syncthreads();
+        sfrom[wib][lane] = sv;
+      }
+    } else if (t == 2 && start == 0) {
+      dense_write_rows<true>(a, i0, Hm1, Hm2, cs, acc);
+    } else {
+      dense_write_rows<false>(a, i0, Hm1, Hm2, cs, acc);
+    }
+#pragma unroll
+    for (int r = 0; r < kDenseRows; ++r) {
+      const float v = warp_sum(acc[r]);
+      if (lane == 0) red[r][wib] = v;
+    }
+    __syncthreads();
+    if (threadIdx.x < kDenseRows && i0 + (int)threadIdx.x < a.n) {
+      const int i = i0 + threadIdx.x;
+      float v = 0.f;
+#pragma unroll
+      for (int q = 0; q < kBlock / 32; ++q) v += red[threadIdx.x][q];
+      if (!write && t > 1) {
+        float sv = 0.f;
+#pragma unroll
+        for (int q = 0; q < kBlock / 32; ++q) sv += sfrom[q][kDenseRows * ((g - g0) & 7) + threadIdx.x];
+        v -= sv;
+      }
+      const float hnew = a.rhs[i] + v, ip = a.invP[i];
+      Ht[i] = hnew;
+      const float x = hnew * ip, dx = (hnew - Hm1[i]) * ip;
+      dxx = fmaf(dx, dx, dxx);
+      xx = fmaf(x, x, xx);
+    }
+    __syncthreads();
+  }
+  if (write)
+    for (int c = 4 * threadIdx.x; c < a.ld; c += 4 * kBlock)
+      *reinterpret_cast<float4 *>(a.Sp + (int64_t)blockIdx.x * a.ld + c) = *reinterpret_cast<const float4 *>(cs + c);
+  double v[2] = {(double)dxx, (double)xx}, tot[2];
+  const int modes[2] = {0, 0};
+  block_sum<2>(v);
+  if (last_block_reduce<2>(v, modes, a.partials, &ctl->arrive, tot) && threadIdx.x == 0) mean_decide(a, ctl, t, tot);
 }
 
 // ---------------------------------------------------------------------------- coefficient freeze
@@ -622,6 +805,7 @@ __global__ void k_diag32(int n, const double *__restrict__ ad, const double *__r
 
 __global__ void k_ctl_reset(DevCtl *c, int max_iter, double tol2, int round0 = 0) {
   c->round = round0;
+  c->start = round0;
   c->done = round0 > 0 && round0 >= max_iter;
   c->status = GABP_NOT_CONVERGED;
   c->iters = round0;
@@ -709,7 +893,11 @@ gabp_status ensure_w32(gabp_handle h, int R) {
     w.R = 0;
     GABP_CUDA(cudaMalloc(&w.H[0], sizeof(float) * E * R));
     GABP_CUDA(cudaMalloc(&w.H[1], sizeof(float) * E * R));
-    for (int j = 0; j < 3; ++j) GABP_CUDA(cudaMalloc(&w.NH[j], sizeof(float) * n * R));
+    for (int j = 0; j < 3; ++j) {  // room for the dense rounds' padding columns, finite values there
+      const size_t rows = (n + 31) / 32 * 32;
+      GABP_CUDA(cudaMalloc(&w.NH[j], sizeof(float) * rows * R));
+      GABP_CUDA(cudaMemsetAsync(w.NH[j], 0, sizeof(float) * rows * R, h->stream));
+    }
     GABP_CUDA(cudaMalloc(&w.rhs32, sizeof(float) * n * R));
     GABP_CUDA(cudaMalloc(&w.X, sizeof(double) * n * R));
     w.R = R;
@@ -732,6 +920,7 @@ void free_w32(gabp_handle h) {
   cudaFree(w.CF); cudaFree(w.invP); cudaFree(w.H[0]); cudaFree(w.H[1]);
   cudaFree(w.rhs32); cudaFree(w.X); cudaFree(w.Rs); cudaFree(w.Bt); cudaFree(w.colnorm);
   cudaFree(w.ctlR); cudaFree(w.rhs_active); cudaFree(w.rc); cudaFree(w.Bd);
+  cudaFree(w.dCin); cudaFree(w.dCout); cudaFree(w.dH); cudaFree(w.dSp);
   if (w.rc_host) cudaFreeHost(w.rc_host);
   w = Work32{};
 }
@@ -742,6 +931,7 @@ static Args32 args32(gabp_handle h) {
   Work32 &w = h->w32;
   a.n = g.n; a.rp = g.rp; a.ci = g.ci; a.av = g.av32; a.ad = g.ad32;
   a.dense = g.n > 1 && (int64_t)g.E == (int64_t)g.n * (g.n - 1);  // every off-diagonal entry stored
+  a.ld = w.dense_ld; a.Cin = w.dCin; a.Cout = w.dCout; a.Hd = w.dH; a.Sp = w.dSp;
   a.MP0 = w.MP[0]; a.MP1 = w.MP[1];
   a.NP0 = w.NP[0]; a.NP1 = w.NP[1]; a.NP2 = w.NP[2];
   a.CF = w.CF; a.invP = w.invP;
@@ -756,12 +946,48 @@ static Args32 args32(gabp_handle h) {
   return a;
 }
 
-// A mean round of shape (LL, UU) on stream st: the complete-pattern variant when the
-// matrix is dense.
+// The dense mean rounds' arrays (complete patterns of kDenseMin rows or more, unless the shape of the
+// round kernels is pinned): sets w.dense_ld when they run the mean rounds.
+static gabp_status ensure_dense32(gabp_handle h) {
+  Work32 &w = h->w32;
+  const Graph &g = h->g;
+  w.dense_ld = 0;
+  if (h->opt.lanes || g.n < kDenseMin || (int64_t)g.E != (int64_t)g.n * (g.n - 1)) return GABP_OK;
+  const int ld = (g.n + 31) / 32 * 32;
+  if (!w.dCin) {
+    const int smem = (int)sizeof(float) * ld;
+    int optin = 0, nb = 0;
+    cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, h->device);
+    constexpr int kStaticRoom = 4096;  // the kernel's static shared memory
+    if (smem > optin - kStaticRoom) return GABP_OK;
+    GABP_CUDA(cudaFuncSetAttribute(k32_dense, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - kStaticRoom));
+    GABP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k32_dense, kBlock, smem));
+    if (nb < 1) return GABP_OK;
+    const int grid = blocks_for(g.n, kDenseRows, std::min(nb * h->num_sms, h->max_blocks));
+    const size_t bytes = sizeof(float) * (size_t)g.n * ld;
+    if (cudaMalloc(&w.dCin, bytes) != cudaSuccess || cudaMalloc(&w.dCout, bytes) != cudaSuccess ||
+        cudaMalloc(&w.dH, bytes) != cudaSuccess ||
+        cudaMalloc(&w.dSp, sizeof(float) * (size_t)grid * ld) != cudaSuccess) {
+      cudaGetLastError();  // no room for them: k32_mean needs none
+      cudaFree(w.dCin); cudaFree(w.dCout); cudaFree(w.dH); cudaFree(w.dSp);
+      w.dCin = w.dCout = w.dH = w.dSp = nullptr;
+      return GABP_OK;
+    }
+    w.dense_grid = grid;
+    w.dense_packed = false;
+  }
+  w.dense_ld = ld;
+  return GABP_OK;
+}
+
+// A mean round of shape (LL, UU) on stream st: the dense rounds or the complete-pattern
+// variant when the matrix is dense.
 template <int LL, int UU>
 static void launch_mean(gabp_handle h, const Args32 &a, cudaStream_t st) {
   const int n = h->g.n;
-  if (a.dense)
+  if (a.ld)
+    k32_dense<<<h->w32.dense_grid, kBlock, sizeof(float) * a.ld, st>>>(a);
+  else if (a.dense)
     k32_mean<LL, UU, true><<<blocks_for(n, kBlock / LL, resident_grid(h->num_sms, k32_mean<LL, UU, true>)), kBlock, 0,
                              st>>>(a);
   else
@@ -866,6 +1092,7 @@ gabp_status precision_phase32(gabp_handle h, const double *gamma_diag) {
   GABP_CUDA(cudaGetLastError());
   w.prec_round = c.result_round;
   w.coef_ready = true;
+  w.dense_packed = false;
   return GABP_OK;
 }
 
@@ -926,12 +1153,24 @@ static gabp_status freeze32(gabp_handle h, int T) {
     k32_freeze<LL, UU><<<blocks_for(g.n, kBlock / LL, resident_grid(h->num_sms, k32_freeze<LL, UU>)), kBlock, 0,
                          h->stream>>>(a);
   });
+  if (a.ld) k32_dense_pack<<<blocks_for(g.n, 1, h->max_blocks), kBlock, 0, h->stream>>>(a, 1);
   prof_end(h);
   GABP_CUDA(cudaGetLastError());
   prof_collect(h, PH_FREEZE32, 1);
-  h->prof.launches += 1;
+  h->prof.launches += a.ld ? 2 : 1;
   w.prec_round = T;
   w.coef_ready = true;
+  w.dense_packed = a.ld > 0;
+  return GABP_OK;
+}
+
+// The packed coefficients for a solve that takes them as they are (no joint rounds).
+static gabp_status dense_pack(gabp_handle h) {
+  if (h->w32.dense_packed) return GABP_OK;
+  k32_dense_pack<<<blocks_for(h->g.n, 1, h->max_blocks), kBlock, 0, h->stream>>>(args32(h), 0);
+  GABP_CUDA(cudaGetLastError());
+  h->prof.launches += 1;
+  h->w32.dense_packed = true;
   return GABP_OK;
 }
 
@@ -970,6 +1209,7 @@ struct RefineParams {
 
 __device__ void ctl_arm(DevCtl *c, int round0, int max_iter, double tol2) {
   c->round = round0;
+  c->start = round0;
   c->done = round0 >= max_iter;
   c->status = GABP_NOT_CONVERGED;
   c->iters = round0;
@@ -1057,8 +1297,8 @@ constexpr int kLoopK = 2;
 // The joint rounds' while loop ran ceil(rounds / kLoopK) bodies; with the prep, the
 // joint-after, the freeze and this kernel: the launches of the joint block.  Marks
 // the round from which the first inner solve's loop continues.
-__global__ void k_joint_mark(RefineCtl *rc, const DevCtl *ctl) {
-  rc->launches += 2 + 2 + 1 + kLoopK * ((rc->joint_rounds + kLoopK - 1) / kLoopK);
+__global__ void k_joint_mark(RefineCtl *rc, const DevCtl *ctl, int pack) {
+  rc->launches += 2 + 2 + 1 + pack + kLoopK * ((rc->joint_rounds + kLoopK - 1) / kLoopK);
   rc->inner_start = ctl->round;
 }
 
@@ -1138,6 +1378,16 @@ static cudaError_t seq_conditional(SeqGraph &seq, cudaGraphConditionalHandle han
   return cudaSuccess;
 }
 
+// Lanes per row of the FP64 residual: narrow (its per-row epilogue is FP64), but enough to fill the GPU
+// where the rows are few and long (dense 8192 x 8192 matrix: 2 lanes 1.09 ms, 32 lanes 0.14).
+static int residual_lanes(gabp_handle h) {
+  if (h->opt.lanes) return h->opt.lanes;
+  const Graph &g = h->g;
+  int L = g.avg_deg >= 12.0 ? 2 : 1;
+  while (L < 32 && (int64_t)g.n * L < (int64_t)h->num_sms * 2048 && g.avg_deg >= 16.0 * L) L *= 2;
+  return L;
+}
+
 static gabp_status build_refine_graph(gabp_handle h, int SHm, int SHj, int LR) {
   Graph &g = h->g;
   Work32 &w = h->w32;
@@ -1173,13 +1423,16 @@ static gabp_status build_refine_graph(gabp_handle h, int SHm, int SHj, int LR) {
   SeqGraph outer{}, joint{}, jw{}, inner{};
   if (e == cudaSuccess) e = seq_conditional(top, h_outer, cudaGraphCondTypeWhile, &outer);
   if (e == cudaSuccess)
-    e = seq_capture(outer, st, [&] { cudaMemsetAsync(w.H[0], 0, sizeof(float) * E, st); });
+    e = seq_capture(outer, st, [&] {
+      if (!a.ld) cudaMemsetAsync(w.H[0], 0, sizeof(float) * E, st);
+    });
   // precision state computed together with the first inner solve
   if (e == cudaSuccess) e = seq_conditional(outer, h_joint, cudaGraphCondTypeIf, &joint);
   if (e == cudaSuccess)
     e = seq_capture(joint, st, [&] {
       cudaMemsetAsync(w.MP[0], 0, sizeof(float) * E, st);
       cudaMemsetAsync(w.MP[1], 0, sizeof(float) * E, st);
+      if (a.ld) cudaMemsetAsync(w.H[0], 0, sizeof(float) * E, st);
       k32_joint_init<<<nb1, kBlock, 0, st>>>(g.n, g.ad32, w.rhs32, w.NQ[0], w.NP[0]);
       k_joint_prep<<<1, 1, 0, st>>>(rc, h->ctl, h_jw);
     });
@@ -1207,7 +1460,8 @@ static gabp_status build_refine_graph(gabp_handle h, int SHm, int SHj, int LR) {
         k32_freeze<LL, UU><<<blocks_for(g.n, kBlock / LL, resident_grid(h->num_sms, k32_freeze<LL, UU>)), kBlock, 0,
                              st>>>(af);
       });
-      k_joint_mark<<<1, 1, 0, st>>>(rc, h->ctl);
+      if (a.ld) k32_dense_pack<<<blocks_for(g.n, 1, h->max_blocks), kBlock, 0, st>>>(af, 1);
+      k_joint_mark<<<1, 1, 0, st>>>(rc, h->ctl, a.ld ? 1 : 0);
     });
   // the inner solve's frozen-coefficient rounds
   if (e == cudaSuccess) e = seq_conditional(outer, h_inner, cudaGraphCondTypeWhile, &inner);
@@ -1250,9 +1504,12 @@ static gabp_status solve32_device_loop(gabp_handle h, const double *B, double *X
     GABP_CUDA(cudaMallocHost(&w.rc_host, sizeof(RefineCtl)));
     GABP_CUDA(cudaMalloc(&w.Bd, sizeof(double) * (size_t)g.n));
   }
+  gabp_status sd = ensure_dense32(h);
+  if (sd != GABP_OK) return sd;
   const bool joint = !w.coef_ready || !h->opt.reuse_precisions;
   if (joint) {
     w.coef_ready = false;
+    w.dense_packed = false;
     if (!h->opt.overlap_precision) {
       gabp_status s = precision_phase32(h, nullptr);
       if (s != GABP_OK) return s;
@@ -1273,11 +1530,12 @@ static gabp_status solve32_device_loop(gabp_handle h, const double *B, double *X
     }
   }
   const bool run_joint = joint && h->opt.overlap_precision;
-  gabp_status s = autotune32(h, K32_MEAN);
+  gabp_status s = w.dense_ld ? GABP_OK : autotune32(h, K32_MEAN);
   if (s != GABP_OK) return s;
+  if (w.dense_ld && !run_joint && (s = dense_pack(h)) != GABP_OK) return s;
   const int SHm = shape32(h, K32_MEAN), SHj = shape32(h, K32_JOINT);
-  const int LR = h->opt.lanes ? h->opt.lanes : (g.avg_deg >= 12.0 ? 2 : 1);
-  const long long key = (long long)SHm | ((long long)SHj << 16) | ((long long)LR << 32);
+  const int LR = residual_lanes(h);
+  const long long key = (long long)SHm | ((long long)SHj << 16) | ((long long)LR << 32) | ((long long)w.dense_ld << 40);
   if (!h->gRef || h->gRef_key != key) {
     if ((s = build_refine_graph(h, SHm, SHj, LR)) != GABP_OK) return s;
     h->gRef_key = key;
@@ -1304,6 +1562,7 @@ static gabp_status solve32_device_loop(gabp_handle h, const double *B, double *X
     if (r.prec_round >= 0) {
       w.prec_round = r.prec_round;
       w.coef_ready = true;
+      w.dense_packed = w.dense_ld > 0;
     } else if (r.status != GABP_BREAKDOWN && r.status != GABP_DIVERGED) {
       // stopped before any inner solve (b = 0): the precision state is still provided
       if ((s = precision_phase32(h, nullptr)) != GABP_OK) return s;
@@ -1335,8 +1594,11 @@ gabp_status solve32_refine(gabp_handle h, int R, const double *B, double *X, int
   // has to be computed, it is either computed first (precision-only rounds) or
   // together with the first inner solve (joint rounds, overlap_precision)
   bool joint = false;
+  if (serial) w.dense_ld = 0;
+  else if ((s = ensure_dense32(h)) != GABP_OK) return s;
   if (!w.coef_ready || gamma_diag || !h->opt.reuse_precisions) {
     w.coef_ready = false;
+    w.dense_packed = false;
     joint = h->opt.overlap_precision != 0 && !serial;
     if (!joint) {
       if ((s = precision_phase32(h, gamma_diag)) != GABP_OK) return s;
@@ -1344,10 +1606,10 @@ gabp_status solve32_refine(gabp_handle h, int R, const double *B, double *X, int
     }
   }
   if (serial && (s = serial_freeze32(h, w.CF, w.invP)) != GABP_OK) return s;  // coefficients in the serial order
-  if (!serial && (s = autotune32(h, K32_MEAN)) != GABP_OK) return s;
+  if (!serial && !w.dense_ld && (s = autotune32(h, K32_MEAN)) != GABP_OK) return s;
+  if (!serial && w.dense_ld && !joint && (s = dense_pack(h)) != GABP_OK) return s;
   const int SH = shape32(h, K32_MEAN);
-  // FP64 residual: narrow sub-warps (its per-row epilogue is FP64)
-  const int LR = h->opt.lanes ? h->opt.lanes : (g.avg_deg >= 12.0 ? 2 : 1);
+  const int LR = residual_lanes(h);
   int nbr = 1;
   GABP_DISPATCH_L(LR, nbr = blocks_for(g.n, kBlock / LL, resident_grid(h->num_sms, k64_residual<LL>)));
   GABP_CUDA(cudaMemsetAsync(X, 0, sizeof(double) * g.n, h->stream));
@@ -1411,7 +1673,7 @@ gabp_status solve32_refine(gabp_handle h, int R, const double *B, double *X, int
       h->prof.launches += 1;
       if ((s = freeze32(h, T)) != GABP_OK) return s;
       if (gamma_diag) w.coef_ready = false;  // do not reuse a loaded state for a plain solve
-    } else {
+    } else if (!w.dense_ld) {
       GABP_CUDA(cudaMemsetAsync(w.H[0], 0, sizeof(float) * E, h->stream));
     }
     int result_round = T;
@@ -1423,7 +1685,7 @@ gabp_status solve32_refine(gabp_handle h, int R, const double *B, double *X, int
       GABP_CUDA(cudaGetLastError());
       with_shape(SH, [&](auto Lc, auto Uc) {
         constexpr int LL = decltype(Lc)::value, UU = decltype(Uc)::value;
-        s = run_rounds(h, &h->gH32, &h->gH32_L, SH, [&] {
+        s = run_rounds(h, &h->gH32, &h->gH32_L, w.dense_ld ? -1 : SH, [&] {
           launch_mean<LL, UU>(h, a, h->stream);
         }, cap - T, PH_MEAN32, T > 0 ? T + 1 : 0);
       });
