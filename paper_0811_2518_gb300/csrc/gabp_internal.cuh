@@ -179,6 +179,19 @@ struct Work32 {
   double *Bd = nullptr;                           // [n] right-hand side staged for the device loop
 };
 
+// FP64 serial sweeps of two colours (serial2.cu) on a sliced layout of their own, colour 0's slices first.
+// Rows of colour 0 use N[0] and M[0]; rows of colour 1 N[1 + (t & 1)] and M[t & 1] in sweep t.
+struct WorkS2 {
+  Sell64 sl;
+  int ns0 = 0;                                       // slices of colour 0
+  double2 *M[2] = {nullptr, nullptr};                // [Es] messages {c, v}
+  NodeRec64 *N[3] = {nullptr, nullptr, nullptr};     // [n] node records
+  double *C = nullptr;                               // [Es] frozen coefficients (options.freeze_precisions)
+  double *b = nullptr;                               // [n] right-hand side of the captured sweeps
+  cudaGraphExec_t graph = nullptr;
+  long long graph_key = -1;
+};
+
 // Serial schedule (serial.cu): colouring, colour-grouped relabelling,
 // colour-sorted slot layout, state.
 struct WorkS {
@@ -213,6 +226,8 @@ struct WorkS {
   int chip_S = 0;              // slots of the largest CTA there
   bool valid = false;
   int result_round = 0;
+  WorkS2 two;                  // the sweeps of two colours
+  bool last_two = false;       // the last FP64 serial solve ran them
   float2 *sCF = nullptr;       // [E] frozen coefficients in serial order
   float *sH = nullptr;         // [E] FP32 mean messages
   float *hfire = nullptr;      // [n] FP32 firing aggregates h~
@@ -560,6 +575,13 @@ void free_ws(gabp_handle h);
 gabp_status serial_prepare(gabp_handle h);
 gabp_status serial_colours(gabp_handle h, int *colour_dev, int *ncolours);
 gabp_status serial_refresh_values(gabp_handle h);
+// serial2.cu: the FP64 sweeps of a graph of two colours; GABP_NOT_RUN where b = 0 (nothing was done)
+constexpr gabp_status GABP_NOT_RUN = (gabp_status)-100;
+gabp_status solve64_two_colours(gabp_handle h, const double *b, double *x, double tol, int max_iter, int *iters,
+                                double *relres);
+gabp_status two_colours_messages(gabp_handle h, double2 *M_input_layout);
+gabp_status two_colours_marginals(gabp_handle h, double *Pi);
+void free_serial2(WorkS &s);
 gabp_status solve64_serial(gabp_handle h, const double *b, double *x, double tol, int max_iter, int *iters,
                            double *relres);
 gabp_status serial_messages64(gabp_handle h, double2 *M_input_layout);

@@ -878,6 +878,7 @@ void free_ws(gabp_handle h) {
   cudaFree(s.SM); cudaFree(s.fire); cudaFree(s.sPm); cudaFree(s.sCF); cudaFree(s.sH); cudaFree(s.hfire);
   cudaFree(s.srhs); cudaFree(s.sinvP); cudaFree(s.bin); cudaFree(s.xin); cudaFree(s.sh1); cudaFree(s.sx0);
   cudaFree(s.sx1); cudaFree(s.coef); cudaFree(s.dcstart);
+  free_serial2(s);
   if (h->gS64) cudaGraphExecDestroy(h->gS64);
   if (h->gS32) cudaGraphExecDestroy(h->gS32);
   h->gS64 = h->gS32 = nullptr;
@@ -1022,6 +1023,7 @@ gabp_status serial_refresh_values(gabp_handle h) {
   WorkS &s = h->ws;
   if (!s.ready) return GABP_OK;
   Graph &g = h->g;
+  s.two.sl.vals_ok = false;
   if (g.E > 0)
     ks_refresh<<<(g.E + kBlock - 1) / kBlock, kBlock, 0, h->stream>>>(g.E, s.sperm, g.av, s.sav);
   ks_perm64<<<(g.n + kBlock - 1) / kBlock, kBlock, 0, h->stream>>>(g.n, s.oid, g.ad, s.sad);
@@ -1212,6 +1214,21 @@ gabp_status solve64_serial(gabp_handle h, const double *b, double *x, double tol
   Graph &g = h->g;
   WorkS &s = h->ws;
   const size_t Ea = (size_t)(g.E > 0 ? g.E : 1);
+  const int L = serial_lanes64(g);
+  const bool stf = h->opt.accel == 2;
+  if ((L == 1 || L == 2 || L == 4) && s.clu < 0) {
+    if (L == 1) serial_cluster_size<1>(h);
+    else if (L == 2) serial_cluster_size<2>(h);
+    else serial_cluster_size<4>(h);
+  }
+  // small graphs: every sweep in one thread-block cluster (Steffensen's step only with the state on chip)
+  const bool one_launch = (L == 1 || L == 2 || L == 4) && s.clu > 0 && (!stf || s.chip_bytes_stf > 0);
+  // larger graphs of two colours: two fused passes a sweep (serial2.cu)
+  s.last_two = false;
+  if (!one_launch && !stf && s.C == 2) {
+    st = solve64_two_colours(h, b, x, tol, max_iter, iters, relres);
+    if (st != GABP_NOT_RUN) return st;
+  }
   if (!s.SM) {
     GABP_CUDA(cudaMalloc(&s.SM, sizeof(double2) * Ea));
     GABP_CUDA(cudaMalloc(&s.fire, sizeof(double2) * g.n));
@@ -1244,7 +1261,6 @@ gabp_status solve64_serial(gabp_handle h, const double *b, double *x, double tol
   h->stats.refine_steps = 0;
   s.valid = true;
   s.result_round = 0;
-  const int L = serial_lanes64(g);
   if (bb == 0.0) {  // x = 0 after zero sweeps; P from the zero messages
     ks64_ctl<<<1, 1, 0, h->stream>>>(h->ctl, 1, 1.0, 0.0);
     GABP_DISPATCH_L(L, (ks64_final<LL><<<blocks_for(g.n, kBlock / LL, resident_grid(h->num_sms, ks64_final<LL>)),
@@ -1258,25 +1274,13 @@ gabp_status solve64_serial(gabp_handle h, const double *b, double *x, double tol
   }
   ks64_ctl<<<1, 1, 0, h->stream>>>(h->ctl, std::max(1, max_iter), bb, tol * tol);
   GABP_CUDA(cudaGetLastError());
-  const bool stf = h->opt.accel == 2;
   const int key = L | (s.C << 8) | (stf ? 1 << 30 : 0) | (a.freeze ? 1 << 29 : 0);
   gabp_status rs = GABP_OK;
-  // small graphs: every sweep in one thread-block cluster (Steffensen's step only with the state
-  // on chip)
-  bool one_launch = false;
-  if (L == 1 || L == 2 || L == 4) {
-    if (s.clu < 0) {
-      if (L == 1) serial_cluster_size<1>(h);
-      else if (L == 2) serial_cluster_size<2>(h);
-      else serial_cluster_size<4>(h);
-    }
-    one_launch = s.clu > 0 && (!stf || s.chip_bytes_stf > 0);
-    if (one_launch) {
-      const int ms = std::max(1, max_iter);
-      rs = L == 1 ? serial_cluster_dispatch<1>(h, a, ms)
-           : L == 2 ? serial_cluster_dispatch<2>(h, a, ms) : serial_cluster_dispatch<4>(h, a, ms);
-      if (rs != GABP_OK) return rs;
-    }
+  if (one_launch) {
+    const int ms = std::max(1, max_iter);
+    rs = L == 1 ? serial_cluster_dispatch<1>(h, a, ms)
+         : L == 2 ? serial_cluster_dispatch<2>(h, a, ms) : serial_cluster_dispatch<4>(h, a, ms);
+    if (rs != GABP_OK) return rs;
   }
   if (!one_launch) GABP_DISPATCH_L(L, {
     const int nb = blocks_for(g.n, kBlock / LL, resident_grid(h->num_sms, ks64_pass<LL>));
@@ -1307,6 +1311,7 @@ gabp_status solve64_serial(gabp_handle h, const double *b, double *x, double tol
 
 gabp_status serial_messages64(gabp_handle h, double2 *M_input_layout) {
   WorkS &s = h->ws;
+  if (s.last_two) return two_colours_messages(h, M_input_layout);
   if (!s.valid || !s.SM) return GABP_ERR_INVALID;
   if (h->g.E > 0)
     ks_unpermute<<<(h->g.E + kBlock - 1) / kBlock, kBlock, 0, h->stream>>>(h->g.E, s.sperm, s.SM, M_input_layout);
@@ -1316,6 +1321,7 @@ gabp_status serial_messages64(gabp_handle h, double2 *M_input_layout) {
 
 gabp_status serial_marginals64(gabp_handle h, double *Pi) {
   WorkS &s = h->ws;
+  if (s.last_two) return two_colours_marginals(h, Pi);
   if (!s.valid || !s.sPm) return GABP_ERR_INVALID;
   ks_unperm64<<<(h->g.n + kBlock - 1) / kBlock, kBlock, 0, h->stream>>>(h->g.n, s.oid, s.sPm, Pi);
   GABP_CUDA(cudaGetLastError());

@@ -38,7 +38,7 @@
 // 113; 309 us with 11 FP64 instructions a slot); 2^20 rows of degree 16: 250 us (FP64 195, HBM 131;
 // 505 us with 11 and with gathered reverse messages).
 #include "gabp_internal.cuh"
-#include "devutil.cuh"
+#include "sell64.cuh"
 #include "cluster.cuh"
 
 #include <cooperative_groups.h>
@@ -48,8 +48,6 @@
 #include <vector>
 
 namespace gabp {
-
-constexpr int kSellWindow = 4096;  // rows sorted by degree within windows of this many (a multiple of 32)
 
 // Slots per lane whose loads a round issues together, and the blocks per SM its register budget
 // is sized for (__launch_bounds__).  Recompute form on the 2^20 random graph of degree 16: 2 slots and
@@ -78,26 +76,6 @@ struct Args64 {
   int wide;    // plain node rounds of a matrix of long rows: k64_wide
   int rec;     // plain node rounds with a launch each: the recompute form
 };
-
-// Warp / lane of the calling thread and the number of warps in the grid.
-struct WarpPos {
-  int lane, warp, nwarps;
-};
-__device__ __forceinline__ WarpPos warp_pos() {
-  return WarpPos{(int)(threadIdx.x & 31), (int)((blockIdx.x * kBlock + threadIdx.x) >> 5),
-                 (int)((gridDim.x * kBlock) >> 5)};
-}
-
-// The slice a warp takes in its pass m over the grid (ns or more: none).  Inside a window of kSellWindow
-// rows the slices get narrower (rows sorted by degree), and a fixed stride would hand a warp slices of
-// like width in every pass (28 % of the round with idle warps on the 2^20 random graph); turning each
-// pass by the golden section of a window's 128 slices spreads every warp's slices over the window:
-// 347 -> 286 us per round there, unchanged on grids.
-__device__ __forceinline__ int pass_slice(const WarpPos &w, int m) {
-  constexpr int kSlices = kSellWindow / 32, kGolden = 79;  // 128 / 1.618
-  const int turn = (kGolden + kSlices - w.nwarps % kSlices) % kSlices;
-  return m * w.nwarps + (w.warp + m * turn) % w.nwarps;
-}
 
 // Round bookkeeping shared by the FP64 round kernels: this round checked
 // x^{(t-1)} with squared residual rr; 'bad' counts zero cavities / precisions
@@ -183,13 +161,6 @@ template <bool COOP> __device__ __forceinline__ NodeRec64 ld_rec(const NodeRec64
   return NodeRec64{q.x, q.y, q1.x, q1.y};
 }
 
-// Message k -> i of round t as {c, v} from node k's record at t-1 and the reverse message rv
-// (i -> k at t-1).  bad: a cavity precision P_{k\i} of exactly 0.
-__device__ __forceinline__ double2 message64(double A, const NodeRec64 &nk, const double2 &rv, int &bad) {
-  const double den = fma(A, rv.x, nk.P);  // cavity precision P_{k\i}
-  bad |= is_zero64(den);
-  return make_double2(div64(A, den), fma(rv.x, rv.y, nk.h));
-}
 // The reverse message i -> k of round t-1 by the same formula, from row i's aggregates at t-2
 // (P2, h2) and the slot's own in-message at t-2 (recompute form; its cavity was checked by row k).
 __device__ __forceinline__ double2 reverse64(double A, double P2, double h2, const double2 &m2) {
@@ -1223,67 +1194,111 @@ static void cluster_setup(gabp_handle h, const std::vector<int> &sp) {
   cudaGetLastError();
 }
 
+void sort_degree_windows(const std::vector<int> &rp, std::vector<int> &rows, size_t b, size_t e) {
+  std::vector<int> out, fill;
+  for (size_t w0 = b; w0 < e; w0 += kSellWindow) {
+    const size_t w1 = std::min(e, w0 + kSellWindow);
+    auto deg = [&](size_t q) { return rp[rows[q] + 1] - rp[rows[q]]; };
+    int lo = deg(w0), hi = lo;
+    for (size_t q = w0; q < w1; ++q) {
+      lo = std::min(lo, deg(q));
+      hi = std::max(hi, deg(q));
+    }
+    if (hi == lo) continue;
+    if (hi - lo > 4 * kSellWindow) {
+      std::stable_sort(rows.begin() + w0, rows.begin() + w1,
+                       [&](int x, int y) { return rp[x + 1] - rp[x] > rp[y + 1] - rp[y]; });
+      continue;
+    }
+    fill.assign(hi - lo + 2, 0);  // counting sort, the largest degree first
+    out.resize(w1 - w0);
+    for (size_t q = w0; q < w1; ++q) ++fill[hi - deg(q) + 1];
+    for (int d = 0; d <= hi - lo; ++d) fill[d + 1] += fill[d];
+    for (size_t q = w0; q < w1; ++q) out[fill[hi - deg(q)]++] = rows[q];
+    std::copy(out.begin(), out.end(), rows.begin() + w0);
+  }
+}
+
+gabp_status sell64_values(gabp_handle h, Sell64 &S) {
+  const Graph &g = h->g;
+  if (g.E > 0)
+    k_sell_rev_vals<<<(g.E + kBlock - 1) / kBlock, kBlock, 0, h->stream>>>(g.E, S.c2s, g.rev, g.av, S.srev, S.sav,
+                                                                             nullptr);
+  GABP_CUDA(cudaGetLastError());
+  S.vals_ok = true;
+  return GABP_OK;
+}
+
+void free_sell64(Sell64 &S) {
+  cudaFree(S.srow); cudaFree(S.sp); cudaFree(S.sci); cudaFree(S.srev); cudaFree(S.sav); cudaFree(S.c2s);
+  S = Sell64{};
+}
+
+gabp_status build_sell64(gabp_handle h, Sell64 &S, const std::vector<int> &rp, const std::vector<int> &srow,
+                         std::vector<int> *sp_out) {
+  const Graph &g = h->g;
+  const int E = g.E, ns = (int)(srow.size() / 32);
+  std::vector<int> sp((size_t)ns + 1, 0);
+  int64_t pos = 0;
+  for (int sl = 0; sl < ns; ++sl) {
+    sp[sl] = (int)pos;
+    int wd = 0;
+    for (int l = 0; l < 32; ++l) {
+      const int i = srow[(size_t)sl * 32 + l];
+      if (i >= 0) wd = std::max(wd, rp[i + 1] - rp[i]);
+    }
+    pos += 32 * (int64_t)wd;
+    if (pos >= INT32_MAX) {
+      set_last_error("FP64 rounds: the sliced layout does not fit int32 positions");
+      return GABP_ERR_INVALID;
+    }
+  }
+  sp[ns] = (int)pos;
+  S.ns = ns;
+  S.Es = (int)pos;
+  const size_t Ea = (size_t)std::max(S.Es, 1), Ec = (size_t)std::max(E, 1);
+  GABP_CUDA(cudaMalloc(&S.srow, sizeof(int) * srow.size()));
+  GABP_CUDA(cudaMalloc(&S.sp, sizeof(int) * sp.size()));
+  GABP_CUDA(cudaMalloc(&S.sci, sizeof(int) * Ea));
+  GABP_CUDA(cudaMalloc(&S.srev, sizeof(int) * Ea));
+  GABP_CUDA(cudaMalloc(&S.sav, sizeof(double) * Ea));
+  GABP_CUDA(cudaMalloc(&S.c2s, sizeof(int) * Ec));
+  GABP_CUDA(cudaMemcpyAsync(S.srow, srow.data(), sizeof(int) * srow.size(), cudaMemcpyHostToDevice, h->stream));
+  GABP_CUDA(cudaMemcpyAsync(S.sp, sp.data(), sizeof(int) * sp.size(), cudaMemcpyHostToDevice, h->stream));
+  GABP_CUDA(cudaMemsetAsync(S.sci, 0xff, sizeof(int) * Ea, h->stream));  // -1: padding
+  GABP_CUDA(cudaMemsetAsync(S.srev, 0, sizeof(int) * Ea, h->stream));
+  GABP_CUDA(cudaMemsetAsync(S.sav, 0, sizeof(double) * Ea, h->stream));
+  const int nq = ns * 32;
+  k_sell_fill<<<(nq + kBlock - 1) / kBlock, kBlock, 0, h->stream>>>(nq, S.srow, S.sp, g.rp, g.ci, S.c2s, S.sci);
+  unsigned far = 0;
+  unsigned *dfar = &h->ctl->arrive;  // the control block is idle here; every run clears it
+  GABP_CUDA(cudaMemsetAsync(dfar, 0, sizeof(unsigned), h->stream));
+  if (E > 0)
+    k_sell_rev_vals<<<(E + kBlock - 1) / kBlock, kBlock, 0, h->stream>>>(E, S.c2s, g.rev, g.av, S.srev, S.sav, dfar);
+  GABP_CUDA(cudaGetLastError());
+  GABP_CUDA(cudaMemcpyAsync(&far, dfar, sizeof(unsigned), cudaMemcpyDeviceToHost, h->stream));
+  GABP_CUDA(cudaMemsetAsync(dfar, 0, sizeof(unsigned), h->stream));
+  GABP_CUDA(cudaStreamSynchronize(h->stream));  // the host vectors are released on return
+  S.far = far;
+  S.ready = true;
+  S.vals_ok = true;
+  if (sp_out) *sp_out = sp;
+  return GABP_OK;
+}
+
 static gabp_status ensure_sell64(gabp_handle h) {
   Sell64 &S = h->w64.sl;
   Graph &g = h->g;
-  const int n = g.n, E = g.E;
+  const int n = g.n;
   if (!S.ready) {
-    std::vector<int> rp((size_t)n + 1);
+    std::vector<int> rp((size_t)n + 1), sp;
     GABP_CUDA(cudaMemcpy(rp.data(), g.rp, sizeof(int) * rp.size(), cudaMemcpyDeviceToHost));
     const int ns = (n + 31) / 32;
-    std::vector<int> srow((size_t)ns * 32, -1), sp((size_t)ns + 1, 0);
-    std::vector<int> idx;
-    for (int w0 = 0; w0 < n; w0 += kSellWindow) {  // a window is a whole number of slices
-      const int w1 = std::min(n, w0 + kSellWindow);
-      idx.resize(w1 - w0);
-      for (int i = w0; i < w1; ++i) idx[i - w0] = i;
-      std::stable_sort(idx.begin(), idx.end(),
-                       [&](int x, int y) { return rp[x + 1] - rp[x] > rp[y + 1] - rp[y]; });
-      std::copy(idx.begin(), idx.end(), srow.begin() + w0);
-    }
-    int64_t pos = 0;
-    for (int sl = 0; sl < ns; ++sl) {
-      sp[sl] = (int)pos;
-      int wd = 0;
-      for (int l = 0; l < 32; ++l) {
-        const int i = srow[(size_t)sl * 32 + l];
-        if (i >= 0) wd = std::max(wd, rp[i + 1] - rp[i]);
-      }
-      pos += 32 * (int64_t)wd;
-      if (pos >= INT32_MAX) {
-        set_last_error("FP64 rounds: the sliced layout does not fit int32 positions");
-        return GABP_ERR_INVALID;
-      }
-    }
-    sp[ns] = (int)pos;
-    S.ns = ns;
-    S.Es = (int)pos;
-    const size_t Ea = (size_t)std::max(S.Es, 1), Ec = (size_t)std::max(E, 1);
-    GABP_CUDA(cudaMalloc(&S.srow, sizeof(int) * srow.size()));
-    GABP_CUDA(cudaMalloc(&S.sp, sizeof(int) * sp.size()));
-    GABP_CUDA(cudaMalloc(&S.sci, sizeof(int) * Ea));
-    GABP_CUDA(cudaMalloc(&S.srev, sizeof(int) * Ea));
-    GABP_CUDA(cudaMalloc(&S.sav, sizeof(double) * Ea));
-    GABP_CUDA(cudaMalloc(&S.c2s, sizeof(int) * Ec));
-    GABP_CUDA(cudaMemcpyAsync(S.srow, srow.data(), sizeof(int) * srow.size(), cudaMemcpyHostToDevice, h->stream));
-    GABP_CUDA(cudaMemcpyAsync(S.sp, sp.data(), sizeof(int) * sp.size(), cudaMemcpyHostToDevice, h->stream));
-    GABP_CUDA(cudaMemsetAsync(S.sci, 0xff, sizeof(int) * Ea, h->stream));  // -1: padding
-    GABP_CUDA(cudaMemsetAsync(S.srev, 0, sizeof(int) * Ea, h->stream));
-    GABP_CUDA(cudaMemsetAsync(S.sav, 0, sizeof(double) * Ea, h->stream));
-    const int nq = ns * 32;
-    k_sell_fill<<<(nq + kBlock - 1) / kBlock, kBlock, 0, h->stream>>>(nq, S.srow, S.sp, g.rp, g.ci, S.c2s, S.sci);
-    unsigned far = 0;
-    unsigned *dfar = &h->ctl->arrive;  // the control block is idle here; every run clears it
-    GABP_CUDA(cudaMemsetAsync(dfar, 0, sizeof(unsigned), h->stream));
-    if (E > 0)
-      k_sell_rev_vals<<<(E + kBlock - 1) / kBlock, kBlock, 0, h->stream>>>(E, S.c2s, g.rev, g.av, S.srev, S.sav, dfar);
-    GABP_CUDA(cudaGetLastError());
-    GABP_CUDA(cudaMemcpyAsync(&far, dfar, sizeof(unsigned), cudaMemcpyDeviceToHost, h->stream));
-    GABP_CUDA(cudaMemsetAsync(dfar, 0, sizeof(unsigned), h->stream));
-    GABP_CUDA(cudaStreamSynchronize(h->stream));  // the host vectors are released on return
-    S.far = far;
-    S.ready = true;
-    S.vals_ok = true;
+    std::vector<int> srow((size_t)ns * 32, -1);
+    for (int i = 0; i < n; ++i) srow[i] = i;
+    sort_degree_windows(rp, srow, 0, n);  // a window is a whole number of slices
+    const gabp_status bs = build_sell64(h, S, rp, srow, &sp);
+    if (bs != GABP_OK) return bs;
     h->tuned_L64 = 1;  // one row per lane
     // one cluster of up to 16 CTAs (a slice per warp) for the smallest graphs, its state on chip
     // where it fits
@@ -1313,11 +1328,7 @@ static gabp_status ensure_sell64(gabp_handle h) {
       cudaGetLastError();
     }
   } else if (!S.vals_ok) {
-    if (E > 0)
-      k_sell_rev_vals<<<(E + kBlock - 1) / kBlock, kBlock, 0, h->stream>>>(E, S.c2s, g.rev, g.av, S.srev, S.sav,
-                                                                           nullptr);
-    GABP_CUDA(cudaGetLastError());
-    S.vals_ok = true;
+    return sell64_values(h, S);
   }
   return GABP_OK;
 }
@@ -1338,8 +1349,7 @@ gabp_status ensure_w64(gabp_handle h) {
 void free_w64(gabp_handle h) {
   Work64 &w = h->w64;
   cudaFree(w.M[0]); cudaFree(w.M[1]); cudaFree(w.N[0]); cudaFree(w.N[1]); cudaFree(w.bar); cudaFree(w.C);
-  Sell64 &S = w.sl;
-  cudaFree(S.srow); cudaFree(S.sp); cudaFree(S.sci); cudaFree(S.srev); cudaFree(S.sav); cudaFree(S.c2s);
+  free_sell64(w.sl);
   w = Work64{};
 }
 
