@@ -121,9 +121,8 @@ __global__ void __launch_bounds__(kBlock) ksl_decide(ArgsSL a) {
     }
   }
   double v[1] = {rr}, tot[1];
-  const int modes[1] = {0};
   block_sum<1>(v);
-  if (last_block_reduce<1>(v, modes, a.partials, &ctl->arrive, tot) && threadIdx.x == 0) {
+  if (last_block_reduce<1>(v, a.partials, &ctl->arrive, tot) && threadIdx.x == 0) {
     const int t = ctl->round + 1;
     ctl->round = t;
     ctl->rr = tot[0];
@@ -145,9 +144,8 @@ __global__ void ksl_bb(int n, const double *__restrict__ b, DevCtl *ctl, double 
   double sacc = 0.0;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) sacc = fma(b[i], b[i], sacc);
   double v[1] = {sacc}, tot[1];
-  const int modes[1] = {0};
   block_sum<1>(v);
-  if (last_block_reduce<1>(v, modes, partials, &ctl->arrive, tot) && threadIdx.x == 0) {
+  if (last_block_reduce<1>(v, partials, &ctl->arrive, tot) && threadIdx.x == 0) {
     ctl->round = 0;
     ctl->done = tot[0] == 0.0;
     ctl->status = tot[0] == 0.0 ? GABP_OK : GABP_NOT_CONVERGED;

@@ -41,9 +41,8 @@ __global__ void __launch_bounds__(kBlock) k_ig_residual(int n, const int *__rest
     }
   }
   double v[2] = {rr, bb}, tot[2];
-  const int modes[2] = {0, 0};
   block_sum<2>(v);
-  if (last_block_reduce<2>(v, modes, partials, arrive, tot) && threadIdx.x == 0) {
+  if (last_block_reduce<2>(v, partials, arrive, tot) && threadIdx.x == 0) {
     sums[0] = tot[0];
     sums[1] = tot[1];
     *arrive = 0;

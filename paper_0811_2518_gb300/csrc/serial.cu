@@ -339,9 +339,8 @@ __global__ void __launch_bounds__(kBlock) ks64_decide(ArgsS64 a) {
   const int warp = (blockIdx.x * kBlock + threadIdx.x) >> 5;
   const int nwarps = (gridDim.x * kBlock) >> 5;
   double v[1] = {s64_resid_rows<L, false>(a, warp, nwarps)}, tot[1];
-  const int modes[1] = {0};
   block_sum<1>(v);
-  if (last_block_reduce<1>(v, modes, a.partials, &ctl->arrive, tot) && threadIdx.x == 0) {
+  if (last_block_reduce<1>(v, a.partials, &ctl->arrive, tot) && threadIdx.x == 0) {
     const int t = ctl->round + 1;
     ctl->round = t;
     ctl->rr = tot[0];
@@ -643,9 +642,8 @@ __global__ void __launch_bounds__(kBlock) ks64_steff_a(ArgsS64 a, int E) {
     sDD = fma(D, D, sDD);
   }
   double v[2] = {sdD, sDD}, tot[2];
-  const int modes[2] = {0, 0};
   block_sum<2>(v);
-  if (last_block_reduce<2>(v, modes, a.partials, &ctl->arrive, tot) && threadIdx.x == 0) {
+  if (last_block_reduce<2>(v, a.partials, &ctl->arrive, tot) && threadIdx.x == 0) {
     const double lam = tot[1] > 0.0 ? tot[0] / tot[1] : 0.0;
     ctl->lam = isfinite(lam) ? lam : 0.0;
     ctl->arrive = 0;
@@ -714,9 +712,8 @@ __global__ void ks_bb(int n, const double *__restrict__ b, DevCtl *ctl, double *
   double s = 0.0;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) s = fma(b[i], b[i], s);
   double v[1] = {s}, tot[1];
-  const int modes[1] = {0};
   block_sum<1>(v);
-  if (last_block_reduce<1>(v, modes, partials, &ctl->arrive, tot) && threadIdx.x == 0) {
+  if (last_block_reduce<1>(v, partials, &ctl->arrive, tot) && threadIdx.x == 0) {
     ctl->bb = tot[0];
     ctl->arrive = 0;
     __threadfence();
@@ -821,9 +818,8 @@ __global__ void __launch_bounds__(kBlock) ks32_pass(ArgsS32 a, int c, int skip0,
     }
   }
   double v[2] = {(double)dxx, (double)xx}, tot[2];
-  const int modes[2] = {0, 0};
   block_sum<2>(v);
-  if (last_block_reduce<2>(v, modes, a.partials, &ctl->arrive, tot) && threadIdx.x == 0) {
+  if (last_block_reduce<2>(v, a.partials, &ctl->arrive, tot) && threadIdx.x == 0) {
     ctl->rr += tot[0];
     ctl->xx += tot[1];
     if (c == a.C - 1) {  // the sweep is complete

@@ -148,9 +148,8 @@ __global__ void __launch_bounds__(kBlock, MODE == 2 ? 3 : kMinBlocks2) ks2_pass(
   if (w.lane == 0 && fb) atomicOr(&ctl->edge_bad, (int)fb);
   if (w.lane == 0 && fm) atomicOr(&ctl->fmove, 1);
   double v[1] = {rr}, tot[1];
-  const int modes[1] = {0};
   block_sum<1>(v);
-  if (last_block_reduce<1>(v, modes, a.partials, &ctl->arrive, tot) && threadIdx.x == 0) {
+  if (last_block_reduce<1>(v, a.partials, &ctl->arrive, tot) && threadIdx.x == 0) {
     ctl->stable = 1 - PASS;  // the pass to come (the freeze's state may change after pass 1: not another of its modes)
     if (PASS == 1) {  // the sweep is complete but for the residual of colour 1
       ctl->round = t;
@@ -197,9 +196,8 @@ __global__ void __launch_bounds__(kBlock) ks2_init(ArgsS2 a, const double *__res
     bb = fma(bi, bi, bb);
   }
   double v[1] = {bb}, tot[1];
-  const int modes[1] = {0};
   block_sum<1>(v);
-  if (last_block_reduce<1>(v, modes, a.partials, &a.ctl->arrive, tot) && threadIdx.x == 0) {
+  if (last_block_reduce<1>(v, a.partials, &a.ctl->arrive, tot) && threadIdx.x == 0) {
     DevCtl *c = a.ctl;
     c->bb = tot[0];
     c->tol2bb = tol * tol * tot[0];

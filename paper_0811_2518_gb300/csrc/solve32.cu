@@ -183,8 +183,7 @@ __global__ void __launch_bounds__(kBlock) k32_prec(Args32 a) {
   }
   double v[3] = {(double)bad, (double)moving, (double)nonfinite}, tot[3];
   block_sum<3>(v);
-  const int modes[3] = {0, 0, 0};
-  if (last_block_reduce<3>(v, modes, a.partials, &ctl->arrive, tot) && threadIdx.x == 0) {
+  if (last_block_reduce<3>(v, a.partials, &ctl->arrive, tot) && threadIdx.x == 0) {
     ctl->round = t;
     ctl->maxrel = tot[1];                      // messages that moved by more than 2^-s
     ctl->stable = tot[1] == 0.0 ? ctl->stable + 1 : 0;
@@ -298,8 +297,7 @@ __global__ void __launch_bounds__(kBlock, 4) k32_joint(Args32 a) {
   }
   double v[3] = {(double)bad, (double)moving, (double)nonfinite}, tot[3];
   block_sum<3>(v);
-  const int modes[3] = {0, 0, 0};
-  if (last_block_reduce<3>(v, modes, a.partials, &ctl->arrive, tot) && threadIdx.x == 0) {
+  if (last_block_reduce<3>(v, a.partials, &ctl->arrive, tot) && threadIdx.x == 0) {
     ctl->round = t;
     ctl->maxrel = tot[1];                      // messages that moved by more than 2^-s
     ctl->stable = tot[1] == 0.0 ? ctl->stable + 1 : 0;
@@ -444,9 +442,8 @@ __global__ void __launch_bounds__(kBlock) k32_mean(Args32 a) {
     }
   }
   double v[2] = {(double)dxx, (double)xx}, tot[2];
-  const int modes[2] = {0, 0};
   block_sum<2>(v);
-  if (last_block_reduce<2>(v, modes, a.partials, &ctl->arrive, tot) && threadIdx.x == 0) {
+  if (last_block_reduce<2>(v, a.partials, &ctl->arrive, tot) && threadIdx.x == 0) {
     mean_decide(a, ctl, t, tot);
   }
 }
@@ -621,9 +618,8 @@ __global__ void __launch_bounds__(kBlock, 2) k32_dense(Args32 a) {
     for (int c = 4 * threadIdx.x; c < a.ld; c += 4 * kBlock)
       *reinterpret_cast<float4 *>(a.Sp + (int64_t)blockIdx.x * a.ld + c) = *reinterpret_cast<const float4 *>(cs + c);
   double v[2] = {(double)dxx, (double)xx}, tot[2];
-  const int modes[2] = {0, 0};
   block_sum<2>(v);
-  if (last_block_reduce<2>(v, modes, a.partials, &ctl->arrive, tot) && threadIdx.x == 0) mean_decide(a, ctl, t, tot);
+  if (last_block_reduce<2>(v, a.partials, &ctl->arrive, tot) && threadIdx.x == 0) mean_decide(a, ctl, t, tot);
 }
 
 // ---------------------------------------------------------------------------- coefficient freeze
@@ -705,9 +701,8 @@ __global__ void __launch_bounds__(kBlock) k32_freeze(Args32 a) {
   }
   if (coef_only) return;
   double v[2] = {(double)dxx, (double)xx}, tot[2];
-  const int modes[2] = {0, 0};
   block_sum<2>(v);
-  if (last_block_reduce<2>(v, modes, a.partials, &ctl->arrive, tot) && threadIdx.x == 0) {
+  if (last_block_reduce<2>(v, a.partials, &ctl->arrive, tot) && threadIdx.x == 0) {
     ctl->round = t;
     ctl->rr = tot[0];
     ctl->xx = tot[1];
@@ -773,9 +768,8 @@ __global__ void __launch_bounds__(kBlock) k64_residual(int n, const int *__restr
     }
   }
   double v[1] = {rr}, tot[1];
-  const int modes[1] = {0};
   block_sum<1>(v);
-  if (last_block_reduce<1>(v, modes, partials, &ctl->arrive, tot) && threadIdx.x == 0) {
+  if (last_block_reduce<1>(v, partials, &ctl->arrive, tot) && threadIdx.x == 0) {
     ctl->rr = tot[0];
     if (set_bb) {
       ctl->bb = tot[0];
@@ -958,9 +952,11 @@ static gabp_status ensure_dense32(gabp_handle h) {
     const int smem = (int)sizeof(float) * ld;
     int optin = 0, nb = 0;
     cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, h->device);
-    constexpr int kStaticRoom = 4096;  // the kernel's static shared memory
-    if (smem > optin - kStaticRoom) return GABP_OK;
-    GABP_CUDA(cudaFuncSetAttribute(k32_dense, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - kStaticRoom));
+    cudaFuncAttributes fa;
+    GABP_CUDA(cudaFuncGetAttributes(&fa, k32_dense));
+    const int room = optin - (int)fa.sharedSizeBytes;  // beside the kernel's static shared memory
+    if (smem > room) return GABP_OK;
+    GABP_CUDA(cudaFuncSetAttribute(k32_dense, cudaFuncAttributeMaxDynamicSharedMemorySize, room));
     GABP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k32_dense, kBlock, smem));
     if (nb < 1) return GABP_OK;
     const int grid = blocks_for(g.n, kDenseRows, std::min(nb * h->num_sms, h->max_blocks));

@@ -299,9 +299,8 @@ __global__ void __launch_bounds__(kBlock) k64_init(Args64 a, double tol, int max
     bb = fma(bi, bi, bb);
   }
   double v[1] = {bb}, tot[1];
-  const int modes[1] = {0};
   block_sum<1>(v);
-  if (last_block_reduce<1>(v, modes, a.partials, &a.ctl->arrive, tot) && threadIdx.x == 0) {
+  if (last_block_reduce<1>(v, a.partials, &a.ctl->arrive, tot) && threadIdx.x == 0) {
     DevCtl *c = a.ctl;
     c->round = 0;
     c->bb = tot[0];
@@ -367,13 +366,11 @@ __device__ __forceinline__ void plain_round(const Args64 &a, DevCtl *ctl, int t,
   else rows(std::integral_constant<RevFrom, REC && MODE < 2 ? kRecZero : kGather>());
   constexpr int NV = MODE > 0 ? 3 : 2;  // the moving count only when the freeze is on
   double v[NV], tot[NV];
-  int modes[NV];
   v[0] = rr;
   v[1] = (double)bad;
   if constexpr (NV > 2) v[2] = (double)moving;
-  for (int q = 0; q < NV; ++q) modes[q] = 0;
   block_sum<NV>(v);
-  if (last_block_reduce<NV>(v, modes, a.partials, &ctl->arrive, tot) && threadIdx.x == 0) {
+  if (last_block_reduce<NV>(v, a.partials, &ctl->arrive, tot) && threadIdx.x == 0) {
     if constexpr (MODE > 0) freeze_step(ctl, MODE - 1, t, tot[2]);
     decide64(ctl, t, tot[0], tot[1]);
   }
@@ -439,9 +436,8 @@ __global__ void __launch_bounds__(kBlock) k64_wide(Args64 a) {
     }
   }
   double v[2] = {rr, (double)bad}, tot[2];
-  const int modes[2] = {0, 0};
   block_sum<2>(v);
-  if (last_block_reduce<2>(v, modes, a.partials, &ctl->arrive, tot) && threadIdx.x == 0) decide64(ctl, t, tot[0], tot[1]);
+  if (last_block_reduce<2>(v, a.partials, &ctl->arrive, tot) && threadIdx.x == 0) decide64(ctl, t, tot[0], tot[1]);
 }
 
 // The plain round with the precision freeze on: MODE 1 (screen), 2 (verify and store)
@@ -548,9 +544,8 @@ __global__ void __launch_bounds__(kBlock, ACC ? 3 : kMinBlocks64) k64_node(Args6
   }
   if (STF) {
     double v[4] = {rr, (double)bad, sdD, sDD}, tot[4];
-    const int modes[4] = {0, 0, 0, 0};
     block_sum<4>(v);
-    if (last_block_reduce<4>(v, modes, a.partials, &ctl->arrive, tot) && threadIdx.x == 0) {
+    if (last_block_reduce<4>(v, a.partials, &ctl->arrive, tot) && threadIdx.x == 0) {
       if (!(t & 1)) {  // the cycle's scalar step; 0 where nothing moves or the quotient is not finite
         const double lam = tot[3] > 0.0 ? tot[2] / tot[3] : 0.0;
         ctl->lam = isfinite(lam) ? lam : 0.0;
@@ -560,9 +555,8 @@ __global__ void __launch_bounds__(kBlock, ACC ? 3 : kMinBlocks64) k64_node(Args6
     return;
   }
   double v[2] = {rr, (double)bad}, tot[2];
-  const int modes[2] = {0, 0};
   block_sum<2>(v);
-  if (last_block_reduce<2>(v, modes, a.partials, &ctl->arrive, tot) && threadIdx.x == 0)
+  if (last_block_reduce<2>(v, a.partials, &ctl->arrive, tot) && threadIdx.x == 0)
     decide64(ctl, t, tot[0], tot[1]);
 }
 
@@ -1041,9 +1035,8 @@ __global__ void __launch_bounds__(kBlock) k64_edge_agg(Args64 a) {
     }
   }
   double v[2] = {rr, (double)bad}, tot[2];
-  const int modes[2] = {0, 0};
   block_sum<2>(v);
-  if (last_block_reduce<2>(v, modes, a.partials, &ctl->arrive, tot) && threadIdx.x == 0) {
+  if (last_block_reduce<2>(v, a.partials, &ctl->arrive, tot) && threadIdx.x == 0) {
     const double eb = ctl->edge_bad ? 1.0 : 0.0;
     ctl->edge_bad = 0;
     decide64(ctl, t, tot[0], tot[1] + eb);
