@@ -271,16 +271,18 @@ gabp_status gabp_solve_batched(gabp_handle h, int32_t nrhs, const double *B, dou
                                double tol, int32_t max_iter, int32_t *iters_out, double *relres_out);
 
 /*
- * gabp_solve_systems -- solve nsys independent systems in ONE persistent launch.
+ * gabp_solve_systems -- solve nsys independent systems in one persistent launch, or two.
  * The handle's A must be block diagonal: system s owns rows and columns
  * [offsets[s], offsets[s+1]) (host array of nsys+1 ints, offsets[0] = 0,
  * offsets[nsys] = n, strictly increasing); an entry coupling two systems gives
  * GABP_ERR_INVALID.  b, x: device arrays of n doubles.  Every system runs its own
  * FP32 precision phase, FP32 mean rounds and FP64 refinement to
  * ||b_s - A_s x_s|| <= tol ||b_s|| (the batching direction of the paper's method:
- * systems share nothing).  Large systems are solved by a thread-block cluster,
- * small ones by a single thread block (a host scheduler balances the work; the
- * size threshold between the two is autotuned on the handle's first call).
+ * systems share nothing).  With the default options systems of up to 17,120 rows
+ * are solved by one SM each from a queue where that pays, and the larger ones by
+ * the grid-persistent kernel; else the kernel and its shape (grid-persistent, or
+ * clusters for large systems and blocks for small ones) are autotuned on the handle's
+ * first call.
  * status_out / iters_out / relres_out: nullable HOST arrays of nsys receiving each
  * system's status, rounds (precision + inner) and final relative residual.
  * Returns the worst status.
@@ -455,7 +457,7 @@ gabp_status gabp_residual_history(gabp_handle h, double *relres, int32_t cap, in
  * shape (the joint precision + mean round when options.overlap_precision = 1,
  * else the precision-only round) and the mean round's shape, packed as
  * lanes | unroll << 8; the multi-system size split;
- * the multi-system kernel (1 grid-persistent, 2 teams) | the grid-persistent
+ * the multi-system kernel (1 grid-persistent, 2 teams or the queue, which tunes no shape) | the grid-persistent
  * kernel's shape << 8 (shape: lanes | unroll << 8, plus 1 << 16 on the sliced
  * layout).  The FP64 and FP32 choices are remembered for the
  * process per (device, n, directed-edge count): a later handle of a matrix of

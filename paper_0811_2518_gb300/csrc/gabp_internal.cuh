@@ -235,16 +235,28 @@ struct WorkS {
   float *sinvP = nullptr;      // [n] 1 / P~ (new order)
 };
 
+// What the queue kernel (multichip.cu) adds to the layout below: rows addressed by position in their system.
+struct TeamSell {
+  int njobs = -1;                 // systems its `order` holds (-1: not built)
+  int2 *sys = nullptr;            // [nsys] first slice and slices of each system
+  int *order = nullptr;           // [nsys] the systems it solves by descending size, then its counters
+  unsigned char *blk = nullptr;   // [10 Es] coefficients and senders' positions, chunk by chunk
+  float *adp = nullptr;           // [32 ns] A_ii by position
+  float *node = nullptr;          // [2][32 ns] right-hand side, 1 / P~
+};
+
 // Sliced layout of the independent-systems grid kernel: every system's rows sorted by
 // degree (descending, stable) in windows of 4096 and cut into 32-row slices, the last
 // slice of a system padded with rows -1, so that a slice belongs to one system; slot j
 // of the slice's rows is the contiguous line sp[s] + 32 j + lane (sender -1 past a
-// row's degree).  Built for one offsets array; the values are refreshed after
-// gabp_set_values.
+// row's degree).  The systems lie by descending size.  Built for one offsets array; the
+// values are refreshed after gabp_set_values.
 struct GSell {
+  TeamSell team;
   std::vector<int> off;        // the offsets the layout was built for
   int ns = 0;                  // slices
   int Es = 0;                  // slots, padding included
+  std::vector<int> order;      // the systems by descending size (stable)
   bool vals_ok = false;
   int *srow = nullptr;         // [32 ns] row of each slice lane, -1 for padding
   int *sp = nullptr;           // [ns + 1] first slot of each slice (multiples of 32)
@@ -605,8 +617,15 @@ constexpr int kGridShapes[12] = {1 | (4 << 8), 2 | (4 << 8), 4 | (2 << 8), 4 | (
                                   kSliced | 1 | (1 << 8), kSliced | 1 | (2 << 8), kSliced | 1 | (4 << 8)};
 gabp_status solve_systems_grid(gabp_handle h, int nsys, const int *d_off, const int *off_host, const double *b,
                                double *x, double tol, int max_iter, int *d_status, int *d_iters, int *d_refine,
-                               double *d_relres, int shape, float *ms_out);
+                               double *d_relres, int shape, float *ms_out, int upto = -1);
 void free_gsell(gabp_handle h);
+gabp_status ensure_gsell(gabp_handle h, int nsys, const int *off);
+// multichip.cu
+void free_team(TeamSell &t);
+int team_rows(gabp_handle h);
+gabp_status solve_systems_team(gabp_handle h, int nsys, const int *off, int from, const double *b, double *x, double tol,
+                               int max_iter, int *d_status, int *d_iters, int *d_refine, double *d_relres,
+                               float *ms_out);
 gabp_status solve_batched32(gabp_handle h, int nrhs, const double *B, double *X, int64_t ld, double tol,
                             int max_iter, int *iters, double *relres_host);
 

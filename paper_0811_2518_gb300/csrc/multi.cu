@@ -22,6 +22,7 @@
 
 #include <algorithm>
 #include <cmath>
+#include <functional>
 #include <numeric>
 #include <vector>
 
@@ -514,6 +515,43 @@ gabp_status solve_systems(gabp_handle h, int nsys, const int *offsets_host, cons
     return solve_systems_grid(h, nsys, d_off, offsets_host, b, x, tol, max_iter, d_res, d_res + nsys, d_res + 2 * nsys,
                               d_rel, shape, t);
   };
+  // The queue kernel (multichip.cu) for the smaller systems and the grid-persistent kernel on the sliced
+  // layout for the larger ones, one after the other, unless an option asks for a kernel or the model below
+  // finds no system for the queue.  Time of a round in us by rows, fitted to geometric graphs of degree 6.
+  // Queue kernel: 3 + the larger of 2.4e-3 a row of its largest system (one SM's rate) and 2.0e-5 a row of
+  // all its systems (HBM): 1 system of 16384 rows 39.7, 152 of 1024 / 4096 / 16384 5.2 / 12.7 / 49.9.  Grid
+  // kernel: 11 + 4.6e-5 a row: 1 of 16384 10.8, 8 of 16384 17.2, 60 of 8192 32.5 (queue 22.7), 152 of
+  // 16384 113.
+  if (h->opt.multi_split == 0 && h->opt.multi_mode == 0 && h->opt.lanes == 0) {
+    std::vector<int> desc(rows);
+    std::sort(desc.begin(), desc.end(), std::greater<int>());
+    const int most = team_rows(h);
+    double left = 0.0, all = 0.0, best = 1e300;
+    for (int r : rows) all += r;
+    int from = nsys;  // systems desc[from ..] go to the queue
+    for (int q = 0; q <= nsys; ++q) {  // desc[0 .. q) on the grid
+      if (q == 0 || q == nsys || desc[q] != desc[q - 1]) {
+        const double grid = q > 0 ? 11.0 + 4.6e-5 * left : 0.0;
+        const double team = q < nsys ? 3.0 + std::max(2.4e-3 * desc[q], 2.0e-5 * (all - left)) : 0.0;
+        if ((q == nsys || desc[q] <= most) && grid + team < best) {
+          best = grid + team;
+          from = q;
+        }
+      }
+      if (q < nsys) left += desc[q];
+    }
+    if (from < nsys) {
+      float ms2 = 0.f;
+      if (from > 0 && (st = solve_systems_grid(h, nsys, d_off, offsets_host, b, x, tol, max_iter, d_res, d_res + nsys,
+                                               d_res + 2 * nsys, d_rel, kSliced | 1 | (4 << 8), &ms, from)) != GABP_OK)
+        return st;
+      st = solve_systems_team(h, nsys, offsets_host, from, b, x, tol, max_iter, d_res, d_res + nsys, d_res + 2 * nsys,
+                              d_rel, &ms2);
+      if (st != GABP_OK) return st;
+      h->multi_mode = 2;
+      return finish(ms + ms2);
+    }
+  }
   // grid-kernel shape: the lanes option, else the tuned one, else tune it now
   // (each candidate one complete run; the fastest is kept)
   const int mode = h->opt.multi_split > 0 ? 2 : h->opt.multi_mode ? h->opt.multi_mode : h->multi_mode;

@@ -21,8 +21,7 @@
 // The barrier spins on a generation counter with a clock-bounded wait: all
 // blocks are co-resident (cooperative launch), so it always completes; if it
 // ever did not within ~2 s, the kernel records GABP_TIMEOUT and returns.
-#include "gabp_internal.cuh"
-#include "devutil.cuh"
+#include "sell64.cuh"
 
 #include <algorithm>
 #include <cmath>
@@ -630,12 +629,14 @@ __global__ void kgs_fill(int nq, const int *__restrict__ srow, const int *__rest
   }
 }
 
-__global__ void kg_init(int nsys, SysState *st, double *acc, const int *__restrict__ offsets, int *sys_of) {
+// rows_min: smaller systems are not this launch's (done from the start)
+__global__ void kg_init(int nsys, SysState *st, double *acc, const int *__restrict__ offsets, int *sys_of,
+                        int rows_min) {
   const int s = blockIdx.x;
   if (s >= nsys) return;
   if (threadIdx.x == 0) {
     SysState S = {};
-    S.phase = PH_PREC;
+    S.phase = offsets[s + 1] - offsets[s] >= rows_min ? PH_PREC : PH_DONE;
     S.t = 1;
     S.status = GABP_NOT_CONVERGED;
     st[s] = S;
@@ -682,13 +683,14 @@ void free_gsell(gabp_handle h) {
   if (!L) return;
   cudaFree(L->srow); cudaFree(L->sp); cudaFree(L->ssys); cudaFree(L->sci); cudaFree(L->sav);
   cudaFree(L->MP[0]); cudaFree(L->MP[1]); cudaFree(L->H[0]); cudaFree(L->H[1]); cudaFree(L->CF);
+  free_team(L->team);
   delete L;
   h->gsl = nullptr;
 }
 
 // The sliced layout for these offsets (rebuilt when they differ from the cached one),
 // its slot values refreshed after gabp_set_values.
-static gabp_status ensure_gsell(gabp_handle h, int nsys, const int *off) {
+gabp_status ensure_gsell(gabp_handle h, int nsys, const int *off) {
   Graph &g = h->g;
   GSell *L = h->gsl;
   if (!(L && (int)L->off.size() == nsys + 1 && std::equal(L->off.begin(), L->off.end(), off))) {
@@ -699,13 +701,15 @@ static gabp_status ensure_gsell(gabp_handle h, int nsys, const int *off) {
     GABP_CUDA(cudaStreamSynchronize(h->stream));
     std::vector<int> srow, sp(1, 0), ssys, rows;
     long long slots = 0;
-    for (int s = 0; s < nsys; ++s) {
+    L->order.resize(nsys);
+    for (int s = 0; s < nsys; ++s) L->order[s] = s;
+    std::stable_sort(L->order.begin(), L->order.end(),
+                     [&](int p, int q) { return off[p + 1] - off[p] > off[q + 1] - off[q]; });
+    for (int s : L->order) {
       const int a0 = off[s], ns = off[s + 1] - off[s];
       rows.resize(ns);
       for (int r = 0; r < ns; ++r) rows[r] = a0 + r;
-      for (int w0 = 0; w0 < ns; w0 += 4096)
-        std::stable_sort(rows.begin() + w0, rows.begin() + std::min(ns, w0 + 4096),
-                         [&](int x, int y) { return rp[x + 1] - rp[x] > rp[y + 1] - rp[y]; });
+      sort_degree_windows(rp, rows, 0, ns);
       for (int q = 0; q < ns; q += 32) {
         int wd = 0;
         for (int l = 0; l < 32; ++l) {
@@ -755,7 +759,7 @@ static gabp_status ensure_gsell(gabp_handle h, int nsys, const int *off) {
 
 gabp_status solve_systems_grid(gabp_handle h, int nsys, const int *d_off, const int *off_host, const double *b,
                                double *x, double tol, int max_iter, int *d_status, int *d_iters, int *d_refine,
-                               double *d_relres, int shape, float *ms_out) {
+                               double *d_relres, int shape, float *ms_out, int upto) {
   Graph &g = h->g;
   Work32 &w = h->w32;
   struct Free {
@@ -776,15 +780,23 @@ gabp_status solve_systems_grid(gabp_handle h, int nsys, const int *d_off, const 
   fr.p.push_back(misc);
   bar = reinterpret_cast<unsigned int *>(misc + 2);
   GABP_CUDA(cudaMemsetAsync(misc, 0, sizeof(int) * 2 + sizeof(unsigned int) * 2, h->stream));
-  kg_init<<<nsys, kBlock, 0, h->stream>>>(nsys, st, acc, d_off, sys_of);
   const bool sliced = (shape & kSliced) != 0;
+  int rows_min = 0, ns_run = 0;  // upto >= 0 (sliced): the first `upto` systems of the layout's order only
   if (sliced) {
     gabp_status e = ensure_gsell(h, nsys, off_host);
     if (e != GABP_OK) return e;
     const size_t Ea = std::max<size_t>(1, (size_t)h->gsl->Es);
     GABP_CUDA(cudaMemsetAsync(h->gsl->MP[0], 0, sizeof(float) * Ea, h->stream));
     GABP_CUDA(cudaMemsetAsync(h->gsl->MP[1], 0, sizeof(float) * Ea, h->stream));
+    ns_run = h->gsl->ns;
+    if (upto > 0) {
+      const std::vector<int> &ord = h->gsl->order;
+      rows_min = off_host[ord[upto - 1] + 1] - off_host[ord[upto - 1]];
+      ns_run = 0;
+      for (int q = 0; q < upto; ++q) ns_run += (off_host[ord[q] + 1] - off_host[ord[q]] + 31) / 32;
+    }
   }
+  kg_init<<<nsys, kBlock, 0, h->stream>>>(nsys, st, acc, d_off, sys_of, rows_min);
   kg_rows_init<<<blocks_for(g.n, kBlock, h->max_blocks), kBlock, 0, h->stream>>>(
       g.n, g.rp, g.ad, g.ad32, w.NP[0], sliced ? nullptr : w.MP[0], sliced ? nullptr : w.MP[1], x);
   GABP_CUDA(cudaGetLastError());
@@ -799,7 +811,7 @@ gabp_status solve_systems_grid(gabp_handle h, int nsys, const int *d_off, const 
   a.ns = 0; a.srow = a.sp = a.ssys = nullptr;
   if (sliced) {  // the slot arrays of the sliced layout
     GSell *L = h->gsl;
-    a.ns = L->ns; a.srow = L->srow; a.sp = L->sp; a.ssys = L->ssys;
+    a.ns = ns_run; a.srow = L->srow; a.sp = L->sp; a.ssys = L->ssys;
     a.ci = L->sci; a.av = L->sav;
     a.MP0 = L->MP[0]; a.MP1 = L->MP[1]; a.H0 = L->H[0]; a.H1 = L->H[1]; a.CF = L->CF;
   }
