@@ -360,6 +360,7 @@ struct gabp_handle_s {
   int chip64_bytes = 0;             // shared memory per CTA of those rounds with all state on chip (0: no fit)
   int chip64_smax = 0, chip64_rmax = 0;  // own slots and own rows of the largest CTA there
   int coop64 = 0;                   // blocks of the FP64 cooperative rounds (0: graph too large or no support)
+  int coop64_u = 2;                 // slots per lane at once of the cooperative rounds
   int coop64f = 0;                  // the same for the cooperative rounds with the precision freeze
   int lsq_m = 0, lsq_k = 0;         // 0: not a least-squares handle
   double *lsq_b = nullptr, *lsq_x = nullptr;  // [k + m] augmented right-hand side and solution

@@ -191,13 +191,13 @@ __device__ __forceinline__ RevFrom round_source(int t, int cold) {
 // FROM: where the reverse messages come from (round_source), a template parameter because a
 // branch on it between a slot's loads would keep them from being issued together.  In the
 // recompute form Nout and Mout hold round t-2 until they are written.
-template <bool COOP, int MODE, RevFrom FROM>
+template <bool COOP, int MODE, RevFrom FROM, int UU = 0>
 __device__ __forceinline__ void plain_slice(const Args64 &a, int sl, int lane, const double *__restrict__ b,
                                             const double2 *__restrict__ Min, double2 *__restrict__ Mout,
                                             const NodeRec64 *__restrict__ Nin, NodeRec64 *__restrict__ Nout,
                                             double &rr, int &bad, int &moving) {
   constexpr bool REC = FROM == kRec || FROM == kRecZero;
-  constexpr int U = COOP ? kUCoop : REC ? kURec : kUGather;
+  constexpr int U = UU ? UU : COOP ? kUCoop : REC ? kURec : kUGather;
   const int i = COOP ? __ldg(a.srow + sl * 32 + lane) : a.srow[sl * 32 + lane];
   const int q0 = COOP ? __ldg(a.sp + sl) : a.sp[sl];
   const int p0 = q0 + lane, wd = ((COOP ? __ldg(a.sp + sl + 1) : a.sp[sl + 1]) - q0) >> 5;
@@ -574,29 +574,34 @@ __global__ void __launch_bounds__(kBlock, ACC ? 3 : kMinBlocks64) k64_node(Args6
 // The barrier's wait is bounded (kCoopBarrierLimit clock cycles, ~2 s; all blocks are
 // co-resident, so it always completes): if it ever gave up, the kernel raises *err and
 // every block returns.  The loop is bounded by max_rounds.
-#ifndef GABP_COOP_THREADS
-#define GABP_COOP_THREADS 64
-#endif
-#ifndef GABP_COOP_SLEEP
-#define GABP_COOP_SLEEP 32
-#endif
-constexpr int kCoopThreads = GABP_COOP_THREADS;
+//
+// A round is a chain of latencies, so: the round index, the stopping parameters and the freeze state stay
+// in registers, and the word that releases the blocks carries the decision and the next state (no read of
+// the control block on either side of the barrier); U slots of a row have their loads issued together, as
+// many as registers allow with a warp for every slice resident.  Whole solves over their rounds: 20011-row
+// random graph of degree 8 21.5 -> 17.4 us, 181 x 181 grid 11 -> 9.2, 40^3 grid 19 -> 15.1.
+constexpr int kCoopThreads = 64;
 constexpr int kCoopMaxSlices = 4096;
 constexpr long long kCoopBarrierLimit = 4000000000LL;
 
-template <bool FRZ>
-__global__ void __launch_bounds__(kCoopThreads, FRZ ? 8 : 12) k64_coop(Args64 a, unsigned *bar, int *err, int max_rounds) {
+// Blocks per SM that a kernel of U slots is sized for: 255 registers for 8 slots, 128 for 4, 80 for 2.
+__host__ __device__ constexpr int coop_blocks(bool frz, int U) { return frz ? 8 : U == 8 ? 4 : U == 4 ? 8 : 12; }
+
+template <bool FRZ, int U>
+__global__ void __launch_bounds__(kCoopThreads, coop_blocks(FRZ, U))
+    k64_coop(Args64 a, unsigned *bar, int *err, int max_rounds) {
   DevCtl *ctl = a.ctl;
-  __shared__ int s_last, s_go;
-  __shared__ unsigned s_gen;
+  __shared__ int s_last;
+  __shared__ unsigned s_word;
   const int lane = threadIdx.x & 31;
   const int warp = (blockIdx.x * kCoopThreads + threadIdx.x) >> 5;
   const int nwarps = (gridDim.x * kCoopThreads) >> 5;
   const double *__restrict__ b = ctl->b;
-  const int cold = ctl->cold;
+  const int cold = ctl->cold, t0 = ctl->round;
+  const StopRule rule = stop_rule(ctl);
+  int fs = FRZ ? ctl->fstate : 0;
   for (int iter = 0; iter < max_rounds; ++iter) {
-    const int t = __ldcg(&ctl->round) + 1;
-    const int fs = FRZ ? __ldcg(&ctl->fstate) : -1;
+    const int t = t0 + 1 + iter;
     const double2 *__restrict__ Min = (t & 1) ? a.M0 : a.M1;
     double2 *__restrict__ Mout = (t & 1) ? a.M1 : a.M0;
     const NodeRec64 *__restrict__ Nin = (t & 1) ? a.N0 : a.N1;
@@ -604,61 +609,69 @@ __global__ void __launch_bounds__(kCoopThreads, FRZ ? 8 : 12) k64_coop(Args64 a,
     double rr = 0.0;
     int bad = 0, moving = 0;
     for (int sl = warp; sl < a.ns; sl += nwarps) {
-      if (!FRZ && t == 1 && cold) plain_slice<true, 0, kZero>(a, sl, lane, b, Min, Mout, Nin, Nout, rr, bad, moving);
-      else if (!FRZ) plain_slice<true, 0, kGather>(a, sl, lane, b, Min, Mout, Nin, Nout, rr, bad, moving);
-      else if (fs == 0) plain_slice<true, 1, kGather>(a, sl, lane, b, Min, Mout, Nin, Nout, rr, bad, moving);
-      else if (fs == 1) plain_slice<true, 2, kGather>(a, sl, lane, b, Min, Mout, Nin, Nout, rr, bad, moving);
-      else plain_slice<true, 3, kGather>(a, sl, lane, b, Min, Mout, Nin, Nout, rr, bad, moving);
+      if (!FRZ && t == 1 && cold)
+        plain_slice<true, 0, kZero, U>(a, sl, lane, b, Min, Mout, Nin, Nout, rr, bad, moving);
+      else if (!FRZ) plain_slice<true, 0, kGather, U>(a, sl, lane, b, Min, Mout, Nin, Nout, rr, bad, moving);
+      else if (fs == 0) plain_slice<true, 1, kGather, U>(a, sl, lane, b, Min, Mout, Nin, Nout, rr, bad, moving);
+      else if (fs == 1) plain_slice<true, 2, kGather, U>(a, sl, lane, b, Min, Mout, Nin, Nout, rr, bad, moving);
+      else plain_slice<true, 3, kGather, U>(a, sl, lane, b, Min, Mout, Nin, Nout, rr, bad, moving);
     }
-    // grid barrier; the last block to arrive reduces and decides
-    constexpr int NV = FRZ ? 3 : 2;
-    double v[NV];
-    v[0] = rr;
-    v[1] = (double)bad;
-    if constexpr (FRZ) v[2] = (double)moving;
-    block_sum_nt<NV, kCoopThreads>(v);
+    // grid barrier; the last block to arrive reduces and decides.  partials: the blocks' sums, then their
+    // flags (bit 0 a zero precision, bit 1 a precision moved).
+    const int flags = (__syncthreads_or(bad) ? 1 : 0) | (FRZ && __syncthreads_or(moving) ? 2 : 0);
+    double v[1] = {rr};
+    block_sum_nt<1, kCoopThreads>(v);
+    int *const bflags = reinterpret_cast<int *>(a.partials + gridDim.x);
     if (threadIdx.x == 0) {
       a.partials[blockIdx.x] = v[0];
-      a.partials[gridDim.x + blockIdx.x] = v[1];
-      if constexpr (FRZ) a.partials[2 * gridDim.x + blockIdx.x] = v[2];
-      const unsigned g = *(volatile unsigned *)(bar + 1);
+      bflags[blockIdx.x] = flags;
       __threadfence();
       s_last = atomicAdd(bar, 1u) == gridDim.x - 1;
-      s_gen = g;
     }
     __syncthreads();
+    const unsigned mine = (unsigned)t << 3;  // the release of this round: t, the freeze state, done
     if (s_last) {
       __threadfence();
-      double w[NV];
-      for (int q = 0; q < NV; ++q) w[q] = 0.0;
+      double w[1] = {0.0};
+      int f = 0;
       for (int q = threadIdx.x; q < (int)gridDim.x; q += kCoopThreads) {
         w[0] += __ldcg(a.partials + q);
-        w[1] += __ldcg(a.partials + gridDim.x + q);
-        if constexpr (FRZ) w[2] += __ldcg(a.partials + 2 * gridDim.x + q);
+        f |= __ldcg(bflags + q);
       }
-      block_sum_nt<NV, kCoopThreads>(w);
+      const int fbad = __syncthreads_or(f & 1), fmove = FRZ ? __syncthreads_or(f & 2) : 0;
+      block_sum_nt<1, kCoopThreads>(w);
       if (threadIdx.x == 0) {
-        if constexpr (FRZ) freeze_step(ctl, fs, t, w[2]);
-        decide64(ctl, t, w[0], w[1]);
-        s_go = !ctl->done;
+        const double nbad = fbad ? 1.0 : 0.0;
+        if constexpr (FRZ) {
+          freeze_step(ctl, fs, t, fmove ? 1.0 : 0.0);
+          fs = ctl->fstate;
+        }
+        record64<true>(ctl, rule, t, w[0], nbad);
+        const unsigned word = mine | ((unsigned)fs << 1) | (stops64(rule, t, w[0], nbad) ? 1u : 0u);
         bar[0] = 0;
         __threadfence();
-        atomicAdd(bar + 1, 1u);
+        atomicExch(bar + 1, word);
+        s_word = word;
       }
     } else if (threadIdx.x == 0) {
-      volatile unsigned *gen = bar + 1;
-      const long long t0 = clock64();
-      int ok = 1;
-      while (*gen == s_gen) {
-        if (*(volatile int *)err || clock64() - t0 > kCoopBarrierLimit) { ok = 0; break; }
-        if (GABP_COOP_SLEEP) __nanosleep(GABP_COOP_SLEEP);
+      const long long c0 = clock64();
+      unsigned word;
+      while (((word = *(volatile unsigned *)(bar + 1)) & ~7u) != mine) {
+        if (*(volatile int *)err || clock64() - c0 > kCoopBarrierLimit) {
+          atomicExch(err, 1);
+          word = mine | 1u;
+          break;
+        }
+        __nanosleep(32);
       }
-      if (!ok) atomicExch(err, 1);
       __threadfence();
-      s_go = ok && !__ldcg(&ctl->done);
+      s_word = word;
     }
     __syncthreads();
-    if (!s_go) break;
+    const unsigned word = s_word;
+    if (word & 1u) break;
+    fs = (int)((word >> 1) & 3u);
+    __syncthreads();  // s_word is read by all before the next round's
   }
 }
 
@@ -1310,14 +1323,18 @@ static gabp_status ensure_sell64(gabp_handle h) {
     cudaDeviceGetAttribute(&coop_attr, cudaDevAttrCooperativeLaunch, h->device);
     if (coop_attr && S.ns <= kCoopMaxSlices) {
       const int want = (S.ns * 32 + kCoopThreads - 1) / kCoopThreads;
-      int per_sm = 0;
-      if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k64_coop<false>, kCoopThreads, 0) == cudaSuccess &&
-          per_sm > 0)
-        h->coop64 = std::min(want, std::min(per_sm * h->num_sms, h->max_blocks));
-      per_sm = 0;
-      if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k64_coop<true>, kCoopThreads, 0) == cudaSuccess &&
-          per_sm > 0)
-        h->coop64f = std::min(want, std::min(per_sm * h->num_sms, h->max_blocks));
+      auto fits = [&](auto kern) {
+        int per_sm = 0;
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kCoopThreads, 0) != cudaSuccess) per_sm = 0;
+        return std::min(per_sm * h->num_sms, h->max_blocks);
+      };
+      // as many slots at once as leave a warp for every slice
+      int most = fits(k64_coop<false, 8>);
+      h->coop64_u = 8;
+      if (most < want) { most = fits(k64_coop<false, 4>); h->coop64_u = 4; }
+      if (most < want) { most = fits(k64_coop<false, 2>); h->coop64_u = 2; }
+      h->coop64 = std::min(want, most);
+      h->coop64f = std::min(want, fits(k64_coop<true, 2>));
       cudaGetLastError();
     }
   } else if (!S.vals_ok) {
@@ -1553,8 +1570,10 @@ gabp_status solve64(gabp_handle h, const double *b, double *x, double tol, int m
     int max_rounds = max_iter + 2;
     void *args[] = {(void *)&a, (void *)&bar, (void *)&err, (void *)&max_rounds};
     prof_begin(h);
-    cudaError_t le = cudaLaunchCooperativeKernel(a.freeze ? (void *)k64_coop<true> : (void *)k64_coop<false>,
-                                                 dim3(coop_grid), dim3(kCoopThreads), args, 0, h->stream);
+    void *kern = a.freeze ? (void *)k64_coop<true, 2>
+                 : h->coop64_u == 8 ? (void *)k64_coop<false, 8>
+                 : h->coop64_u == 4 ? (void *)k64_coop<false, 4> : (void *)k64_coop<false, 2>;
+    cudaError_t le = cudaLaunchCooperativeKernel(kern, dim3(coop_grid), dim3(kCoopThreads), args, 0, h->stream);
     if (le != cudaSuccess) return cuda_fail(le, "FP64 cooperative rounds");
     prof_end(h);
     h->prof.launches += 1;
