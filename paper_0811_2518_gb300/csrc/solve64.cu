@@ -276,8 +276,8 @@ __device__ __forceinline__ void plain_slice(const Args64 &a, int sl, int lane, c
 // solve's, or imported ones) and forms the aggregates from them with this b:
 // any starting messages lead to the same fixed point when the iteration converges.
 // cold = 1: M0 was not cleared, and the rounds take zero starting messages without reading it.
-__global__ void __launch_bounds__(kBlock) k64_init(Args64 a, double tol, int max_iter, int warm, int cold) {
-  const double *b = a.ctl->b;
+__global__ void __launch_bounds__(kBlock) k64_init(Args64 a, const double *__restrict__ b, double tol, int max_iter,
+                                                   int warm, int cold, double *hist, int hist_cap) {
   const WarpPos w = warp_pos();
   double bb = 0.0;
   for (int sl = w.warp; sl < a.ns; sl += w.nwarps) {
@@ -302,6 +302,9 @@ __global__ void __launch_bounds__(kBlock) k64_init(Args64 a, double tol, int max
   block_sum<1>(v);
   if (last_block_reduce<1>(v, a.partials, &a.ctl->arrive, tot) && threadIdx.x == 0) {
     DevCtl *c = a.ctl;
+    c->b = b;
+    c->hist = hist;
+    c->hist_cap = hist_cap;
     c->round = 0;
     c->bb = tot[0];
     c->tol2bb = tol * tol * tot[0];
@@ -596,6 +599,7 @@ __global__ void __launch_bounds__(kCoopThreads, coop_blocks(FRZ, U))
   const int lane = threadIdx.x & 31;
   const int warp = (blockIdx.x * kCoopThreads + threadIdx.x) >> 5;
   const int nwarps = (gridDim.x * kCoopThreads) >> 5;
+  if (ctl->done) return;  // b = 0 (the same in every block: only an earlier kernel writes it)
   const double *__restrict__ b = ctl->b;
   const int cold = ctl->cold, t0 = ctl->round;
   const StopRule rule = stop_rule(ctl);
@@ -713,6 +717,7 @@ __global__ void __launch_bounds__(32 * NW) k64_cluster(Args64 a, int max_rounds)
   const unsigned rank = cl.block_rank(), csize = cl.num_blocks();
   __shared__ ClusterPart part[2][NW];  // [round parity][warp]
   DevCtl *ctl = a.ctl;
+  if (ctl->done) return;  // b = 0 (the same in every CTA: only an earlier kernel writes it)
   const double *__restrict__ b = ctl->b;
   const int t0 = ctl->round;  // read by every CTA before the first barrier, written only after it
   const int cold = ctl->cold;
@@ -795,6 +800,7 @@ __global__ void __launch_bounds__(32 * NW) k64_chip(Args64 a, ChipShape c, int m
   int *inv = reinterpret_cast<int *>(tab + a.ns);        // per row: its slice position (set-up only)
   __shared__ ClusterPart part[2][NW];
   DevCtl *ctl = a.ctl;
+  if (ctl->done) return;
   const double *__restrict__ b = ctl->b;
   const int t0 = ctl->round;
   const StopRule rule = stop_rule(ctl);  // CTA 0 writes none of these fields
@@ -1056,9 +1062,12 @@ __global__ void __launch_bounds__(kBlock) k64_edge_agg(Args64 a) {
   }
 }
 
-__global__ void k64_finalize(int n, const NodeRec64 *__restrict__ N, double *__restrict__ x, int aitken) {
-  int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) x[i] = aitken ? N[i].pad : N[i].x;
+// The iterate of the returned round; x = 0 for b = 0 (the warm round-0 records hold the old messages' mean).
+__global__ void k64_finalize(int n, const NodeRec64 *__restrict__ N0, const NodeRec64 *__restrict__ N1,
+                             double *__restrict__ x, int aitken, const DevCtl *__restrict__ ctl) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  const NodeRec64 *N = (ctl->result_round & 1) ? N1 : N0;
+  if (i < n) x[i] = ctl->bb == 0.0 ? 0.0 : aitken ? N[i].pad : N[i].x;
 }
 
 // Messages of the returned round in the layout of the input CSR.  With the sliced
@@ -1484,26 +1493,18 @@ gabp_status solve64(gabp_handle h, const double *b, double *x, double tol, int m
   // round-0 state (Algorithm 1 step 1): control block pointed at b, zero messages
   auto init = [&]() -> gabp_status {
     GABP_CUDA(cudaMemsetAsync(h->ctl, 0, sizeof(DevCtl), h->stream));
-    const double *bptr = b;
-    GABP_CUDA(cudaMemcpyAsync(&h->ctl->b, &bptr, sizeof(bptr), cudaMemcpyHostToDevice, h->stream));
-    if (h->opt.history > 0) {  // per-round residual history (options.history entries)
-      if (h->hist_alloc < h->opt.history) {
-        cudaFree(h->hist);
-        h->hist = nullptr;
-        h->hist_alloc = 0;
-        GABP_CUDA(cudaMalloc(&h->hist, sizeof(double) * (size_t)h->opt.history));
-        h->hist_alloc = h->opt.history;
-      }
-      double *hp = h->hist;
-      const int cap = h->opt.history;
-      GABP_CUDA(cudaMemcpyAsync(&h->ctl->hist, &hp, sizeof(hp), cudaMemcpyHostToDevice, h->stream));
-      GABP_CUDA(cudaMemcpyAsync(&h->ctl->hist_cap, &cap, sizeof(cap), cudaMemcpyHostToDevice, h->stream));
+    if (h->opt.history > 0 && h->hist_alloc < h->opt.history) {  // per-round residual history
+      cudaFree(h->hist);
+      h->hist = nullptr;
+      h->hist_alloc = 0;
+      GABP_CUDA(cudaMalloc(&h->hist, sizeof(double) * (size_t)h->opt.history));
+      h->hist_alloc = h->opt.history;
     }
     if (!warm && !cold) GABP_CUDA(cudaMemsetAsync(h->w64.M[0], 0, sizeof(double2) * Es, h->stream));
-    k64_init<<<blocks_for(a.ns, kBlock / 32, h->max_blocks), kBlock, 0, h->stream>>>(a, tol, max_iter, warm ? 1 : 0,
-                                                                                       cold ? 1 : 0);
+    k64_init<<<blocks_for(a.ns, kBlock / 32, h->max_blocks), kBlock, 0, h->stream>>>(
+        a, b, tol, max_iter, warm ? 1 : 0, cold ? 1 : 0, h->opt.history > 0 ? h->hist : nullptr,
+        h->opt.history > 0 ? h->opt.history : 0);
     GABP_CUDA(cudaGetLastError());
-    GABP_CUDA(cudaStreamSynchronize(h->stream));  // also retires the pageable copy of bptr
     return GABP_OK;
   };
   if ((s = init()) != GABP_OK) return s;
@@ -1516,14 +1517,17 @@ gabp_status solve64(gabp_handle h, const double *b, double *x, double tol, int m
   }
   const int K = h->opt.check_every;
   const int64_t max_batches = (int64_t)(max_iter + 2) / K + 3;
-  bool done = false;
-  if ((s = read_ctl(h)) != GABP_OK) return s;
-  done = h->ctl_host->done;
+  bool done = false;  // b = 0 is decided by k64_init: the round kernels return at once
+  auto finalize = [&]() {
+    k64_finalize<<<(g.n + kBlock - 1) / kBlock, kBlock, 0, h->stream>>>(g.n, h->w64.N[0], h->w64.N[1], x,
+                                                                       h->opt.accel == ACC_AITKEN, h->ctl);
+    h->prof.launches += 1;
+  };
   const int per_round =
       a.freeze ? 3 : h->opt.variant == GABP_VARIANT_EDGE || h->opt.accel == ACC_STEFFENSEN ? 2 : 1;
   h->prof.launches += 1;  // k64_init
   int prev_round = 0;
-  if (!done && clus) {
+  if (clus) {
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeClusterDimension;
@@ -1557,11 +1561,12 @@ gabp_status solve64(gabp_handle h, const double *b, double *x, double tol, int m
     if (le != cudaSuccess) return cuda_fail(le, "FP64 cluster rounds");
     prof_end(h);
     h->prof.launches += 1;
+    finalize();
     if ((s = read_ctl(h)) != GABP_OK) return s;
     prof_collect(h, PH_FP64, h->ctl_host->round);
     done = h->ctl_host->done;
   }
-  if (!done && coop) {
+  if (coop) {
     Work64 &w = h->w64;
     if (!w.bar) GABP_CUDA(cudaMalloc(&w.bar, 16));  // [0] arrivals, [1] generation, [2] error flag
     GABP_CUDA(cudaMemsetAsync(w.bar, 0, 16, h->stream));
@@ -1577,6 +1582,7 @@ gabp_status solve64(gabp_handle h, const double *b, double *x, double tol, int m
     if (le != cudaSuccess) return cuda_fail(le, "FP64 cooperative rounds");
     prof_end(h);
     h->prof.launches += 1;
+    finalize();
     int herr = 0;
     GABP_CUDA(cudaMemcpyAsync(&herr, err, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
     if ((s = read_ctl(h)) != GABP_OK) return s;
@@ -1618,15 +1624,9 @@ gabp_status solve64(gabp_handle h, const double *b, double *x, double tol, int m
   h->stats.freeze_checks = a.freeze ? c.fchecks : 0;
   if (cold && c.result_round == 0)  // the messages of round 0
     GABP_CUDA(cudaMemsetAsync(h->w64.M[0], 0, sizeof(double2) * Es, h->stream));
-  if (warm && c.bb == 0.0) {  // b = 0: x = 0 (the warm round-0 records hold the old messages' mean)
-    GABP_CUDA(cudaMemsetAsync(x, 0, sizeof(double) * g.n, h->stream));
-  } else {
-    k64_finalize<<<(g.n + kBlock - 1) / kBlock, kBlock, 0, h->stream>>>(g.n, h->w64.N[c.result_round & 1], x,
-                                                                       h->opt.accel == ACC_AITKEN);
-    h->prof.launches += 1;
-  }
+  if (!coop && !clus) finalize();
   GABP_CUDA(cudaGetLastError());
-  GABP_CUDA(cudaStreamSynchronize(h->stream));
+  if ((!coop && !clus) || c.result_round == 0) GABP_CUDA(cudaStreamSynchronize(h->stream));
   if (iters) *iters = c.iters;
   if (relres) *relres = c.bb > 0.0 ? sqrt(c.rr / c.bb) : 0.0;
   return (gabp_status)c.status;
