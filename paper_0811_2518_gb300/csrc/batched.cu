@@ -875,8 +875,9 @@ gabp_status solve_batched32(gabp_handle h, int nrhs, const double *B, double *X,
   h->stats.rounds = 0;
   h->stats.edge_updates = 0;
   h->stats.refine_steps = 0;
+  if (h->opt.reuse_precisions && (s = csr_coef32(h)) != GABP_OK) return s;
   if (!h->w32.coef_ready || !h->opt.reuse_precisions) {
-    h->w32.coef_ready = false;
+    drop_coef32(h);
     if ((s = precision_phase32(h, nullptr)) != GABP_OK) return s;
     h->stats.edge_updates += h->stats.rounds * (int64_t)h->g.E;  // precision rounds serve every column
   }

@@ -151,6 +151,24 @@ struct Work64 {
   double *C = nullptr;      // [Es] frozen coefficients c = A / (P~ - P) (options.freeze_precisions)
 };
 
+// The sliced layout of the FP32 rounds (solve32.cu): rows by degree, 32 a slice, node arrays by position.
+struct Sell32 {
+  bool tried = false;       // built, or found not to fit (ns = 0)
+  bool vals_ok = false;     // sav matches the graph's values (cleared by gabp_set_values)
+  bool coef_ready = false;  // CF, invP hold frozen coefficients
+  int ns = 0, Es = 0;       // slices, positions (slots + padding)
+  int *srow = nullptr;      // [32 ns] row of each position, -1 past n
+  int *pos = nullptr;       // [n] position of each row
+  int *sp = nullptr;        // [ns + 1] first slot of each slice
+  int *sci = nullptr;       // [Es] position of the sender, -1 for padding
+  float *sav = nullptr;     // [Es] A
+  float2 *CF = nullptr;     // [Es] {c_in, c_out}
+  float *nodes = nullptr;   // the arrays below, [32 ns] each
+  float2 *NQ[3] = {nullptr, nullptr, nullptr};
+  float *NP[3] = {nullptr, nullptr, nullptr}, *NH[3] = {nullptr, nullptr, nullptr};
+  float *invP = nullptr, *rhs = nullptr, *ad = nullptr;
+};
+
 struct Work32 {
   // precision phase (recompute form): chains + node ring of 3
   float *MP[2] = {nullptr, nullptr};
@@ -159,6 +177,9 @@ struct Work32 {
   float *invP = nullptr;  // 1 / P~_i (frozen)
   bool coef_ready = false;
   int prec_round = -1;    // round of the frozen precision state
+  bool prec_sliced = false;  // it lies in sl.NP
+  Sell32 sl;
+  bool sl_on = false;     // the current solve's rounds run on sl
   int R = 0;              // RHS capacity of the mean buffers
   float *H[2] = {nullptr, nullptr};               // [E][R]
   float *NH[3] = {nullptr, nullptr, nullptr};     // [n][R] h~ ring
@@ -599,6 +620,8 @@ gabp_status solve64_serial(gabp_handle h, const double *b, double *x, double tol
                            double *relres);
 gabp_status serial_messages64(gabp_handle h, double2 *M_input_layout);
 gabp_status serial_marginals64(gabp_handle h, double *Pi);
+void drop_coef32(gabp_handle h);         // the frozen coefficients no longer hold
+gabp_status csr_coef32(gabp_handle h);  // makes them ready in CSR order if they are in the sliced one
 gabp_status serial_freeze32(gabp_handle h, const float2 *CF, const float *invP);
 gabp_status serial_inner32(gabp_handle h, const float *rhs, int cap, double itol, int *sweeps, int *status);
 gabp_status serial_update32(gabp_handle h, double *X);

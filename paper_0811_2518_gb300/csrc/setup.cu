@@ -433,7 +433,8 @@ extern "C" gabp_status gabp_set_values(gabp_handle h, const double *val, int mem
   h->w64.valid = false;  // and no warm start from them
   h->w64.sl.vals_ok = false;  // the sliced copy of the values is refreshed by the next FP64 solve
   if (h->gsl) h->gsl->vals_ok = false;  // and the independent-systems one by the next such solve
-  h->w32.coef_ready = false;
+  drop_coef32(h);
+  h->w32.sl.vals_ok = false;  // and the FP32 one by the next FP32 solve
   h->w32.prec_round = -1;
   int *dflag = nullptr;
   GABP_CUDA(cudaMalloc(&dflag, sizeof(int)));

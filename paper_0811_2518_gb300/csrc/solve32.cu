@@ -24,6 +24,7 @@
 // computing h_{i->k}^{(t-1)} once and storing it.
 #include "gabp_internal.cuh"
 #include "devutil.cuh"
+#include "sell64.cuh"
 
 #include <algorithm>
 #include <cmath>
@@ -93,11 +94,13 @@ struct Args32 {
   float2 *NQ0, *NQ1, *NQ2;        // {P~, h~} ring of the joint rounds
   DevCtl *ctl;
   double *partials;
+  int ns;                           // slices of the sliced layout (0: row kernels); node arrays by position then
+  const int *sp;                    // [ns + 1] first slot of each slice
   cudaGraphConditionalHandle cond;  // while-node condition cleared when the run is decided
   int use_cond;                     // (only inside the device-loop graph)
 };
 
-__device__ __forceinline__ float *ring3(float *a, float *b, float *c, int t) {
+__host__ __device__ __forceinline__ float *ring3(float *a, float *b, float *c, int t) {
   int m = t % 3;
   return m == 0 ? a : (m == 1 ? b : c);
 }
@@ -216,6 +219,26 @@ __global__ void __launch_bounds__(kBlock) k32_prec(Args32 a) {
 // the coefficients at any round T and continue with k32_mean from round T + 1.
 // Stop rule: the precision phase's (relative change <= 2^-s in two consecutive
 // rounds, zero cavity, max_iter).
+__device__ __forceinline__ void joint_decide(const Args32 &a, DevCtl *ctl, int t, const double (&tot)[3]) {
+  ctl->round = t;
+  ctl->maxrel = tot[1];                      // messages that moved by more than 2^-s
+  ctl->stable = tot[1] == 0.0 ? ctl->stable + 1 : 0;
+  if (ctl->no_stop) {
+    // autotuning run: no decision
+  } else if (tot[0] > 0.0) {
+    ctl->status = GABP_BREAKDOWN; ctl->iters = t; ctl->result_round = t; ctl->done = 1;
+  } else if (tot[2] > 0.0 && t > 1) {
+    ctl->status = GABP_DIVERGED; ctl->iters = t; ctl->result_round = t; ctl->done = 1;
+  } else if (ctl->stable >= 2) {
+    ctl->status = GABP_OK; ctl->iters = t; ctl->result_round = t; ctl->done = 1;
+  } else if (t >= ctl->max_iter) {
+    ctl->status = GABP_NOT_CONVERGED; ctl->iters = t; ctl->result_round = t; ctl->done = 1;
+  }
+  if (a.use_cond && ctl->done) cudaGraphSetConditional(a.cond, 0);
+  ctl->arrive = 0;
+  __threadfence();
+}
+
 template <int L, int U>
 __global__ void __launch_bounds__(kBlock, 4) k32_joint(Args32 a) {
   DevCtl *ctl = a.ctl;
@@ -297,25 +320,86 @@ __global__ void __launch_bounds__(kBlock, 4) k32_joint(Args32 a) {
   }
   double v[3] = {(double)bad, (double)moving, (double)nonfinite}, tot[3];
   block_sum<3>(v);
-  if (last_block_reduce<3>(v, a.partials, &ctl->arrive, tot) && threadIdx.x == 0) {
-    ctl->round = t;
-    ctl->maxrel = tot[1];                      // messages that moved by more than 2^-s
-    ctl->stable = tot[1] == 0.0 ? ctl->stable + 1 : 0;
-    if (ctl->no_stop) {
-      // autotuning run: no decision
-    } else if (tot[0] > 0.0) {
-      ctl->status = GABP_BREAKDOWN; ctl->iters = t; ctl->result_round = t; ctl->done = 1;
-    } else if (tot[2] > 0.0 && t > 1) {
-      ctl->status = GABP_DIVERGED; ctl->iters = t; ctl->result_round = t; ctl->done = 1;
-    } else if (ctl->stable >= 2) {
-      ctl->status = GABP_OK; ctl->iters = t; ctl->result_round = t; ctl->done = 1;
-    } else if (t >= ctl->max_iter) {
-      ctl->status = GABP_NOT_CONVERGED; ctl->iters = t; ctl->result_round = t; ctl->done = 1;
+  if (last_block_reduce<3>(v, a.partials, &ctl->arrive, tot) && threadIdx.x == 0) joint_decide(a, ctl, t, tot);
+}
+
+// The same on the sliced layout (ensure_sell32): lane by row.  The sums are those of the row kernel with 4 lanes a
+// row, bit for bit: systems whose FP32 rounds go one way or the other by their rounding (indefinite augmented ones of
+// least squares) go the same way on both.  U slots a lane in flight and the registers for them
+// (whole 2^20-row solves in us): U 4 at 3 blocks 2396, 3 at 4 2382, 2 at 5 2430, 4 at 4 (spills) 2535, 1 at 8 2786.
+// 130 us a round at 16.8 M slots, 157 with the row kernel (the streams and gathers alone, without rows: 101).
+__global__ void __launch_bounds__(kBlock, 3) ks32_joint(Args32 a) {
+  constexpr int U = 4;  // slots a lane in flight
+  DevCtl *ctl = a.ctl;
+  if (ctl->done) return;
+  const int t = ctl->round + 1;
+  float *Mc = (t & 1) ? a.MP1 : a.MP0;        // P chain: holds t-2, becomes t
+  const float *Mo = (t & 1) ? a.MP0 : a.MP1;  // P at t-1
+  float *Hc = (t & 1) ? a.H1 : a.H0;          // h chain: holds t-2, becomes t
+  const float2 *__restrict__ Qm1 = ring3(a.NQ0, a.NQ1, a.NQ2, t + 2);
+  const float2 *__restrict__ Qm2 = ring3(a.NQ0, a.NQ1, a.NQ2, t + 1);
+  float2 *__restrict__ Qt = ring3(a.NQ0, a.NQ1, a.NQ2, t);
+  float *__restrict__ Pt = ring3(a.NP0, a.NP1, a.NP2, t);
+  float *__restrict__ Ht = ring3(a.NH0, a.NH1, a.NH2, t);
+  const WarpPos w = warp_pos();
+  const float thr = (float)ctl->tol2bb;  // 2^-prec_stop_log2
+  int bad = 0, moving = 0, nonfinite = 0;
+  for (int m = 0; m * (int64_t)w.nwarps < a.ns; ++m) {
+    const int s = pass_slice(w, m);
+    if (s >= a.ns) continue;
+    const int p = 32 * s + w.lane, q1 = a.sp[s + 1];
+    const float2 q2 = t >= 2 ? Qm2[p] : make_float2(0.f, 0.f);
+    const float ad = a.ad[p], rhs = a.rhs[p];
+    float aP[4] = {}, aH[4] = {};  // as by 4 lanes a row
+    for (int qb = a.sp[s] + w.lane; qb < q1; qb += 32 * U) {
+      int k[U];
+      float A[U], Ps[U], Pp[U], hs[U];
+      float2 qk[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int q = qb + 32 * u;
+        k[u] = -1;
+        if (q < q1) {
+          k[u] = __ldcs(a.ci + q); A[u] = __ldcs(a.av + q);
+          Ps[u] = __ldcs(Mc + q); Pp[u] = __ldcs(Mo + q); hs[u] = __ldcs(Hc + q);
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        if (k[u] >= 0) qk[u] = __ldcg(Qm1 + k[u]);  // random gather, L2 only
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        if (k[u] >= 0) {
+          float Pout = 0.f, hout = 0.f;
+          if (t >= 2) {  // message i -> k of round t-1
+            const float d1 = q2.x - Ps[u];
+            bad |= (d1 == 0.f);
+            const float r1 = __fdividef(1.f, d1);
+            Pout = -A[u] * A[u] * r1;
+            hout = -A[u] * (q2.y - hs[u]) * r1;
+          }
+          const float d2 = qk[u].x - Pout;  // message k -> i of round t
+          bad |= (d2 == 0.f);
+          const float r2 = __fdividef(1.f, d2);
+          const float Pn = -A[u] * A[u] * r2;
+          const float hn = -A[u] * (qk[u].y - hout) * r2;
+          __stcs(Mc + qb + 32 * u, Pn);
+          __stcs(Hc + qb + 32 * u, hn);
+          aP[u] += Pn;
+          aH[u] += hn;
+          moving |= !(fabsf(Pn - Pp[u]) <= thr * fabsf(Pn));  // a NaN counts as moving
+          nonfinite |= !isfinite(Pn);
+        }
     }
-    if (a.use_cond && ctl->done) cudaGraphSetConditional(a.cond, 0);
-    ctl->arrive = 0;
-    __threadfence();
+    const float P = ad + ((aP[0] + aP[2]) + (aP[1] + aP[3])), hh = rhs + ((aH[0] + aH[2]) + (aH[1] + aH[3]));
+    bad |= (P == 0.f);
+    Qt[p] = make_float2(P, hh);
+    Pt[p] = P;
+    Ht[p] = hh;
   }
+  double v[3] = {(double)bad, (double)moving, (double)nonfinite}, tot[3];
+  block_sum<3>(v);
+  if (last_block_reduce<3>(v, a.partials, &ctl->arrive, tot) && threadIdx.x == 0) joint_decide(a, ctl, t, tot);
 }
 
 // round-0 state of the joint rounds: zero messages, {P~, h~} = {A_ii (+ Gamma_ii), r}
@@ -446,6 +530,58 @@ __global__ void __launch_bounds__(kBlock) k32_mean(Args32 a) {
   if (last_block_reduce<2>(v, a.partials, &ctl->arrive, tot) && threadIdx.x == 0) {
     mean_decide(a, ctl, t, tot);
   }
+}
+
+// The same on the sliced layout (ensure_sell32): lane by row.  95 us a round at 16.8 M slots, 117 with the row
+// kernel (the streams and gathers alone, without rows: 86).
+__global__ void __launch_bounds__(kBlock, 4) ks32_mean(Args32 a) {
+  constexpr int U = 4;  // slots a lane in flight
+  DevCtl *ctl = a.ctl;
+  if (ctl->done) return;
+  const int t = ctl->round + 1;
+  float *Hc = (t & 1) ? a.H1 : a.H0;  // holds t-2, becomes t
+  const float *__restrict__ Hm1 = ring3(a.NH0, a.NH1, a.NH2, t + 2);
+  const float *__restrict__ Hm2 = ring3(a.NH0, a.NH1, a.NH2, t + 1);
+  float *__restrict__ Ht = ring3(a.NH0, a.NH1, a.NH2, t);
+  const WarpPos w = warp_pos();
+  float dxx = 0.f, xx = 0.f;
+  for (int m = 0; m * (int64_t)w.nwarps < a.ns; ++m) {
+    const int s = pass_slice(w, m);
+    if (s >= a.ns) continue;
+    const int p = 32 * s + w.lane, q1 = a.sp[s + 1];
+    const float hi2 = t >= 2 ? Hm2[p] : 0.f, rhs = a.rhs[p], ip = a.invP[p], hprev = Hm1[p];
+    float acc[4] = {};  // as by 4 lanes a row
+    for (int qb = a.sp[s] + w.lane; qb < q1; qb += 32 * U) {
+      int k[U];
+      float2 cf[U];
+      float hs[U], hk[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int q = qb + 32 * u;
+        k[u] = -1;
+        if (q < q1) { k[u] = __ldcs(a.ci + q); cf[u] = __ldcs(a.CF + q); hs[u] = __ldcs(Hc + q); }
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        if (k[u] >= 0) hk[u] = __ldcg(Hm1 + k[u]);  // random gather, L2 only
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        if (k[u] >= 0) {
+          const float hout = t >= 2 ? cf[u].y * (hi2 - hs[u]) : 0.f;  // message i -> k at t-1
+          const float hn = cf[u].x * (hk[u] - hout);                  // message k -> i at t
+          __stcs(Hc + qb + 32 * u, hn);
+          acc[u] += hn;
+        }
+    }
+    const float hnew = rhs + ((acc[0] + acc[2]) + (acc[1] + acc[3]));
+    Ht[p] = hnew;
+    const float x = hnew * ip, dx = (hnew - hprev) * ip;
+    dxx = fmaf(dx, dx, dxx);
+    xx = fmaf(x, x, xx);
+  }
+  double v[2] = {(double)dxx, (double)xx}, tot[2];
+  block_sum<2>(v);
+  if (last_block_reduce<2>(v, a.partials, &ctl->arrive, tot) && threadIdx.x == 0) mean_decide(a, ctl, t, tot);
 }
 
 // ---------------------------------------------------------------------------- mean phase, dense matrix
@@ -702,21 +838,71 @@ __global__ void __launch_bounds__(kBlock) k32_freeze(Args32 a) {
   if (coef_only) return;
   double v[2] = {(double)dxx, (double)xx}, tot[2];
   block_sum<2>(v);
-  if (last_block_reduce<2>(v, a.partials, &ctl->arrive, tot) && threadIdx.x == 0) {
-    ctl->round = t;
-    ctl->rr = tot[0];
-    ctl->xx = tot[1];
-    if (!isfinite(tot[0]) || !isfinite(tot[1])) {
-      ctl->status = GABP_DIVERGED; ctl->iters = t; ctl->result_round = t; ctl->done = 1;
-    } else if (t >= 2 && tot[0] <= ctl->tol2bb * tot[1]) {
-      ctl->status = GABP_OK; ctl->iters = t; ctl->result_round = t; ctl->done = 1;
-    } else if (t >= ctl->max_iter) {
-      ctl->status = GABP_NOT_CONVERGED; ctl->iters = t; ctl->result_round = t; ctl->done = 1;
+  if (last_block_reduce<2>(v, a.partials, &ctl->arrive, tot) && threadIdx.x == 0) mean_decide(a, ctl, t, tot);
+}
+
+// The same on the sliced layout (118 us at 16.8 M slots, 158 with the row kernel).
+__global__ void __launch_bounds__(kBlock, 4) ks32_freeze(Args32 a) {
+  constexpr int U = 4;  // slots a lane in flight
+  DevCtl *ctl = a.ctl;
+  const bool coef_only = ctl->done;
+  const int T = ctl->round, t = T + 1;
+  const float *__restrict__ Ms = (T & 1) ? a.MP1 : a.MP0;  // P_ki of round T
+  const float2 *__restrict__ QT = ring3(a.NQ0, a.NQ1, a.NQ2, T);
+  float *Hc = (t & 1) ? a.H1 : a.H0;  // holds t-2, becomes t
+  const float *__restrict__ Hm2 = ring3(a.NH0, a.NH1, a.NH2, t + 1);
+  float *__restrict__ Ht = ring3(a.NH0, a.NH1, a.NH2, t);
+  const WarpPos w = warp_pos();
+  float dxx = 0.f, xx = 0.f;
+  for (int m = 0; m * (int64_t)w.nwarps < a.ns; ++m) {
+    const int s = pass_slice(w, m);
+    if (s >= a.ns) continue;
+    const int p = 32 * s + w.lane, q1 = a.sp[s + 1];
+    const float2 qi = QT[p];
+    const float hi2 = t >= 2 ? Hm2[p] : 0.f, rhs = a.rhs[p];
+    float acc[4] = {};  // as by 4 lanes a row
+    for (int qb = a.sp[s] + w.lane; qb < q1; qb += 32 * U) {
+      int k[U];
+      float A[U], Ps[U], hs[U];
+      float2 qk[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int q = qb + 32 * u;
+        k[u] = -1;
+        if (q < q1) { k[u] = __ldcs(a.ci + q); A[u] = __ldcs(a.av + q); Ps[u] = __ldcs(Ms + q); hs[u] = __ldcs(Hc + q); }
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        if (k[u] >= 0) qk[u] = __ldcg(QT + k[u]);  // random gather, L2 only
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        if (k[u] >= 0) {
+          const float cout = -A[u] / (qi.x - Ps[u]);
+          const float Pout = cout * A[u];
+          const float cin = -A[u] / (qk[u].x - Pout);
+          a.CF[qb + 32 * u] = make_float2(cin, cout);
+          if (!coef_only) {
+            const float hout = t >= 2 ? cout * (hi2 - hs[u]) : 0.f;  // message i -> k at t-1
+            const float hn = cin * (qk[u].y - hout);                 // message k -> i at t
+            __stcs(Hc + qb + 32 * u, hn);
+            acc[u] += hn;
+          }
+        }
     }
-    if (a.use_cond && ctl->done) cudaGraphSetConditional(a.cond, 0);
-    ctl->arrive = 0;
-    __threadfence();
+    const float ip = 1.f / qi.x;
+    a.invP[p] = ip;
+    if (!coef_only) {
+      const float hnew = rhs + ((acc[0] + acc[2]) + (acc[1] + acc[3]));
+      Ht[p] = hnew;
+      const float x = hnew * ip, dx = (hnew - qi.y) * ip;
+      dxx = fmaf(dx, dx, dxx);
+      xx = fmaf(x, x, xx);
+    }
   }
+  if (coef_only) return;
+  double v[2] = {(double)dxx, (double)xx}, tot[2];
+  block_sum<2>(v);
+  if (last_block_reduce<2>(v, a.partials, &ctl->arrive, tot) && threadIdx.x == 0) mean_decide(a, ctl, t, tot);
 }
 
 // ---------------------------------------------------------------------------- FP64 outer steps
@@ -728,7 +914,8 @@ __global__ void __launch_bounds__(kBlock) k64_residual(int n, const int *__restr
                                                        const double *__restrict__ b, const double *__restrict__ x,
                                                        float *__restrict__ rhs32, float *__restrict__ nh0,
                                                        DevCtl *ctl, double *partials, int set_bb,
-                                                       const int *skip = nullptr, int x_zero = 0) {
+                                                       const int *__restrict__ pos, const int *skip = nullptr,
+                                                       int x_zero = 0) {
   if (skip && *skip) return;  // device-loop graph: the loop already stopped
   constexpr int RPW = 32 / L;
   const int lane = threadIdx.x & 31, sl = lane & (L - 1), sw = lane / L;
@@ -763,8 +950,9 @@ __global__ void __launch_bounds__(kBlock) k64_residual(int n, const int *__restr
       const double r = bi - ax;
       rr = fma(r, r, rr);
       const float rf = (float)r;
-      rhs32[i] = rf;
-      nh0[i] = rf;
+      const int at = pos ? pos[i] : i;  // position in the sliced layout
+      rhs32[at] = rf;
+      nh0[at] = rf;
     }
   }
   double v[1] = {rr}, tot[1];
@@ -781,9 +969,11 @@ __global__ void __launch_bounds__(kBlock) k64_residual(int n, const int *__restr
 
 // x <- x + d, d_i = h~_i / P~_i of the inner solve's final round (FP64 accumulate).
 __global__ void k64_update(int n, double *__restrict__ x, const float *__restrict__ hT,
-                           const float *__restrict__ invP) {
+                           const float *__restrict__ invP, const int *__restrict__ pos) {
   int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) x[i] += (double)(hT[i] * invP[i]);
+  if (i >= n) return;
+  const int at = pos ? pos[i] : i;
+  x[i] += (double)(hT[at] * invP[at]);
 }
 
 __global__ void k_to_f32(int64_t m, const double *__restrict__ s, float *__restrict__ d) {
@@ -834,9 +1024,119 @@ __global__ void k_gamma(int n, int mode, double gamma, const int *__restrict__ r
   }
 }
 
-__global__ void k32_marginals(int n, const float *__restrict__ P, double *__restrict__ Pi) {
+__global__ void k32_marginals(int n, const float *__restrict__ P, const int *__restrict__ pos, double *__restrict__ Pi) {
   int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) Pi[i] = (double)P[i];
+  if (i < n) Pi[i] = (double)P[pos ? pos[i] : i];
+}
+
+// ---------------------------------------------------------------------------- sliced layout
+// Rows sorted by degree (descending, stable) in windows of kSellWindow, one window a block: srow, its inverse
+// pos, and the width of each slice at sp[slice + 1].
+constexpr int kMaxKeyDegree = 0xfffff;
+__global__ void __launch_bounds__(1024) k_sort32(int n, int npos, const int *__restrict__ rp, int *__restrict__ srow,
+                                                 int *__restrict__ pos, int *__restrict__ sp) {
+  __shared__ unsigned key[kSellWindow];
+  const int w0 = blockIdx.x * kSellWindow;
+  for (int j = threadIdx.x; j < kSellWindow; j += 1024) {
+    const int d = w0 + j < n ? rp[w0 + j + 1] - rp[w0 + j] : 0;
+    key[j] = ((unsigned)(kMaxKeyDegree - min(d, kMaxKeyDegree)) << 12) | (unsigned)j;
+  }
+  for (int k = 2; k <= kSellWindow; k <<= 1)
+    for (int d = k >> 1; d > 0; d >>= 1) {
+      __syncthreads();
+      for (int x = threadIdx.x; x < kSellWindow / 2; x += 1024) {
+        const int lo = 2 * x - (x & (d - 1)), hi = lo + d;
+        const unsigned u = key[lo], v = key[hi];
+        if ((u > v) == ((lo & k) == 0)) {
+          key[lo] = v;
+          key[hi] = u;
+        }
+      }
+    }
+  __syncthreads();
+  for (int j = threadIdx.x; j < kSellWindow; j += 1024) {
+    const int p = w0 + j, i = w0 + (int)(key[j] & (kSellWindow - 1));
+    if (p >= npos) continue;
+    srow[p] = i < n ? i : -1;
+    if (i < n) pos[i] = p;
+    if ((p & 31) == 0) sp[p / 32 + 1] = kMaxKeyDegree - (int)(key[j] >> 12);
+  }
+}
+
+// Widths at sp[1 ..] to first slots; out: slots in all, the widest slice.  One block.
+__global__ void __launch_bounds__(1024) k_scan32(int ns, int *__restrict__ sp, long long *__restrict__ out) {
+  __shared__ long long sum[1024];
+  __shared__ int top[1024];
+  const int c = (ns + 1023) / 1024, s0 = min(ns, (int)threadIdx.x * c), s1 = min(ns, s0 + c);
+  long long v = 0;
+  int wmax = 0;
+  for (int s = s0; s < s1; ++s) {
+    v += 32LL * sp[s + 1];
+    wmax = max(wmax, sp[s + 1]);
+  }
+  sum[threadIdx.x] = v;
+  top[threadIdx.x] = wmax;
+  for (int d = 1; d < 1024; d <<= 1) {
+    __syncthreads();
+    const long long u = threadIdx.x >= d ? sum[threadIdx.x - d] : 0;
+    const int x = threadIdx.x >= d ? top[threadIdx.x - d] : 0;
+    __syncthreads();
+    sum[threadIdx.x] += u;
+    top[threadIdx.x] = max(top[threadIdx.x], x);
+  }
+  __syncthreads();
+  long long at = sum[threadIdx.x] - v;
+  for (int s = s0; s < s1; ++s) {
+    at += 32LL * sp[s + 1];
+    sp[s + 1] = (int)at;
+  }
+  if (threadIdx.x == 0) sp[0] = 0;
+  if (threadIdx.x == 1023) {
+    out[0] = sum[1023];
+    out[1] = top[1023];
+  }
+}
+
+// f(position, slot of the CSR or -1) for every position of the slices, a warp a slice; g(p, i) for its rows.
+template <typename F, typename G>
+__device__ __forceinline__ void for_slices(int ns, const int *__restrict__ srow, const int *__restrict__ sp,
+                                           const int *__restrict__ rp, F &&f, G &&g) {
+  const WarpPos w = warp_pos();
+  for (int s = w.warp; s < ns; s += w.nwarps) {
+    const int p = 32 * s + w.lane, i = srow[p], q1 = sp[s + 1];
+    const int e0 = i < 0 ? 0 : rp[i], e1 = i < 0 ? 0 : rp[i + 1];
+    g(p, i);
+    int e = e0;
+    for (int q = sp[s] + w.lane; q < q1; q += 32, ++e) f(q, e < e1 ? e : -1);
+  }
+}
+__global__ void __launch_bounds__(kBlock) k_fill32(Sell32 S, const int *__restrict__ rp, const int *__restrict__ ci,
+                                                   const double *__restrict__ av, int columns) {
+  for_slices(S.ns, S.srow, S.sp, rp,
+             [&](int q, int e) {
+               if (columns) S.sci[q] = e < 0 ? -1 : S.pos[ci[e]];
+               S.sav[q] = e < 0 ? 0.f : (float)av[e];
+             },
+             [](int, int) {});
+}
+// Frozen coefficients from the CSR order to the sliced one, and back.
+__global__ void __launch_bounds__(kBlock) k_coef_slice(Sell32 S, const int *__restrict__ rp, const float2 *__restrict__ CF,
+                                                       const float *__restrict__ invP) {
+  for_slices(S.ns, S.srow, S.sp, rp, [&](int q, int e) { if (e >= 0) S.CF[q] = CF[e]; },
+             [&](int p, int i) { S.invP[p] = i < 0 ? 1.f : invP[i]; });
+}
+__global__ void __launch_bounds__(kBlock) k_coef_unslice(Sell32 S, const int *__restrict__ rp, float2 *__restrict__ CF,
+                                                         float *__restrict__ invP) {
+  for_slices(S.ns, S.srow, S.sp, rp, [&](int q, int e) { if (e >= 0) CF[e] = S.CF[q]; },
+             [&](int p, int i) { if (i >= 0) invP[i] = S.invP[p]; });
+}
+// Diagonal (+ loading) by position, 1 where there is no row.
+__global__ void k_diag32_sliced(int npos, const int *__restrict__ srow, const double *__restrict__ ad,
+                                const double *__restrict__ gam, float *__restrict__ d32) {
+  const int p = blockIdx.x * blockDim.x + threadIdx.x;
+  if (p >= npos) return;
+  const int i = srow[p];
+  d32[p] = i < 0 ? 1.f : (float)(ad[i] + (gam ? gam[i] : 0.0));
 }
 
 // ---------------------------------------------------------------------------- host side
@@ -852,20 +1152,24 @@ gabp_status marginals32(gabp_handle h, double *Pi) {
   Work32 &w = h->w32;
   if (!w.MP[0] || w.prec_round < 0) return GABP_ERR_INVALID;
   Graph &g = h->g;
-  const float *P = w.NP[w.prec_round % 3];
-  k32_marginals<<<(g.n + kBlock - 1) / kBlock, kBlock, 0, h->stream>>>(g.n, P, Pi);
+  const float *P = w.prec_sliced ? w.sl.NP[w.prec_round % 3] : w.NP[w.prec_round % 3];
+  k32_marginals<<<(g.n + kBlock - 1) / kBlock, kBlock, 0, h->stream>>>(g.n, P, w.prec_sliced ? w.sl.pos : nullptr, Pi);
   GABP_CUDA(cudaGetLastError());
   GABP_CUDA(cudaStreamSynchronize(h->stream));
   return GABP_OK;
 }
 
+// Positions of the sliced layout that the message chains have room for: E and 3 % for its padding.
+static size_t sell32_room(int64_t E) { return (size_t)(E + E / 32 + 4096); }
+
 gabp_status ensure_w32(gabp_handle h, int R) {
   Work32 &w = h->w32;
   Graph &g = h->g;
   size_t E = (size_t)(g.E > 0 ? g.E : 1), n = (size_t)g.n;
+  const size_t Es = sell32_room(g.E);  // the chains serve the sliced layout, too
   if (!w.MP[0]) {
-    GABP_CUDA(cudaMalloc(&w.MP[0], sizeof(float) * E));
-    GABP_CUDA(cudaMalloc(&w.MP[1], sizeof(float) * E));
+    GABP_CUDA(cudaMalloc(&w.MP[0], sizeof(float) * Es));
+    GABP_CUDA(cudaMalloc(&w.MP[1], sizeof(float) * Es));
     for (int j = 0; j < 3; ++j) GABP_CUDA(cudaMalloc(&w.NP[j], sizeof(float) * n));
     GABP_CUDA(cudaMalloc(&w.CF, sizeof(float2) * E));
     GABP_CUDA(cudaMalloc(&w.invP, sizeof(float) * n));
@@ -885,8 +1189,8 @@ gabp_status ensure_w32(gabp_handle h, int R) {
     w.NH[0] = w.NH[1] = w.NH[2] = nullptr;
     w.rhs32 = nullptr; w.X = w.Rs = w.Bt = nullptr;
     w.R = 0;
-    GABP_CUDA(cudaMalloc(&w.H[0], sizeof(float) * E * R));
-    GABP_CUDA(cudaMalloc(&w.H[1], sizeof(float) * E * R));
+    GABP_CUDA(cudaMalloc(&w.H[0], sizeof(float) * Es * R));
+    GABP_CUDA(cudaMalloc(&w.H[1], sizeof(float) * Es * R));
     for (int j = 0; j < 3; ++j) {  // room for the dense rounds' padding columns, finite values there
       const size_t rows = (n + 31) / 32 * 32;
       GABP_CUDA(cudaMalloc(&w.NH[j], sizeof(float) * rows * R));
@@ -907,6 +1211,12 @@ gabp_status ensure_w32(gabp_handle h, int R) {
   return GABP_OK;
 }
 
+static void free_sell32(Sell32 &S) {
+  cudaFree(S.srow); cudaFree(S.pos); cudaFree(S.sp); cudaFree(S.sci); cudaFree(S.sav); cudaFree(S.CF);
+  cudaFree(S.nodes);
+  S = Sell32{};
+}
+
 void free_w32(gabp_handle h) {
   Work32 &w = h->w32;
   cudaFree(w.MP[0]); cudaFree(w.MP[1]);
@@ -915,6 +1225,7 @@ void free_w32(gabp_handle h) {
   cudaFree(w.rhs32); cudaFree(w.X); cudaFree(w.Rs); cudaFree(w.Bt); cudaFree(w.colnorm);
   cudaFree(w.ctlR); cudaFree(w.rhs_active); cudaFree(w.rc); cudaFree(w.Bd);
   cudaFree(w.dCin); cudaFree(w.dCout); cudaFree(w.dH); cudaFree(w.dSp);
+  free_sell32(w.sl);
   if (w.rc_host) cudaFreeHost(w.rc_host);
   w = Work32{};
 }
@@ -933,11 +1244,136 @@ static Args32 args32(gabp_handle h) {
   a.NH0 = w.NH[0]; a.NH1 = w.NH[1]; a.NH2 = w.NH[2];
   a.rhs = w.rhs32;
   a.NQ0 = w.NQ[0]; a.NQ1 = w.NQ[1]; a.NQ2 = w.NQ[2];
+  a.ns = 0;
+  a.sp = nullptr;
   a.cond = 0;
   a.use_cond = 0;
   a.ctl = h->ctl;
   a.partials = h->partials;
   return a;
+}
+
+// The arguments of the joint, freeze and mean rounds: the sliced layout's arrays where it is in use.
+static Args32 round_args32(gabp_handle h) {
+  Args32 a = args32(h);
+  Work32 &w = h->w32;
+  if (!w.sl_on) return a;
+  const Sell32 &S = w.sl;
+  a.n = 32 * S.ns; a.ns = S.ns; a.sp = S.sp; a.ci = S.sci; a.av = S.sav; a.ad = S.ad;
+  a.NP0 = S.NP[0]; a.NP1 = S.NP[1]; a.NP2 = S.NP[2];
+  a.CF = S.CF; a.invP = S.invP; a.rhs = S.rhs;
+  a.NH0 = S.NH[0]; a.NH1 = S.NH[1]; a.NH2 = S.NH[2];
+  a.NQ0 = S.NQ[0]; a.NQ1 = S.NQ[1]; a.NQ2 = S.NQ[2];
+  return a;
+}
+
+// The sliced layout of the FP32 rounds (sets w.sl_on when they run on it): 32 rows a slice, lane by row, so that a
+// warp's load of a stream is one line.  The row kernels' loads are cut at the rows (16 slots a row, 8 lanes: 4 to 8
+// lines a load), and the L1, which takes a line a cycle, bounds them: the gathers alone need 65 us of it for 16.8 M
+// slots.  Whole solves, row kernels / sliced: 2^20 rows of 16 slots 2907 / 2396 us, 1.6 M rows of 10 (least squares)
+// 7548 / 5844, 2^22 rows of 6 with new values, forward and adjoint 13597 / 10459; the first solve of a 400 K-row
+// graph 13.8 / 2.5 ms (no shapes to tune).
+// Not where there are too few rows for a lane each: the row kernels give a row up to 16.  6 slots a row: 20 K rows
+// 448 / 472 us, 40 K 507 / 499, 80 K 556 / 523; 16 slots: 80 K 521 / 544, 160 K 710 / 723, 400 K 1316 / 1194: from
+// kSellRowsSlot rows a slot of the average row on.  Not where a lane's row would be long, where the padding exceeds the
+// chains' room, or where there is no memory for it.
+constexpr int kSellWidth32 = 96;
+constexpr double kSellRowsSlot = 12000.0;
+static gabp_status ensure_sell32(gabp_handle h) {
+  Work32 &w = h->w32;
+  Sell32 &S = w.sl;
+  const Graph &g = h->g;
+  w.sl_on = false;
+  if (h->opt.lanes || w.dense_ld || g.E == 0 || g.n < kSellRowsSlot * g.avg_deg) return GABP_OK;
+  if (!S.tried) {
+    S.tried = true;
+    const int ns = (g.n - 1) / 32 + 1, npos = 32 * ns;
+    long long out[2] = {0, 0};
+    bool room = cudaMalloc(&S.srow, sizeof(int) * npos) == cudaSuccess &&
+                cudaMalloc(&S.pos, sizeof(int) * (size_t)g.n) == cudaSuccess &&
+                cudaMalloc(&S.sp, sizeof(int) * ((size_t)ns + 1)) == cudaSuccess;
+    if (room) {
+      k_sort32<<<(g.n - 1) / kSellWindow + 1, 1024, 0, h->stream>>>(g.n, npos, g.rp, S.srow, S.pos, S.sp);
+      long long *dout = reinterpret_cast<long long *>(h->partials);  // idle between runs
+      k_scan32<<<1, 1024, 0, h->stream>>>(ns, S.sp, dout);
+      GABP_CUDA(cudaGetLastError());
+      GABP_CUDA(cudaMemcpyAsync(out, dout, sizeof(out), cudaMemcpyDeviceToHost, h->stream));
+      GABP_CUDA(cudaStreamSynchronize(h->stream));
+      room = out[1] <= kSellWidth32 && out[0] < INT32_MAX - 4096 && (size_t)out[0] <= sell32_room(g.E);
+    }
+    if (room) {
+      const size_t Es = (size_t)out[0], nodes = sizeof(float) * 15 * (size_t)npos;
+      room = cudaMalloc(&S.sci, sizeof(int) * Es) == cudaSuccess && cudaMalloc(&S.sav, sizeof(float) * Es) == cudaSuccess &&
+             cudaMalloc(&S.CF, sizeof(float2) * Es) == cudaSuccess && cudaMalloc(&S.nodes, nodes) == cudaSuccess;
+      if (room) {
+        GABP_CUDA(cudaMemsetAsync(S.nodes, 0, nodes, h->stream));  // zeros where there is no row
+        float *at = S.nodes;
+        for (int j = 0; j < 3; ++j, at += 2 * (size_t)npos) S.NQ[j] = reinterpret_cast<float2 *>(at);
+        for (int j = 0; j < 3; ++j, at += npos) S.NP[j] = at;
+        for (int j = 0; j < 3; ++j, at += npos) S.NH[j] = at;
+        S.invP = at; S.rhs = at + npos; S.ad = at + 2 * (size_t)npos;
+        S.ns = ns;
+        S.Es = (int)Es;
+        k_fill32<<<blocks_for(ns, kBlock / 32, h->max_blocks), kBlock, 0, h->stream>>>(S, g.rp, g.ci, g.av, 1);
+        GABP_CUDA(cudaGetLastError());
+        S.vals_ok = true;
+      }
+    }
+    if (!room) {
+      cudaGetLastError();
+      free_sell32(S);
+      S.tried = true;
+    }
+  }
+  if (!S.ns) return GABP_OK;
+  if (!S.vals_ok) {
+    k_fill32<<<blocks_for(S.ns, kBlock / 32, h->max_blocks), kBlock, 0, h->stream>>>(S, g.rp, g.ci, g.av, 0);
+    GABP_CUDA(cudaGetLastError());
+    h->prof.launches += 1;
+    S.vals_ok = true;
+  }
+  w.sl_on = true;
+  return GABP_OK;
+}
+
+// The diagonal (+ loading) that the FP32 rounds run on.
+static void diag32(gabp_handle h, const double *gamma_diag) {
+  const Graph &g = h->g;
+  const Sell32 &S = h->w32.sl;
+  if (h->w32.sl_on)
+    k_diag32_sliced<<<(32 * S.ns + kBlock - 1) / kBlock, kBlock, 0, h->stream>>>(32 * S.ns, S.srow, g.ad, gamma_diag, S.ad);
+  else
+    k_diag32<<<(g.n + kBlock - 1) / kBlock, kBlock, 0, h->stream>>>(g.n, g.ad, gamma_diag, g.ad32);
+}
+
+void drop_coef32(gabp_handle h) { h->w32.coef_ready = h->w32.sl.coef_ready = false; }
+
+// Coefficients that are frozen in one order, in the other.
+gabp_status csr_coef32(gabp_handle h) {
+  Work32 &w = h->w32;
+  if (w.coef_ready || !w.sl.coef_ready) return GABP_OK;
+  k_coef_unslice<<<blocks_for(w.sl.ns, kBlock / 32, h->max_blocks), kBlock, 0, h->stream>>>(w.sl, h->g.rp, w.CF, w.invP);
+  GABP_CUDA(cudaGetLastError());
+  h->prof.launches += 1;
+  w.coef_ready = true;
+  return GABP_OK;
+}
+static gabp_status sliced_coef32(gabp_handle h) {
+  Work32 &w = h->w32;
+  if (w.sl.coef_ready || !w.coef_ready) return GABP_OK;
+  k_coef_slice<<<blocks_for(w.sl.ns, kBlock / 32, h->max_blocks), kBlock, 0, h->stream>>>(w.sl, h->g.rp, w.CF, w.invP);
+  GABP_CUDA(cudaGetLastError());
+  h->prof.launches += 1;
+  w.sl.coef_ready = true;
+  return GABP_OK;
+}
+static gabp_status ready_coef32(gabp_handle h) { return h->w32.sl_on ? sliced_coef32(h) : csr_coef32(h); }
+static void frozen32(gabp_handle h, int T) {  // the joint rounds' precisions of round T are frozen
+  Work32 &w = h->w32;
+  w.prec_round = T;
+  w.prec_sliced = w.sl_on;
+  w.coef_ready = !w.sl_on;
+  w.sl.coef_ready = w.sl_on;
 }
 
 // The dense mean rounds' arrays (complete patterns of kDenseMin rows or more, unless the shape of the
@@ -983,11 +1419,29 @@ static void launch_mean(gabp_handle h, const Args32 &a, cudaStream_t st) {
   const int n = h->g.n;
   if (a.ld)
     k32_dense<<<h->w32.dense_grid, kBlock, sizeof(float) * a.ld, st>>>(a);
+  else if (a.ns)
+    ks32_mean<<<blocks_for(a.ns, kBlock / 32, resident_grid(h->num_sms, ks32_mean)), kBlock, 0, st>>>(a);
   else if (a.dense)
     k32_mean<LL, UU, true><<<blocks_for(n, kBlock / LL, resident_grid(h->num_sms, k32_mean<LL, UU, true>)), kBlock, 0,
                              st>>>(a);
   else
     k32_mean<LL, UU><<<blocks_for(n, kBlock / LL, resident_grid(h->num_sms, k32_mean<LL, UU>)), kBlock, 0, st>>>(a);
+}
+
+// A joint round, and the freeze fused with the first mean round, in the same forms.
+template <int LL, int UU>
+static void launch_joint(gabp_handle h, const Args32 &a, cudaStream_t st) {
+  if (a.ns)
+    ks32_joint<<<blocks_for(a.ns, kBlock / 32, resident_grid(h->num_sms, ks32_joint)), kBlock, 0, st>>>(a);
+  else
+    k32_joint<LL, UU><<<blocks_for(a.n, kBlock / LL, resident_grid(h->num_sms, k32_joint<LL, UU>)), kBlock, 0, st>>>(a);
+}
+template <int LL, int UU>
+static void launch_freeze(gabp_handle h, const Args32 &a, cudaStream_t st) {
+  if (a.ns)
+    ks32_freeze<<<blocks_for(a.ns, kBlock / 32, resident_grid(h->num_sms, ks32_freeze)), kBlock, 0, st>>>(a);
+  else
+    k32_freeze<LL, UU><<<blocks_for(a.n, kBlock / LL, resident_grid(h->num_sms, k32_freeze<LL, UU>)), kBlock, 0, st>>>(a);
 }
 
 // Shape (lanes per row, unroll) of an FP32 round kernel: the option if set, else
@@ -1087,7 +1541,9 @@ gabp_status precision_phase32(gabp_handle h, const double *gamma_diag) {
   h->prof.launches += 1;
   GABP_CUDA(cudaGetLastError());
   w.prec_round = c.result_round;
+  w.prec_sliced = false;
   w.coef_ready = true;
+  w.sl.coef_ready = false;
   w.dense_packed = false;
   return GABP_OK;
 }
@@ -1099,34 +1555,33 @@ gabp_status precision_phase32(gabp_handle h, const double *gamma_diag) {
 static gabp_status joint_phase32(gabp_handle h, const double *gamma_diag, int cap, int *T_out) {
   Work32 &w = h->w32;
   Graph &g = h->g;
-  size_t E = (size_t)(g.E > 0 ? g.E : 1);
-  k_diag32<<<(g.n + kBlock - 1) / kBlock, kBlock, 0, h->stream>>>(g.n, g.ad, gamma_diag, g.ad32);
+  const Args32 a = round_args32(h);
+  const size_t E = a.ns ? (size_t)w.sl.Es : (size_t)(g.E > 0 ? g.E : 1);
+  diag32(h, gamma_diag);
   auto init = [&]() -> gabp_status {
     GABP_CUDA(cudaMemsetAsync(w.MP[0], 0, sizeof(float) * E, h->stream));
     GABP_CUDA(cudaMemsetAsync(w.MP[1], 0, sizeof(float) * E, h->stream));
     GABP_CUDA(cudaMemsetAsync(w.H[0], 0, sizeof(float) * E, h->stream));
-    k32_joint_init<<<(g.n + kBlock - 1) / kBlock, kBlock, 0, h->stream>>>(g.n, g.ad32, w.rhs32, w.NQ[0], w.NP[0]);
+    k32_joint_init<<<(a.n + kBlock - 1) / kBlock, kBlock, 0, h->stream>>>(a.n, a.ad, a.rhs, a.NQ0, a.NP0);
     GABP_CUDA(cudaGetLastError());
     return GABP_OK;
   };
   gabp_status st = init();
   if (st != GABP_OK) return st;
-  if (!h->opt.lanes && !h->tuned_Lj32) {
+  if (!a.ns && !h->opt.lanes && !h->tuned_Lj32) {
     if ((st = autotune32(h, K32_JOINT)) != GABP_OK) return st;
     if ((st = init()) != GABP_OK) return st;
   }
-  const int SH = shape32(h, K32_JOINT);
+  const int SH = shape32(h, K32_JOINT), key = a.ns ? -2 : SH;
   const int rounds = std::max(1, std::min(kPrecMaxRounds, cap));
   k_ctl_reset<<<1, 1, 0, h->stream>>>(h->ctl, rounds, std::ldexp(1.0, -h->opt.prec_stop_log2));
   h->prof.launches += 3;
   GABP_CUDA(cudaGetLastError());
-  Args32 a = args32(h);
   gabp_status s;
   with_shape(SH, [&](auto Lc, auto Uc) {
     constexpr int LL = decltype(Lc)::value, UU = decltype(Uc)::value;
-    s = run_rounds(h, &h->gJ32, &h->gJ32_L, SH, [&] {
-      const int nb = blocks_for(g.n, kBlock / LL, resident_grid(h->num_sms, k32_joint<LL, UU>));
-      k32_joint<LL, UU><<<nb, kBlock, 0, h->stream>>>(a);
+    s = run_rounds(h, &h->gJ32, &h->gJ32_L, key, [&] {
+      launch_joint<LL, UU>(h, a, h->stream);
     }, rounds, PH_PREC32);
   });
   if (s != GABP_OK) return s;
@@ -1141,21 +1596,19 @@ static gabp_status joint_phase32(gabp_handle h, const double *gamma_diag, int ca
 static gabp_status freeze32(gabp_handle h, int T) {
   Graph &g = h->g;
   Work32 &w = h->w32;
-  Args32 a = args32(h);
+  const Args32 a = round_args32(h);
   const int SH = shape32(h, K32_JOINT);
   prof_begin(h);
   with_shape(SH, [&](auto Lc, auto Uc) {
     constexpr int LL = decltype(Lc)::value, UU = decltype(Uc)::value;
-    k32_freeze<LL, UU><<<blocks_for(g.n, kBlock / LL, resident_grid(h->num_sms, k32_freeze<LL, UU>)), kBlock, 0,
-                         h->stream>>>(a);
+    launch_freeze<LL, UU>(h, a, h->stream);
   });
   if (a.ld) k32_dense_pack<<<blocks_for(g.n, 1, h->max_blocks), kBlock, 0, h->stream>>>(a, 1);
   prof_end(h);
   GABP_CUDA(cudaGetLastError());
   prof_collect(h, PH_FREEZE32, 1);
   h->prof.launches += a.ld ? 2 : 1;
-  w.prec_round = T;
-  w.coef_ready = true;
+  frozen32(h, T);
   w.dense_packed = a.ld > 0;
   return GABP_OK;
 }
@@ -1314,12 +1767,15 @@ __global__ void k_ref_after_inner(RefineCtl *rc, const DevCtl *ctl) {
 
 // x <- x + d with d from the inner solve's final round (read on the device)
 __global__ void k64_update_ctl(int n, double *__restrict__ x, const float *NH0, const float *NH1, const float *NH2,
-                               const float *__restrict__ invP, const DevCtl *ctl, const int *skip) {
+                               const float *__restrict__ invP, const int *__restrict__ pos, const DevCtl *ctl,
+                               const int *skip) {
   if (*skip) return;
   const int m = ctl->result_round % 3;
   const float *__restrict__ hT = m == 0 ? NH0 : (m == 1 ? NH1 : NH2);
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) x[i] += (double)(hT[i] * invP[i]);
+  if (i >= n) return;
+  const int at = pos ? pos[i] : i;
+  x[i] += (double)(hT[at] * invP[at]);
 }
 
 // A graph under construction: nodes are appended in sequence after `last`.
@@ -1387,7 +1843,6 @@ static int residual_lanes(gabp_handle h) {
 static gabp_status build_refine_graph(gabp_handle h, int SHm, int SHj, int LR) {
   Graph &g = h->g;
   Work32 &w = h->w32;
-  const size_t E = (size_t)(g.E > 0 ? g.E : 1);
   cudaStream_t st = h->stream;
   cudaGraph_t root;
   GABP_CUDA(cudaGraphCreate(&root, 0));
@@ -1400,15 +1855,18 @@ static gabp_status build_refine_graph(gabp_handle h, int SHm, int SHj, int LR) {
   GABP_CUDA(cudaGraphConditionalHandleCreate(&h_joint, root, 0, cudaGraphCondAssignDefault));
   GABP_CUDA(cudaGraphConditionalHandleCreate(&h_jw, root, 0, cudaGraphCondAssignDefault));
   GABP_CUDA(cudaGraphConditionalHandleCreate(&h_inner, root, 0, cudaGraphCondAssignDefault));
-  Args32 a = args32(h);
+  const Args32 a = round_args32(h);
+  const size_t E = a.ns ? (size_t)w.sl.Es : (size_t)(g.E > 0 ? g.E : 1);
+  const int *pos = a.ns ? w.sl.pos : nullptr;
+  float *rhs32 = const_cast<float *>(a.rhs);
   int nbr = 1;
   GABP_DISPATCH_L(LR, nbr = blocks_for(g.n, kBlock / LL, resident_grid(h->num_sms, k64_residual<LL>)));
   RefineCtl *rc = w.rc;
   const int nb1 = (g.n + kBlock - 1) / kBlock;
   auto residual = [&](int first) {
-    GABP_DISPATCH_L(LR, (k64_residual<LL><<<nbr, kBlock, 0, st>>>(g.n, g.rowptr, g.col, g.val, w.Bd, w.X, w.rhs32,
-                                                                    w.NH[0], w.ctlR, h->partials, first,
-                                                                    &rc->skip, first)));
+    GABP_DISPATCH_L(LR, (k64_residual<LL><<<nbr, kBlock, 0, st>>>(g.n, g.rowptr, g.col, g.val, w.Bd, w.X, rhs32, a.NH0,
+                                                                    w.ctlR, h->partials, first, pos, &rc->skip,
+                                                                    first)));
   };
   SeqGraph top{root, nullptr};
   cudaError_t e = seq_capture(top, st, [&] {
@@ -1429,7 +1887,7 @@ static gabp_status build_refine_graph(gabp_handle h, int SHm, int SHj, int LR) {
       cudaMemsetAsync(w.MP[0], 0, sizeof(float) * E, st);
       cudaMemsetAsync(w.MP[1], 0, sizeof(float) * E, st);
       if (a.ld) cudaMemsetAsync(w.H[0], 0, sizeof(float) * E, st);
-      k32_joint_init<<<nb1, kBlock, 0, st>>>(g.n, g.ad32, w.rhs32, w.NQ[0], w.NP[0]);
+      k32_joint_init<<<(a.n + kBlock - 1) / kBlock, kBlock, 0, st>>>(a.n, a.ad, a.rhs, a.NQ0, a.NP0);
       k_joint_prep<<<1, 1, 0, st>>>(rc, h->ctl, h_jw);
     });
   if (e == cudaSuccess) e = seq_conditional(joint, h_jw, cudaGraphCondTypeWhile, &jw);
@@ -1440,8 +1898,7 @@ static gabp_status build_refine_graph(gabp_handle h, int SHm, int SHj, int LR) {
       aj.use_cond = 1;
       with_shape(SHj, [&](auto Lc, auto Uc) {
         constexpr int LL = decltype(Lc)::value, UU = decltype(Uc)::value;
-        const int nb = blocks_for(g.n, kBlock / LL, resident_grid(h->num_sms, k32_joint<LL, UU>));
-        for (int k = 0; k < kLoopK; ++k) k32_joint<LL, UU><<<nb, kBlock, 0, st>>>(aj);
+        for (int k = 0; k < kLoopK; ++k) launch_joint<LL, UU>(h, aj, st);
       });
     });
   if (e == cudaSuccess)
@@ -1453,8 +1910,7 @@ static gabp_status build_refine_graph(gabp_handle h, int SHm, int SHj, int LR) {
       af.use_cond = 1;
       with_shape(SHj, [&](auto Lc, auto Uc) {
         constexpr int LL = decltype(Lc)::value, UU = decltype(Uc)::value;
-        k32_freeze<LL, UU><<<blocks_for(g.n, kBlock / LL, resident_grid(h->num_sms, k32_freeze<LL, UU>)), kBlock, 0,
-                             st>>>(af);
+        launch_freeze<LL, UU>(h, af, st);
       });
       if (a.ld) k32_dense_pack<<<blocks_for(g.n, 1, h->max_blocks), kBlock, 0, st>>>(af, 1);
       k_joint_mark<<<1, 1, 0, st>>>(rc, h->ctl, a.ld ? 1 : 0);
@@ -1474,7 +1930,7 @@ static gabp_status build_refine_graph(gabp_handle h, int SHm, int SHj, int LR) {
   if (e == cudaSuccess)
     e = seq_capture(outer, st, [&] {
       k_ref_after_inner<<<1, 1, 0, st>>>(rc, h->ctl);
-      k64_update_ctl<<<nb1, kBlock, 0, st>>>(g.n, w.X, w.NH[0], w.NH[1], w.NH[2], w.invP, h->ctl, &rc->skip);
+      k64_update_ctl<<<nb1, kBlock, 0, st>>>(g.n, w.X, a.NH0, a.NH1, a.NH2, a.invP, pos, h->ctl, &rc->skip);
       residual(0);
       k_ref_decide<<<1, 1, 0, st>>>(rc, w.ctlR, h->ctl, 0, h_outer, h_joint, h_inner);
     });
@@ -1502,17 +1958,18 @@ static gabp_status solve32_device_loop(gabp_handle h, const double *B, double *X
   }
   gabp_status sd = ensure_dense32(h);
   if (sd != GABP_OK) return sd;
-  const bool joint = !w.coef_ready || !h->opt.reuse_precisions;
+  if ((sd = ensure_sell32(h)) != GABP_OK) return sd;
+  const bool joint = !(w.coef_ready || w.sl.coef_ready) || !h->opt.reuse_precisions;
   if (joint) {
-    w.coef_ready = false;
+    drop_coef32(h);
     w.dense_packed = false;
     if (!h->opt.overlap_precision) {
       gabp_status s = precision_phase32(h, nullptr);
       if (s != GABP_OK) return s;
     } else {
-      k_diag32<<<(g.n + kBlock - 1) / kBlock, kBlock, 0, h->stream>>>(g.n, g.ad, nullptr, g.ad32);
+      diag32(h, nullptr);
       GABP_CUDA(cudaGetLastError());
-      if (!h->opt.lanes && !h->tuned_Lj32) {
+      if (!w.sl_on && !h->opt.lanes && !h->tuned_Lj32) {
         // the autotuner runs a few joint rounds on scratch state (re-initialised by the graph)
         const size_t E = (size_t)(g.E > 0 ? g.E : 1);
         GABP_CUDA(cudaMemsetAsync(w.rhs32, 0, sizeof(float) * g.n, h->stream));
@@ -1526,12 +1983,13 @@ static gabp_status solve32_device_loop(gabp_handle h, const double *B, double *X
     }
   }
   const bool run_joint = joint && h->opt.overlap_precision;
-  gabp_status s = w.dense_ld ? GABP_OK : autotune32(h, K32_MEAN);
-  if (s != GABP_OK) return s;
+  gabp_status s = w.dense_ld || w.sl_on ? GABP_OK : autotune32(h, K32_MEAN);
+  if (s != GABP_OK || (!run_joint && (s = ready_coef32(h)) != GABP_OK)) return s;
   if (w.dense_ld && !run_joint && (s = dense_pack(h)) != GABP_OK) return s;
   const int SHm = shape32(h, K32_MEAN), SHj = shape32(h, K32_JOINT);
   const int LR = residual_lanes(h);
-  const long long key = (long long)SHm | ((long long)SHj << 16) | ((long long)LR << 32) | ((long long)w.dense_ld << 40);
+  const long long key = (long long)SHm | ((long long)SHj << 16) | ((long long)LR << 32) | ((long long)w.dense_ld << 40) |
+                        ((long long)w.sl_on << 62);
   if (!h->gRef || h->gRef_key != key) {
     if ((s = build_refine_graph(h, SHm, SHj, LR)) != GABP_OK) return s;
     h->gRef_key = key;
@@ -1556,8 +2014,7 @@ static gabp_status solve32_device_loop(gabp_handle h, const double *B, double *X
   h->prof.launches += 3 + (int64_t)r.launches;  // k_ref_setup, the first residual and decision, the loop
   if (run_joint) {
     if (r.prec_round >= 0) {
-      w.prec_round = r.prec_round;
-      w.coef_ready = true;
+      frozen32(h, r.prec_round);
       w.dense_packed = w.dense_ld > 0;
     } else if (r.status != GABP_BREAKDOWN && r.status != GABP_DIVERGED) {
       // stopped before any inner solve (b = 0): the precision state is still provided
@@ -1590,29 +2047,32 @@ gabp_status solve32_refine(gabp_handle h, int R, const double *B, double *X, int
   // has to be computed, it is either computed first (precision-only rounds) or
   // together with the first inner solve (joint rounds, overlap_precision)
   bool joint = false;
-  if (serial) w.dense_ld = 0;
-  else if ((s = ensure_dense32(h)) != GABP_OK) return s;
-  if (!w.coef_ready || gamma_diag || !h->opt.reuse_precisions) {
-    w.coef_ready = false;
+  if (serial) { w.dense_ld = 0; w.sl_on = false; }
+  else if ((s = ensure_dense32(h)) != GABP_OK || (s = ensure_sell32(h)) != GABP_OK) return s;
+  if (!(w.coef_ready || w.sl.coef_ready) || gamma_diag || !h->opt.reuse_precisions) {
+    drop_coef32(h);
     w.dense_packed = false;
     joint = h->opt.overlap_precision != 0 && !serial;
     if (!joint) {
       if ((s = precision_phase32(h, gamma_diag)) != GABP_OK) return s;
-      if (gamma_diag) w.coef_ready = false;  // do not reuse a loaded state for a plain solve
     }
   }
+  if (!joint && (s = ready_coef32(h)) != GABP_OK) return s;
+  if (gamma_diag) drop_coef32(h);  // do not reuse a loaded state for a plain solve
   if (serial && (s = serial_freeze32(h, w.CF, w.invP)) != GABP_OK) return s;  // coefficients in the serial order
-  if (!serial && !w.dense_ld && (s = autotune32(h, K32_MEAN)) != GABP_OK) return s;
+  if (!serial && !w.dense_ld && !w.sl_on && (s = autotune32(h, K32_MEAN)) != GABP_OK) return s;
   if (!serial && w.dense_ld && !joint && (s = dense_pack(h)) != GABP_OK) return s;
   const int SH = shape32(h, K32_MEAN);
   const int LR = residual_lanes(h);
   int nbr = 1;
   GABP_DISPATCH_L(LR, nbr = blocks_for(g.n, kBlock / LL, resident_grid(h->num_sms, k64_residual<LL>)));
+  const Args32 a = round_args32(h);
+  const int *pos = a.ns ? w.sl.pos : nullptr;
+  float *rhs32 = const_cast<float *>(a.rhs);
   GABP_CUDA(cudaMemsetAsync(X, 0, sizeof(double) * g.n, h->stream));
   GABP_CUDA(cudaMemsetAsync(w.ctlR, 0, sizeof(DevCtl), h->stream));
-  GABP_DISPATCH_L(LR, (k64_residual<LL><<<nbr, kBlock, 0, h->stream>>>(g.n, g.rowptr, g.col, g.val, B, X, w.rhs32,
-                                                                          w.NH[0], w.ctlR, h->partials, 1, nullptr,
-                                                                          1)));
+  GABP_DISPATCH_L(LR, (k64_residual<LL><<<nbr, kBlock, 0, h->stream>>>(g.n, g.rowptr, g.col, g.val, B, X, rhs32, a.NH0,
+                                                                          w.ctlR, h->partials, 1, pos, nullptr, 1)));
   h->prof.launches += 1;
   GABP_CUDA(cudaGetLastError());
   DevCtl cr;
@@ -1625,13 +2085,12 @@ gabp_status solve32_refine(gabp_handle h, int R, const double *B, double *X, int
   if (bb == 0.0) {
     // x = 0; the precision state is still made available (marginal precisions)
     if (joint && (s = precision_phase32(h, gamma_diag)) != GABP_OK) return s;
-    if (gamma_diag) w.coef_ready = false;
+    if (gamma_diag) drop_coef32(h);
     if (iters) *iters = 0;
     if (relres) *relres = 0.0;
     return GABP_OK;
   }
-  Args32 a = args32(h);
-  const size_t E = (size_t)(g.E > 0 ? g.E : 1);
+  const size_t E = a.ns ? (size_t)w.sl.Es : (size_t)(g.E > 0 ? g.E : 1);
   const double itol = h->opt.inner_tol;
   for (int step = 0; step < h->opt.max_refine; ++step) {
     if (rr <= tol * tol * bb) { result = GABP_OK; break; }
@@ -1648,8 +2107,8 @@ gabp_status solve32_refine(gabp_handle h, int R, const double *B, double *X, int
       if (ist == GABP_DIVERGED) { result = GABP_DIVERGED; break; }
       prof_begin(h);
       if ((s = serial_update32(h, X)) != GABP_OK) return s;
-      GABP_DISPATCH_L(LR, (k64_residual<LL><<<nbr, kBlock, 0, h->stream>>>(g.n, g.rowptr, g.col, g.val, B, X, w.rhs32,
-                                                                              w.NH[0], w.ctlR, h->partials, 0)));
+      GABP_DISPATCH_L(LR, (k64_residual<LL><<<nbr, kBlock, 0, h->stream>>>(g.n, g.rowptr, g.col, g.val, B, X, rhs32, a.NH0,
+                                                                              w.ctlR, h->partials, 0, pos)));
       prof_end(h);
       h->prof.launches += 2;
       GABP_CUDA(cudaGetLastError());
@@ -1668,7 +2127,7 @@ gabp_status solve32_refine(gabp_handle h, int R, const double *B, double *X, int
       k_ctl_reset<<<1, 1, 0, h->stream>>>(h->ctl, cap, it_tol * it_tol, T);
       h->prof.launches += 1;
       if ((s = freeze32(h, T)) != GABP_OK) return s;
-      if (gamma_diag) w.coef_ready = false;  // do not reuse a loaded state for a plain solve
+      if (gamma_diag) drop_coef32(h);  // do not reuse a loaded state for a plain solve
     } else if (!w.dense_ld) {
       GABP_CUDA(cudaMemsetAsync(w.H[0], 0, sizeof(float) * E, h->stream));
     }
@@ -1681,7 +2140,7 @@ gabp_status solve32_refine(gabp_handle h, int R, const double *B, double *X, int
       GABP_CUDA(cudaGetLastError());
       with_shape(SH, [&](auto Lc, auto Uc) {
         constexpr int LL = decltype(Lc)::value, UU = decltype(Uc)::value;
-        s = run_rounds(h, &h->gH32, &h->gH32_L, w.dense_ld ? -1 : SH, [&] {
+        s = run_rounds(h, &h->gH32, &h->gH32_L, w.dense_ld ? -1 : (a.ns ? -2 : SH), [&] {
           launch_mean<LL, UU>(h, a, h->stream);
         }, cap - T, PH_MEAN32, T > 0 ? T + 1 : 0);
       });
@@ -1697,11 +2156,11 @@ gabp_status solve32_refine(gabp_handle h, int R, const double *B, double *X, int
     }
     total_inner += result_round;
     h->stats.rounds += result_round;
-    float *hT = result_round % 3 == 0 ? w.NH[0] : (result_round % 3 == 1 ? w.NH[1] : w.NH[2]);
+    const float *hT = ring3(a.NH0, a.NH1, a.NH2, result_round);
     prof_begin(h);
-    k64_update<<<(g.n + kBlock - 1) / kBlock, kBlock, 0, h->stream>>>(g.n, X, hT, w.invP);
-    GABP_DISPATCH_L(LR, (k64_residual<LL><<<nbr, kBlock, 0, h->stream>>>(g.n, g.rowptr, g.col, g.val, B, X, w.rhs32,
-                                                                            w.NH[0], w.ctlR, h->partials, 0)));
+    k64_update<<<(g.n + kBlock - 1) / kBlock, kBlock, 0, h->stream>>>(g.n, X, hT, a.invP, pos);
+    GABP_DISPATCH_L(LR, (k64_residual<LL><<<nbr, kBlock, 0, h->stream>>>(g.n, g.rowptr, g.col, g.val, B, X, rhs32, a.NH0,
+                                                                            w.ctlR, h->partials, 0, pos)));
     prof_end(h);
     h->prof.launches += 2;
     GABP_CUDA(cudaGetLastError());
