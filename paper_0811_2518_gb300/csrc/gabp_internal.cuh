@@ -178,6 +178,7 @@ struct Work32 {
   bool coef_ready = false;
   int prec_round = -1;    // round of the frozen precision state
   bool prec_sliced = false;  // it lies in sl.NP
+  bool av32_ok = false;   // g.av32 matches the graph's values
   Sell32 sl;
   bool sl_on = false;     // the current solve's rounds run on sl
   int R = 0;              // RHS capacity of the mean buffers
@@ -620,6 +621,7 @@ gabp_status solve64_serial(gabp_handle h, const double *b, double *x, double tol
                            double *relres);
 gabp_status serial_messages64(gabp_handle h, double2 *M_input_layout);
 gabp_status serial_marginals64(gabp_handle h, double *Pi);
+gabp_status csr_values32(gabp_handle h);  // g.av32 up to date
 void drop_coef32(gabp_handle h);         // the frozen coefficients no longer hold
 gabp_status csr_coef32(gabp_handle h);  // makes them ready in CSR order if they are in the sliced one
 gabp_status serial_freeze32(gabp_handle h, const float2 *CF, const float *invP);

@@ -389,7 +389,7 @@ gabp_status solve_systems(gabp_handle h, int nsys, const int *offsets_host, cons
   for (int s = 0; s < nsys; ++s)
     if (offsets_host[s + 1] <= offsets_host[s]) return GABP_ERR_INVALID;
   gabp_status st = ensure_w32(h, 1);
-  if (st != GABP_OK) return st;
+  if (st != GABP_OK || (st = csr_values32(h)) != GABP_OK) return st;
   Work32 &w = h->w32;
   // per-system sizes from the host copy of the off-diagonal row pointer
   std::vector<int> rp_h(g.n + 1);

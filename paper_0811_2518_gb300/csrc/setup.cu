@@ -99,15 +99,31 @@ __global__ void k_compact(int n, const int *__restrict__ rowptr, const int *__re
   }
 }
 
-// New values on the existing pattern: A_ik == A_ki bit for bit through rev[].
-__global__ void k_values_to_f32(int64_t E, const double *__restrict__ s, float *__restrict__ d) {
-  const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (e < E) d[e] = (float)s[e];
+// New values on the existing pattern: checked and split off the diagonal in one pass.  HBM bounds it (16 bytes an
+// entry); 29 M entries, 25 M of them off the diagonal: k_check_rows and k_compact, which read and write the columns
+// as well, took 301 us.
+__global__ void k_new_values(int n, const int *__restrict__ rowptr, const double *__restrict__ val,
+                             const int *__restrict__ dpos, double *__restrict__ av, double *__restrict__ ad, int *flag) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  const int a = rowptr[i], b = rowptr[i + 1], d = a + dpos[i];
+  int f = 0;
+  for (int p = a; p < b; ++p) {
+    const double v = val[p];
+    if (v == 0.0 || !isfinite(v)) f |= p == d ? BAD_DIAG : BAD_OFFDIAG;
+    if (p == d) ad[i] = v;
+    else av[p - i - (p > d)] = v;
+  }
+  if (f) atomicOr(flag, f);
 }
 
+// A_ik == A_ki bit for bit through rev[], each pair from its first slot (the gather of the other one is a DRAM
+// access of its own; from both slots 25 M slots took 317 us).
 __global__ void k_check_sym(int64_t E, const double *__restrict__ av, const int *__restrict__ rev, int *flag) {
   const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (e < E && __double_as_longlong(av[e]) != __double_as_longlong(av[rev[e]])) atomicOr(flag, (int)BAD_VALUE);
+  if (e >= E) return;
+  const int r = rev[e];
+  if (e < r && __double_as_longlong(av[e]) != __double_as_longlong(av[r])) atomicOr(flag, (int)BAD_VALUE);
 }
 
 // rev[e] for slot e = (row i, column k): binary search of i among row k's columns.
@@ -453,27 +469,19 @@ extern "C" gabp_status gabp_set_values(gabp_handle h, const double *val, int mem
                             mem_space == 0 ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice, h->stream));
   GABP_CUDA(cudaMemsetAsync(dflag, 0, sizeof(int), h->stream));
   const int nb = (g.n + kBlock - 1) / kBlock;
-  k_check_rows<<<nb, kBlock, 0, h->stream>>>(g.n, g.rowptr, g.col, g.val, g.dpos, dflag);
+  k_new_values<<<nb, kBlock, 0, h->stream>>>(g.n, g.rowptr, g.val, g.dpos, g.av, g.ad, dflag);
+  if (g.E > 0)
+    k_check_sym<<<(int)(((int64_t)g.E + kBlock - 1) / kBlock), kBlock, 0, h->stream>>>(g.E, g.av, g.rev, dflag);
+  GABP_CUDA(cudaGetLastError());
   gabp_status s = read_flag();
   if (s != GABP_OK) return s;
   if (hflag) {
     set_last_error(hflag & BAD_DIAG ? "gabp_set_values: a diagonal entry is zero or non-finite"
-                                    : "gabp_set_values: zero or non-finite off-diagonal entry");
+                   : hflag & BAD_OFFDIAG ? "gabp_set_values: zero or non-finite off-diagonal entry"
+                                         : "gabp_set_values: A_ij != A_ji");
     return GABP_ERR_INVALID;
   }
-  k_compact<<<(g.n + 1 + kBlock - 1) / kBlock, kBlock, 0, h->stream>>>(g.n, g.rowptr, g.col, g.val, g.dpos, g.rp,
-                                                                        g.ci, g.av, g.ad);
-  if (g.E > 0)
-    k_check_sym<<<(int)(((int64_t)g.E + kBlock - 1) / kBlock), kBlock, 0, h->stream>>>(g.E, g.av, g.rev, dflag);
-  if ((s = read_flag()) != GABP_OK) return s;
-  if (hflag) {
-    set_last_error("gabp_set_values: A_ij != A_ji");
-    return GABP_ERR_INVALID;
-  }
-  if (g.av32 && g.E > 0) {
-    k_values_to_f32<<<(int)(((int64_t)g.E + kBlock - 1) / kBlock), kBlock, 0, h->stream>>>(g.E, g.av, g.av32);
-    GABP_CUDA(cudaGetLastError());
-  }
+  h->w32.av32_ok = false;  // refreshed by the next call that runs on the row CSR in FP32
   if ((s = serial_refresh_values(h)) != GABP_OK) return s;
   h->values_ok = true;
   return GABP_OK;

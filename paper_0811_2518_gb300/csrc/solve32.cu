@@ -1174,12 +1174,11 @@ gabp_status ensure_w32(gabp_handle h, int R) {
     GABP_CUDA(cudaMalloc(&w.CF, sizeof(float2) * E));
     GABP_CUDA(cudaMalloc(&w.invP, sizeof(float) * n));
     GABP_CUDA(cudaMalloc(&g.av32, sizeof(float) * E));
+    w.av32_ok = false;
     GABP_CUDA(cudaMalloc(&g.ad32, sizeof(float) * n));
     GABP_CUDA(cudaMalloc(&w.ctlR, sizeof(DevCtl)));
     GABP_CUDA(cudaMemsetAsync(w.ctlR, 0, sizeof(DevCtl), h->stream));
     for (int j = 0; j < 3; ++j) GABP_CUDA(cudaMalloc(&w.NQ[j], sizeof(float2) * n));
-    k_to_f32<<<(int)((E + kBlock - 1) / kBlock), kBlock, 0, h->stream>>>((int64_t)g.E, g.av, g.av32);
-    GABP_CUDA(cudaGetLastError());
   }
   if (w.R < R) {
     cudaFree(w.H[0]); cudaFree(w.H[1]);
@@ -1208,6 +1207,16 @@ gabp_status ensure_w32(gabp_handle h, int R) {
     h->gRefG = nullptr;
     h->gRef_key = -1;
   }
+  return GABP_OK;
+}
+
+// The FP32 values of the row CSR (the sliced layout has its own).
+gabp_status csr_values32(gabp_handle h) {
+  Graph &g = h->g;
+  if (h->w32.av32_ok) return GABP_OK;
+  if (g.E > 0) k_to_f32<<<(int)(((int64_t)g.E + kBlock - 1) / kBlock), kBlock, 0, h->stream>>>((int64_t)g.E, g.av, g.av32);
+  GABP_CUDA(cudaGetLastError());
+  h->w32.av32_ok = true;
   return GABP_OK;
 }
 
@@ -1504,6 +1513,8 @@ gabp_status precision_phase32(gabp_handle h, const double *gamma_diag) {
   Work32 &w = h->w32;
   Graph &g = h->g;
   size_t E = (size_t)(g.E > 0 ? g.E : 1);
+  gabp_status st = csr_values32(h);
+  if (st != GABP_OK) return st;
   k_diag32<<<(g.n + kBlock - 1) / kBlock, kBlock, 0, h->stream>>>(g.n, g.ad, gamma_diag, g.ad32);
   // round-0 state: zero precision messages, P~ = diagonal
   auto init = [&]() -> gabp_status {
@@ -1512,7 +1523,7 @@ gabp_status precision_phase32(gabp_handle h, const double *gamma_diag) {
     GABP_CUDA(cudaMemcpyAsync(w.NP[0], g.ad32, sizeof(float) * g.n, cudaMemcpyDeviceToDevice, h->stream));
     return GABP_OK;
   };
-  gabp_status st = init();
+  st = init();
   if (st != GABP_OK) return st;
   if (!h->opt.lanes && !h->tuned_Lp32) {
     if ((st = autotune32(h, K32_PREC)) != GABP_OK) return st;
@@ -1958,7 +1969,7 @@ static gabp_status solve32_device_loop(gabp_handle h, const double *B, double *X
   }
   gabp_status sd = ensure_dense32(h);
   if (sd != GABP_OK) return sd;
-  if ((sd = ensure_sell32(h)) != GABP_OK) return sd;
+  if ((sd = ensure_sell32(h)) != GABP_OK || (!w.sl_on && (sd = csr_values32(h)) != GABP_OK)) return sd;
   const bool joint = !(w.coef_ready || w.sl.coef_ready) || !h->opt.reuse_precisions;
   if (joint) {
     drop_coef32(h);
@@ -2049,6 +2060,7 @@ gabp_status solve32_refine(gabp_handle h, int R, const double *B, double *X, int
   bool joint = false;
   if (serial) { w.dense_ld = 0; w.sl_on = false; }
   else if ((s = ensure_dense32(h)) != GABP_OK || (s = ensure_sell32(h)) != GABP_OK) return s;
+  if (!w.sl_on && (s = csr_values32(h)) != GABP_OK) return s;
   if (!(w.coef_ready || w.sl.coef_ready) || gamma_diag || !h->opt.reuse_precisions) {
     drop_coef32(h);
     w.dense_packed = false;
