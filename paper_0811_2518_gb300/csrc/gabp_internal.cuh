@@ -278,7 +278,8 @@ struct GSell {
   std::vector<int> off;        // the offsets the layout was built for
   int ns = 0;                  // slices
   int Es = 0;                  // slots, padding included
-  std::vector<int> order;      // the systems by descending size (stable)
+  bool by_size = false;
+  std::vector<int> order;      // the systems in the layout's order: as given, or by descending size (stable)
   bool vals_ok = false;
   int *srow = nullptr;         // [32 ns] row of each slice lane, -1 for padding
   int *sp = nullptr;           // [ns + 1] first slot of each slice (multiples of 32)
@@ -645,7 +646,7 @@ gabp_status solve_systems_grid(gabp_handle h, int nsys, const int *d_off, const 
                                double *x, double tol, int max_iter, int *d_status, int *d_iters, int *d_refine,
                                double *d_relres, int shape, float *ms_out, int upto = -1);
 void free_gsell(gabp_handle h);
-gabp_status ensure_gsell(gabp_handle h, int nsys, const int *off);
+gabp_status ensure_gsell(gabp_handle h, int nsys, const int *off, bool by_size);
 // multichip.cu
 void free_team(TeamSell &t);
 int team_rows(gabp_handle h);

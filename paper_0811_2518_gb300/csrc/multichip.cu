@@ -492,7 +492,7 @@ int team_rows(gabp_handle h) {
 gabp_status solve_systems_team(gabp_handle h, int nsys, const int *off, int from, const double *b, double *x, double tol,
                                int max_iter, int *d_status, int *d_iters, int *d_refine, double *d_relres,
                                float *ms_out) {
-  gabp_status st = ensure_gsell(h, nsys, off);
+  gabp_status st = ensure_gsell(h, nsys, off, true);
   if (st != GABP_OK) return st;
   Graph &g = h->g;
   GSell *L = h->gsl;
