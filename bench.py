@@ -394,12 +394,13 @@ def main():
     impl_bytes = (20 * E + 24 * n) if ph == "mean32" else (28 * E + 36 * n)
     dur_ms = prof["ms"][ph] / max(prof["rounds"][ph], 1)
     achieved = bytes_launch / (dur_ms / 1e3) / 1e9
-    kname = "k32_mean" if ph == "mean32" else "k32_joint"
-    _ts = s32.tuned()
-    tuned = {"k32_mean": _ts["mean32"], "k32_joint": _ts["prec32"]}  # (lanes per row, slots per lane)
+    # without a pinned or tuned shape the rounds run on the sliced layout: a lane a row, 4 slots in flight
+    shape = s32.tuned()["mean32" if ph == "mean32" else "prec32"]
     if args.lanes:  # pinned: the library's mapping of (lanes, unroll)
         _L = min(args.lanes, 16)
-        tuned = {k: (_L, args.unroll or (1 if _L >= 16 else 4)) for k in tuned}
+        shape = (_L, args.unroll or (1 if _L >= 16 else 4))
+    kname = ("k32" if shape[0] else "ks32") + ("_mean" if ph == "mean32" else "_joint")
+    shape = shape if shape[0] else (1, 4)
 
     legs = set(args.legs.split(","))
 
@@ -534,16 +535,16 @@ def main():
                 cpu_b = oracle_rounds_sample(mg, synth.rhs_batch(mg.n, 1, 3)[0])
             msb, pb, stats_b, stb, itb, maxrel, ncol = res[1]
             mean_ms = pb["ms"]["mean32"] / max(pb["rounds"]["mean32"], 1)  # one sweep (all colour passes)
-            # per sweep: every slot once (R messages read + written, coefficient pair, sender) and every row once
-            # (R firing aggregates read + written, R right-hand sides, segment bounds / colour / row pointer)
-            bytes_b = Eg * (8 * Rb + 12) + ng * (12 * Rb + 20)
+            # per sweep of two colours: every slot once (R messages read, those of one direction written, coefficient
+            # pair, sender) and every row once (R firing aggregates read + written, R right-hand sides, row data)
+            bytes_b = Eg * (6 * Rb + 12) + ng * (12 * Rb + 20)
             # the method's own bytes per sweep: per edge R mean messages read and written (8 R) and the frozen
             # coefficient with the reverse index (8), per node the R aggregates (8 R)
             alg_b = Eg * (8 * Rb + 8) + 8 * Rb * ng
             # DRAM bytes from a capture of the 64^3 case (a few GB on the device; the 128^3 x 64 workload is
             # too large to capture under ncu), scaled to this sweep by the implementation's bytes
             traffic_b = _profiled_traffic("kbs_pass_grid3d_64_64rhs.md", "paper_0811_2518_gb300/csrc/batched.cu",
-                                          "kbs_pass", scale_to=bytes_b)
+                                          "kbs2_pass", scale_to=bytes_b)
             traffic_note_b = ("DRAM bytes per sweep, scaled from one captured pass of the 64^3 case (the two "
                               "red-black passes move equal bytes) by the implementation's bytes")
             batched = {"workload": f"{args.batched_grid}^3 7-point grid, face coefficients LogNormal(0,1), diagonal 1.05 x "
@@ -556,7 +557,7 @@ def main():
                                              "max_relres": res[0][5]},
                        "fp64_plain_one_rhs": fp64_one, "cpu_oracle_one_rhs": cpu_b,
                        "batched_vs_64_fp64": {k: v["ms_x64"] / msb for k, v in fp64_one.items()},
-                       "roofline": {"bound": "hbm", "kernel": "kbs_pass (one sweep = all colour passes)",
+                       "roofline": {"bound": "hbm", "kernel": "kbs2_pass (one sweep = both colour passes)",
                                     "achieved": alg_b / (mean_ms / 1e3) / 1e9, "peak": peak, "unit": "GB/s",
                                     "frac": alg_b / (mean_ms / 1e3) / 1e9 / peak,
                                     "algorithmic_bytes_per_sweep": alg_b,
@@ -843,14 +844,15 @@ def main():
                     sdn.solve(bdt, tol=TOL, max_iter=2000, x=xd_)
                     pd = sdn.profile(reset=True)
                     mean_ms = pd["ms"]["mean32"] / max(pd["rounds"]["mean32"], 1)
-                    alg = 16 * Edn + 8 * nd
-                    entry["roofline"] = {"bound": "hbm", "kernel": "k32_mean", "launch_ms": mean_ms,
+                    # write rounds (16 B an edge: both coefficients, message read and written) and product
+                    # rounds (4 B: one coefficient) in turn
+                    alg = 10 * Edn + 8 * nd
+                    entry["roofline"] = {"bound": "hbm", "kernel": "k32_dense", "launch_ms": mean_ms,
                                          "algorithmic_bytes_per_launch": alg,
-                                         "algorithmic_bytes_rule": "16 B per directed edge + 8 B per node",
+                                         "algorithmic_bytes_rule": "16 and 4 B per directed edge in turn + 8 B per node",
                                          "achieved": alg / (mean_ms / 1e3) / 1e9, "peak": peak, "unit": "GB/s",
                                          "frac": alg / (mean_ms / 1e3) / 1e9 / peak,
-                                         # a complete pattern's mean round reads no column indices
-                                         "impl_frac": (16 * Edn + 24 * nd) / (mean_ms / 1e3) / 1e9 / peak}
+                                         "impl_frac": (10 * Edn + 24 * nd) / (mean_ms / 1e3) / 1e9 / peak}
                     x32 = xh
                 else:
                     entry["max_abs_diff_fp32_refine_vs_fp64"] = float(np.max(np.abs(xh - x32)))
@@ -940,7 +942,7 @@ def main():
                          "impl_bytes_per_launch": impl_bytes, "impl_frac": impl_bytes / (dur_ms / 1e3) / 1e9 / peak,
                          "traffic_over_algorithmic": None if traffic_main is None else traffic_main / bytes_launch,
                          "launch_ms": dur_ms,
-                         "shape": {"lanes_per_row": tuned[kname][0], "slots_per_lane": tuned[kname][1]},
+                         "shape": {"lanes_per_row": shape[0], "slots_per_lane": shape[1]},
                          "random_gather_reference": gather},
             "phases_ms_per_step": {k: v / args.steps for k, v in prof["ms"].items()},
             "rounds_per_step_by_phase": {k: v / args.steps for k, v in prof["rounds"].items()},
@@ -952,12 +954,12 @@ def main():
                 "ms_per_solve": ms64, "rounds": r64 / k64, "edge_updates_per_s": E * (r64 / k64) / (ms64 / 1e3),
                 "phase_ms": p64["ms"]["fp64"] / k64,
                 "roofline": {"bound": "fp64 alu", "kernel": "k64_node",
-                             # FP64 instructions of a round, counted by ncu's per-opcode counters: per message
-                             # 4 DADD + 4 DFMA + 3 DMUL, per row 3 + 5 + 1; GB300 retires 2 FP64 operations per
+                             # FP64 instructions of a round of the recompute form: 7 a message (the division
+                             # runs on the integer units), 9 a row; GB300 retires 2 FP64 operations per
                              # SM and clock (1.25 TFLOP/s FMA at 2.07 GHz on 152 SMs)
-                             "fp64_ops_per_round": 11 * E + 9 * n,
+                             "fp64_ops_per_round": 7 * E + 9 * n,
                              "fp64_peak_ops_per_s": 2.0 * n_sms * clk_mhz * 1e6,
-                             "alu_frac": (11 * E + 9 * n) / (p64["ms"]["fp64"] / max(p64["rounds"]["fp64"], 1) / 1e3)
+                             "alu_frac": (7 * E + 9 * n) / (p64["ms"]["fp64"] / max(p64["rounds"]["fp64"], 1) / 1e3)
                                          / (2.0 * n_sms * clk_mhz * 1e6),
                              "algorithmic_bytes_per_round": 48 * E + 24 * n,
                              "algorithmic_bytes_rule": "48 B per directed edge (A 8, sender 4, reverse index 4, "

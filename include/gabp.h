@@ -103,8 +103,9 @@ typedef struct {
                            the mean messages only (the precisions do not depend on b), else the
                            screen resumes.  Every round up to the stored one is bitwise the plain
                            solve's; after it x differs from the plain iterate by rounding only.
-                           Pays on solves that need many more rounds than the precisions do
-                           (FP64-bound rounds); the screen costs a few percent per round.  0 =
+                           The plain rounds are no longer bound by the precisions' arithmetic: on the 128^3
+                           grid a frozen solve takes 34.7 ms (parallel) and 23.0 (serial), a plain one
+                           30.8 and 18.7.  0 =
                            every round updates both (Algorithm 2 as printed).  The edge variant
                            and the accelerated solves ignore it (the FP32 path always freezes).
                            Default 0 */

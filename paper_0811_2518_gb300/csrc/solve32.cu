@@ -22,6 +22,9 @@
 // values h~_k^{(t-1)} are gathered (they stay in L2).  In exact arithmetic this
 // is the synchronous schedule of Algorithm 2; in FP32 it rounds the same way as
 // computing h_{i->k}^{(t-1)} once and storing it.
+//
+// Large graphs of short rows run these rounds on a sliced layout (ks32_*, ensure_sell32), dense matrices on
+// arrays of their own (k32_dense), the rest and pinned shapes with L lanes a row (k32_*).
 #include "gabp_internal.cuh"
 #include "devutil.cuh"
 #include "sell64.cuh"
