@@ -271,8 +271,8 @@ struct TeamSell {
 // degree (descending, stable) in windows of 4096 and cut into 32-row slices, the last
 // slice of a system padded with rows -1, so that a slice belongs to one system; slot j
 // of the slice's rows is the contiguous line sp[s] + 32 j + lane (sender -1 past a
-// row's degree).  The systems lie by descending size.  Built for one offsets array; the
-// values are refreshed after gabp_set_values.
+// row's degree).  The systems lie as given, or by descending size where the queue kernel takes some of
+// them.  Built for one offsets array; the values are refreshed after gabp_set_values.
 struct GSell {
   TeamSell team;
   std::vector<int> off;        // the offsets the layout was built for
@@ -288,6 +288,7 @@ struct GSell {
   float *sav = nullptr;        // [Es] A_ij (FP32), 0 for padding
   float *MP[2] = {nullptr, nullptr}, *H[2] = {nullptr, nullptr};  // [Es] precision / mean chains
   float2 *CF = nullptr;        // [Es] frozen coefficients
+  float *node = nullptr;       // [4][n] P~ ring of three rounds, 1 / P~ (the handle's own belong to its kept precisions)
 };
 
 // Single-loop convergence fix (fixloop.cu)

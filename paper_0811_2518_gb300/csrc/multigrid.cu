@@ -682,7 +682,7 @@ void free_gsell(gabp_handle h) {
   GSell *L = h->gsl;
   if (!L) return;
   cudaFree(L->srow); cudaFree(L->sp); cudaFree(L->ssys); cudaFree(L->sci); cudaFree(L->sav);
-  cudaFree(L->MP[0]); cudaFree(L->MP[1]); cudaFree(L->H[0]); cudaFree(L->H[1]); cudaFree(L->CF);
+  cudaFree(L->MP[0]); cudaFree(L->MP[1]); cudaFree(L->H[0]); cudaFree(L->H[1]); cudaFree(L->CF); cudaFree(L->node);
   free_team(L->team);
   delete L;
   h->gsl = nullptr;
@@ -743,6 +743,7 @@ gabp_status ensure_gsell(gabp_handle h, int nsys, const int *off, bool by_size) 
       GABP_CUDA(cudaMalloc(&L->H[c], sizeof(float) * Ea));
     }
     GABP_CUDA(cudaMalloc(&L->CF, sizeof(float2) * Ea));
+    GABP_CUDA(cudaMalloc(&L->node, sizeof(float) * 4 * (size_t)g.n));
     GABP_CUDA(cudaMemcpyAsync(L->srow, srow.data(), sizeof(int) * srow.size(), cudaMemcpyHostToDevice, h->stream));
     GABP_CUDA(cudaMemcpyAsync(L->sp, sp.data(), sizeof(int) * sp.size(), cudaMemcpyHostToDevice, h->stream));
     GABP_CUDA(cudaMemcpyAsync(L->ssys, ssys.data(), sizeof(int) * ssys.size(), cudaMemcpyHostToDevice, h->stream));
@@ -801,7 +802,7 @@ gabp_status solve_systems_grid(gabp_handle h, int nsys, const int *d_off, const 
   }
   kg_init<<<nsys, kBlock, 0, h->stream>>>(nsys, st, acc, d_off, sys_of, rows_min);
   kg_rows_init<<<blocks_for(g.n, kBlock, h->max_blocks), kBlock, 0, h->stream>>>(
-      g.n, g.rp, g.ad, g.ad32, w.NP[0], sliced ? nullptr : w.MP[0], sliced ? nullptr : w.MP[1], x);
+      g.n, g.rp, g.ad, g.ad32, sliced ? h->gsl->node : w.NP[0], sliced ? nullptr : w.MP[0], sliced ? nullptr : w.MP[1], x);
   GABP_CUDA(cudaGetLastError());
   GridArgs a;
   a.n = g.n; a.nsys = nsys; a.sys_of = sys_of;
@@ -812,8 +813,9 @@ gabp_status solve_systems_grid(gabp_handle h, int nsys, const int *d_off, const 
   a.H0 = w.H[0]; a.H1 = w.H[1]; a.NH0 = w.NH[0]; a.NH1 = w.NH[1]; a.NH2 = w.NH[2];
   a.rhs = w.rhs32; a.b = b; a.x = x;
   a.ns = 0; a.srow = a.sp = a.ssys = nullptr;
-  if (sliced) {  // the slot arrays of the sliced layout
+  if (sliced) {  // the slot arrays of the sliced layout, its precisions
     GSell *L = h->gsl;
+    a.NP0 = L->node; a.NP1 = L->node + g.n; a.NP2 = L->node + 2 * (size_t)g.n; a.invP = L->node + 3 * (size_t)g.n;
     a.ns = ns_run; a.srow = L->srow; a.sp = L->sp; a.ssys = L->ssys;
     a.ci = L->sci; a.av = L->sav;
     a.MP0 = L->MP[0]; a.MP1 = L->MP[1]; a.H0 = L->H[0]; a.H1 = L->H[1]; a.CF = L->CF;

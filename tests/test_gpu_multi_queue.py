@@ -129,3 +129,23 @@ def test_large_systems_beside_small_ones(gb):
         sl = slice(off[k], off[k + 1])
         ref = oracle.gabp_broadcast(mats[k], b[sl], max_iter=5000, tol=1e-13)
         assert np.linalg.norm(x[sl] - ref["x"]) <= 1e-9 * np.linalg.norm(ref["x"])
+
+
+@pytest.mark.parametrize("stop", [10, 11, 12, 14, 16])
+def test_kept_precisions_survive_a_batch_on_both_kernels(gb, stop):
+    """The precisions a handle keeps between solves are the same before and after a call whose small systems
+    go to the queue and whose large ones to the grid kernel (the stops end them at rounds of every
+    remainder modulo three, the length of their ring)."""
+    mats = synth.rgg_batch(400, 1024, 1100, 2.0, 4) + synth.rgg_batch(2, 20000, 30000, 2.0, 5)
+    big = synth.block_diag(mats)
+    off = big.meta["offsets"]
+    b = torch.from_numpy(synth.rhs(big.n, 6)).cuda()
+    s = gb.Solver.from_csr(big, prec_stop_log2=stop)
+    B = b.reshape(1, -1)
+    s.solve_batched(B, tol=1e-6)
+    before = s.marginal_precisions()
+    assert s.solve_systems(b, off, tol=1e-10)[1] == gb.GABP_OK
+    assert s.tuned()["multi_mode"] == 2 and s.tuned()["multi_grid"] == (0, 0)  # both kernels ran
+    s.solve_batched(B, tol=1e-6)
+    assert torch.equal(s.marginal_precisions(), before)
+    s.close()
