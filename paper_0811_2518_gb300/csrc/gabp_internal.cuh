@@ -375,7 +375,8 @@ struct gabp_handle_s {
   long long multi_big = 0;          // autotuned cluster / single-CTA size split of the multi-system kernel
   int multi_nt = 0;                 // autotuned block size of the multi-system kernel
   bool values_ok = true;            // false after a rejected gabp_set_values
-  int multi_mode = 0;               // 0 untuned, 1 grid-persistent kernel, 2 cluster / single-block teams
+  bool multi_queue = false;         // the last call on independent systems ran the queue kernel
+  int multi_mode = 0;               // timed choice: 0 untuned, 1 grid-persistent kernel, 2 cluster / single-block teams
   int multi_grid_shape = 0;         // autotuned shape of the grid-persistent kernel (0 untuned)
   gabp::GSell *gsl = nullptr;       // sliced layout of the grid-persistent kernel (built on first use)
   // least squares (gabp_create_lsq): the handle's matrix is [[I_k, J^T], [J, -gamma I_m]]

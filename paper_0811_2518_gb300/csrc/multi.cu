@@ -522,6 +522,7 @@ gabp_status solve_systems(gabp_handle h, int nsys, const int *offsets_host, cons
   // all its systems (HBM): 1 system of 16384 rows 39.7, 152 of 1024 / 4096 / 16384 5.2 / 12.7 / 49.9.  Grid
   // kernel: 11 + 4.6e-5 a row: 1 of 16384 10.8, 8 of 16384 17.2, 60 of 8192 32.5 (queue 22.7), 152 of
   // 16384 113.
+  h->multi_queue = false;
   if (h->opt.multi_split == 0 && h->opt.multi_mode == 0 && h->opt.lanes == 0) {
     std::vector<int> desc(rows);
     std::sort(desc.begin(), desc.end(), std::greater<int>());
@@ -548,7 +549,7 @@ gabp_status solve_systems(gabp_handle h, int nsys, const int *offsets_host, cons
       st = solve_systems_team(h, nsys, offsets_host, from, b, x, tol, max_iter, d_res, d_res + nsys, d_res + 2 * nsys,
                               d_rel, &ms2);
       if (st != GABP_OK) return st;
-      h->multi_mode = 2;
+      h->multi_queue = true;
       return finish(ms + ms2);
     }
   }

@@ -149,3 +149,22 @@ def test_kept_precisions_survive_a_batch_on_both_kernels(gb, stop):
     s.solve_batched(B, tol=1e-6)
     assert torch.equal(s.marginal_precisions(), before)
     s.close()
+
+
+@pytest.mark.parametrize("opts", [{}, {"lanes": 4}])
+def test_the_queue_is_not_taken_for_a_timed_choice(gb, opts):
+    """After a call on the queue, offsets that make one large system of all of them (or a pinned shape) run
+    the grid kernel, which one team of blocks cannot match there (one cluster against every SM)."""
+    mats = synth.rgg_batch(300, 1024, 1100, 2.0, 4)
+    big = synth.block_diag(mats)
+    b = torch.from_numpy(synth.rhs(big.n, 6)).cuda()
+    s = gb.Solver.from_csr(big)
+    x = s.solve_systems(b, big.meta["offsets"], tol=1e-11)[0]
+    assert s.tuned()["multi_mode"] == 2 and s.tuned()["multi_grid"] == (0, 0)  # the queue
+    s.set_options(**opts)
+    one, st, _, _, rel = s.solve_systems(b, np.array([0, big.n], dtype=np.int32), tol=1e-11)
+    assert st == gb.GABP_OK and rel[0] <= 1e-11
+    assert torch.allclose(one, x, rtol=0, atol=1e-8 * float(x.abs().max()))
+    t = s.tuned()
+    assert t["multi_mode"] == 1 and (t["multi_grid"] != (0, 0)) == (not opts)  # timed; a pinned shape is not tuned
+    s.close()
