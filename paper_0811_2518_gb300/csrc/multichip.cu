@@ -101,9 +101,8 @@ __device__ __noinline__ void mbar_wait_slow(unsigned long long *bar, unsigned pa
 // This thread's writes to global memory come before later bulk copies (another proxy) by the CTA.
 __device__ __forceinline__ void fence_bulk() { asm volatile("fence.proxy.async;" ::: "memory"); }
 
-// What a round's sums decide, the same bits in every thread.
-struct TeamSums {
-  float a, b;
+// What a precision round's flags decide, the same bits in every thread.
+struct TeamFlags {
   unsigned m, f;
 };
 
@@ -111,27 +110,41 @@ struct TeamShared {
   float2 part[2][kTWarps];
   uint2 flag[2][kTWarps];
   double rr[kTWarps];
+  double tot[2];
   int job;
   unsigned long long bar[kTWarps][kStagesMax];  // one phase per chunk
   TeamArgs args;  // the launch's arguments, read from here in the solves
 };
 
-// Posts this thread's sums and flags, passes the CTA's barrier, and adds what all warps posted.
-__device__ __forceinline__ TeamSums team_sums(TeamShared &sh, int parity, float va, float vb, unsigned m, unsigned f) {
+// Posts this thread's flags, passes the CTA's barrier, and joins what all warps posted.
+__device__ __forceinline__ TeamFlags team_flags(TeamShared &sh, int parity, unsigned m, unsigned f) {
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  m = __reduce_max_sync(0xffffffffu, m);
+  f = __reduce_or_sync(0xffffffffu, f);
+  if (lane == 0) sh.flag[parity][w] = make_uint2(m, f);
+  __syncthreads();
+  const uint2 g = lane < kTWarps ? sh.flag[parity][lane] : make_uint2(0u, 0u);
+  return TeamFlags{__reduce_max_sync(0xffffffffu, g.x), __reduce_or_sync(0xffffffffu, g.y)};
+}
+
+// The CTA's sums of two values, within a warp in FP32, over the warps in FP64 (a sum over a whole system
+// overflows FP32 long before its entries do).  One warp adds them, 16 lanes a value: in every warp the
+// FP64 unit would need four times as long as this and the second barrier.
+__device__ __forceinline__ double2 team_sums(TeamShared &sh, int parity, float va, float vb) {
+  static_assert(kTWarps == 16, "16 lanes a value");
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   va = warp_sum(va);
   vb = warp_sum(vb);
-  m = __reduce_max_sync(0xffffffffu, m);
-  f = __reduce_or_sync(0xffffffffu, f);
-  if (lane == 0) {
-    sh.part[parity][w] = make_float2(va, vb);
-    sh.flag[parity][w] = make_uint2(m, f);
+  if (lane == 0) sh.part[parity][w] = make_float2(va, vb);
+  __syncthreads();
+  if (w == 0) {
+    double s = (double)(lane < 16 ? sh.part[parity][lane].x : sh.part[parity][lane - 16].y);
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if ((lane & 15) == 0) sh.tot[lane >> 4] = s;
   }
   __syncthreads();
-  const float2 p = lane < kTWarps ? sh.part[parity][lane] : make_float2(0.f, 0.f);
-  const uint2 g = lane < kTWarps ? sh.flag[parity][lane] : make_uint2(0u, 0u);
-  return TeamSums{warp_sum(p.x), warp_sum(p.y), __reduce_max_sync(0xffffffffu, g.x),
-                  __reduce_or_sync(0xffffffffu, g.y)};
+  return make_double2(sh.tot[0], sh.tot[1]);
 }
 
 __device__ __forceinline__ double team_sum64(TeamShared &sh, double v) {
@@ -228,7 +241,7 @@ __device__ __noinline__ unsigned team_solve(TeamShared &sh, unsigned char *smem,
       hn[p] = P;
     }
     parity ^= 1;
-    return team_sums(sh, parity, 0.f, 0.f, rel & 0x7fffffffu, bad);
+    return team_flags(sh, parity, rel & 0x7fffffffu, bad);
   };
 
   // The fetch cursor over this warp's chunks: slice and chunk of it (an empty slice has one, of no lines),
@@ -326,14 +339,14 @@ __device__ __noinline__ unsigned team_solve(TeamShared &sh, unsigned char *smem,
     }
     fence_bulk();  // the messages written here are fetched for round t + 2, from the next round on
     parity ^= 1;
-    return team_sums(sh, parity, dxx, xx, 0u, 0u);
+    return team_sums(sh, parity, dxx, xx);
   };
 
   bool run = true;
   {
     int stable = 0;
     for (int t = 1;; ++t) {
-      const TeamSums r = t <= 2 ? prec_round(t, std::true_type()) : prec_round(t, std::false_type());
+      const TeamFlags r = t <= 2 ? prec_round(t, std::true_type()) : prec_round(t, std::false_type());
       const float rel = __uint_as_float(r.m);
       stable = (double)rel <= a.prec_thr ? stable + 1 : 0;  // a NaN is not stationary
       Tp = t;
@@ -389,15 +402,15 @@ __device__ __noinline__ unsigned team_solve(TeamShared &sh, unsigned char *smem,
     if (!isfinite(rr)) { status = GABP_DIVERGED; break; }
     if (steps >= a.max_refine || inner >= a.max_iter) { status = GABP_NOT_CONVERGED; break; }
     const double itol = fmin(a.inner_tol, fmax(1e-6, 0.1 * a.tol * sqrt(bb / rr)));
-    const float it2 = (float)(itol * itol);
+    const double it2 = itol * itol;
     const int cap = min(a.inner_max, max(1, a.max_iter - inner));
     int t = 1;
     bool ok = true;
     pm = w; pc = 0; ft = 1;
     for (;; ++t) {
-      const TeamSums r = t <= 2 ? mean_round(t, std::true_type()) : mean_round(t, std::false_type());
-      if (!isfinite(r.a) || !isfinite(r.b)) { ok = false; break; }
-      if ((t >= 2 && r.a <= it2 * r.b) || t >= cap) break;
+      const double2 r = t <= 2 ? mean_round(t, std::true_type()) : mean_round(t, std::false_type());
+      if (!isfinite(r.x) || !isfinite(r.y)) { ok = false; break; }
+      if ((t >= 2 && r.x <= it2 * r.y) || t >= cap) break;
     }
     while (out > 0) {  // chunks fetched for a round that does not come
       arrive();

@@ -168,3 +168,28 @@ def test_the_queue_is_not_taken_for_a_timed_choice(gb, opts):
     t = s.tuned()
     assert t["multi_mode"] == 1 and (t["multi_grid"] != (0, 0)) == (not opts)  # timed; a pinned shape is not tuned
     s.close()
+
+
+def test_iterates_beyond_the_square_root_of_fp32(gb):
+    """Solutions whose sum of squares is half again FP32's largest value, though no entry's square and no warp's
+    sum (a sixteenth of the rows) comes near it, converge as on the grid kernel."""
+    mats = synth.rgg_batch(300, 1024, 1100, 2.0, 8)
+    big = synth.block_diag(mats)
+    off = big.meta["offsets"]
+    b = synth.rhs(big.n, 9)
+    for k, m in enumerate(mats):
+        sl = slice(off[k], off[k + 1])
+        if k < 3:  # three systems of this kind, the others as drawn
+            x = np.linalg.solve(synth.to_dense(m), b[sl])
+            b[sl] *= np.sqrt(5e38) / np.linalg.norm(x)
+    got = []
+    for mode in (0, 3):
+        s = gb.Solver.from_csr(big, multi_mode=mode)
+        x, st, sts, its, rel = _solve(gb, s, mats, b, off, tol=1e-11, check=False)
+        assert s.tuned()["multi_mode"] == (0 if mode else 2)  # 2: the queue
+        s.close()
+        assert st == gb.GABP_OK and np.all(sts == gb.GABP_OK) and np.all(rel <= 1e-11)
+        got.append(x)
+    for k in range(5):
+        sl = slice(off[k], off[k + 1])
+        assert np.linalg.norm(got[0][sl] - got[1][sl]) <= 1e-9 * np.linalg.norm(got[1][sl])
