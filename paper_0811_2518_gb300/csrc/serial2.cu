@@ -80,7 +80,7 @@ __device__ __forceinline__ void s2_slice(const ArgsS2 &a, int sl, int lane, cons
       const int pos = p0 + 32 * (j + u);
       if (MODE == 3) {
         const double v = fma(rv[u].x, rv[u].y, nk[u].h);
-        __stcs(reinterpret_cast<double *>(Mout + pos) + 1, v);
+        __stcs(Mout + pos, make_double2(c[u], v));  // with c, as in solve64.cu
         acch = fma(-c[u], v, acch);
       } else {
         const double2 m = message64(A[u], nk[u], rv[u], bad);

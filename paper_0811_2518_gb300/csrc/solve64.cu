@@ -236,8 +236,8 @@ __device__ __forceinline__ void plain_slice(const Args64 &a, int sl, int lane, c
       const int pos = p0 + 32 * (j + u);
       if (MODE == 3) {
         const double v = fma(rv[u].x, rv[u].y, nk[u].h);
-        double *dst = reinterpret_cast<double *>(Mout + pos) + 1;
-        if (COOP) *dst = v; else __stcs(dst, v);
+        const double2 m = make_double2(c[u], v);  // with c: both stores hold the frozen one, which the cavities take
+        if (COOP) Mout[pos] = m; else __stcs(Mout + pos, m);
         acch = fma(-c[u], v, acch);
       } else {
         if (REC) rv[u] = reverse64(A[u], P2, h2, rv[u]);

@@ -244,3 +244,26 @@ def test_serial_freeze(gb, name, make, tol):
         else:
             r = oracle.gabp_serial(m, b, max_iter=t, tol=0.0)
             assert np.allclose(g["x"], r["x"], rtol=1e-12, atol=1e-14 * np.max(np.abs(r["x"]))), t
+
+
+@pytest.mark.parametrize("make,opts", [(lambda: synth.grid2d(32, -1.0, 4.5), {}),
+                                       (lambda: synth.random_sym(20011, 8, 1.1, 2), {}),
+                                       (lambda: synth.random_sym(1 << 18, 8, 1.1, 2), {}),
+                                       (lambda: synth.grid3d(64, 1.1, 2), {}),
+                                       (lambda: synth.grid3d(33, 1.1, 3), {"schedule": 1})],
+                         ids=["cluster", "coop", "recompute", "gather", "serial_two_colours"])
+def test_frozen_rounds_keep_the_stored_precisions(gb, make, opts):
+    """The precision messages after the freeze are those of its round, bit for bit, whichever of the two message
+    stores the last round wrote."""
+    m = make()
+    b = torch.from_numpy(synth.rhs(m.n, 2)).cuda()
+    s = gb.Solver.from_csr(m, freeze_precisions=1, **opts)
+    s.solve(b, tol=0.0, max_iter=300)
+    F = s.stats()["freeze_round"]
+    assert 0 < F < 250
+    s.solve(b, tol=0.0, max_iter=F)
+    P = s.messages()[0]
+    for t in (F + 1, F + 2, F + 3, F + 8):
+        s.solve(b, tol=0.0, max_iter=t)
+        assert torch.equal(s.messages()[0], P), t - F
+    s.close()
