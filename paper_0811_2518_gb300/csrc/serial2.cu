@@ -230,11 +230,20 @@ __global__ void ks2_messages(int n, const int *__restrict__ rp, const int *__res
   }
 }
 
+// The layout, its values and the state; GABP_NOT_RUN, now and from then on, where there is no room for them
+// (the general passes need one message store and no padding).
 gabp_status ensure_two(gabp_handle h) {
   WorkS &s = h->ws;
   WorkS2 &w = s.two;
   const Graph &g = h->g;
   const size_t n = (size_t)g.n;
+  if (w.refused) return GABP_NOT_RUN;
+  auto refuse = [&] {
+    cudaGetLastError();
+    free_serial2(s);
+    w.refused = true;
+    return GABP_NOT_RUN;
+  };
   if (!w.sl.ready) {
     std::vector<int> rp(n + 1), rows(n);
     GABP_CUDA(cudaMemcpyAsync(rp.data(), g.rp, sizeof(int) * rp.size(), cudaMemcpyDeviceToHost, h->stream));
@@ -247,22 +256,20 @@ gabp_status ensure_two(gabp_handle h) {
     std::vector<int> srow(p0 + p1, -1);
     std::copy(rows.begin(), rows.begin() + n0, srow.begin());
     std::copy(rows.begin() + n0, rows.end(), srow.begin() + p0);
-    free_sell64(w.sl);  // of a failed attempt
     w.ns0 = (int)(p0 / 32);
-    const gabp_status bs = build_sell64(h, w.sl, rp, srow, nullptr);
-    if (bs != GABP_OK) return bs;
+    if (build_sell64(h, w.sl, rp, srow, nullptr) != GABP_OK) return refuse();
   } else if (!w.sl.vals_ok) {
     const gabp_status vs = sell64_values(h, w.sl);
     if (vs != GABP_OK) return vs;
   }
   const size_t Es = (size_t)std::max(w.sl.Es, 1);
-  for (int q = 0; q < 2; ++q)
-    if (!w.M[q]) GABP_CUDA(cudaMalloc(&w.M[q], sizeof(double2) * Es));
-  for (int q = 0; q < 3; ++q)
-    if (!w.N[q]) GABP_CUDA(cudaMalloc(&w.N[q], sizeof(NodeRec64) * n));
-  if (!w.b) GABP_CUDA(cudaMalloc(&w.b, sizeof(double) * n));
-  if (h->opt.freeze_precisions && !w.C) GABP_CUDA(cudaMalloc(&w.C, sizeof(double) * Es));
-  return GABP_OK;
+  bool room = true;
+  auto get = [&](auto *&p, size_t m) { room = room && (p || cudaMalloc(&p, sizeof(*p) * m) == cudaSuccess); };
+  for (int q = 0; q < 2; ++q) get(w.M[q], Es);
+  for (int q = 0; q < 3; ++q) get(w.N[q], n);
+  get(w.b, n);
+  if (h->opt.freeze_precisions) get(w.C, Es);
+  return room ? GABP_OK : refuse();
 }
 
 ArgsS2 args_two(gabp_handle h) {

@@ -140,3 +140,26 @@ def test_breakdown(gb):
     assert st == r["status"]
     if r["status"] == oracle.BREAKDOWN:
         assert it == r["iters"]
+
+
+def test_no_room_for_the_two_colour_layout(gb):
+    """Where the device has room for the general passes only (about 130 MB here, the two-colour layout and state
+    360 MB), they run, with the same sweeps."""
+    m = synth.grid3d(96, 1.05, 3)
+    b = torch.from_numpy(synth.rhs(m.n, 7)).cuda()
+    s = gb.Solver.from_csr(m, schedule=1)
+    ref, st, sweeps, _ = s.solve(b, tol=1e-10, max_iter=500)
+    assert st == gb.GABP_OK
+    s.close()
+    s = gb.Solver.from_csr(m, schedule=1)
+    s.serial_colours()
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    keep = torch.empty(torch.cuda.mem_get_info()[0] - (250 << 20), dtype=torch.uint8, device="cuda")
+    out = torch.empty_like(b)
+    x, st, it, _ = s.solve(b, tol=1e-10, max_iter=500, x=out)
+    del keep
+    torch.cuda.empty_cache()
+    assert st == gb.GABP_OK and it == sweeps
+    assert torch.allclose(x, ref, rtol=0, atol=1e-10 * float(ref.abs().max()))
+    s.close()
