@@ -440,7 +440,9 @@ gabp_status gabp_solve_noalloc(int32_t n, int64_t nnz, const int32_t *rowptr, co
  * ignored).  The next gabp_solve with options.warm_start = 1 (FP64 parallel
  * rounds) starts from them; any finite messages are a valid start, a poor one
  * costs rounds (or, outside the convergent cases, convergence).  The handle
- * keeps its own copy.  GABP_ERR_INVALID for null pointers or host arrays. */
+ * keeps its own copy, as factors of the messages: they are products on export and
+ * quotients on loading, so a resumed run agrees with the run it resumes to
+ * rounding, not bit for bit.  GABP_ERR_INVALID for null pointers or host arrays. */
 gabp_status gabp_set_messages(gabp_handle h, const double *P, const double *hm);
 
 /* Residual history of the last solve (options.history > 0, plain FP64 parallel

@@ -1642,9 +1642,9 @@ gabp_status messages64(gabp_handle h, double *P, double *hm) {
   return GABP_OK;
 }
 
-// Inverse of k64_messages: input-layout messages into the sliced positions as {c, v}.  A
-// mean message without a precision message (P = 0, h != 0) takes a c of 2^-300, whose
-// precision vanishes against any aggregate.
+// Inverse of k64_messages, to rounding: input-layout messages into the sliced positions as {c, v}.  A
+// mean message with (next to) no precision message takes a c of 2^-300, whose precision vanishes
+// against any aggregate (c has no unit: A over a cavity precision) and whose v stays finite.
 __global__ void k64_load_messages(int n, const int *__restrict__ rowptr, const int *__restrict__ dpos,
                                   const int *__restrict__ rp, const int *__restrict__ c2s,
                                   const double *__restrict__ av, const double *__restrict__ P,
@@ -1655,7 +1655,7 @@ __global__ void k64_load_messages(int n, const int *__restrict__ rowptr, const i
   for (int q = 0; q < deg; ++q) {
     int p = a + q + (q >= d ? 1 : 0);
     double c = -P[p] / av[e0 + q];
-    if (c == 0.0 && hm[p] != 0.0) c = 0x1p-300;
+    if (hm[p] != 0.0 && fabs(c) < 0x1p-300) c = copysign(0x1p-300, c);
     M[c2s[e0 + q]] = make_double2(c, hm[p] == 0.0 ? 0.0 : -hm[p] / c);
   }
 }

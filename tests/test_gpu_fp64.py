@@ -455,3 +455,18 @@ def test_cluster_rounds_small_graphs(gb, n, deg):
     assert st == gb.GABP_OK and it == ref["iters"]
     assert _relerr(x.cpu().numpy(), ref["x"]) <= 1e-12
     assert launches == 3
+
+
+@pytest.mark.parametrize("P0", [0.0, 1e-300, -1e-300, 5e-324])
+def test_warm_start_from_mean_messages_without_precision(gb, P0):
+    """Mean messages with a vanishing precision message are a valid start like any finite ones."""
+    m = synth.random_sym(3001, 8, 1.1, 2)
+    b = synth.rhs(m.n, 3)
+    s = gb.Solver.from_csr(m, warm_start=1)
+    hm = torch.full((m.nnz,), 1e10, dtype=torch.float64, device="cuda")
+    s.set_messages(torch.full_like(hm, P0), hm)
+    x, st, it, _ = s.solve(torch.from_numpy(b).cuda(), tol=1e-12)
+    s.close()
+    assert st == gb.GABP_OK
+    ref = oracle.gabp_broadcast(m, b, max_iter=1000, tol=1e-13)
+    assert _relerr(x.cpu().numpy(), ref["x"]) <= 1e-10
