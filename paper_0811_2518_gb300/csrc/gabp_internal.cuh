@@ -172,6 +172,7 @@ struct Sell32 {
 struct Work32 {
   // precision phase (recompute form): chains + node ring of 3
   float *MP[2] = {nullptr, nullptr};
+  size_t chain = 0;       // floats a chain of one right-hand side has room for
   float *NP[3] = {nullptr, nullptr, nullptr};
   float2 *CF = nullptr;   // {c_in, c_out} per slot
   float *invP = nullptr;  // 1 / P~_i (frozen)

@@ -1162,14 +1162,17 @@ gabp_status marginals32(gabp_handle h, double *Pi) {
   return GABP_OK;
 }
 
-// Positions of the sliced layout that the message chains have room for: E and 3 % for its padding.
-static size_t sell32_room(int64_t E) { return (size_t)(E + E / 32 + 4096); }
+// Graphs whose FP32 rounds may run on the sliced layout (ensure_sell32).
+constexpr double kSellRowsSlot = 12000.0;
+static bool sell32_size(const Graph &g) { return g.E > 0 && g.n >= kSellRowsSlot * g.avg_deg; }
 
 gabp_status ensure_w32(gabp_handle h, int R) {
   Work32 &w = h->w32;
   Graph &g = h->g;
   size_t E = (size_t)(g.E > 0 ? g.E : 1), n = (size_t)g.n;
-  const size_t Es = sell32_room(g.E);  // the chains serve the sliced layout, too
+  // the chains serve the sliced layout, too: 3 % for its padding where it may be built
+  const size_t Es = sell32_size(g) ? E + E / 32 + 4096 : E;
+  w.chain = Es;
   if (!w.MP[0]) {
     GABP_CUDA(cudaMalloc(&w.MP[0], sizeof(float) * Es));
     GABP_CUDA(cudaMalloc(&w.MP[1], sizeof(float) * Es));
@@ -1290,13 +1293,12 @@ static Args32 round_args32(gabp_handle h) {
 // kSellRowsSlot rows a slot of the average row on.  Not where a lane's row would be long, where the padding exceeds the
 // chains' room, or where there is no memory for it.
 constexpr int kSellWidth32 = 96;
-constexpr double kSellRowsSlot = 12000.0;
 static gabp_status ensure_sell32(gabp_handle h) {
   Work32 &w = h->w32;
   Sell32 &S = w.sl;
   const Graph &g = h->g;
   w.sl_on = false;
-  if (h->opt.lanes || w.dense_ld || g.E == 0 || g.n < kSellRowsSlot * g.avg_deg) return GABP_OK;
+  if (h->opt.lanes || w.dense_ld || !sell32_size(g)) return GABP_OK;
   if (!S.tried) {
     S.tried = true;
     const int ns = (g.n - 1) / 32 + 1, npos = 32 * ns;
@@ -1311,7 +1313,7 @@ static gabp_status ensure_sell32(gabp_handle h) {
       GABP_CUDA(cudaGetLastError());
       GABP_CUDA(cudaMemcpyAsync(out, dout, sizeof(out), cudaMemcpyDeviceToHost, h->stream));
       GABP_CUDA(cudaStreamSynchronize(h->stream));
-      room = out[1] <= kSellWidth32 && out[0] < INT32_MAX - 4096 && (size_t)out[0] <= sell32_room(g.E);
+      room = out[1] <= kSellWidth32 && out[0] < INT32_MAX - 4096 && (size_t)out[0] <= w.chain;
     }
     if (room) {
       const size_t Es = (size_t)out[0], nodes = sizeof(float) * 15 * (size_t)npos;

@@ -112,3 +112,26 @@ def test_handle_moves_between_the_orders(gb):
                 assert np.linalg.norm(x[c] - direct(bs[c])) <= 1e-11 / 0.15 * np.linalg.norm(bs[c])
         s.set_options(overlap_precision=1)
     s.close()
+
+
+def test_no_room_reserved_where_the_layout_cannot_be(gb):
+    """A graph of long rows (500 entries, 2 x 10^8 in all) takes the memory of the row kernels alone: per entry four
+    message chains, a coefficient pair and the FP32 value, 28 bytes, per row 25 words.  Allocations are rounded to 2
+    MB and graphs take some memory: 50 MB, half of 3 % of the four chains."""
+    _check(gb, _graph(25000, 40, 3), _solver(gb, _graph(25000, 40, 3)), 1)  # kernels are loaded
+    n, half = 400000, 250
+    d = torch.cat([torch.arange(-half, 0, device="cuda"), torch.arange(0, half + 1, device="cuda")])
+    col = (torch.arange(n, device="cuda")[:, None] + d[None, :]).remainder(n).int().sort(dim=1)[0]
+    val = torch.where(col == torch.arange(n, device="cuda", dtype=torch.int32)[:, None], 2.0 * 600, -1.0).double()
+    rowptr = torch.arange(n + 1, device="cuda", dtype=torch.int32) * (2 * half + 1)
+    s = gb.Solver(n, rowptr, col.reshape(-1), val.reshape(-1), precision=gb.GABP_PREC_FP32_REFINE, lanes=8)
+    del col, val
+    b = torch.ones(n, dtype=torch.float64, device="cuda")
+    x = torch.empty_like(b)
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    free = torch.cuda.mem_get_info()[0]
+    assert s.solve(b, tol=1e-8, x=x)[1] == gb.GABP_OK
+    assert free - torch.cuda.mem_get_info()[0] <= 28 * 500 * n + 100 * n + (50 << 20)
+    s.close()
+    assert float((x - 1.0 / 700).abs().max()) <= 1e-9
