@@ -282,6 +282,7 @@ struct GSell {
   int Es = 0;                  // slots, padding included
   bool by_size = false;
   std::vector<int> order;      // the systems in the layout's order: as given, or by descending size (stable)
+  std::vector<int> pad, wide;  // slots of each system, padding included, and its widest slice
   bool vals_ok = false;
   int *srow = nullptr;         // [32 ns] row of each slice lane, -1 for padding
   int *sp = nullptr;           // [ns + 1] first slot of each slice (multiples of 32)
@@ -378,6 +379,8 @@ struct gabp_handle_s {
   int multi_nt = 0;                 // autotuned block size of the multi-system kernel
   bool values_ok = true;            // false after a rejected gabp_set_values
   bool multi_queue = false;         // the last call on independent systems ran the queue kernel
+  std::vector<int> multi_off;       // the offsets that multi_from was decided for
+  int multi_from = 0;               // systems, by descending size, that the queue kernel does not take
   int multi_mode = 0;               // timed choice: 0 untuned, 1 grid-persistent kernel, 2 cluster / single-block teams
   int multi_grid_shape = 0;         // autotuned shape of the grid-persistent kernel (0 untuned)
   gabp::GSell *gsl = nullptr;       // sliced layout of the grid-persistent kernel (built on first use)

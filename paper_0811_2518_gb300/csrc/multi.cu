@@ -22,7 +22,6 @@
 
 #include <algorithm>
 #include <cmath>
-#include <functional>
 #include <numeric>
 #include <vector>
 
@@ -381,6 +380,76 @@ static gabp_status collect_systems(gabp_handle h, int nsys, const std::vector<in
                                    const double *d_rel, float ms, int *status_host, int *iters_host,
                                    double *relres_host);
 
+// Systems, by descending size, before the first that the queue kernel takes (nsys: none, the kernels are timed).
+// A model of a round in us, fitted to graphs of degree 3 to 300 with and without one hub row a system (geometric ones up
+// to 30, banded above); S slots, P with the sliced layout's padding, w the widest slice.
+//   queue kernel, one system: 3 + 7.2e-4 a row + 2.75e-4 a slot of P (one SM's rate) + 0.085 a slot that w exceeds
+//     the mean row (the chunks of a hub row, one warp); the longest of them, their sum over the SMs, or HBM's 18
+//     bytes a slot of P and 20 a row, whichever is most;
+//   timed choice: 9 + 0.12 a slot of w (40 at most) + 5.6e-6 a slot of S + 2e-5 a row + 0.035 a slot that w exceeds
+//     the mean row + 1.34e-5 a slot of padding;
+//   grid kernel on the sliced layout beside the queue: 11 + 5.6e-6 S + 2e-5 a row + 0.22 a slot of w above 16.
+// Measured, queue / timed choice (degree, systems of rows): 3, 1 of 4096 9.0 / 9.2 and 152 of 16384 34 / 76; 6, 8 of
+// 2048 7.3 / 10.7 and 8 of 16384 42 / 18; 12, 60 of 8192 39 / 57; 30, 8 of 2048 20 / 16 and 152 of 1024 13 / 38; 100,
+// 8 of 2048 59 / 21 and 152 of 4096 191 / 292; 300, 8 of 2048 169 / 34; 6 and a hub of 500, 8 of 4096 56 / 36 and 152 of
+// 4096 61 / 109.  Not where a row is wider than kQueueWidth: a lane's FP32 sum over 2000 slots cost 152 systems 227
+// rounds for the 190 of the row kernels' 8 lanes (500 slots: 161 and 161).
+constexpr int kQueueWidth = 512;
+static gabp_status queue_from(gabp_handle h, int nsys, const int *off, const std::vector<int> &rows,
+                              const std::vector<int> &slots, int *from) {
+  if ((int)h->multi_off.size() == nsys + 1 && std::equal(h->multi_off.begin(), h->multi_off.end(), off)) {
+    *from = h->multi_from;
+    return GABP_OK;
+  }
+  const int most = team_rows(h);
+  *from = nsys;
+  if (*std::min_element(rows.begin(), rows.end()) > most) return GABP_OK;
+  gabp_status st = ensure_gsell(h, nsys, off, true);
+  if (st != GABP_OK) return st;
+  const GSell &L = *h->gsl;
+  // of the systems order[0 .. q): slots, rows and widest slice; of order[q ..): what the queue's three bounds add up
+  double S = 0.0, R = 0.0, P = 0.0;
+  int wide = 0;
+  for (int s = 0; s < nsys; ++s) {
+    S += slots[s];
+    R += rows[s];
+    P += L.pad[s];
+    wide = std::max(wide, L.wide[s]);
+  }
+  double best = 9.0 + 0.12 * std::min(wide, 40) + 5.6e-6 * S + 2e-5 * R + 0.035 * std::max(0.0, wide - S / R) +
+                1.34e-5 * (P - S);
+  std::vector<double> gridt(nsys + 1, 0.0);
+  double gS = 0.0, gR = 0.0;
+  int gw = 0;
+  for (int q = 0; q < nsys; ++q) {
+    const int s = L.order[q];
+    gS += slots[s];
+    gR += rows[s];
+    gw = std::max(gw, L.wide[s]);
+    gridt[q + 1] = 11.0 + 5.6e-6 * gS + 2e-5 * gR + 0.22 * std::max(0, gw - 16);
+  }
+  double top = 0.0, sum = 0.0, bytes = 0.0;
+  for (int q = nsys - 1; q >= 0; --q) {
+    const int s = L.order[q];
+    if (rows[s] > most || L.wide[s] > kQueueWidth) break;
+    const double t = 3.0 + 7.2e-4 * rows[s] + 2.75e-4 * L.pad[s] +
+                     0.085 * std::max(0.0, L.wide[s] - (double)slots[s] / rows[s]);
+    top = std::max(top, t);
+    sum += t;
+    bytes += 18.0 * L.pad[s] + 20.0 * rows[s];
+    // a launch of the grid kernel takes all systems of a size
+    if (q > 0 && rows[L.order[q - 1]] == rows[s]) continue;
+    const double all = gridt[q] + std::max(std::max(top, sum / h->num_sms), bytes / 5.8e6);
+    if (all * (q > 0 ? 1.05 : 1.0) < best) {  // two launches for a gain that the model can tell
+      best = all;
+      *from = q;
+    }
+  }
+  h->multi_off.assign(off, off + nsys + 1);
+  h->multi_from = *from;
+  return GABP_OK;
+}
+
 gabp_status solve_systems(gabp_handle h, int nsys, const int *offsets_host, const double *b, double *x, double tol,
                           int max_iter, int *status_host, int *iters_host, double *relres_host) {
   NvtxRange nvtx_("gabp independent systems");
@@ -516,31 +585,12 @@ gabp_status solve_systems(gabp_handle h, int nsys, const int *offsets_host, cons
                               d_rel, shape, t);
   };
   // The queue kernel (multichip.cu) for the smaller systems and the grid-persistent kernel on the sliced
-  // layout for the larger ones, one after the other, unless an option asks for a kernel or the model below
-  // finds no system for the queue.  Time of a round in us by rows, fitted to geometric graphs of degree 6.
-  // Queue kernel: 3 + the larger of 2.4e-3 a row of its largest system (one SM's rate) and 2.0e-5 a row of
-  // all its systems (HBM): 1 system of 16384 rows 39.7, 152 of 1024 / 4096 / 16384 5.2 / 12.7 / 49.9.  Grid
-  // kernel: 11 + 4.6e-5 a row: 1 of 16384 10.8, 8 of 16384 17.2, 60 of 8192 32.5 (queue 22.7), 152 of
-  // 16384 113.
+  // layout for the larger ones, one after the other, unless an option asks for a kernel or queue_from finds
+  // no system for the queue.
   h->multi_queue = false;
   if (h->opt.multi_split == 0 && h->opt.multi_mode == 0 && h->opt.lanes == 0) {
-    std::vector<int> desc(rows);
-    std::sort(desc.begin(), desc.end(), std::greater<int>());
-    const int most = team_rows(h);
-    double left = 0.0, all = 0.0, best = 1e300;
-    for (int r : rows) all += r;
-    int from = nsys;  // systems desc[from ..] go to the queue
-    for (int q = 0; q <= nsys; ++q) {  // desc[0 .. q) on the grid
-      if (q == 0 || q == nsys || desc[q] != desc[q - 1]) {
-        const double grid = q > 0 ? 11.0 + 4.6e-5 * left : 0.0;
-        const double team = q < nsys ? 3.0 + std::max(2.4e-3 * desc[q], 2.0e-5 * (all - left)) : 0.0;
-        if ((q == nsys || desc[q] <= most) && grid + team < best) {
-          best = grid + team;
-          from = q;
-        }
-      }
-      if (q < nsys) left += desc[q];
-    }
+    int from = nsys;
+    if ((st = queue_from(h, nsys, offsets_host, rows, slots, &from)) != GABP_OK) return st;
     if (from < nsys) {
       float ms2 = 0.f;
       if (from > 0 && (st = solve_systems_grid(h, nsys, d_off, offsets_host, b, x, tol, max_iter, d_res, d_res + nsys,

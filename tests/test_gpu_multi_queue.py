@@ -193,3 +193,43 @@ def test_iterates_beyond_the_square_root_of_fp32(gb):
     for k in range(5):
         sl = slice(off[k], off[k + 1])
         assert np.linalg.norm(got[0][sl] - got[1][sl]) <= 1e-9 * np.linalg.norm(got[1][sl])
+
+
+def _hub(m, width, seed):
+    """m with its first row joined to ``width`` others (the diagonal keeps its dominance)."""
+    rng = np.random.default_rng(seed)
+    rows = np.repeat(np.arange(m.n), np.diff(m.rowptr))
+    off = rows != m.col
+    j = np.setdiff1d(rng.choice(np.arange(1, m.n), width, replace=False), m.col[m.rowptr[0]:m.rowptr[1]])
+    i = np.concatenate([rows[off], np.zeros(j.size, int), j])
+    k = np.concatenate([m.col[off], j, np.zeros(j.size, int)])
+    v = np.concatenate([m.val[off], np.full(2 * j.size, -0.7)])
+    d = 1.1 * np.bincount(i, np.abs(v), minlength=m.n)
+    return synth.from_coo(m.n, np.concatenate([i, np.arange(m.n)]), np.concatenate([k, np.arange(m.n)]),
+                          np.concatenate([v, np.where(d > 0, d, 1.0)]))
+
+
+@pytest.mark.parametrize("make,queue", [
+    (lambda: [synth.random_sym(2048, 50, 1.1, q) for q in range(8)], False),   # few systems of wide rows
+    (lambda: [synth.random_sym(1024, 15, 1.1, q) for q in range(152)], True),  # an SM for each
+    (lambda: [_hub(m, 500, 3) for m in synth.rgg_batch(8, 4000, 4096, 2.0, 4)], False),  # hub rows, SMs idle
+    (lambda: [_hub(m, 500, 3) for m in synth.rgg_batch(152, 2000, 2048, 2.0, 4)], True),
+    (lambda: [_hub(m, 1000, 3) for m in synth.rgg_batch(152, 2000, 2048, 2.0, 4)], False),  # too wide for a lane
+], ids=["wide8", "wide152", "hub8", "hub152", "hub_too_wide"])
+def test_choice_by_slots_and_widths(gb, make, queue):
+    """Systems go to the queue where one SM each is enough for their slots and widest rows."""
+    mats = make()
+    big = synth.block_diag(mats)
+    off = big.meta["offsets"]
+    b = synth.rhs(big.n, 6)
+    s = gb.Solver.from_csr(big)
+    for _ in range(2):
+        x, st, sts, its, rel = _solve(gb, s, mats, b, off, tol=1e-11)
+        assert st == gb.GABP_OK and np.all(rel <= 1e-11)
+    t = s.tuned()
+    assert t["multi_mode"] in ((2,) if queue else (1, 2)) and (t["multi_grid"] == (0, 0)) == queue
+    s.close()
+    for k in (0, 5):
+        sl = slice(off[k], off[k + 1])
+        ref = np.linalg.solve(synth.to_dense(mats[k]), b[sl])
+        assert np.linalg.norm(x[sl] - ref) <= 1e-9 * np.linalg.norm(ref)
