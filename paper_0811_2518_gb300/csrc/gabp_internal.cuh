@@ -618,7 +618,8 @@ void free_ws(gabp_handle h);
 gabp_status serial_prepare(gabp_handle h);
 gabp_status serial_colours(gabp_handle h, int *colour_dev, int *ncolours);
 gabp_status serial_refresh_values(gabp_handle h);
-// serial2.cu: the FP64 sweeps of a graph of two colours; GABP_NOT_RUN where b = 0 or there is no room (nothing was done)
+// serial2.cu: the FP64 sweeps of a graph of two colours; GABP_NOT_RUN where b = 0, there is no
+// room or the general passes are faster (nothing was done)
 constexpr gabp_status GABP_NOT_RUN = (gabp_status)-100;
 gabp_status solve64_two_colours(gabp_handle h, const double *b, double *x, double tol, int max_iter, int *iters,
                                 double *relres);

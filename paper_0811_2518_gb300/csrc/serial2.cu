@@ -272,6 +272,18 @@ gabp_status ensure_two(gabp_handle h) {
   return room ? GABP_OK : refuse();
 }
 
+// Where the general passes (2 lanes a row from 8 slots a row, 4 from 24) are the faster ones: rows that are long for
+// a lane each, and too few of them to hide that behind other warps.  Bipartite graphs of two equal sides, whole solves
+// in ms, general / these: 24 slots a row or more, 2 x 6,000 rows of 40 2.95 / 4.70, 2 x 10,000 of 25 2.87 / 3.65, 2 x
+// 20,000 of 100 8.43 / 9.64, 2 x 40,000 of 100 15.6 / 12.1 and of 40 7.40 / 5.29; 16 slots, 2 x 3,000 rows 2.35 / 2.10.
+// With the freeze, whose empty launches weigh on these: 8 slots a row or more, 2 x 20,000 rows of 16 2.36 / 3.14, 2 x
+// 40,000 of 100 14.1 / 14.8 and of 40 6.75 / 6.49, 2 x 60,000 of 16 4.63 / 3.55; below 8, 2 x 6,000 rows 2.10 / 1.59.
+bool two_pays(gabp_handle h) {
+  const int slices = h->g.n / 32;
+  return h->opt.freeze_precisions ? h->g.avg_deg < 8.0 || slices >= 20 * h->num_sms
+                                  : h->g.avg_deg < 24.0 || slices >= 16 * h->num_sms;
+}
+
 ArgsS2 args_two(gabp_handle h) {
   WorkS2 &w = h->ws.two;
   ArgsS2 a;
@@ -304,6 +316,7 @@ void free_serial2(WorkS &s) {
 
 gabp_status solve64_two_colours(gabp_handle h, const double *b, double *x, double tol, int max_iter, int *iters,
                                 double *relres) {
+  if (!two_pays(h)) return GABP_NOT_RUN;
   gabp_status st = ensure_two(h);
   if (st != GABP_OK) return st;
   Graph &g = h->g;

@@ -163,3 +163,34 @@ def test_no_room_for_the_two_colour_layout(gb):
     assert st == gb.GABP_OK and it == sweeps
     assert torch.allclose(x, ref, rtol=0, atol=1e-10 * float(ref.abs().max()))
     s.close()
+
+
+def _regular(side, deg):
+    """A bipartite graph of two sides, every row with ``deg`` neighbours around its place on the other side."""
+    i = np.repeat(np.arange(side), deg)
+    j = side + (i + np.tile(np.arange(deg), side)) % side
+    w = -np.random.default_rng(1).uniform(0.1, 1.0, i.size)
+    d = 1.2 * (np.bincount(i, -w, minlength=2 * side) + np.bincount(j, -w, minlength=2 * side))
+    a = np.arange(2 * side)
+    return synth.from_coo(2 * side, np.concatenate([i, j, a]), np.concatenate([j, i, a]), np.concatenate([w, w, d]))
+
+
+@pytest.mark.parametrize("side,deg,freeze,two", [(6000, 50, 0, False), (6000, 50, 1, False), (40000, 30, 0, True),
+                                                 (24000, 20, 0, True), (24000, 20, 1, False), (50000, 12, 1, True)])
+def test_long_rows_run_the_general_passes(gb, side, deg, freeze, two):
+    """Rows long for a lane each, and few of them, run the general passes: seen by the memory of their state (16
+    bytes a slot, 24 with the freeze, where the two-colour layout and state take 52 and 60)."""
+    m = _regular(side, deg)
+    b = synth.rhs(m.n, 7)
+    s = gb.Solver.from_csr(m, schedule=1, freeze_precisions=freeze)
+    assert s.serial_colours()[1] == 2
+    tb, x = torch.from_numpy(b).cuda(), torch.empty(m.n, dtype=torch.float64, device="cuda")
+    torch.cuda.synchronize()
+    free = torch.cuda.mem_get_info()[0]
+    st, it = s.solve(tb, tol=1e-11, max_iter=3000, x=x)[1:3]
+    taken = free - torch.cuda.mem_get_info()[0]
+    assert (taken > 40 * 2 * side * deg) == two
+    r = oracle.gabp_serial(m, b, max_iter=3000, tol=1e-11)
+    assert st == gb.GABP_OK and it == r["iters"]
+    assert np.linalg.norm(x.cpu().numpy() - r["x"]) <= 1e-11 * np.linalg.norm(r["x"])
+    s.close()
