@@ -186,12 +186,16 @@ __device__ __forceinline__ RevFrom round_source(int t, int cold) {
 // verification of a solve takes a bar of 8 units in the last place, which tells a message
 // that still converges from one that rounds; where the stagnant messages jitter by more
 // (3D grids: up to 16), the later ones, after longer screens, take the screen's 16.  MODE 3 (frozen precisions): only the mean
-// messages, h_ki = -c v, with the stored coefficients; P~ and 1/P~ carried over.
+// messages, h_ki = -c v, with the stored coefficients; P~ and 1/P~ carried over.  WHOLE: it stores
+// c beside v, so that the cavities, which take the store's c, take the frozen one; needed in
+// the first such round (the other store holds the frozen c already), and the faster form where the
+// stores go to HBM (128^3 grid 33.9 -> 31.7 ms, 2^20 random rows 35.7 -> 32.3), but not from L2 (6,000 rows of
+// 300 slots in one launch 18.9 -> 21.4).
 // All modes form x and the residual of the previous iterate as the round kernels do.
 // FROM: where the reverse messages come from (round_source), a template parameter because a
 // branch on it between a slot's loads would keep them from being issued together.  In the
 // recompute form Nout and Mout hold round t-2 until they are written.
-template <bool COOP, int MODE, RevFrom FROM, int UU = 0>
+template <bool COOP, int MODE, RevFrom FROM, int UU = 0, bool WHOLE = true>
 __device__ __forceinline__ void plain_slice(const Args64 &a, int sl, int lane, const double *__restrict__ b,
                                             const double2 *__restrict__ Min, double2 *__restrict__ Mout,
                                             const NodeRec64 *__restrict__ Nin, NodeRec64 *__restrict__ Nout,
@@ -236,8 +240,12 @@ __device__ __forceinline__ void plain_slice(const Args64 &a, int sl, int lane, c
       const int pos = p0 + 32 * (j + u);
       if (MODE == 3) {
         const double v = fma(rv[u].x, rv[u].y, nk[u].h);
-        const double2 m = make_double2(c[u], v);  // with c: both stores hold the frozen one, which the cavities take
-        if (COOP) Mout[pos] = m; else __stcs(Mout + pos, m);
+        if (WHOLE) {
+          const double2 m = make_double2(c[u], v);
+          if (COOP) Mout[pos] = m; else __stcs(Mout + pos, m);
+        } else {
+          reinterpret_cast<double *>(Mout + pos)[1] = v;
+        }
         acch = fma(-c[u], v, acch);
       } else {
         if (REC) rv[u] = reverse64(A[u], P2, h2, rv[u]);
@@ -603,9 +611,11 @@ __global__ void __launch_bounds__(kCoopThreads, coop_blocks(FRZ, U))
   const double *__restrict__ b = ctl->b;
   const int cold = ctl->cold, t0 = ctl->round;
   const StopRule rule = stop_rule(ctl);
-  int fs = FRZ ? ctl->fstate : 0;
+  int fs = FRZ ? ctl->fstate : 0, fprev = 0, fnow = 0;  // the freeze state of this round, of the last one
   for (int iter = 0; iter < max_rounds; ++iter) {
     const int t = t0 + 1 + iter;
+    fprev = fnow;
+    fnow = fs;
     const double2 *__restrict__ Min = (t & 1) ? a.M0 : a.M1;
     double2 *__restrict__ Mout = (t & 1) ? a.M1 : a.M0;
     const NodeRec64 *__restrict__ Nin = (t & 1) ? a.N0 : a.N1;
@@ -618,7 +628,8 @@ __global__ void __launch_bounds__(kCoopThreads, coop_blocks(FRZ, U))
       else if (!FRZ) plain_slice<true, 0, kGather, U>(a, sl, lane, b, Min, Mout, Nin, Nout, rr, bad, moving);
       else if (fs == 0) plain_slice<true, 1, kGather, U>(a, sl, lane, b, Min, Mout, Nin, Nout, rr, bad, moving);
       else if (fs == 1) plain_slice<true, 2, kGather, U>(a, sl, lane, b, Min, Mout, Nin, Nout, rr, bad, moving);
-      else plain_slice<true, 3, kGather, U>(a, sl, lane, b, Min, Mout, Nin, Nout, rr, bad, moving);
+      else if (fprev != 2) plain_slice<true, 3, kGather, U>(a, sl, lane, b, Min, Mout, Nin, Nout, rr, bad, moving);
+      else plain_slice<true, 3, kGather, U, false>(a, sl, lane, b, Min, Mout, Nin, Nout, rr, bad, moving);
     }
     // grid barrier; the last block to arrive reduces and decides.  partials: the blocks' sums, then their
     // flags (bit 0 a zero precision, bit 1 a precision moved).
