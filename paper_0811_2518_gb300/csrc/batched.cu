@@ -147,6 +147,11 @@ __device__ bool col_reduce(const double (&acc)[NV][VEC], int RP, double *red, do
 #endif
 template <int VEC>
 constexpr int kBU = VEC == 4 ? 2 : GABP_KB_U;
+// Graphs of few rows leave an SM a few warps, each waiting for its loads: more slots of a row together.  (With 2, the
+// rounds that read the reverse messages through rev cost such graphs more than the store they save: 200 rows of 40
+// slots, 16 columns 2.51 ms with four messages a pair of rounds, 2.71 with three, 2.37 with three and 8 slots; 1,000 rows
+// of 100 4.53, 4.68, 3.51; 2,000 rows of 100 6.3, 6.4.  With 64 columns, two a lane, 2 slots are enough.)
+constexpr int kBUFew = 8, kBFewRowsSm = 8;
 
 // Rounds by what their reverse messages come from: none in round 1 (zero messages), the row's own
 // aggregate in round 2 (its stored messages are the zero ones, not read), then as above.
@@ -187,10 +192,9 @@ __device__ __forceinline__ void kb_slots(const ArgsB &a, int e, int c0, const fl
   }
 }
 
-template <int VEC, BKind KIND>
+template <int VEC, BKind KIND, int NU>
 __device__ __forceinline__ void kb_rows(const ArgsB &a, const float *__restrict__ Hm1, const float *__restrict__ Hm2,
                                         float *__restrict__ Ht, float (&acc2)[2][VEC]) {
-  constexpr int NU = kBU<VEC>;
   const int RP = a.RP;
   const int c0 = (threadIdx.x & 31) * VEC;
   const int warp = (blockIdx.x * kBlock + threadIdx.x) >> 5;
@@ -203,6 +207,8 @@ __device__ __forceinline__ void kb_rows(const ArgsB &a, const float *__restrict_
     int e = a.rp[i];
     const int e1 = a.rp[i + 1];
     for (; e + NU <= e1; e += NU) kb_slots<VEC, KIND, NU>(a, e, c0, Hm1, hi2, acc);
+    if (NU > 4 && e + 4 <= e1) { kb_slots<VEC, KIND, 4>(a, e, c0, Hm1, hi2, acc); e += 4; }
+    if (NU > 2 && e + 2 <= e1) { kb_slots<VEC, KIND, 2>(a, e, c0, Hm1, hi2, acc); e += 2; }
     for (; e < e1; ++e) kb_slots<VEC, KIND, 1>(a, e, c0, Hm1, hi2, acc);
     float rh[VEC], hp[VEC], hnew[VEC];
     ldv<VEC>(a.rhs + (size_t)i * RP + c0, rh);
@@ -221,8 +227,8 @@ __device__ __forceinline__ void kb_rows(const ArgsB &a, const float *__restrict_
 
 // Round t of the batched frozen-precision mean iteration (one warp per row).
 // Stops when every column with a nonzero iterate has ||dx_r|| <= inner_tol ||x_r||.
-template <int VEC>
-__global__ void __launch_bounds__(kBlock, GABP_KB_MINB) kb_mean(ArgsB a) {
+template <int VEC, int NU>
+__global__ void __launch_bounds__(kBlock, NU > 2 ? 2 : GABP_KB_MINB) kb_mean(ArgsB a) {
   DevCtl *ctl = a.ctl;
   if (ctl->done) return;
   const int t = ctl->round + 1;
@@ -234,11 +240,11 @@ __global__ void __launch_bounds__(kBlock, GABP_KB_MINB) kb_mean(ArgsB a) {
 #pragma unroll
   for (int v = 0; v < VEC; ++v) acc2[0][v] = acc2[1][v] = 0.f;
   if (t & 1) {
-    if (t == 1) kb_rows<VEC, kBFirst>(a, Hm1, Hm2, Ht, acc2);
-    else kb_rows<VEC, kBOdd>(a, Hm1, Hm2, Ht, acc2);
+    if (t == 1) kb_rows<VEC, kBFirst, NU>(a, Hm1, Hm2, Ht, acc2);
+    else kb_rows<VEC, kBOdd, NU>(a, Hm1, Hm2, Ht, acc2);
   } else {
-    if (t == 2) kb_rows<VEC, kBSecond>(a, Hm1, Hm2, Ht, acc2);
-    else kb_rows<VEC, kBEven>(a, Hm1, Hm2, Ht, acc2);
+    if (t == 2) kb_rows<VEC, kBSecond, NU>(a, Hm1, Hm2, Ht, acc2);
+    else kb_rows<VEC, kBEven, NU>(a, Hm1, Hm2, Ht, acc2);
   }
   double accd[2][VEC];
 #pragma unroll
@@ -740,7 +746,9 @@ static gabp_status batched_chunk(gabp_handle h, int R, const double *B, double *
     }
     return blocks_for(g.n, kBlock / 32, nb * h->num_sms);
   };
-  const int nb_mean = grid_of(kb_mean<VEC>);
+  void (*const mean)(ArgsB) =
+      VEC == 1 && g.n <= kBFewRowsSm * h->num_sms ? kb_mean<VEC, VEC == 1 ? kBUFew : kBU<VEC>> : kb_mean<VEC, kBU<VEC>>;
+  const int nb_mean = grid_of(mean);
   const int nb_res = grid_of(kb_residual<VEC>);
   dim3 tb(32, 8), tg((g.n + 31) / 32, RP / 32);
   kb_gather_cols<<<tg, tb, 0, h->stream>>>(g.n, R, RP, B, ld, w.Bt);
@@ -820,7 +828,7 @@ static gabp_status batched_chunk(gabp_handle h, int R, const double *B, double *
       kb_ctl_reset<<<1, 1, 0, h->stream>>>(h->ctl, cap, it_tol * it_tol);
       h->prof.launches += 1;
       GABP_CUDA(cudaGetLastError());
-      s = run_rounds(h, &w.graph, &w.graph_key, RP, [&] { kb_mean<VEC><<<nb_mean, kBlock, shmem, h->stream>>>(a); },
+      s = run_rounds(h, &w.graph, &w.graph_key, RP, [&] { mean<<<nb_mean, kBlock, shmem, h->stream>>>(a); },
                      cap, PH_MEAN32);
     }
     if (s != GABP_OK) return s;

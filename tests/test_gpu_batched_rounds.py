@@ -64,3 +64,30 @@ def test_batched_rounds_reach_the_dense_solution(gb, kind, schedule, R, cap):
         ref = np.linalg.solve(A, B.T).T
         assert np.max(np.abs(X.cpu().numpy() - ref)) <= 1e-9 * np.max(np.abs(ref))
     s.close()
+
+
+@pytest.mark.parametrize("R", [1, 32])
+@pytest.mark.parametrize("kind", ["tree", "random", "dense rows"])
+def test_few_rows_and_many_rows_give_the_same_bits(gb, kind, R):
+    """A graph alone (few rows: eight slots of a row together) and in eight copies (two slots) after equal rounds:
+    rows of none to 29 slots, every remainder."""
+    if kind == "dense rows":
+        n = 203
+        A = np.triu(np.random.default_rng(2).uniform(-1, 1, (n, n)), 1)
+        A *= (np.arange(n)[:, None] + np.arange(n)[None, :]) % 7 == 0
+        A[:46, :46] = A[46:92, :46] = A[:46, 46:92] = 0.0
+        A = A + A.T
+        A[np.diag_indices(n)] = 1.3 * np.maximum(np.abs(A).sum(1), 1.0)
+    else:
+        A = _matrix(kind)
+    m = synth.from_dense(A)
+    n = m.n
+    B = np.random.default_rng(R).standard_normal((R, n))
+    out = []
+    for copies in (1, 8):
+        big = synth.block_diag([m] * copies)
+        s = gb.Solver.from_csr(big, lanes=4, inner_max_iter=9, inner_tol=1e-30, max_refine=2)
+        X = s.solve_batched(torch.from_numpy(np.tile(B, (1, copies))).cuda(), tol=0.0, max_iter=1000, check=False)[0]
+        out.append(X.cpu().numpy()[:, :n])
+        s.close()
+    assert np.any(out[0]) and np.array_equal(out[0], out[1])
