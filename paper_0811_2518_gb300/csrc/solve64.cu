@@ -190,7 +190,7 @@ __device__ __forceinline__ RevFrom round_source(int t, int cold) {
 // c beside v, so that the cavities, which take the store's c, take the frozen one; needed in
 // the first such round (the other store holds the frozen c already), and the faster form where the
 // stores go to HBM (128^3 grid 33.9 -> 31.7 ms, 2^20 random rows 35.7 -> 32.3), but not from L2 (6,000 rows of
-// 300 slots in one launch 18.9 -> 21.4).
+// 300 slots in one launch 18.9 -> 21.4): the cooperative rounds fill in c once instead.
 // All modes form x and the residual of the previous iterate as the round kernels do.
 // FROM: where the reverse messages come from (round_source), a template parameter because a
 // branch on it between a slot's loads would keep them from being issued together.  In the
@@ -611,24 +611,26 @@ __global__ void __launch_bounds__(kCoopThreads, coop_blocks(FRZ, U))
   const double *__restrict__ b = ctl->b;
   const int cold = ctl->cold, t0 = ctl->round;
   const StopRule rule = stop_rule(ctl);
-  int fs = FRZ ? ctl->fstate : 0, fprev = 0, fnow = 0;  // the freeze state of this round, of the last one
+  int fs = FRZ ? ctl->fstate : 0;
+  bool fresh = false;  // the last round verified
   for (int iter = 0; iter < max_rounds; ++iter) {
     const int t = t0 + 1 + iter;
-    fprev = fnow;
-    fnow = fs;
     const double2 *__restrict__ Min = (t & 1) ? a.M0 : a.M1;
     double2 *__restrict__ Mout = (t & 1) ? a.M1 : a.M0;
     const NodeRec64 *__restrict__ Nin = (t & 1) ? a.N0 : a.N1;
     NodeRec64 *__restrict__ Nout = (t & 1) ? a.N1 : a.N0;
     double rr = 0.0;
     int bad = 0, moving = 0;
+    if (FRZ && fs == 2 && fresh)  // the own slots' c, in the store that the last round did not write
+      for (int sl = warp; sl < a.ns; sl += nwarps)
+        for (int pos = a.sp[sl] + lane; pos < a.sp[sl + 1]; pos += 32) Mout[pos].x = __ldcg(a.C + pos);
+    if (FRZ) fresh = fs == 1;
     for (int sl = warp; sl < a.ns; sl += nwarps) {
       if (!FRZ && t == 1 && cold)
         plain_slice<true, 0, kZero, U>(a, sl, lane, b, Min, Mout, Nin, Nout, rr, bad, moving);
       else if (!FRZ) plain_slice<true, 0, kGather, U>(a, sl, lane, b, Min, Mout, Nin, Nout, rr, bad, moving);
       else if (fs == 0) plain_slice<true, 1, kGather, U>(a, sl, lane, b, Min, Mout, Nin, Nout, rr, bad, moving);
       else if (fs == 1) plain_slice<true, 2, kGather, U>(a, sl, lane, b, Min, Mout, Nin, Nout, rr, bad, moving);
-      else if (fprev != 2) plain_slice<true, 3, kGather, U>(a, sl, lane, b, Min, Mout, Nin, Nout, rr, bad, moving);
       else plain_slice<true, 3, kGather, U, false>(a, sl, lane, b, Min, Mout, Nin, Nout, rr, bad, moving);
     }
     // grid barrier; the last block to arrive reduces and decides.  partials: the blocks' sums, then their
