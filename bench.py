@@ -581,9 +581,9 @@ def main():
             offm = bigm.meta["offsets"]
             bm = torch.from_numpy(synth.rhs(bigm.n, 4 + rank)).to(dev)
             sm = gb.Solver.from_csr(bigm, multi_mode=args.multi_mode, **gkw)
-            xm, stm, stsm, itsm, relm = sm.solve_systems(bm, offm, tol=TOL)  # first call autotunes the split
+            xm, stm, stsm, itsm, relm = sm.solve_systems(bm, offm, tol=TOL)  # the first call lays out or tunes
             sm.profile(reset=True)
-            reps_m = 5  # timed batches (each one launch); the median is reported
+            reps_m = 5  # timed batches; the median is reported
             times_m = []
             for _ in range(reps_m):
                 barrier()
@@ -622,13 +622,15 @@ def main():
                                  "weights -U(0.5,1), diagonal 1.1 x row abs-sum, one b ~ N(0,1) each",
                      "systems": len(mats), "n_total": bigm.n, "edges_total": bigm.num_edges, "status": int(stm),
                      "ms_per_batch": msm, "ms_per_batch_all": times_m, "kernel_ms": pm["ms"]["multi"] / reps_m,
-                     "kernel": "grid-persistent" if (args.multi_mode in (1, 3) or tuned_m["multi_mode"] == 1) else "teams",
+                     "kernel": ("grid-persistent" if (args.multi_mode in (1, 3) or tuned_m["multi_mode"] == 1) else
+                                "queue (largest systems: grid-persistent)" if not args.multi_mode
+                                and tuned_m["multi_split"] == 0 else "teams"),
                      "grid_shape": {"lanes_per_row": tuned_m["multi_grid"][0], "slots_per_lane": tuned_m["multi_grid"][1],
                                     "sliced_layout": tuned_m["multi_grid_sliced"]},
                      "edge_updates": stm_["edge_updates"],
                      "edge_updates_per_s": stm_["edge_updates"] / (msm / 1e3),
                      "rounds_per_system": {"min": int(itsm.min()), "median": int(np.median(itsm)), "max": int(itsm.max())},
-                     "max_relres": float(relm.max()), "launches_per_batch": 1,
+                     "max_relres": float(relm.max()), "launches_per_batch": pm["launches"] // reps_m,
                      "fp64_plain_per_system": {"ms_all_systems": ms_per_sys, "rounds_total": rounds_p,
                                                "how": "one FP64 handle per system, solved one after another"},
                      "batch_vs_fp64_per_system": ms_per_sys / msm,

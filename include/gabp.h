@@ -104,8 +104,8 @@ typedef struct {
                            screen resumes.  Every round up to the stored one is bitwise the plain
                            solve's; after it x differs from the plain iterate by rounding only.
                            The plain rounds are no longer bound by the precisions' arithmetic: on the 128^3
-                           grid a frozen solve takes 34.7 ms (parallel) and 23.0 (serial), a plain one
-                           30.8 and 18.7.  0 =
+                           grid a frozen solve takes 31.8 ms (parallel) and 21.4 (serial), a plain one
+                           30.7 and 18.5.  0 =
                            every round updates both (Algorithm 2 as printed).  The edge variant
                            and the accelerated solves ignore it (the FP32 path always freezes).
                            Default 0 */
@@ -129,7 +129,9 @@ typedef struct {
                            thread-block cluster, smaller ones to one block; 0 = autotune.  Default 0 */
   int prec_stop_log2;   /* FP32 precision phase stops at a max relative change <= 2^-prec_stop_log2 in
                            two consecutive rounds (10..23).  Default 16 */
-  int multi_mode;       /* gabp_solve_systems kernel: 0 autotune, 1 grid-persistent (every round sweeps
+  int multi_mode;       /* gabp_solve_systems kernel: 0 by a model of the batch (a queue of one-SM
+                           solves where that pays, beside the grid-persistent kernel for the largest
+                           systems), else timed (kernel and shape); 1 grid-persistent (every round sweeps
                            all running systems; its shape autotuned over the row-CSR and the sliced
                            layouts), 2 cluster / single-block teams, 3 grid-persistent on the sliced
                            layout only (each system's rows sorted by degree and cut into 32-row
@@ -280,8 +282,8 @@ gabp_status gabp_solve_batched(gabp_handle h, int32_t nrhs, const double *B, dou
  * FP32 precision phase, FP32 mean rounds and FP64 refinement to
  * ||b_s - A_s x_s|| <= tol ||b_s|| (the batching direction of the paper's method:
  * systems share nothing).  With the default options systems of up to 17,120 rows
- * are solved by one SM each from a queue where that pays, and the larger ones by
- * the grid-persistent kernel; else the kernel and its shape (grid-persistent, or
+ * and 512 entries a row are solved by one SM each from a queue where that pays, and the
+ * larger ones by the grid-persistent kernel; else the kernel and its shape (grid-persistent, or
  * clusters for large systems and blocks for small ones) are autotuned on the handle's
  * first call.
  * status_out / iters_out / relres_out: nullable HOST arrays of nsys receiving each

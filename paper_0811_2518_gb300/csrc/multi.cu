@@ -1,5 +1,6 @@
-// multi.cu -- many independent systems (a block-diagonal A) solved by ONE
-// persistent launch: FP32 precision phase, frozen coefficients, FP32 mean
+// multi.cu -- many independent systems (a block-diagonal A): the choice of kernels (the queue of one-SM
+// solves of multichip.cu, the grid-persistent kernel of multigrid.cu, the teams below), and the teams,
+// which solve all systems in ONE persistent launch: FP32 precision phase, frozen coefficients, FP32 mean
 // rounds and FP64 iterative refinement of every system run inside the kernel.
 //
 // Each system is solved by a team: either a whole thread-block cluster (kCS
@@ -634,9 +635,9 @@ gabp_status solve_systems(gabp_handle h, int nsys, const int *offsets_host, cons
     h->multi_grid_shape = shape;
     return run_grid_shape(shape, t);
   };
-  // kernel choice: the options may force the grid-persistent kernel (mode 1) or
-  // teams (mode 2, or any fixed split); otherwise the first call on a handle
-  // times both and later calls reuse the faster one
+  // timed choice: the options may force the grid-persistent kernel (modes 1 and 3) or
+  // teams (mode 2, or any fixed split); otherwise (no system for the queue) the first such call on a
+  // handle times both and later ones reuse the faster
   if (mode == 1 || mode == 3) {
     if ((st = run_grid(&ms)) != GABP_OK) return st;
     return finish(ms);

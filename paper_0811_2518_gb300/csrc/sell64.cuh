@@ -22,7 +22,7 @@ __device__ __forceinline__ WarpPos warp_pos() {
 // rows the slices get narrower (rows sorted by degree), and a fixed stride would hand a warp slices of
 // like width in every pass (28 % of the round with idle warps on the 2^20 random graph); turning each
 // pass by the golden section of a window's 128 slices spreads every warp's slices over the window:
-// 347 -> 286 us per round there, unchanged on grids.
+// 307 -> 240 us per round there, unchanged on grids.
 __device__ __forceinline__ int pass_slice(const WarpPos &w, int m) {
   constexpr int kSlices = kSellWindow / 32, kGolden = 79;  // 128 / 1.618
   const int turn = (kGolden + kSlices - w.nwarps % kSlices) % kSlices;

@@ -34,9 +34,9 @@
 // degree share a warp, and the row epilogue runs on all 32 lanes.
 //
 // What bounds a round: the FP64 pipe (629 G operations/s at 2070 MHz), 5 instructions a slot and 5 a
-// row in the gather form, 7 a slot in the recompute form.  128^3 grid: 164 us per round (FP64 116, HBM
-// 113; 309 us with 11 FP64 instructions a slot); 2^20 rows of degree 16: 250 us (FP64 195, HBM 131;
-// 505 us with 11 and with gathered reverse messages).
+// row in the gather form, 7 a slot in the recompute form.  128^3 grid: 160 us per round (FP64 116, HBM
+// 113; 309 us with 11 FP64 instructions a slot); 2^20 rows of degree 16: 240 us (FP64 195, HBM 131;
+// 506 us with 11 and with gathered reverse messages).  (Device time of the rounds over their number.)
 #include "gabp_internal.cuh"
 #include "sell64.cuh"
 #include "cluster.cuh"
@@ -51,9 +51,9 @@ namespace gabp {
 
 // Slots per lane whose loads a round issues together, and the blocks per SM its register budget
 // is sized for (__launch_bounds__).  Recompute form on the 2^20 random graph of degree 16: 2 slots and
-// 4 blocks (64 registers, 32 warps an SM) 276 us per round; 3 blocks 286; 1 slot with 4 blocks 284, with
-// 5 blocks 282.  Gather form on the 128^3 grid: 3 slots and 4 blocks 164 us per round, 2 slots 169,
-// 3 slots with 3 or 5 blocks 170 / 185.
+// 4 blocks (64 registers, 32 warps an SM) 240 us per round; 3 blocks 242; 1 slot with 4 blocks 257, with
+// 5 blocks 248.  Gather form on the 128^3 grid: 3 slots and 4 blocks 160 us per round, 2 slots 165,
+// 3 slots with 3 or 5 blocks 165 / 177.
 constexpr int kURec = 2, kUGather = 3, kUCoop = 2, kU64 = 2;
 constexpr int kMinBlocks64 = 4;
 
@@ -185,8 +185,8 @@ __device__ __forceinline__ RevFrom round_source(int t, int cold) {
 // c = A / (P~_k - P_ik) and each row's 1/P~ (the record's spare slot).  The first
 // verification of a solve takes a bar of 8 units in the last place, which tells a message
 // that still converges from one that rounds; where the stagnant messages jitter by more
-// (3D grids: up to 16), the later ones, after longer screens, take the screen's 16.  MODE 3 (frozen precisions): only the mean
-// messages, h_ki = -c v, with the stored coefficients; P~ and 1/P~ carried over.  WHOLE: it stores
+// (3D grids: up to 16), the later ones, after longer screens, take the screen's 16.
+// MODE 3 (frozen precisions): only the mean messages, h_ki = -c v, with the stored coefficients; P~ and 1/P~ carried over.  WHOLE: it stores
 // c beside v, so that the cavities, which take the store's c, take the frozen one; needed in
 // the first such round (the other store holds the frozen c already), and the faster form where the
 // stores go to HBM (128^3 grid 33.9 -> 31.7 ms, 2^20 random rows 35.7 -> 32.3), but not from L2 (6,000 rows of
@@ -1408,9 +1408,9 @@ static Args64 args64(gabp_handle h) {
              h->w64.C != nullptr;
   // Recompute the reverse messages when more than a quarter of them lie further than kFarSlots positions
   // (32 MB of messages) from the slot that needs them: such reads come from DRAM, a 32-byte sector each.
-  // Both forms measured, gather / recompute: random graphs of degree 16 with 200,000 rows (12 % far) 76 / 79
-  // us per round, 400,000 (45 %) 145 / 128, 2^20 (77 %) 449 / 276; 10^6 rows of degree 6 (42 %) 193 / 122;
-  // 64^3 and 128^3 grids (none far) 34 / 39 and 164 / 203.
+  // Both forms measured, gather / recompute: random graphs of degree 16 with 200,000 rows (12 % far) 70 / 71
+  // us per round, 400,000 (45 %) 130 / 109, 2^20 (77 %) 411 / 240; 10^6 rows of degree 6 (42 %) 155 / 105;
+  // 64^3 and 128^3 grids (none far) 28 / 33 and 160 / 186.
   a.rec = S.far > (int64_t)h->g.E / 4;
   // long rows and too few slices to give every SM eight warps: a warp per row instead
   a.wide = !a.freeze && h->opt.variant == GABP_VARIANT_NODE && h->opt.accel == ACC_NONE && S.ns > 0 &&
