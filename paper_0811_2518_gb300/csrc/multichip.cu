@@ -110,7 +110,6 @@ struct TeamShared {
   float2 part[2][kTWarps];
   uint2 flag[2][kTWarps];
   double rr[kTWarps];
-  double tot[2];
   int job;
   unsigned long long bar[kTWarps][kStagesMax];  // one phase per chunk
   TeamArgs args;  // the launch's arguments, read from here in the solves
@@ -127,24 +126,62 @@ __device__ __forceinline__ TeamFlags team_flags(TeamShared &sh, int parity, unsi
   return TeamFlags{__reduce_max_sync(0xffffffffu, g.x), __reduce_or_sync(0xffffffffu, g.y)};
 }
 
-// The CTA's sums of two values, within a warp in FP32, over the warps in FP64 (a sum over a whole system
-// overflows FP32 long before its entries do).  One warp adds them, 16 lanes a value: in every warp the
-// FP64 unit would need four times as long as this and the second barrier.
-__device__ __forceinline__ double2 team_sums(TeamShared &sh, int parity, float va, float vb) {
-  static_assert(kTWarps == 16, "16 lanes a value");
+// A sum over the warps of their FP32 values (not negative), on the integer units: the 24-bit significands are
+// aligned to the largest value's, 32 bits below its last place kept, and added exactly: s 2^(e - 182).  A sum over a whole system
+// overflows FP32 long before its entries do, and FP64 additions would hold every warp's scheduler 64 cycles each
+// (in one warp, with a second barrier: 0.4 to 0.8 us a round of 10 to 45).
+struct TeamSum {
+  unsigned long long s;
+  int e;  // 255: a value is not finite
+};
+__device__ __forceinline__ TeamSum team_sum(float v) {
+  const unsigned u = __float_as_uint(v) & 0x7fffffffu;
+  const int em = max(1, (int)(__reduce_max_sync(0xffffffffu, u) >> 23)), eu = max(1, (int)(u >> 23));
+  const unsigned long long m = (u & 0x7fffffu) | (u >= 0x800000u ? 0x800000u : 0u);
+  const unsigned long long x = em - eu < 56 ? (m << 32) >> (em - eu) : 0ull;  // below 2^56
+  const unsigned lo = __reduce_add_sync(0xffffffffu, (unsigned)x & 0xfffffffu);
+  const unsigned hi = __reduce_add_sync(0xffffffffu, (unsigned)(x >> 28));
+  return TeamSum{lo + ((unsigned long long)hi << 28), em};
+}
+
+// A positive factor as m 2^e with the top bit of m set (m = 0: zero).
+struct TeamFactor {
+  unsigned long long m;
+  int e;
+};
+__device__ __forceinline__ TeamFactor team_factor(double f) {
+  if (!(f > 0.0)) return TeamFactor{0ull, 0};
+  int e;
+  const double r = frexp(f, &e);  // f = r 2^e, r in [1/2, 1)
+  return TeamFactor{(unsigned long long)(r * 0x1p53) << 11, e - 64};
+}
+// a <= f b, to 2^-62.
+__device__ __forceinline__ bool team_below(const TeamSum &a, const TeamFactor &f, const TeamSum &b) {
+  if (a.s == 0ull) return true;
+  if (b.s == 0ull || f.m == 0ull) return false;
+  const int la = __clzll((long long)a.s), lb = __clzll((long long)b.s);
+  const unsigned long long A = a.s << la;
+  unsigned long long P = __umul64hi(f.m, b.s << lb);  // f b = P 2^64 at b's exponent, less lb, and f's
+  int ep = 64 + f.e + b.e - lb;
+  if (!(P >> 63)) {
+    P <<= 1;
+    --ep;
+  }
+  const int ea = a.e - la;
+  return ea != ep ? ea < ep : A <= P;
+}
+
+// Posts this thread's squared update and iterate, passes the CTA's barrier, and decides: bit 0 a sum is not
+// finite, bit 1 the update is small against the iterate.
+__device__ __forceinline__ int team_stop(TeamShared &sh, int parity, float va, float vb, const TeamFactor &f) {
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   va = warp_sum(va);
   vb = warp_sum(vb);
   if (lane == 0) sh.part[parity][w] = make_float2(va, vb);
   __syncthreads();
-  if (w == 0) {
-    double s = (double)(lane < 16 ? sh.part[parity][lane].x : sh.part[parity][lane - 16].y);
-#pragma unroll
-    for (int o = 8; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if ((lane & 15) == 0) sh.tot[lane >> 4] = s;
-  }
-  __syncthreads();
-  return make_double2(sh.tot[0], sh.tot[1]);
+  const float2 p = lane < kTWarps ? sh.part[parity][lane] : make_float2(0.f, 0.f);
+  const TeamSum a = team_sum(p.x), b = team_sum(p.y);
+  return (a.e >= 255 || b.e >= 255 ? 1 : 0) | (team_below(a, f, b) ? 2 : 0);
 }
 
 __device__ __forceinline__ double team_sum64(TeamShared &sh, double v) {
@@ -283,7 +320,7 @@ __device__ __noinline__ unsigned team_solve(TeamShared &sh, unsigned char *smem,
     __syncwarp();  // every lane has read the stage before it is filled again
   };
 
-  auto mean_round = [&](int t, auto zero) {
+  auto mean_round = [&](int t, const TeamFactor &f, auto zero) {
     constexpr bool ZERO = decltype(zero)::value;
     float *__restrict__ Hc = ((t & 1) ? a.H1 : a.H0) + slot0;
     const float *hp = (t & 1) ? h0 : h1;
@@ -339,7 +376,7 @@ __device__ __noinline__ unsigned team_solve(TeamShared &sh, unsigned char *smem,
     }
     fence_bulk();  // the messages written here are fetched for round t + 2, from the next round on
     parity ^= 1;
-    return team_sums(sh, parity, dxx, xx);
+    return team_stop(sh, parity, dxx, xx, f);
   };
 
   bool run = true;
@@ -402,15 +439,15 @@ __device__ __noinline__ unsigned team_solve(TeamShared &sh, unsigned char *smem,
     if (!isfinite(rr)) { status = GABP_DIVERGED; break; }
     if (steps >= a.max_refine || inner >= a.max_iter) { status = GABP_NOT_CONVERGED; break; }
     const double itol = fmin(a.inner_tol, fmax(1e-6, 0.1 * a.tol * sqrt(bb / rr)));
-    const double it2 = itol * itol;
+    const TeamFactor it2 = team_factor(itol * itol);
     const int cap = min(a.inner_max, max(1, a.max_iter - inner));
     int t = 1;
     bool ok = true;
     pm = w; pc = 0; ft = 1;
     for (;; ++t) {
-      const double2 r = t <= 2 ? mean_round(t, std::true_type()) : mean_round(t, std::false_type());
-      if (!isfinite(r.x) || !isfinite(r.y)) { ok = false; break; }
-      if ((t >= 2 && r.x <= it2 * r.y) || t >= cap) break;
+      const int r = t <= 2 ? mean_round(t, it2, std::true_type()) : mean_round(t, it2, std::false_type());
+      if (r & 1) { ok = false; break; }
+      if ((t >= 2 && (r & 2)) || t >= cap) break;
     }
     while (out > 0) {  // chunks fetched for a round that does not come
       arrive();
