@@ -653,6 +653,7 @@ constexpr int kGridShapes[12] = {1 | (4 << 8), 2 | (4 << 8), 4 | (2 << 8), 4 | (
 gabp_status solve_systems_grid(gabp_handle h, int nsys, const int *d_off, const int *off_host, const double *b,
                                double *x, double tol, int max_iter, int *d_status, int *d_iters, int *d_refine,
                                double *d_relres, int shape, float *ms_out, int upto = -1);
+int grid_steps(gabp_handle h, long long ns);
 void free_gsell(gabp_handle h);
 gabp_status ensure_gsell(gabp_handle h, int nsys, const int *off, bool by_size);
 // multichip.cu

@@ -382,19 +382,22 @@ static gabp_status collect_systems(gabp_handle h, int nsys, const std::vector<in
                                    double *relres_host);
 
 // Systems, by descending size, before the first that the queue kernel takes (nsys: none, the kernels are timed).
-// A model of a round in us, fitted to graphs of degree 3 to 300 with and without one hub row a system (geometric ones up
-// to 30, banded above); S slots, P with the sliced layout's padding, w the widest slice.
-//   queue kernel, one system: 3 + 7.2e-4 a row + 2.75e-4 a slot of P (one SM's rate) + 0.085 a slot that w exceeds
-//     the mean row (the chunks of a hub row, one warp); the longest of them, their sum over the SMs, or HBM's 18
-//     bytes a slot of P and 20 a row, whichever is most;
-//   timed choice: 9 + 0.12 a slot of w (40 at most) + 5.6e-6 a slot of S + 2e-5 a row + 0.035 a slot that w exceeds
-//     the mean row + 1.34e-5 a slot of padding;
-//   grid kernel on the sliced layout beside the queue: 11 + 5.6e-6 S + 2e-5 a row + 0.22 a slot of w above 16.
-// Measured, queue / timed choice (degree, systems of rows): 3, 1 of 4096 9.0 / 9.2 and 152 of 16384 34 / 76; 6, 8 of
-// 2048 7.3 / 10.7 and 8 of 16384 42 / 18; 12, 60 of 8192 39 / 57; 30, 8 of 2048 20 / 16 and 152 of 1024 13 / 38; 100,
-// 8 of 2048 59 / 21 and 152 of 4096 191 / 292; 300, 8 of 2048 169 / 34; 6 and a hub of 500, 8 of 4096 56 / 36 and 152 of
-// 4096 61 / 109.  Not where a row is wider than kQueueWidth: a lane's FP32 sum over 2000 slots cost 152 systems 227
-// rounds for the 190 of the row kernels' 8 lanes (500 slots: 161 and 161).
+// A model of a round in us (kernels alone), fitted to graphs of degree 3 to 300 with and without one hub row a system
+// (geometric ones up to 30, banded above) and to batches of mixed sizes; S slots, P with the sliced layout's padding, w
+// the widest slice, m the mean row.
+//   queue kernel, one system: 0.7 + 8e-4 a row + 2.88e-4 a slot of P (one SM's rate) + 0.083 a slot that w exceeds m
+//     (the chunks of a hub row, one warp); the longest of them, their sum over the SMs, or HBM's 18 bytes a slot
+//     of P and 20 a row, whichever is most;
+//   timed choice: 5.1 + 0.18 a slot of m + 14 (40 at most) + 4.9e-6 a slot of S + 1.8e-5 a row + 0.038 a slot that w
+//     exceeds m + 20 + 1.95e-5 a slot of padding;
+//   grid kernel on the sliced layout beside the queue: 6.4 + 5.9e-6 S + 1.7 a slice of its busiest warp + 0.19 a slot
+//     of w above 16.
+// Measured, queue / timed choice (degree, systems of rows): 3, 1 of 4096 8.2 / 8.0 and 152 of 16384 32 / 73; 6, 8 of
+// 2048 6.6 / 9.7 and 8 of 16384 41 / 17; 12, 60 of 8192 37 / 54; 30, 8 of 2048 19 / 15 and 152 of 1024 12 / 36; 100,
+// 8 of 2048 57 / 19 and 152 of 4096 191 / 284; 300, 8 of 2048 169 / 29; 6 and a hub of 500, 8 of 4096 55 / 34 and 152 of
+// 4096 60 / 104.  512 systems of 1024 to 65536 rows, the grid kernel on the 23 / 31 / 39 / 63 largest: 89 / 85 / 84 / 89
+// (model 88 / 83 / 83 / 86).  Not where a row is wider than kQueueWidth: a lane's FP32 sum over 2000 slots cost 152
+// systems 227 rounds for the 190 of the row kernels' 8 lanes (500 slots: 161 and 161).
 constexpr int kQueueWidth = 512;
 static gabp_status queue_from(gabp_handle h, int nsys, const int *off, const std::vector<int> &rows,
                               const std::vector<int> &slots, int *from) {
@@ -417,32 +420,37 @@ static gabp_status queue_from(gabp_handle h, int nsys, const int *off, const std
     P += L.pad[s];
     wide = std::max(wide, L.wide[s]);
   }
-  double best = 9.0 + 0.12 * std::min(wide, 40) + 5.6e-6 * S + 2e-5 * R + 0.035 * std::max(0.0, wide - S / R) +
-                1.34e-5 * (P - S);
+  const double timed = 5.1 + 0.18 * std::min(S / R + 14.0, 40.0) + 4.9e-6 * S + 1.8e-5 * R +
+                       0.038 * std::max(0.0, wide - S / R - 20.0) + 1.95e-5 * (P - S);
+  double best = timed;
   std::vector<double> gridt(nsys + 1, 0.0);
-  double gS = 0.0, gR = 0.0;
+  double gS = 0.0;
+  long long gns = 0;
   int gw = 0;
   for (int q = 0; q < nsys; ++q) {
     const int s = L.order[q];
     gS += slots[s];
-    gR += rows[s];
+    gns += (rows[s] + 31) / 32;
     gw = std::max(gw, L.wide[s]);
-    gridt[q + 1] = 11.0 + 5.6e-6 * gS + 2e-5 * gR + 0.22 * std::max(0, gw - 16);
+    gridt[q + 1] = 6.4 + 5.9e-6 * gS + 1.7 * grid_steps(h, gns) + 0.19 * std::max(0, gw - 16);
   }
   double top = 0.0, sum = 0.0, bytes = 0.0;
   for (int q = nsys - 1; q >= 0; --q) {
     const int s = L.order[q];
     if (rows[s] > most || L.wide[s] > kQueueWidth) break;
-    const double t = 3.0 + 7.2e-4 * rows[s] + 2.75e-4 * L.pad[s] +
-                     0.085 * std::max(0.0, L.wide[s] - (double)slots[s] / rows[s]);
+    const double t = 0.7 + 8e-4 * rows[s] + 2.88e-4 * L.pad[s] +
+                     0.083 * std::max(0.0, L.wide[s] - (double)slots[s] / rows[s]);
     top = std::max(top, t);
     sum += t;
     bytes += 18.0 * L.pad[s] + 20.0 * rows[s];
     // a launch of the grid kernel takes all systems of a size
     if (q > 0 && rows[L.order[q - 1]] == rows[s]) continue;
     const double all = gridt[q] + std::max(std::max(top, sum / h->num_sms), bytes / 5.8e6);
-    if (all * (q > 0 ? 1.05 : 1.0) < best) {  // two launches for a gain that the model can tell
-      best = all;
+    // two launches (0.3 ms a call, some 180 rounds) for a gain that the model can tell; the queue alone, which needs
+    // no timing, where it ties
+    const double cost = q > 0 ? 1.05 * (all + 1.6) : all;
+    if (cost < (q == 0 && *from == nsys ? 1.08 * timed : best)) {
+      best = cost;
       *from = q;
     }
   }

@@ -106,10 +106,17 @@ struct TeamFlags {
   unsigned m, f;
 };
 
+// A positive factor as m 2^e with the top bit of m set (m = 0: zero).
+struct TeamFactor {
+  unsigned long long m;
+  int e;
+};
+
 struct TeamShared {
   float2 part[2][kTWarps];
   uint2 flag[2][kTWarps];
   double rr[kTWarps];
+  TeamFactor tol2;  // the inner solve's squared tolerance
   int job;
   unsigned long long bar[kTWarps][kStagesMax];  // one phase per chunk
   TeamArgs args;  // the launch's arguments, read from here in the solves
@@ -127,9 +134,9 @@ __device__ __forceinline__ TeamFlags team_flags(TeamShared &sh, int parity, unsi
 }
 
 // A sum over the warps of their FP32 values (not negative), on the integer units: the 24-bit significands are
-// aligned to the largest value's, 32 bits below its last place kept, and added exactly: s 2^(e - 182).  A sum over a whole system
-// overflows FP32 long before its entries do, and FP64 additions would hold every warp's scheduler 64 cycles each
-// (in one warp, with a second barrier: 0.4 to 0.8 us a round of 10 to 45).
+// aligned to the largest value's, 32 bits below its last place kept, and added exactly: s 2^(e - 182).  A sum
+// over a whole system overflows FP32 long before its entries do, and FP64 additions hold a scheduler 64 cycles
+// each (one warp's, with a second barrier: 0.4 to 0.8 us a round of 10 to 45).
 struct TeamSum {
   unsigned long long s;
   int e;  // 255: a value is not finite
@@ -144,11 +151,7 @@ __device__ __forceinline__ TeamSum team_sum(float v) {
   return TeamSum{lo + ((unsigned long long)hi << 28), em};
 }
 
-// A positive factor as m 2^e with the top bit of m set (m = 0: zero).
-struct TeamFactor {
-  unsigned long long m;
-  int e;
-};
+// f as a factor.
 __device__ __forceinline__ TeamFactor team_factor(double f) {
   if (!(f > 0.0)) return TeamFactor{0ull, 0};
   int e;
@@ -171,17 +174,26 @@ __device__ __forceinline__ bool team_below(const TeamSum &a, const TeamFactor &f
   return ea != ep ? ea < ep : A <= P;
 }
 
+// The decision from all warps' sums p; out of line, to leave the rounds their registers.
+__device__ __noinline__ int team_decide(float2 p, const TeamFactor &f) {
+  const TeamSum a = team_sum(p.x), b = team_sum(p.y);
+  return (a.e >= 255 || b.e >= 255 ? 1 : 0) | (team_below(a, f, b) ? 2 : 0);
+}
+
 // Posts this thread's squared update and iterate, passes the CTA's barrier, and decides: bit 0 a sum is not
-// finite, bit 1 the update is small against the iterate.
-__device__ __forceinline__ int team_stop(TeamShared &sh, int parity, float va, float vb, const TeamFactor &f) {
+// finite, bit 1 the update is small against the iterate.  Most rounds are far from that, which FP32 sums of the 16
+// values tell (16 2^-24 off; the bound is 2^-16 wide, and values near FP32's smallest go the exact way).
+// The tolerance is sh.tol2; above: an FP32 value 2^-16 above it.
+__device__ __forceinline__ int team_stop(TeamShared &sh, int parity, float va, float vb, float above) {
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   va = warp_sum(va);
   vb = warp_sum(vb);
   if (lane == 0) sh.part[parity][w] = make_float2(va, vb);
   __syncthreads();
   const float2 p = lane < kTWarps ? sh.part[parity][lane] : make_float2(0.f, 0.f);
-  const TeamSum a = team_sum(p.x), b = team_sum(p.y);
-  return (a.e >= 255 || b.e >= 255 ? 1 : 0) | (team_below(a, f, b) ? 2 : 0);
+  const float fa = warp_sum(p.x), fb = warp_sum(p.y);
+  if (isfinite(fa) && isfinite(fb) && fa > 0x1p-100f && fa > above * fb) return 0;
+  return team_decide(p, sh.tol2);
 }
 
 __device__ __forceinline__ double team_sum64(TeamShared &sh, double v) {
@@ -320,7 +332,7 @@ __device__ __noinline__ unsigned team_solve(TeamShared &sh, unsigned char *smem,
     __syncwarp();  // every lane has read the stage before it is filled again
   };
 
-  auto mean_round = [&](int t, const TeamFactor &f, auto zero) {
+  auto mean_round = [&](int t, float above, auto zero) {
     constexpr bool ZERO = decltype(zero)::value;
     float *__restrict__ Hc = ((t & 1) ? a.H1 : a.H0) + slot0;
     const float *hp = (t & 1) ? h0 : h1;
@@ -376,7 +388,7 @@ __device__ __noinline__ unsigned team_solve(TeamShared &sh, unsigned char *smem,
     }
     fence_bulk();  // the messages written here are fetched for round t + 2, from the next round on
     parity ^= 1;
-    return team_stop(sh, parity, dxx, xx, f);
+    return team_stop(sh, parity, dxx, xx, above);
   };
 
   bool run = true;
@@ -439,7 +451,8 @@ __device__ __noinline__ unsigned team_solve(TeamShared &sh, unsigned char *smem,
     if (!isfinite(rr)) { status = GABP_DIVERGED; break; }
     if (steps >= a.max_refine || inner >= a.max_iter) { status = GABP_NOT_CONVERGED; break; }
     const double itol = fmin(a.inner_tol, fmax(1e-6, 0.1 * a.tol * sqrt(bb / rr)));
-    const TeamFactor it2 = team_factor(itol * itol);
+    const float it2 = fmaxf((float)(itol * itol), 0x1p-126f) * (1.f + 0x1p-16f);  // and a little above it
+    if (threadIdx.x == 0) sh.tol2 = team_factor(itol * itol);
     const int cap = min(a.inner_max, max(1, a.max_iter - inner));
     int t = 1;
     bool ok = true;

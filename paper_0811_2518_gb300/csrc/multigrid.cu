@@ -765,6 +765,19 @@ gabp_status ensure_gsell(gabp_handle h, int nsys, const int *off, bool by_size) 
   return GABP_OK;
 }
 
+// Warp steps per chunk: about four chunks per warp or more, so that the round's slowest warp has little more
+// work than the average one; longer chunks (fewer accumulator flushes) when the steps allow.
+static int grid_chunk(long long steps, long long warps) {
+  return (int)std::max(1LL, std::min<long long>(kGChunkMax, (steps + warps - 1) / warps / 4));
+}
+
+// Slices that the round's busiest warp runs, of ns slices on the shape that runs beside the queue kernel.
+int grid_steps(gabp_handle h, long long ns) {
+  const long long warps = (long long)resident_grid(h->num_sms, grid_kernel(kSliced | 1 | (4 << 8))) * (kBlock / 32);
+  const int chunk = grid_chunk(ns, warps);
+  return (int)(((ns + chunk - 1) / chunk + warps - 1) / warps * chunk);
+}
+
 gabp_status solve_systems_grid(gabp_handle h, int nsys, const int *d_off, const int *off_host, const double *b,
                                double *x, double tol, int max_iter, int *d_status, int *d_iters, int *d_refine,
                                double *d_relres, int shape, float *ms_out, int upto) {
@@ -832,21 +845,9 @@ gabp_status solve_systems_grid(gabp_handle h, int nsys, const int *d_off, const 
                           (long long)h->opt.max_refine * (std::min(h->opt.inner_max_iter, std::max(1, max_iter)) + 2) + 1;
   a.max_rounds = (int)std::min<long long>(bound, 0x7fffffff);
   void (*kern)(GridArgs) = grid_kernel(shape);
-  int per_sm = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kBlock, 0) != cudaSuccess || per_sm < 1) {
-    cudaGetLastError();
-    per_sm = 1;
-  }
-  const int grid = per_sm * h->num_sms;
-  {
-    // about four chunks per warp or more, so that the round's slowest warp has little more work
-    // than the average one; longer chunks (fewer accumulator flushes) when the rows allow
-    const int lanes = shape & 0xff;
-    const long long warps = (long long)grid * (kBlock / 32);
-    const long long steps_per_warp = sliced ? ((long long)a.ns + warps - 1) / warps
-                                            : ((long long)g.n * lanes + 32LL * warps - 1) / (32LL * warps);
-    a.chunk = (int)std::max(1LL, std::min<long long>(kGChunkMax, steps_per_warp / 4));
-  }
+  const int grid = resident_grid(h->num_sms, kern);
+  const long long warps = (long long)grid * (kBlock / 32);
+  a.chunk = grid_chunk(sliced ? a.ns : ((long long)g.n * (shape & 0xff) + 31) / 32, warps);
   cudaEvent_t e0, e1;
   GABP_CUDA(cudaEventCreate(&e0));
   GABP_CUDA(cudaEventCreate(&e1));
