@@ -282,7 +282,6 @@ struct GSell {
   int Es = 0;                  // slots, padding included
   bool by_size = false;
   std::vector<int> order;      // the systems in the layout's order: as given, or by descending size (stable)
-  std::vector<int> pad, wide;  // slots of each system, padding included, and its widest slice
   bool vals_ok = false;
   int *srow = nullptr;         // [32 ns] row of each slice lane, -1 for padding
   int *sp = nullptr;           // [ns + 1] first slot of each slice (multiples of 32)

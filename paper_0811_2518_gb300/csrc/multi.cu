@@ -17,7 +17,7 @@
 // precision phase to a 2^-20 stationary point, inner solves to
 // ||dx|| <= inner_tol ||x||, outer loop to ||b_s - A_s x_s|| <= tol ||b_s||.
 #include "gabp_internal.cuh"
-#include "devutil.cuh"
+#include "sell64.cuh"
 
 #include <cooperative_groups.h>
 
@@ -381,6 +381,30 @@ static gabp_status collect_systems(gabp_handle h, int nsys, const std::vector<in
                                    const double *d_rel, float ms, int *status_host, int *iters_host,
                                    double *relres_host);
 
+// Slots of rows [b, e) on the sliced layout (degree-sorted windows of kSellWindow rows, 32 rows a slice), padding
+// included, and the widest slice.  Windows of rows up to 64 slots: to half the most that sorted rows can waste.
+static double slice_widths(const std::vector<int> &rp, int b, int e, int *wide) {
+  std::vector<int> count;
+  double pad = 0.0;
+  *wide = 0;
+  for (int w0 = b; w0 < e; w0 += kSellWindow) {
+    const int w1 = std::min(e, w0 + kSellWindow);
+    int hi = 0;
+    for (int r = w0; r < w1; ++r) hi = std::max(hi, rp[r + 1] - rp[r]);
+    *wide = std::max(*wide, hi);
+    if (hi <= 64) {
+      pad += rp[w1] - rp[w0] + 16.0 * hi;
+      continue;
+    }
+    count.assign((size_t)hi + 1, 0);
+    for (int r = w0; r < w1; ++r) ++count[rp[r + 1] - rp[r]];
+    int seen = 0, first = 0;  // rows of larger degree, the next slice's first row
+    for (int d = hi; d >= 0; --d)
+      for (seen += count[d]; first < seen; first += 32) pad += 32.0 * d;
+  }
+  return pad;
+}
+
 // Systems, by descending size, before the first that the queue kernel takes (nsys: none, the kernels are timed).
 // A model of a round in us (kernels alone), fitted to graphs of degree 3 to 300 with and without one hub row a system
 // (geometric ones up to 30, banded above) and to batches of mixed sizes; S slots, P with the sliced layout's padding, w
@@ -388,7 +412,7 @@ static gabp_status collect_systems(gabp_handle h, int nsys, const std::vector<in
 //   queue kernel, one system: 0.7 + 8e-4 a row + 2.88e-4 a slot of P (one SM's rate) + 0.083 a slot that w exceeds m
 //     (the chunks of a hub row, one warp); the longest of them, their sum over the SMs, or HBM's 18 bytes a slot
 //     of P and 20 a row, whichever is most;
-//   timed choice: 5.1 + 0.18 a slot of m + 14 (40 at most) + 4.9e-6 a slot of S + 1.8e-5 a row + 0.038 a slot that w
+//   timed choice: 5.1 (and 0.5 of host work more) + 0.18 a slot of m + 14 (40 at most) + 4.9e-6 a slot of S + 1.8e-5 a row + 0.038 a slot that w
 //     exceeds m + 20 + 1.95e-5 a slot of padding;
 //   grid kernel on the sliced layout beside the queue: 6.4 + 5.9e-6 S + 1.7 a slice of its busiest warp + 0.19 a slot
 //     of w above 16.
@@ -399,28 +423,29 @@ static gabp_status collect_systems(gabp_handle h, int nsys, const std::vector<in
 // (model 88 / 83 / 83 / 86).  Not where a row is wider than kQueueWidth: a lane's FP32 sum over 2000 slots cost 152
 // systems 227 rounds for the 190 of the row kernels' 8 lanes (500 slots: 161 and 161).
 constexpr int kQueueWidth = 512;
-static gabp_status queue_from(gabp_handle h, int nsys, const int *off, const std::vector<int> &rows,
-                              const std::vector<int> &slots, int *from) {
-  if ((int)h->multi_off.size() == nsys + 1 && std::equal(h->multi_off.begin(), h->multi_off.end(), off)) {
-    *from = h->multi_from;
-    return GABP_OK;
-  }
+static int queue_from(gabp_handle h, int nsys, const int *off, const std::vector<int> &rp, const std::vector<int> &rows,
+                      const std::vector<int> &slots) {
+  if ((int)h->multi_off.size() == nsys + 1 && std::equal(h->multi_off.begin(), h->multi_off.end(), off))
+    return h->multi_from;
   const int most = team_rows(h);
-  *from = nsys;
-  if (*std::min_element(rows.begin(), rows.end()) > most) return GABP_OK;
-  gabp_status st = ensure_gsell(h, nsys, off, true);
-  if (st != GABP_OK) return st;
-  const GSell &L = *h->gsl;
+  int from = nsys;
+  std::vector<int> order(nsys), wide_of(nsys);
+  std::vector<double> pad(nsys);
+  for (int s = 0; s < nsys; ++s) {
+    order[s] = s;
+    pad[s] = slice_widths(rp, off[s], off[s + 1], &wide_of[s]);
+  }
+  std::stable_sort(order.begin(), order.end(), [&](int p, int q) { return rows[p] > rows[q]; });
   // of the systems order[0 .. q): slots, rows and widest slice; of order[q ..): what the queue's three bounds add up
   double S = 0.0, R = 0.0, P = 0.0;
   int wide = 0;
   for (int s = 0; s < nsys; ++s) {
     S += slots[s];
     R += rows[s];
-    P += L.pad[s];
-    wide = std::max(wide, L.wide[s]);
+    P += pad[s];
+    wide = std::max(wide, wide_of[s]);
   }
-  const double timed = 5.1 + 0.18 * std::min(S / R + 14.0, 40.0) + 4.9e-6 * S + 1.8e-5 * R +
+  const double timed = 5.6 + 0.18 * std::min(S / R + 14.0, 40.0) + 4.9e-6 * S + 1.8e-5 * R +
                        0.038 * std::max(0.0, wide - S / R - 20.0) + 1.95e-5 * (P - S);
   double best = timed;
   std::vector<double> gridt(nsys + 1, 0.0);
@@ -428,35 +453,35 @@ static gabp_status queue_from(gabp_handle h, int nsys, const int *off, const std
   long long gns = 0;
   int gw = 0;
   for (int q = 0; q < nsys; ++q) {
-    const int s = L.order[q];
+    const int s = order[q];
     gS += slots[s];
     gns += (rows[s] + 31) / 32;
-    gw = std::max(gw, L.wide[s]);
+    gw = std::max(gw, wide_of[s]);
     gridt[q + 1] = 6.4 + 5.9e-6 * gS + 1.7 * grid_steps(h, gns) + 0.19 * std::max(0, gw - 16);
   }
   double top = 0.0, sum = 0.0, bytes = 0.0;
   for (int q = nsys - 1; q >= 0; --q) {
-    const int s = L.order[q];
-    if (rows[s] > most || L.wide[s] > kQueueWidth) break;
-    const double t = 0.7 + 8e-4 * rows[s] + 2.88e-4 * L.pad[s] +
-                     0.083 * std::max(0.0, L.wide[s] - (double)slots[s] / rows[s]);
+    const int s = order[q];
+    if (rows[s] > most || wide_of[s] > kQueueWidth) break;
+    const double t = 0.7 + 8e-4 * rows[s] + 2.88e-4 * pad[s] +
+                     0.083 * std::max(0.0, wide_of[s] - (double)slots[s] / rows[s]);
     top = std::max(top, t);
     sum += t;
-    bytes += 18.0 * L.pad[s] + 20.0 * rows[s];
+    bytes += 18.0 * pad[s] + 20.0 * rows[s];
     // a launch of the grid kernel takes all systems of a size
-    if (q > 0 && rows[L.order[q - 1]] == rows[s]) continue;
+    if (q > 0 && rows[order[q - 1]] == rows[s]) continue;
     const double all = gridt[q] + std::max(std::max(top, sum / h->num_sms), bytes / 5.8e6);
-    // two launches (0.3 ms a call, some 180 rounds) for a gain that the model can tell; the queue alone, which needs
-    // no timing, where it ties
+    // two launches (0.3 ms a call, some 180 rounds) for a gain that the model can tell; the queue alone where it
+    // ties with the timed choice, whose first call takes some thirty times as long
     const double cost = q > 0 ? 1.05 * (all + 1.6) : all;
-    if (cost < (q == 0 && *from == nsys ? 1.08 * timed : best)) {
+    if (cost < (q == 0 && from == nsys ? 1.08 * timed : best)) {
       best = cost;
-      *from = q;
+      from = q;
     }
   }
   h->multi_off.assign(off, off + nsys + 1);
-  h->multi_from = *from;
-  return GABP_OK;
+  h->multi_from = from;
+  return from;
 }
 
 gabp_status solve_systems(gabp_handle h, int nsys, const int *offsets_host, const double *b, double *x, double tol,
@@ -598,8 +623,7 @@ gabp_status solve_systems(gabp_handle h, int nsys, const int *offsets_host, cons
   // no system for the queue.
   h->multi_queue = false;
   if (h->opt.multi_split == 0 && h->opt.multi_mode == 0 && h->opt.lanes == 0) {
-    int from = nsys;
-    if ((st = queue_from(h, nsys, offsets_host, rows, slots, &from)) != GABP_OK) return st;
+    const int from = queue_from(h, nsys, offsets_host, rp_h, rows, slots);
     if (from < nsys) {
       float ms2 = 0.f;
       if (from > 0 && (st = solve_systems_grid(h, nsys, d_off, offsets_host, b, x, tol, max_iter, d_res, d_res + nsys,

@@ -705,8 +705,6 @@ gabp_status ensure_gsell(gabp_handle h, int nsys, const int *off, bool by_size) 
     L->order.resize(nsys);
     for (int s = 0; s < nsys; ++s) L->order[s] = s;
     L->by_size = by_size;
-    L->pad.assign(nsys, 0);
-    L->wide.assign(nsys, 0);
     if (by_size)
       std::stable_sort(L->order.begin(), L->order.end(),
                        [&](int p, int q) { return off[p + 1] - off[p] > off[q + 1] - off[q]; });
@@ -723,8 +721,6 @@ gabp_status ensure_gsell(gabp_handle h, int nsys, const int *off, bool by_size) 
           if (r >= 0) wd = std::max(wd, rp[r + 1] - rp[r]);
         }
         slots += 32LL * wd;
-        L->pad[s] += 32 * wd;
-        L->wide[s] = std::max(L->wide[s], wd);
         if (slots > 0x7fffffffLL) {
           set_last_error("gabp_solve_systems: the sliced layout would exceed 2^31 slots");
           free_gsell(h);
