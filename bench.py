@@ -543,10 +543,10 @@ def main():
             alg_b = Eg * (8 * Rb + 8) + 8 * Rb * ng
             # DRAM bytes from a capture of the 64^3 case (a few GB on the device; the 128^3 x 64 workload is
             # too large to capture under ncu), scaled to this sweep by the implementation's bytes
-            traffic_b = _profiled_traffic("kbs_pass_grid3d_64_64rhs.md", "paper_0811_2518_gb300/csrc/batched.cu",
+            traffic_b = _profiled_traffic("kbs2_pass_grid3d_64_64rhs.md", "paper_0811_2518_gb300/csrc/batched.cu",
                                           "kbs2_pass", scale_to=bytes_b)
-            traffic_note_b = ("DRAM bytes per sweep, scaled from one captured pass of the 64^3 case (the two "
-                              "red-black passes move equal bytes) by the implementation's bytes")
+            traffic_note_b = ("DRAM bytes per sweep, scaled from both captured passes of a sweep of the 64^3 "
+                              "case by the implementation's bytes")
             batched = {"workload": f"{args.batched_grid}^3 7-point grid, face coefficients LogNormal(0,1), diagonal 1.05 x "
                                    "row abs-sum, 64 right-hand sides N(0,1)", "n": ng, "edges": Eg, "rhs": Rb,
                        "schedule": f"serial (one message store, {ncol} colours: red-black on this grid)",

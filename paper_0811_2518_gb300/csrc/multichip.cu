@@ -9,10 +9,10 @@
 // fetches the chunks of its slices by bulk copies into its part of a ring, several ahead (one SM's share of
 // the HBM rate times the copies' ~1.8 us of latency is 80 KB in flight), into the next round too: what
 // that round streams was written a round ago.
-// Bound by HBM when every SM has a system (152 graphs of 16384 rows and degree 6: 50 us a round, 6.2 TB/s of
-// slots and row vectors; the grid-persistent kernel 113), by one SM's rate of 2.4 ns a row and round when
+// Bound by HBM when every SM has a system (152 graphs of 16384 rows and degree 6: 54 us a round, 5.9 TB/s of
+// slots and row vectors; the grid-persistent kernel 138), by one SM's rate of 2.4 ns a row of degree 6 and round when
 // few have.  Systems above kTRowsMost rows go to the grid-persistent kernel.  512 geometric graphs of 1024
-// to 65536 rows to 1e-10: 22.0 -> 16.5 ms, half of it for the 17 largest on the grid-persistent kernel.
+// to 65536 rows to 1e-10: 22.0 -> 16.0 ms, 9 of it for the 38 largest on the grid-persistent kernel.
 //
 // Rows are addressed by position (slice, lane) of the sliced layout within their system, so own rows'
 // accesses are contiguous; padding slots hold zero coefficients, padding rows a unit precision and a zero
