@@ -149,11 +149,17 @@ __device__ bool col_reduce(const double (&acc)[NV][VEC], int RP, double *red, do
 #endif
 template <int VEC>
 constexpr int kBU = VEC == 4 ? 2 : GABP_KB_U;
-// Graphs of few rows leave an SM a few warps, each waiting for its loads: more slots of a row together.  (With 2, the
-// rounds that read the reverse messages through rev cost such graphs more than the store they save: 200 rows of 40
-// slots, 16 columns 2.51 ms with four messages a pair of rounds, 2.71 with three, 2.37 with three and 8 slots; 1,000 rows
-// of 100 4.53, 4.68, 3.51; 2,000 rows of 100 6.3, 6.4.  With 64 columns, two a lane, 2 slots are enough.)
-constexpr int kBUFew = 8, kBFewRowsSm = 8;
+// Rounds that last as long as their longest row, one warp waiting for its loads (few rows, or a hub among many), take more
+// slots of a row together.  With 2, the rounds that read the reverse messages through rev cost such graphs more than
+// the store they save; whole solves in ms with four messages a pair of rounds / with three / with three and 8 slots, 16
+// columns: 200 rows of 40 slots 2.51 / 2.71 / 2.37, 1,000 rows of 100 4.55 / 4.31 / 3.24, 60,000 rows of
+// 6 with a hub of 1,000 45.8 / 47.0 / 25.1, 100,000 rows of a heavy tail 168 / 182 / 86.
+constexpr int kBULong = 8;
+// A slot of the longest row takes 0.35 us of a round with 2 slots at a time; the round's bytes as below.
+static bool long_row_round(const Graph &g, int max_deg, int RP) {
+  const double bytes = (double)g.E * (6.0 * RP + 14.0) + (double)g.n * (16.0 * RP + 8.0);
+  return 0.35 * max_deg > bytes / 6.8e6;
+}
 
 // Rounds by what their reverse messages come from: none in round 1 (zero messages), the row's own
 // aggregate in round 2 (its stored messages are the zero ones, not read), then as above.
@@ -670,6 +676,13 @@ __global__ void kbs_ctl_reset(DevCtl *c, int max_iter, double tol2, double *col,
   for (int r = 2 * RP; r < 5 * RP; ++r) col[r] = 0.0;  // sweep sums and previous steps
 }
 
+__global__ void __launch_bounds__(kBlock) kb_max_degree(int n, const int *__restrict__ rp, unsigned *most) {
+  unsigned d = 0;
+  for (int i = blockIdx.x * kBlock + threadIdx.x; i < n; i += gridDim.x * kBlock) d = max(d, (unsigned)(rp[i + 1] - rp[i]));
+  d = __reduce_max_sync(0xffffffffu, d);
+  if ((threadIdx.x & 31) == 0) atomicMax(most, d);
+}
+
 __global__ void kb_ctl_reset(DevCtl *c, int max_iter, double tol2) {
   c->round = 0;
   c->done = 0;
@@ -688,6 +701,7 @@ __global__ void kb_ctl_reset(DevCtl *c, int max_iter, double tol2) {
 
 struct WorkB {
   int RP = 0;
+  int max_deg = 0;  // longest row
   float *H = nullptr;
   float *NH[3] = {nullptr, nullptr, nullptr};
   float *rhs = nullptr;
@@ -728,6 +742,11 @@ static gabp_status ensure_wb(gabp_handle h, int RP) {
   GABP_CUDA(cudaMalloc(&w->col, sizeof(double) * 5 * RP));
   GABP_CUDA(cudaMalloc(&w->arrive, sizeof(unsigned int)));
   GABP_CUDA(cudaMemsetAsync(w->arrive, 0, sizeof(unsigned int), h->stream));
+  kb_max_degree<<<blocks_for(h->g.n, kBlock, h->max_blocks), kBlock, 0, h->stream>>>(h->g.n, h->g.rp, w->arrive);
+  GABP_CUDA(cudaGetLastError());
+  GABP_CUDA(cudaMemcpyAsync(&w->max_deg, w->arrive, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
+  GABP_CUDA(cudaMemsetAsync(w->arrive, 0, sizeof(unsigned int), h->stream));
+  GABP_CUDA(cudaStreamSynchronize(h->stream));
   w->RP = RP;
   return GABP_OK;
 }
@@ -753,7 +772,7 @@ static gabp_status batched_chunk(gabp_handle h, int R, const double *B, double *
     return blocks_for(g.n, kBlock / 32, nb * h->num_sms);
   };
   void (*const mean)(ArgsB) =
-      VEC == 1 && g.n <= kBFewRowsSm * h->num_sms ? kb_mean<VEC, VEC == 1 ? kBUFew : kBU<VEC>> : kb_mean<VEC, kBU<VEC>>;
+      VEC < 4 && long_row_round(g, w.max_deg, RP) ? kb_mean<VEC, VEC < 4 ? kBULong : kBU<VEC>> : kb_mean<VEC, kBU<VEC>>;
   const int nb_mean = grid_of(mean);
   const int nb_res = grid_of(kb_residual<VEC>);
   dim3 tb(32, 8), tg((g.n + 31) / 32, RP / 32);

@@ -66,11 +66,11 @@ def test_batched_rounds_reach_the_dense_solution(gb, kind, schedule, R, cap):
     s.close()
 
 
-@pytest.mark.parametrize("R", [1, 32])
+@pytest.mark.parametrize("R", [1, 32, 40])
 @pytest.mark.parametrize("kind", ["tree", "random", "dense rows"])
 def test_few_rows_and_many_rows_give_the_same_bits(gb, kind, R):
-    """A graph alone (few rows: eight slots of a row together) and in eight copies (two slots) after equal rounds:
-    rows of none to 29 slots, every remainder."""
+    """A graph alone (rounds as long as their longest row: eight slots of a row together) and in 250 copies (rounds
+    bound by their bytes: two slots) after equal rounds: rows of none to 29 slots, every remainder."""
     if kind == "dense rows":
         n = 203
         A = np.triu(np.random.default_rng(2).uniform(-1, 1, (n, n)), 1)
@@ -84,7 +84,7 @@ def test_few_rows_and_many_rows_give_the_same_bits(gb, kind, R):
     n = m.n
     B = np.random.default_rng(R).standard_normal((R, n))
     out = []
-    for copies in (1, 8):
+    for copies in (1, 250):
         big = synth.block_diag([m] * copies)
         s = gb.Solver.from_csr(big, lanes=4, inner_max_iter=9, inner_tol=1e-30, max_refine=2)
         X = s.solve_batched(torch.from_numpy(np.tile(B, (1, copies))).cuda(), tol=0.0, max_iter=1000, check=False)[0]
