@@ -156,10 +156,11 @@ def test_no_room_for_the_two_colour_layout(gb):
     torch.cuda.synchronize()
     torch.cuda.empty_cache()
     keep = torch.empty(torch.cuda.mem_get_info()[0] - (250 << 20), dtype=torch.uint8, device="cuda")
-    out = torch.empty_like(b)
-    x, st, it, _ = s.solve(b, tol=1e-10, max_iter=500, x=out)
-    del keep
-    torch.cuda.empty_cache()
+    try:
+        x, st, it, _ = s.solve(b, tol=1e-10, max_iter=500, x=torch.empty_like(b))
+    finally:
+        del keep
+        torch.cuda.empty_cache()
     assert st == gb.GABP_OK and it == sweeps
     assert torch.allclose(x, ref, rtol=0, atol=1e-10 * float(ref.abs().max()))
     s.close()
